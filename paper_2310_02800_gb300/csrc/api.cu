@@ -125,6 +125,8 @@ tm_status build_plan(const tm_graph* g, const tm_motif* m, Plan* out) {
     p.elabel0 = m->elabel[0];
     p.nl_x0 = m->nlabel[m->esrc[0]];
     p.nl_y0 = m->nlabel[m->edst[0]];
+    p.lv[0].elabel = p.lv[0].nl0 = p.lv[0].nl1 = -1;   // level 0 carries its labels above
+    p.lv[0].gap = INT64_MAX;
     int slot[TM_MAX_NODES], bound_at[TM_MAX_NODES];
     for (int j = 0; j < TM_MAX_NODES; ++j) slot[j] = bound_at[j] = -1;
     slot[m->esrc[0]] = 0;
@@ -144,7 +146,7 @@ tm_status build_plan(const tm_graph* g, const tm_motif* m, Plan* out) {
         if (anti_level[a] == 0) p.anti_mask0 |= (uint8_t)(1u << a);
     }
     int nb = 2;
-    int off_c = 0, off_f = 0;
+    int off_c = ROOT_BUF_BYTES, off_f = ROOT_BUF_BYTES;
     for (int i = 1; i < k; ++i) {
         LevelPlan& lp = p.lv[i];
         const int x = m->esrc[i], y = m->edst[i];
@@ -211,10 +213,24 @@ tm_status build_plan(const tm_graph* g, const tm_motif* m, Plan* out) {
         L.look_v[L.n_look] = (int8_t)slot[y];
         L.n_look++;
     }
-    p.warp_smem = std::max(16, (off_c + 15) & ~15);
-    p.warp_smem_fill = std::max(16, (off_f + 15) & ~15);
+    for (int i = 0; i < k; ++i) p.lv[i].hot = Hot::pack(p.lv[i]);
+    p.warp_smem = (off_c + 15) & ~15;
+    p.warp_smem_fill = (off_f + 15) & ~15;
+    // lists of the root's two nodes that some later edge is drawn from or closes
+    // into: each needs an entry in (t_root, t_root + delta], else the root has no match
+    auto word_span = [](int64_t d) { return (uint32_t)std::min<int64_t>(d, (int64_t)SUCC_FAR); };
+    p.root_span = word_span(m->delta);
+    p.root_span_next = k > 1 ? word_span(std::min(m->delta, m->gap[0])) : p.root_span;
+    for (int j = 1; j < k; ++j) {
+        const int sh = j == 1 ? 4 : 0;
+        if (m->esrc[j] == m->esrc[0]) p.root_need |= (uint8_t)(1u << (NX_OUT_SRC + sh));
+        if (m->esrc[j] == m->edst[0]) p.root_need |= (uint8_t)(1u << (NX_OUT_DST + sh));
+        if (m->edst[j] == m->edst[0]) p.root_need |= (uint8_t)(1u << (NX_IN_DST + sh));
+        if (m->edst[j] == m->esrc[0]) p.root_need |= (uint8_t)(1u << (NX_IN_SRC + sh));
+    }
     p.tune.warps_per_block = 4;
     p.tune.chunk_roots = 64;
+    p.auto_chunk = 1;
     // stars of 5+ edges on a hub grow subtrees of C(window, k-1) matches:
     // smaller root chunks spread the hubs' roots over more warps (the tuner
     // picked 32 for every such shape on the power-law workload)
@@ -341,7 +357,10 @@ static void apply_cached_tuning(tm_graph* g, tm_query* q) {
     while (d > 0) { key.dbucket++; d >>= 1; }
     std::lock_guard<std::mutex> lk(g->tune_mu);
     auto it = g->tuned.find(key);
-    if (it != g->tuned.end()) q->plan.tune = it->second;
+    if (it != g->tuned.end()) {
+        q->plan.tune = it->second;
+        q->plan.auto_chunk = 0;
+    }
 }
 
 const tm_graph* query_graph(const tm_query* q) { return q->g; }
@@ -355,9 +374,9 @@ void query_plan(tm_query* q, Plan* out) {
 // Stage and run one single-query count (optionally with per-root, per-chunk
 // or work outputs).  Leaves results in scratch counters; does not sync.
 static tm_status run_count(tm_graph* g, tm_query* q, uint64_t rb, uint64_t re, cudaStream_t st,
-                           unsigned long long* per_root, bool chunk_counts, bool work, int grid_override = 0) {
+                           unsigned long long* per_root, bool chunk_counts, bool work) {
     Scratch& s = q->scratch;
-    const int cr = q->plan.tune.chunk_roots;
+    const int cr = effective_chunk(g, q->plan, re - rb);
     uint64_t nch = n_chunks(re - rb, cr);
     tm_status r = scratch_reserve(&s, g->device, 1, 1 + (2 + 2 * TM_MAX_EDGES + 1), chunk_counts ? nch : 0,
                                   DEFAULT_TASK_CAP);
@@ -374,6 +393,7 @@ static tm_status run_count(tm_graph* g, tm_query* q, uint64_t rb, uint64_t re, c
     QueryDev* qd = s.qdev_stage();
     memset(qd, 0, sizeof(QueryDev));
     qd->plan = q->plan;
+    qd->plan.tune.chunk_roots = cr;
     qd->root_begin = rb;
     qd->root_end = re;
     qd->n_chunks = nch;
@@ -388,9 +408,9 @@ static tm_status run_count(tm_graph* g, tm_query* q, uint64_t rb, uint64_t re, c
     if (per_root && re > rb) TM_CUDA(cudaMemsetAsync(per_root, 0, (re - rb) * 8, st));
     if (chunk_counts) TM_CUDA(cudaMemsetAsync(s.chunk_cnt, 0, (nch + 2) * 8, st));   // counts + list length
     if (q->profile) TM_CUDA(cudaEventRecord(q->ev[0], st));
+    const LaunchCfg lc = search_launch_cfg(g, MODE_COUNT, q->plan.warp_smem, q->plan.tune.warps_per_block);
     r = launch_search(g, MODE_COUNT, s.qdev(), 1, q->plan.warp_smem, q->plan.tune.warps_per_block,
-                      plan_features(q->plan), &s, st,
-                      grid_override, work);
+                      plan_features(q->plan), &s, st, launch_blocks(g, lc, nch), work);
     if (r != TM_OK) return r;
     if (q->profile) TM_CUDA(cudaEventRecord(q->ev[1], st));
     q->fill_timed = false;
@@ -445,6 +465,7 @@ extern "C" tm_status tm_query_set_tuning(tm_query* q, const tm_tuning* t) {
         return TM_E_INVALID;
     }
     q->plan.tune = *t;
+    q->plan.auto_chunk = 0;
     if (q->plan.n_anti > 0) q->plan.tune.split_depth = 0;   // donated tasks carry no anti-edge times
     q->explicit_tuning = true;
     return TM_OK;
@@ -539,7 +560,7 @@ extern "C" tm_status tm_enumerate(tm_graph* g, tm_query* q, void* stream, int32_
     tm_status s = run_count(g, q, 0, m, st, nullptr, true, false);
     if (s != TM_OK) return s;
     Scratch& sc = q->scratch;
-    const uint64_t nch = n_chunks(m, q->plan.tune.chunk_roots);
+    const uint64_t nch = n_chunks(m, effective_chunk(g, q->plan, m));
     // pass 2: chunk offsets, and the chunks the fill pass must search
     s = exclusive_scan_u64(sc.chunk_cnt, sc.chunk_cnt, nch + 1, sc.scan_tmp, st);
     if (s != TM_OK) return s;
@@ -566,8 +587,9 @@ extern "C" tm_status tm_enumerate(tm_graph* g, tm_query* q, void* stream, int32_
         qd->total = sc.counters + 1;
         TM_CUDA(cudaMemcpyAsync(sc.head, sc.stage, sc.head_bytes(1), cudaMemcpyHostToDevice, st));
         if (q->profile) TM_CUDA(cudaEventRecord(q->ev[2], st));
+        const LaunchCfg lc = search_launch_cfg(g, MODE_FILL, q->plan.warp_smem_fill, q->plan.tune.warps_per_block);
         s = launch_search(g, MODE_FILL, sc.qdev(), 1, q->plan.warp_smem_fill, q->plan.tune.warps_per_block,
-                         plan_features(q->plan), &sc, st);
+                         plan_features(q->plan), &sc, st, launch_blocks(g, lc, nch));
         if (s != TM_OK) return s;
         if (q->profile) { TM_CUDA(cudaEventRecord(q->ev[3], st)); q->fill_timed = true; }
         TM_CUDA(cudaStreamSynchronize(st));
@@ -581,8 +603,8 @@ extern "C" tm_status tm_enumerate(tm_graph* g, tm_query* q, void* stream, int32_
 
 namespace tmg {
 
-std::vector<LaunchGroup> occupancy_groups(const tm_graph* g, Mode mode, const Plan* const* plans, int nq,
-                                          int* order) {
+std::vector<LaunchGroup> occupancy_groups(const tm_graph* g, Mode mode, const Plan* const* plans,
+                                          const uint64_t* nch, int nq, int* order) {
     std::vector<int> grid(nq), wpb(nq);
     for (int j = 0; j < nq; ++j) {
         const Plan& p = *plans[j];
@@ -607,11 +629,16 @@ std::vector<LaunchGroup> occupancy_groups(const tm_graph* g, Mode mode, const Pl
         const int j = order[i];
         const Plan& p = *plans[j];
         if (out.empty() || grid[order[out.back().first]] != grid[j] || wpb[order[out.back().first]] != wpb[j])
-            out.push_back(LaunchGroup{i, 0, 16, wpb[j], 0u});
+            out.push_back(LaunchGroup{i, 0, 16, wpb[j], 0u, 0});
         LaunchGroup& lg = out.back();
         lg.count++;
         lg.warp_smem = std::max(lg.warp_smem, mode == MODE_FILL ? p.warp_smem_fill : p.warp_smem);
         lg.feat |= plan_features(p);
+    }
+    for (LaunchGroup& lg : out) {
+        uint64_t chunks = 0;
+        for (int i = lg.first; i < lg.first + lg.count; ++i) chunks += nch[order[i]];
+        lg.grid = launch_blocks(g, search_launch_cfg(g, mode, lg.warp_smem, lg.warps), chunks);
     }
     return out;
 }
@@ -641,7 +668,7 @@ struct BatchExec {
         if (n != nq || gs.size() != groups.size() || md != mode) return false;
         for (size_t i = 0; i < gs.size(); ++i)
             if (gs[i].count != groups[i].count || gs[i].warp_smem != groups[i].warp_smem ||
-                gs[i].warps != groups[i].warps || gs[i].feat != groups[i].feat)
+                gs[i].warps != groups[i].warps || gs[i].feat != groups[i].feat || gs[i].grid != groups[i].grid)
                 return false;
         return true;
     }
@@ -714,7 +741,7 @@ static tm_status capture_batch(tm_graph* g, BatchExec* b) {
         Scratch v = b->view(gi);
         cudaMemsetAsync(b->ready, 0, DEFAULT_TASK_CAP, cs);
         ls = launch_search(g, MODE_COUNT, b->qdev_dev() + lg.first, lg.count, lg.warp_smem, lg.warps, lg.feat, &v,
-                           cs);
+                           cs, lg.grid);
     }
     cudaMemcpyAsync(b->counters_host, b->counters, (size_t)b->nq * 8, cudaMemcpyDeviceToHost, cs);
     cudaMemcpyAsync(b->stage, b->head, b->ctrl_bytes(), cudaMemcpyDeviceToHost, cs);
@@ -741,12 +768,16 @@ extern "C" tm_status tm_count_batch(tm_graph* g, tm_query* const* qs, int nq, vo
         return TM_OK;
     }
     std::vector<const Plan*> plans(nq);
+    std::vector<uint64_t> nch(nq);
+    std::vector<int> cr(nq);
     for (int j = 0; j < nq; ++j) {
         apply_cached_tuning(g, qs[j]);
         plans[j] = &qs[j]->plan;
+        cr[j] = effective_chunk(g, qs[j]->plan, (uint64_t)g->v.m * (uint64_t)nq);
+        nch[j] = n_chunks((uint64_t)g->v.m, cr[j]);
     }
     std::vector<int> order(nq);
-    std::vector<LaunchGroup> groups = occupancy_groups(g, MODE_COUNT, plans.data(), nq, order.data());
+    std::vector<LaunchGroup> groups = occupancy_groups(g, MODE_COUNT, plans.data(), nch.data(), nq, order.data());
     BatchExec* b = cached_exec(g, nq, groups, MODE_COUNT);
     std::lock_guard<std::mutex> use(b->mu);
     tm_status s = b->alloc();
@@ -759,9 +790,10 @@ extern "C" tm_status tm_count_batch(tm_graph* g, tm_query* const* qs, int nq, vo
             QueryDev* qd = b->qdev_stage() + i;
             memset(qd, 0, sizeof(QueryDev));
             qd->plan = qs[j]->plan;
+            qd->plan.tune.chunk_roots = cr[j];
             qd->root_begin = 0;
             qd->root_end = (uint64_t)g->v.m;
-            qd->n_chunks = n_chunks((uint64_t)g->v.m, qs[j]->plan.tune.chunk_roots);
+            qd->n_chunks = nch[j];
             qd->chunk_base = base;
             base += qd->n_chunks;
             qd->total = b->counters + j;
@@ -817,10 +849,12 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
     }
     std::vector<const Plan*> plans(nq);
     std::vector<uint64_t> nch(nq);
+    std::vector<int> cr(nq);
     for (int j = 0; j < nq; ++j) {
         apply_cached_tuning(g, qs[j]);
         plans[j] = &qs[j]->plan;
-        nch[j] = n_chunks(m, qs[j]->plan.tune.chunk_roots);
+        cr[j] = effective_chunk(g, qs[j]->plan, m * (uint64_t)nq);
+        nch[j] = n_chunks(m, cr[j]);
         // each query's own scratch holds its chunk counts, then their offsets
         tm_status r = scratch_reserve(&qs[j]->scratch, g->device, 1, 1, nch[j], 0);
         if (r != TM_OK) return r;
@@ -828,7 +862,7 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
     }
     // pass 1: per-chunk counts of every query, one persistent launch per occupancy group
     std::vector<int> order(nq);
-    std::vector<LaunchGroup> cg = occupancy_groups(g, MODE_COUNT, plans.data(), nq, order.data());
+    std::vector<LaunchGroup> cg = occupancy_groups(g, MODE_COUNT, plans.data(), nch.data(), nq, order.data());
     BatchExec* bc = cached_exec(g, nq, cg, MODE_COUNT);
     std::lock_guard<std::mutex> lock_c(bc->mu);
     tm_status s = bc->alloc();
@@ -841,6 +875,7 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
             QueryDev* qd = bc->qdev_stage() + i;
             memset(qd, 0, sizeof(QueryDev));
             qd->plan = qs[j]->plan;
+            qd->plan.tune.chunk_roots = cr[j];
             qd->root_end = m;
             qd->n_chunks = nch[j];
             qd->chunk_base = base;
@@ -859,7 +894,7 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
         Scratch v = bc->view(gi);
         TM_CUDA(cudaMemsetAsync(bc->ready, 0, DEFAULT_TASK_CAP, st));
         s = launch_search(g, MODE_COUNT, bc->qdev_dev() + cg[gi].first, cg[gi].count, cg[gi].warp_smem,
-                          cg[gi].warps, cg[gi].feat, &v, st);
+                          cg[gi].warps, cg[gi].feat, &v, st, cg[gi].grid);
         if (s != TM_OK) return s;
     }
     if (kernel_ms) TM_CUDA(cudaEventRecord(bc->ev[1], st));
@@ -883,9 +918,10 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
     if (!fq.empty()) {
         const int nf = (int)fq.size();
         std::vector<const Plan*> fplans(nf);
-        for (int i = 0; i < nf; ++i) fplans[i] = plans[fq[i]];
+        std::vector<uint64_t> fch(nf);
+        for (int i = 0; i < nf; ++i) { fplans[i] = plans[fq[i]]; fch[i] = nch[fq[i]]; }
         std::vector<int> forder(nf);
-        std::vector<LaunchGroup> fg = occupancy_groups(g, MODE_FILL, fplans.data(), nf, forder.data());
+        std::vector<LaunchGroup> fg = occupancy_groups(g, MODE_FILL, fplans.data(), fch.data(), nf, forder.data());
         bf = cached_exec(g, nf, fg, MODE_FILL);
         lock_f = std::unique_lock<std::mutex>(bf->mu);
         s = bf->alloc();
@@ -898,6 +934,7 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
                 QueryDev* qd = bf->qdev_stage() + i;
                 memset(qd, 0, sizeof(QueryDev));
                 qd->plan = qs[j]->plan;
+                qd->plan.tune.chunk_roots = cr[j];
                 qd->root_end = m;
                 qd->n_chunks = nch[j];
                 qd->chunk_base = base;
@@ -916,7 +953,7 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
         for (size_t gi = 0; gi < fg.size(); ++gi) {
             Scratch v = bf->view(gi);
             s = launch_search(g, MODE_FILL, bf->qdev_dev() + fg[gi].first, fg[gi].count, fg[gi].warp_smem,
-                              fg[gi].warps, fg[gi].feat, &v, st);
+                              fg[gi].warps, fg[gi].feat, &v, st, fg[gi].grid);
             if (s != TM_OK) return s;
         }
         if (kernel_ms) TM_CUDA(cudaEventRecord(bf->ev[1], st));
@@ -972,6 +1009,7 @@ extern "C" tm_status tm_autotune(tm_graph* g, tm_query* q, void* stream, tm_tuni
         TM_CUDA(cudaEventCreate(&e1));
         auto time_cfg = [&](const tm_tuning& t, float* ms) -> tm_status {
             q->plan.tune = t;
+            q->plan.auto_chunk = 0;
             float best_ms = 1e30f;
             for (int rep = 0; rep < 3; ++rep) {
                 cudaEventRecord(e0, st);

@@ -99,6 +99,7 @@ extern "C" tm_status tm_count_batch_noalloc(tm_graph* g, tm_query* const* qs, in
     const uint64_t m = (uint64_t)g->v.m;
     int warp_smem = 16, warps = 1;
     unsigned feat = 0;
+    uint64_t total_chunks = 0;
     for (int j = 0; j < nq; ++j)
         if (!qs[j] || query_graph(qs[j]) != g) { set_error("null or mismatched query in batch"); return TM_E_INVALID; }
     // Every call reuses the array: clear the caller's totals, then rewrite the
@@ -115,7 +116,8 @@ extern "C" tm_status tm_count_batch_noalloc(tm_graph* g, tm_query* const* qs, in
             query_plan(qs[j], &qd.plan);
             qd.root_begin = 0;
             qd.root_end = m;
-            qd.n_chunks = (m + (uint64_t)qd.plan.tune.chunk_roots - 1) / (uint64_t)qd.plan.tune.chunk_roots;
+            qd.plan.tune.chunk_roots = effective_chunk(g, qd.plan, m * (uint64_t)nq);
+            qd.n_chunks = n_chunks(m, qd.plan.tune.chunk_roots);
             qd.chunk_base = chunk_base;
             chunk_base += qd.n_chunks;
             qd.total = (unsigned long long*)totals_dev + j;
@@ -123,7 +125,7 @@ extern "C" tm_status tm_count_batch_noalloc(tm_graph* g, tm_query* const* qs, in
             warps = std::max(warps, qd.plan.tune.warps_per_block);
             feat |= plan_features(qd.plan);
         }
-        g_stage.ctrl.total_chunks = chunk_base;
+        g_stage.ctrl.total_chunks = total_chunks = chunk_base;
         // pageable source: the copy has left this buffer when the call returns
         TM_CUDA(cudaMemcpyAsync(base + OFF_CTRL, &g_stage, OFF_QDEV + (size_t)nq * sizeof(QueryDev),
                                 cudaMemcpyHostToDevice, st));
@@ -136,7 +138,8 @@ extern "C" tm_status tm_count_batch_noalloc(tm_graph* g, tm_query* const* qs, in
     view.tasks = (Task*)(base + OFF_TASKS);
     view.ready = base + OFF_READY;
     view.task_cap = NOALLOC_TASKS;
-    s = launch_search(g, MODE_COUNT, (const QueryDev*)(base + OFF_QDEV), nq, warp_smem, warps, feat, &view, st);
+    s = launch_search(g, MODE_COUNT, (const QueryDev*)(base + OFF_QDEV), nq, warp_smem, warps, feat, &view, st,
+                      launch_blocks(g, search_launch_cfg(g, MODE_COUNT, warp_smem, warps), total_chunks));
     if (s != TM_OK) return s;
     Ctrl done;
     TM_CUDA(cudaMemcpyAsync(&done, base + OFF_CTRL, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));

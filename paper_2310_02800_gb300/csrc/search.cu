@@ -5,8 +5,14 @@
 // Section 5.1.2 deciding where candidates come from and which mapped nodes a
 // new node must differ from.  The GPU organisation is our own:
 //
+//  * Roots are filtered before anything else of them is read: 64 at a time, two
+//    successor words per lane and list the motif continues in, since most edges
+//    have no later edge in the window at one of their nodes.  The survivors are
+//    buffered and taken 32 at a time, so the searches that start a window
+//    run on full warps.  (10M-edge power-law graph, 1 h windows: the cycles'
+//    roots fall to the tenth whose source is answered within the window.)
 //  * A warp owns a stack of FRAMES, one per motif edge i >= 1.  Frame i holds
-//    up to 64 partial matches of i edges ("parents"), each with its candidate
+//    up to 48 (count) or 64 (fill) partial matches of i edges ("parents"), each with its candidate
 //    window for edge i: the entries of one time-ordered adjacency list with
 //    t in (t_prev, min(t_root + delta, t_prev + gap_{i-1})], located by a
 //    binary search for the lower end and a galloping search for the upper end
@@ -16,19 +22,30 @@
 //    candidate; its time gap proves most windows empty without further loads.
 //  * The windows of a frame are flattened: lane j of a 32-wide step takes the
 //    j-th remaining candidate across all parents, so lanes stay busy even when
-//    every individual window is short.  Survivors of a step (structure, label
+//    every individual window is short.  Where each window starts in the flattened
+//    order is computed once, when the frame is begun; a step then finds its lanes'
+//    parents with two ballots and one reduction.  Survivors of a step (structure, label
 //    and injectivity checks) are compacted with __ballot_sync into the child
 //    frame, which is drained once it holds cap - 32 parents (16 in count
-//    frames of 48, 32 in fill frames of 64) or its parent frame is exhausted.  Processing frames in order keeps the emitted matches in
+//    frames of 48, 32 in fill frames of 64) or its parent frame is exhausted.
+//    Processing frames in order keeps the emitted matches in
 //    lexicographic order of edge ids (used by enumeration).
-//  * The last motif edge is never expanded: survivors are counted with
-//    __popc(ballot) and added to per-warp accumulators; per-root / per-chunk
-//    counts use __match_any_sync groups and one atomic per group.
+//  * The last motif edge is never expanded.  Counting it, when it extends by a
+//    new node, is a loop of its own that reads only the neighbour column and lets each lane
+//    count; other last edges count __popc(ballot) of the survivors.  Per-root / per-chunk
+//    counts take one atomic per group of lanes with one parent or root.
 //  * Load balance (sub-tree-level parallelism, Section 5.2): root edges are
 //    claimed in chunks from an atomic cursor; when warps sit idle, a warp at a
 //    shallow level donates the upper half of its remaining candidate range to
 //    a device task queue (count mode only), and idle warps pop those tasks.
+//    The launch ends when all claimed chunks and all donated tasks are reported
+//    done.  A launch has no more warps than chunks, and one idle warp per block polls
+//    for work: 5,472 warps going through the same lines cost a small launch 50 us.
 //    Every device-side wait is bounded by a global-timer deadline.
+//    All of it together, against one 32-root batch per claim, prefix sums rebuilt in every step
+//    and every warp polling: 20k-edge 3-cycle 192 -> 110 us per call, 1/61 of
+//    10M edges 202 -> 109 us, four queries' counts and rows on 10M edges
+//    4.76 -> 2.96 ms, 4-edge path over 15 h windows 47 -> 40 ms.
 //  * Look-ahead on chords (our addition): when an edge binds the last node of
 //    a later motif edge whose node pair no earlier motif edge joins, some
 //    graph edge must join their images later in the root's window; the
@@ -60,6 +77,8 @@ constexpr bool PREFETCH = true;
 constexpr uint32_t INLIST = 0x80000000u;    // window in an in-list
 constexpr uint32_t PAIRLIST = 0x40000000u;  // window in the (neighbour, time)-ordered out-list
 constexpr uint32_t POSMASK = 0x3FFFFFFFu;
+constexpr unsigned long long NO_CHUNK = ~0ull;
+constexpr uint32_t NEVER = 0xFFFFFFFFu;      // prefix entry past a frame's last parent
 constexpr uint32_t SPAN_FAR = 0xFFFFFFFFu;   // frame window end: recompute from the root
 constexpr uint32_t PAIR_MIN_DEG = 1024;     // closing lookups on shorter lists scan the time window
 constexpr uint32_t PAIR_MIN_WINDOW = 768;   // ... and so do windows shorter than this
@@ -149,21 +168,27 @@ __device__ __forceinline__ bool pair_after(const GraphView& g, int32_t u, int32_
 
 // ------------------------------------------------------------ frame access
 
+// The block's dynamic shared memory: each warp's frames, back to back.
+extern __shared__ __align__(16) char smem[];
+
 template <int CAP>
 struct FrameT {
     using L = FrameLayout<CAP>;
-    char* p;
-    __device__ int64_t& tprev(int s) const { return ((int64_t*)(p + L::TPREV))[s]; }
+    uint32_t o;      // byte offset in smem
+    __device__ int64_t& tprev(int s) const { return ((int64_t*)(smem + o + L::TPREV))[s]; }
     // window end t_root + delta, as its distance from tprev (SPAN_FAR: too far to hold)
-    __device__ uint32_t& tspan(int s) const { return ((uint32_t*)(p + L::TEND))[s]; }
-    __device__ uint32_t& beg(int s) const { return ((uint32_t*)(p + L::BEG))[s]; }
-    __device__ uint32_t& len(int s) const { return ((uint32_t*)(p + L::LEN))[s]; }
-    __device__ uint32_t& root(int s) const { return ((uint32_t*)(p + L::ROOT))[s]; }
-    __device__ int32_t& node(int j, int s) const { return ((int32_t*)(p + L::NODE))[j * CAP + s]; }
+    __device__ uint32_t& tspan(int s) const { return ((uint32_t*)(smem + o + L::TEND))[s]; }
+    __device__ uint32_t& beg(int s) const { return ((uint32_t*)(smem + o + L::BEG))[s]; }
+    __device__ uint32_t& len(int s) const { return ((uint32_t*)(smem + o + L::LEN))[s]; }
+    // once begin_frame has run, the same row holds where each window starts in the flattened order
+    __device__ uint32_t& pre(int s) const { return ((uint32_t*)(smem + o + L::LEN))[s]; }
+    __device__ uint2& pre2(int lane) const { return ((uint2*)(smem + o + L::LEN))[lane]; }
+    __device__ uint32_t& root(int s) const { return ((uint32_t*)(smem + o + L::ROOT))[s]; }
+    __device__ int32_t& node(int j, int s) const { return ((int32_t*)(smem + o + L::NODE))[j * CAP + s]; }
     // eids follow the nb node rows
-    __device__ int32_t& eid(int nb, int j, int s) const { return ((int32_t*)(p + L::NODE))[(nb + j) * CAP + s]; }
+    __device__ int32_t& eid(int nb, int j, int s) const { return ((int32_t*)(smem + o + L::NODE))[(nb + j) * CAP + s]; }
     // anti-edge attached-edge times, at byte offset `row_off` of the frame
-    __device__ int64_t& anti_t(int row_off, int a, int s) const { return ((int64_t*)(p + row_off))[a * CAP + s]; }
+    __device__ int64_t& anti_t(int row_off, int a, int s) const { return ((int64_t*)(smem + o + row_off))[a * CAP + s]; }
 };
 
 // ------------------------------------------------------------ per-warp state
@@ -173,7 +198,7 @@ constexpr int W_ROOTS = 0, W_NODES = 1, W_ENTRIES = 1 + TM_MAX_EDGES, W_PROBE = 
               W_MATCH = 2 + 2 * TM_MAX_EDGES, W_LEN = 3 + 2 * TM_MAX_EDGES;
 
 struct Acc {             // per-warp accumulators for the current query
-    unsigned long long total;      // warp-uniform
+    unsigned long long total;      // per lane
     unsigned long long w[W_LEN];   // stats launches; lane-0 values except W_PROBE (per lane)
 };
 
@@ -190,36 +215,34 @@ struct Search {
     Task* tasks;
     uint8_t* ready;
     uint64_t task_cap;
-    char* wbase;              // this warp's shared block
+    uint32_t wbase;           // this warp's shared block (byte offset in smem)
     int lane;
     // current query
     int qi;
     const QueryDev* q;
     int k;
-    // level cursors: lane j holds the values for level j
-    uint32_t myP, myOff, myT;
+    // cursors of the suspended levels: lane j holds level j's next candidate and total
+    uint32_t myOff, myT, myNp;
+    uint32_t np1;             // parents in frame 1 (warp-uniform)
+    uint32_t nbuf;            // roots in the root buffer (warp-uniform)
     Acc acc;
     // enumerate fill
     unsigned long long out_base, out_local;
     unsigned polls;           // donation checks (warp-uniform)
+    uint32_t claimed;         // root chunks this warp has claimed (warp-uniform)
 
-    __device__ Search(const GraphView& g_, const QueryDev* qs_, Ctrl* c, Task* t, uint8_t* r, uint64_t cap, char* wb)
+    __device__ Search(const GraphView& g_, const QueryDev* qs_, Ctrl* c, Task* t, uint8_t* r, uint64_t cap, uint32_t wb)
         : g(g_), qs(qs_), ctrl(c), tasks(t), ready(r), task_cap(cap), wbase(wb) {
         lane = threadIdx.x & 31;
         qi = -1; q = nullptr; k = 0;
-        myP = myOff = myT = 0;
+        myOff = myT = myNp = 0;
+        np1 = nbuf = 0;
         acc.total = 0;
         if (STATS) for (int i = 0; i < W_LEN; ++i) acc.w[i] = 0;
         out_base = out_local = 0;
         polls = 0;
+        claimed = 0;
     }
-
-    __device__ uint32_t P(int l) const { return __shfl_sync(FULL, myP, l); }
-    __device__ uint32_t Off(int l) const { return __shfl_sync(FULL, myOff, l); }
-    __device__ uint32_t T(int l) const { return __shfl_sync(FULL, myT, l); }
-    __device__ void setP(int l, uint32_t v) { if (lane == l) myP = v; }
-    __device__ void setOff(int l, uint32_t v) { if (lane == l) myOff = v; }
-    __device__ void setT(int l, uint32_t v) { if (lane == l) myT = v; }
 
     // The window end t_root + delta of entry s of frame f (4 bytes per entry
     // instead of 8: rebuilt from the root edge's time when too far from tprev).
@@ -233,12 +256,14 @@ struct Search {
     }
 
     __device__ Frame frame(int i) const {
-        return Frame{wbase + (MODE == MODE_FILL ? q->plan.lv[i].frame_off_fill : q->plan.lv[i].frame_off)};
+        return Frame{wbase + (uint32_t)__ldg(MODE == MODE_FILL ? &q->plan.lv[i].frame_off_fill : &q->plan.lv[i].frame_off)};
     }
 
     __device__ int anti_off(int i) const {
         return MODE == MODE_FILL ? q->plan.lv[i].anti_row_off_fill : q->plan.lv[i].anti_row_off;
     }
+
+    __device__ uint32_t hot(int i) const { return __ldg(&q->plan.lv[i].hot); }
 
     // Anti-edges in `mask` (Section 2.1): true when none of them has an edge in
     // its window.  Slots of the candidate's partial match are the parent's
@@ -272,6 +297,7 @@ struct Search {
 
     __device__ void flush() {
         if (q == nullptr) return;
+        for (int d = 16; d > 0; d >>= 1) acc.total += __shfl_down_sync(FULL, acc.total, d);
         if (lane == 0 && acc.total) atomicAdd(q->total, acc.total);
         if (STATS) {
             for (int i = 0; i < W_LEN; ++i) {
@@ -319,11 +345,12 @@ struct Search {
     // Successor words of the lists level `ln` draws its window from, after a
     // candidate edge at position cpos of list cdir, read ahead together with
     // the candidate: only those that take one load.  y == 0 means "not read".
-    __device__ void next_words(const LevelPlan& ln, int cdir, uint32_t cpos, uint2& wa, uint2& wb) const {
+    __device__ void next_words(uint32_t hn, int cdir, uint32_t cpos, uint2& wa, uint2& wb) const {
         wa = make_uint2(0u, 0u);
         wb = make_uint2(0u, 0u);
-        if (ln.nx_a >= 0 && successor_direct(ln.nx_a, cdir)) wa = successor(ln.nx_a, cdir, cpos, -1);
-        if (ln.kind == CLOSE && ln.nx_b >= 0 && successor_direct(ln.nx_b, cdir)) wb = successor(ln.nx_b, cdir, cpos, -1);
+        const int na = Hot::nx_a(hn), nb = Hot::nx_b(hn);
+        if (na >= 0 && successor_direct(na, cdir)) wa = successor(na, cdir, cpos, -1);
+        if (Hot::kind(hn) == CLOSE && nb >= 0 && successor_direct(nb, cdir)) wb = successor(nb, cdir, cpos, -1);
     }
     // True when a list whose successor word is w has no entry in (tprev, lim].
     __device__ static bool word_shows_empty(uint2 w, uint64_t span) {
@@ -336,12 +363,12 @@ struct Search {
         return (int32_t)cpos;
     }
 
-    __device__ uint32_t locate(int lv_i, Frame pf, int ps, int nb, int32_t n0, int32_t n1, int32_t prev_e,
+    __device__ uint32_t locate(int lv_i, uint32_t h, Frame pf, int ps, int nb, int32_t n0, int32_t n1, int32_t prev_e,
                                int cdir, uint32_t cpos, int64_t tprev, int64_t tend, uint32_t& beg_out,
                                uint2 wa, uint2 wb) {
-        const LevelPlan& lp = q->plan.lv[lv_i];
         auto slot = [&](int s) -> int32_t { return s < nb ? pf.node(s, ps) : (s == nb ? n0 : n1); };
-        int64_t lim = min(tend, sat_add(tprev, lp.gap));
+        int64_t lim = tend;
+        if (h & Hot::GAP) lim = min(tend, sat_add(tprev, q->plan.lv[lv_i].gap));
         beg_out = 0;
         if (!STATS && lim <= tprev) return 0;
         const uint64_t span = (uint64_t)(lim - tprev);
@@ -350,7 +377,7 @@ struct Search {
         if (!STATS && (word_shows_empty(wa, span) || word_shows_empty(wb, span))) return 0;
         const int64_t* tarr;
         uint32_t b, hi, flag = 0;
-        int kind = lp.kind;
+        const int kind = Hot::kind(h);
         if (kind == FREE) {
             tarr = g.t;
             hi = (uint32_t)g.m;
@@ -361,11 +388,11 @@ struct Search {
             uint32_t lo;
             if (kind == CLOSE) {
                 // the shorter of out(phi(x_i)) and in(phi(y_i))
-                int32_t u = slot(lp.a), w = slot(lp.b);
+                int32_t u = slot(Hot::a(h)), w = slot(Hot::b(h));
                 uint32_t u0 = __ldg(g.off[0] + u), u1 = __ldg(g.off[0] + u + 1);
                 uint32_t w0 = __ldg(g.off[1] + w), w1 = __ldg(g.off[1] + w + 1);
-                if (u1 - u0 <= w1 - w0) { dir = 0; lo = u0; hi = u1; nx = lp.nx_a; }
-                else { dir = 1; lo = w0; hi = w1; nx = lp.nx_b; }
+                if (u1 - u0 <= w1 - w0) { dir = 0; lo = u0; hi = u1; nx = Hot::nx_a(h); }
+                else { dir = 1; lo = w0; hi = w1; nx = Hot::nx_b(h); }
                 if (!STATS && hi - lo >= PAIR_MIN_DEG) {
                     // a long list: if its time window is long too, take the u -> w
                     // edges straight from u's pair-ordered out-list instead of
@@ -394,8 +421,8 @@ struct Search {
                 }
             } else {
                 dir = kind == EXT_IN ? 1 : 0;
-                int32_t v = slot(lp.a);
-                nx = lp.nx_a;
+                int32_t v = slot(Hot::a(h));
+                nx = Hot::nx_a(h);
                 hi = __ldg(g.off[dir] + v + 1);
                 lo = (nx >= 0 && !STATS) ? 0u : __ldg(g.off[dir] + v);
             }
@@ -416,44 +443,45 @@ struct Search {
         return e - b;
     }
 
-    // Exclusive prefix of the window lengths of a frame's parents, kept in
-    // registers: lane j holds parents 2j and 2j+1.
-    struct Prefix {
-        uint32_t preA, preB, lenA, lenB, tot;
-    };
-    __device__ Prefix prefix(Frame f, uint32_t np) const {
-        const uint32_t a = 2u * lane, b = a + 1u;
-        Prefix r;
-        r.lenA = a < np ? f.len(a) : 0u;
-        r.lenB = b < np ? f.len(b) : 0u;
-        uint32_t s = r.lenA + r.lenB, inc = s;
+    // Start frame i, which holds np parents: its window lengths become their
+    // exclusive prefix (the flattened position each window starts at; entries past
+    // np never start), computed once per frame.  Returns the flattened total.
+    __device__ uint32_t begin_frame(Frame f, uint32_t np) const {
+        const uint32_t a = 2u * lane;
+        uint32_t tot = 0;
+        uint2 l = make_uint2(0u, 0u);
+        if (a < (uint32_t)CAP) l = f.pre2(lane);
+        if (a >= np) l.x = 0u;
+        if (a + 1u >= np) l.y = 0u;
+        const uint32_t s = l.x + l.y;
+        uint32_t inc = s;
         for (int d = 1; d < 32; d <<= 1) {
             uint32_t u = __shfl_up_sync(FULL, inc, d);
             if (lane >= d) inc += u;
         }
-        r.preA = inc - s;
-        r.preB = r.preA + r.lenA;
-        r.tot = __shfl_sync(FULL, inc, 31);
-        return r;
+        tot = __shfl_sync(FULL, inc, 31);
+        const uint32_t pa = inc - s;
+        if (a < (uint32_t)CAP) f.pre2(lane) = make_uint2(a < np ? pa : NEVER, a + 1u < np ? pa + l.x : NEVER);
+        __syncwarp();
+        return tot;
     }
 
-    // The parent whose window holds flattened position x (x < total) and its prefix.
-    __device__ void owner(const Prefix& pr, uint32_t x, int& p, uint32_t& pre_p) const {
-        bool oa = pr.lenA && pr.preA <= x && x - pr.preA < pr.lenA;
-        bool ob = pr.lenB && pr.preB <= x && x - pr.preB < pr.lenB;
-        unsigned ba = __ballot_sync(FULL, oa), bb = __ballot_sync(FULL, ob);
-        int src = ba ? __ffs(ba) - 1 : __ffs(bb) - 1;
-        uint32_t va = __shfl_sync(FULL, pr.preA, src), vb = __shfl_sync(FULL, pr.preB, src);
-        p = 2 * src + (ba ? 0 : 1);
-        pre_p = ba ? va : vb;
+    // Parent whose window holds flattened position x (warp-uniform); every
+    // window of a begun frame is non-empty, so it is the last one starting at or before x.
+    __device__ static int parent_of(uint2 pr, uint32_t x) {
+        return __popc(__ballot_sync(FULL, pr.x <= x)) + __popc(__ballot_sync(FULL, pr.y <= x)) - 1;
     }
 
-    // Start a frame: its cursor and flattened total.
-    __device__ uint32_t begin_frame(int i) {
-        Prefix pr = prefix(frame(i), P(i));
-        setOff(i, 0);
-        setT(i, pr.tot);
-        return pr.tot;
+    // This lane's parent for the 32-wide step at off: the parent holding off plus
+    // the windows that start in (off, off + lane].  starts: bit j = a window starts at off + j.
+    __device__ int lane_parent(uint2 pr, uint32_t off, unsigned& starts) const {
+        const int p0 = parent_of(pr, off);
+        unsigned mk = 0;
+        const uint32_t da = pr.x - off, db = pr.y - off;   // a start at or before off wraps or is 0: masked out
+        if (da - 1u < 31u) mk |= 1u << da;
+        if (db - 1u < 31u) mk |= 1u << db;
+        starts = __reduce_or_sync(FULL, mk);
+        return p0 + __popc(starts & ((2u << lane) - 1u));
     }
 
     // Emit survivors of the last level (or of the root level when k == 1).
@@ -462,7 +490,7 @@ struct Search {
         if (!bal) return;
         unsigned cnt = __popc(bal);
         if (MODE == MODE_COUNT) {
-            acc.total += cnt;
+            if (lane == 0) acc.total += cnt;
             if (STATS && lane == 0) acc.w[W_MATCH] += cnt;
             if (q->per_root && ok) {
                 unsigned grp = __match_any_sync(bal, root);
@@ -485,43 +513,33 @@ struct Search {
         }
     }
 
-    // One 32-candidate step of frame i.
-    __device__ void step(int i) {
-        const LevelPlan& lp = q->plan.lv[i];
-        Frame f = frame(i);
-        const int nb = lp.nb;
-        const uint32_t np = P(i), off = Off(i), tot = T(i);
-        uint32_t idx = off + lane;
-        bool act = idx < tot;
-        // Lane -> parent without a search: the parent holding `off`, plus the
-        // parents whose windows start inside this 32-wide step (a start mask).
-        Prefix pr = prefix(f, np);
-        int p0;
-        uint32_t pre0;
-        owner(pr, off, p0, pre0);
-        const int a = 2 * lane, b = a + 1;
-        unsigned mk = 0;
-        if (a > p0 && pr.lenA && pr.preA - off < 32u) mk |= 1u << (pr.preA - off);
-        if (b > p0 && pr.lenB && pr.preB - off < 32u) mk |= 1u << (pr.preB - off);
-        const unsigned starts = __reduce_or_sync(FULL, mk);
-        const unsigned le = starts & ((2u << lane) - 1u);
-        const int p = p0 + __popc(le);
-        const uint32_t within = le ? (uint32_t)(lane - (31 - __clz(le))) : (off - pre0 + (uint32_t)lane);
+    // One 32-candidate step of frame f at level i < k - 1 (or of the last level,
+    // where survivors are emitted): candidates [off, off + 32) of its tot.  h, hc: packed plans of
+    // levels i and i + 1; survivors with a window join child frame c after its cp
+    // parents.  Returns the child frame's new size.
+    __device__ uint32_t step(int i, uint32_t h, uint32_t hc, Frame f, Frame c, uint32_t off, uint32_t tot,
+                                          uint32_t cp) {
+        const int nb = Hot::nb(h), kind = Hot::kind(h);
+        const uint2 pr = f.pre2(2 * lane < CAP ? lane : 0);
+        unsigned starts;
+        const uint32_t idx = off + lane;
+        const bool act = idx < tot;
+        const int pl_ = lane_parent(2 * lane < CAP ? pr : make_uint2(NEVER, NEVER), off, starts);
+        const int p = act ? pl_ : 0;
         int32_t n0 = -1, n1 = -1, ceid = -1;
         int64_t ct = 0;
         bool ok = act;
-        const int kind = lp.kind;
         // the candidate's edge id: written by enumeration and read by edge labels;
         // the next level's successor lookup loads it only if it needs it
-        const bool need_eid = (MODE == MODE_FILL) || lp.elabel >= 0;
+        const bool need_eid = (MODE == MODE_FILL) || (h & Hot::ELABEL);
         int cdir = 2;
         uint32_t pos = 0;
         uint2 wa = make_uint2(0u, 0u), wb = wa;   // next level's successor words, read with the candidate
         if (act) {
             uint32_t bw = f.beg(p);
-            pos = (bw & POSMASK) + within;
+            pos = (bw & POSMASK) + (idx - f.pre(p));
             cdir = (bw & PAIRLIST) ? 3 : (kind == FREE ? 2 : ((bw & INLIST) ? 1 : 0));
-            if (PREFETCH && !STATS && i < k - 1) next_words(q->plan.lv[i + 1], cdir, pos, wa, wb);
+            if (PREFETCH && !STATS && i < k - 1) next_words(hc, cdir, pos, wa, wb);
             if (bw & PAIRLIST) {
                 // closing edge from the pair-ordered list: structure holds by construction
                 ct = __ldg(g.pt + pos);
@@ -536,38 +554,41 @@ struct Search {
                     int32_t x = f.node(j, p);
                     ok &= (x != n0) && (x != n1);
                 }
-                if (lp.nl0 >= 0) ok &= g.nlabel[n0] == (uint8_t)lp.nl0;
-                if (lp.nl1 >= 0) ok &= g.nlabel[n1] == (uint8_t)lp.nl1;
+                if (h & Hot::NLABEL) {
+                    const LevelPlan& lp = q->plan.lv[i];
+                    if (lp.nl0 >= 0) ok &= g.nlabel[n0] == (uint8_t)lp.nl0;
+                    if (lp.nl1 >= 0) ok &= g.nlabel[n1] == (uint8_t)lp.nl1;
+                }
             } else {
                 int dir = (bw & INLIST) ? 1 : 0;
                 ct = __ldg(g.at[dir] + pos);
                 int32_t nbr = __ldg(g.anbr[dir] + pos);
                 if (need_eid) ceid = __ldg(g.aeid[dir] + pos);
                 if (kind == CLOSE) {
-                    ok = nbr == f.node(dir ? lp.a : lp.b, p);
+                    ok = nbr == f.node(dir ? Hot::a(h) : Hot::b(h), p);
                 } else {
                     n0 = nbr;
                     for (int j = 0; j < nb; ++j) ok &= f.node(j, p) != nbr;
-                    if (lp.nl0 >= 0) ok &= g.nlabel[nbr] == (uint8_t)lp.nl0;
+                    if (h & Hot::NLABEL) ok &= g.nlabel[nbr] == (uint8_t)q->plan.lv[i].nl0;
                 }
             }
-            if (lp.elabel >= 0) ok &= g.elabel[ceid] == (uint8_t)lp.elabel;
-            if (ANTI && ok && lp.anti_mask)
-                ok = anti_clear(lp.anti_mask, i, f, p, nb, n0, n1, ct, f.tprev(p), anti_off(i));
-            if (LOOK && ok && lp.n_look) ok = look_ok(lp, f, p, nb, n0, n1, ct, tend_of(f, p));
+            if (h & Hot::ELABEL) ok &= g.elabel[ceid] == (uint8_t)q->plan.lv[i].elabel;
+            if (ANTI && ok && (h & Hot::ANTI))
+                ok = anti_clear(q->plan.lv[i].anti_mask, i, f, p, nb, n0, n1, ct, f.tprev(p), anti_off(i));
+            if (LOOK && ok && (h & Hot::LOOK)) ok = look_ok(q->plan.lv[i], f, p, nb, n0, n1, ct, tend_of(f, p));
         }
         uint32_t root = act ? f.root(p) : 0u;
         if (i == k - 1) {
             emit(ok, root, f, p, nb, ceid);
-            return;
+            return 0u;
         }
         // expand survivors into frame i+1
-        const int nb_c = q->plan.lv[i + 1].nb;
+        const int nb_c = Hot::nb(hc);
         uint32_t cbeg = 0, clen = 0;
         int64_t tend = 0;
         if (ok) {
             tend = tend_of(f, p);
-            clen = locate(i + 1, f, p, nb, n0, n1, ceid, cdir, pos, ct, tend, cbeg, wa, wb);
+            clen = locate(i + 1, hc, f, p, nb, n0, n1, ceid, cdir, pos, ct, tend, cbeg, wa, wb);
         }
         if (STATS) {
             unsigned b = __ballot_sync(FULL, ok);
@@ -580,9 +601,7 @@ struct Search {
         }
         bool keep = ok && clen > 0;
         unsigned kb = __ballot_sync(FULL, keep);
-        if (!kb) return;
-        uint32_t cp = P(i + 1);
-        Frame c = frame(i + 1);
+        if (!kb) return cp;
         if (keep) {
             int s = (int)(cp + __popc(kb & ((1u << lane) - 1u)));
             for (int j = 0; j < nb; ++j) c.node(j, s) = f.node(j, p);
@@ -605,33 +624,29 @@ struct Search {
             }
         }
         __syncwarp();
-        setP(i + 1, cp + __popc(kb));
+        return cp + __popc(kb);
     }
 
-    // Donate the upper half of frame i's remaining candidates as tasks.
-    __device__ void maybe_donate(int i) {
-        const uint32_t np = P(i), off = Off(i), tot = T(i);
+    // Donate the upper half of frame i's remaining candidates [off, tot) as
+    // tasks; returns the frame's new total.  np: its parents (shrunk too).
+    __device__ uint32_t maybe_donate(int i, Frame f, uint32_t& np, uint32_t off, uint32_t tot) {
         const tm_tuning& tu = q->plan.tune;
-        if (i > tu.split_depth || tot - off <= (uint32_t)tu.split_min || (ANTI && q->plan.n_anti)) return;
-        if ((++polls & 15u) != 1u) return;      // look at the idle count every 16th step
+        if (i > tu.split_depth || tot - off <= (uint32_t)tu.split_min || (ANTI && q->plan.n_anti)) return tot;
+        if ((++polls & 15u) != 1u) return tot;      // look at the idle count every 16th step
         int idle = 0;
         if (lane == 0) idle = *(volatile int*)&ctrl->idle;
         idle = __shfl_sync(FULL, idle, 0);
-        if (idle <= 0) return;
-        Frame f = frame(i);
+        if (idle <= 0) return tot;
         uint32_t mid = off + ((tot - off) >> 1);
         mid = (mid + 31u) & ~31u;
-        if (mid >= tot || mid <= off) return;
+        if (mid >= tot || mid <= off) return tot;
         // parent containing mid
-        Prefix pr = prefix(f, np);
-        int p0;
-        uint32_t pre0;
-        owner(pr, mid, p0, pre0);
+        const int p0 = parent_of(2 * lane < CAP ? f.pre2(lane) : make_uint2(NEVER, NEVER), mid);
         const int ntask = (int)np - p0;
         // a task is one parent's window range: donate only when the tasks carry
         // split_min candidates each on average, else the queue traffic costs
         // more than the work it moves
-        if ((tot - mid) < (uint32_t)ntask * (uint32_t)max(tu.split_min, 32)) return;
+        if ((tot - mid) < (uint32_t)ntask * (uint32_t)max(tu.split_min, 32)) return tot;
         unsigned long long base = 0;
         if (lane == 0) base = atomicAdd(&ctrl->q_reserve, (unsigned long long)ntask);
         base = __shfl_sync(FULL, base, 0);
@@ -639,18 +654,18 @@ struct Search {
             // no room: void the reserved slots that exist and keep the work
             for (int j = lane; j < ntask; j += 32)
                 if (base + j < task_cap) *(volatile uint8_t*)&ready[base + j] = 2;
-            return;
+            return tot;
         }
         const int nb = q->plan.lv[i].nb;
         for (int j = lane; j < ntask; j += 32) {
             int p = p0 + j;
-            uint32_t len = f.len(p), bw = f.beg(p);
-            uint32_t skip = (p == p0) ? (mid - pre0) : 0u;
+            const uint32_t pre = f.pre(p), end = p + 1 < (int)np ? f.pre(p + 1) : tot;
+            const uint32_t skip = (p == p0) ? (mid - pre) : 0u;
             Task* t = tasks + base + j;
             t->query = (int16_t)qi;
             t->level = (int16_t)i;
-            t->beg = bw + skip;
-            t->len = len - skip;
+            t->beg = f.beg(p) + skip;
+            t->len = end - pre - skip;
             t->tprev = f.tprev(p);
             t->tend = tend_of(f, p);
             t->root = f.root(p);
@@ -659,47 +674,167 @@ struct Search {
         __threadfence();
         for (int j = lane; j < ntask; j += 32) *(volatile uint8_t*)&ready[base + j] = 1;
         __syncwarp();
-        if (lane == 0) {
-            f.len(p0) = mid - pre0;
-            atomicAdd(&ctrl->donated, (unsigned)ntask);
-        }
-        __syncwarp();
-        setP(i, (uint32_t)p0 + 1);
-        setT(i, mid);
+        if (lane == 0) atomicAdd(&ctrl->donated, (unsigned)ntask);
+        np = (uint32_t)p0 + 1u;
+        return mid;
     }
 
-    // Drain frame `base` (and everything below it) to completion.
-    __device__ void drain(int base) {
-        begin_frame(base);
-        int lvl = base;
-        while (true) {
-            if (Off(lvl) < T(lvl)) {
-                if (MODE == MODE_COUNT) maybe_donate(lvl);
-                if (Off(lvl) < T(lvl)) {
-                    step(lvl);
-                    setOff(lvl, Off(lvl) + 32);
-                    if (lvl < k - 1 && P(lvl + 1) >= DESCEND) { ++lvl; begin_frame(lvl); }
+    // The last level of a count-mode search whose last edge extends by one new
+    // node without labels or anti-edges: a candidate survives when its neighbour is none of the
+    // bound nodes, so only the neighbour column is read and lanes count on their own.
+    __device__ void count_ext(int i, uint32_t h, Frame f, uint32_t np, uint32_t tot) {
+        const int nb = Hot::nb(h);
+        const int32_t* __restrict__ nbr = g.anbr[Hot::kind(h) == EXT_IN ? 1 : 0];
+        const uint2 pr = 2 * lane < CAP ? f.pre2(lane) : make_uint2(NEVER, NEVER);
+        const bool attrib = q->per_root || q->chunk_cnt;
+        uint32_t off = 0;
+        unsigned long long cnt = 0;
+        while (off < tot) {
+            tot = maybe_donate(i, f, np, off, tot);
+            unsigned starts;
+            const uint32_t idx = off + lane;
+            const int pl_ = lane_parent(pr, off, starts);
+            bool ok = idx < tot;
+            const int p = ok ? pl_ : 0;
+            if (ok) {
+                const uint32_t pos = (f.beg(p) & POSMASK) + (idx - f.pre(p));
+                const int32_t x = __ldg(nbr + pos);
+                for (int j = 0; j < nb; ++j) ok &= f.node(j, p) != x;
+            }
+            cnt += ok;
+            if (attrib) {
+                // lanes of one parent share a root: its first lane adds for all of them
+                const unsigned bal = __ballot_sync(FULL, ok);
+                if (bal && (lane == 0 || (starts >> lane & 1u))) {
+                    const unsigned later = starts & ~((2u << lane) - 1u);     // starts after this lane
+                    const unsigned mine = bal & ~((1u << lane) - 1u) & (later ? (later & (0u - later)) - 1u : FULL);
+                    if (mine) attribute(f.root(p), (unsigned long long)__popc(mine));
                 }
+            }
+            off += 32;
+        }
+        acc.total += cnt;
+    }
+
+    // Add n matches to their root's and their chunk's counters (where asked for).
+    __device__ void attribute(uint32_t root, unsigned long long n) const {
+        const uint64_t r = root - q->root_begin;
+        if (q->per_root) atomicAdd(q->per_root + r, n);
+        if (q->chunk_cnt) atomicAdd(q->chunk_cnt + (uint32_t)r / (uint32_t)q->plan.tune.chunk_roots, n);
+    }
+
+    // Drain frame `base`, holding np parents (and everything below it), to completion.
+    __device__ void drain(int base, uint32_t np) {
+        int lvl = base;
+        uint32_t h = hot(lvl), hc = lvl + 1 < k ? hot(lvl + 1) : 0u;
+        Frame f = frame(lvl), c = lvl + 1 < k ? frame(lvl + 1) : f;
+        uint32_t off = 0, tot = begin_frame(f, np), nch = 0;
+        while (true) {
+            if (MODE == MODE_COUNT && !STATS && lvl == k - 1 && Hot::kind(h) <= EXT_IN &&
+                !(h & (Hot::ELABEL | Hot::NLABEL | Hot::ANTI))) {
+                count_ext(lvl, h, f, np, tot);
+                off = tot;
+            }
+            while (off < tot) {
+                if (MODE == MODE_COUNT) tot = maybe_donate(lvl, f, np, off, tot);
+                nch = step(lvl, h, hc, f, c, off, tot, nch);
+                off += 32;
+                if (nch >= DESCEND) break;
+            }
+            if (nch > 0) {
+                // down into the child frame
+                if (lane == lvl) { myOff = off; myT = tot; myNp = np; }
+                ++lvl;
+                np = nch;
+                nch = 0;
+                h = hc;
+                f = c;
+                if (lvl + 1 < k) { hc = hot(lvl + 1); c = frame(lvl + 1); }
+                off = 0;
+                tot = begin_frame(f, np);
                 continue;
             }
-            if (lvl < k - 1 && P(lvl + 1) > 0) { ++lvl; begin_frame(lvl); continue; }
-            setP(lvl, 0);
             if (lvl == base) break;
+            // back to the suspended parent frame, whose child frame is empty again
             --lvl;
+            hc = h;
+            c = f;
+            h = hot(lvl);
+            f = frame(lvl);
+            off = __shfl_sync(FULL, myOff, lvl);
+            tot = __shfl_sync(FULL, myT, lvl);
+            np = __shfl_sync(FULL, myNp, lvl);
         }
     }
 
-    // Roots [r0, r1) of the current query: level 0 of the search.
-    __device__ void roots(uint64_t r0, uint64_t r1, bool flush_at_end) {
+    __device__ uint32_t& root_buf(uint32_t j) const { return ((uint32_t*)(smem + wbase))[j]; }
+
+    // Scan 64 root edges from rb (rounded down to even) up to re: those whose
+    // successor words leave them a chance of a match join the root buffer, in order.  A
+    // root dies when a list the motif draws a later edge from -- any of the out- and
+    // in-lists of its two nodes -- has no entry in (t, t + delta].  The words are
+    // read two per lane and nothing else of a dead root is read.
+    __device__ void scan_roots(uint32_t rb, uint32_t re) {
+        const uint32_t r = (rb & ~1u) + 2u * lane;
+        bool a = r >= rb && r < re, b = r + 1u < re;
+        if (STATS) {
+            if (lane == 0) acc.w[W_ROOTS] += min(re, (rb & ~1u) + 64u) - rb;
+        } else if (a || b) {
+            const Plan& pl = q->plan;
+            if (pl.elabel0 >= 0) {
+                a = a && g.elabel[r] == (uint8_t)pl.elabel0;
+                b = b && g.elabel[r + 1] == (uint8_t)pl.elabel0;
+            }
+            if (a || b) {
+                const unsigned need = __ldg(&pl.root_need);
+                const uint32_t near = __ldg(&pl.root_span_next), far = __ldg(&pl.root_span);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (!(need & (0x11u << j))) continue;
+                    // the column is padded to an even number of words
+                    const uint4 w = __ldg((const uint4*)(g.nxt[j] + r));
+                    const uint32_t span = need & (0x10u << j) ? near : far;
+                    a = a && w.y <= span;
+                    b = b && w.w <= span;
+                }
+            }
+        }
+        const unsigned ba = __ballot_sync(FULL, a), bb = __ballot_sync(FULL, b);
+        if (!(ba | bb)) return;
+        const unsigned lt = (1u << lane) - 1u;
+        const uint32_t at = nbuf + __popc(ba & lt) + __popc(bb & lt);
+        if (a) root_buf(at) = r;
+        if (b) root_buf(at + (a ? 1u : 0u)) = r + 1u;
+        nbuf += __popc(ba) + __popc(bb);
+        __syncwarp();
+    }
+
+    // Drop the first n of the buffered roots.
+    __device__ void pop_roots(uint32_t n) {
+        const uint32_t left = nbuf - n;
+        const uint32_t x = lane < left ? root_buf(n + lane) : 0u, y = lane + 32u < left ? root_buf(n + 32u + lane) : 0u;
+        __syncwarp();
+        if (lane < left) root_buf(lane) = x;
+        if (lane + 32u < left) root_buf(lane + 32u) = y;
+        __syncwarp();
+        nbuf = left;
+    }
+
+    // Level 0 of the search for the first up to 32 buffered roots; those with a
+    // window join frame 1 after its np1 parents.
+    __device__ void root_batch() {
         const Plan& pl = q->plan;
-        for (uint64_t rb = r0; rb < r1; rb += 32) {
-            uint64_t r = rb + lane;
-            bool ok = r < r1;
+        const uint32_t hc = k > 1 ? hot(1) : 0u;
+        const uint32_t n = min(nbuf, 32u);
+        {
+            bool ok = lane < n;
+            const uint32_t r = ok ? root_buf(lane) : 0u;
+            pop_roots(n);
             int32_t s = 0, d = 0;
             int64_t tt = 0;
             uint2 wa = make_uint2(0u, 0u), wb = wa;
             if (ok) {
-                if (PREFETCH && !STATS && k > 1) next_words(pl.lv[1], 2, (uint32_t)r, wa, wb);
+                if (PREFETCH && !STATS && k > 1) next_words(hc, 2, r, wa, wb);
                 s = __ldg(g.src + r);
                 d = __ldg(g.dst + r);
                 tt = __ldg(g.t + r);
@@ -712,16 +847,15 @@ struct Search {
                 if (LOOK && ok && pl.lv[0].n_look)
                     ok = look_ok(pl.lv[0], Frame{wbase}, 0, 0, s, d, tt, sat_add(tt, pl.delta));
             }
-            if (STATS && lane == 0) acc.w[W_ROOTS] += (r1 - rb < 32ull) ? (unsigned long long)(r1 - rb) : 32ull;
             if (k == 1) {
-                emit(ok, (uint32_t)r, Frame{wbase}, 0, 0, (int32_t)r);
-                continue;
+                emit(ok, r, Frame{wbase}, 0, 0, (int32_t)r);
+                return;
             }
             uint32_t cbeg = 0, clen = 0;
             int64_t tend = 0;
             if (ok) {
                 tend = sat_add(tt, pl.delta);
-                clen = locate(1, Frame{wbase}, 0, 0, s, d, (int32_t)r, 2, (uint32_t)r, tt, tend, cbeg, wa, wb);
+                clen = locate(1, hc, Frame{wbase}, 0, 0, s, d, (int32_t)r, 2, (uint32_t)r, tt, tend, cbeg, wa, wb);
             }
             if (STATS) {
                 unsigned b = __ballot_sync(FULL, ok);
@@ -735,10 +869,9 @@ struct Search {
             bool keep = ok && clen > 0;
             unsigned kb = __ballot_sync(FULL, keep);
             if (kb) {
-                uint32_t cp = P(1);
                 Frame c = frame(1);
                 if (keep) {
-                    int sl = (int)(cp + __popc(kb & ((1u << lane) - 1u)));
+                    int sl = (int)(np1 + __popc(kb & ((1u << lane) - 1u)));
                     c.node(0, sl) = s;
                     c.node(1, sl) = d;
                     c.tprev(sl) = tt;
@@ -751,29 +884,30 @@ struct Search {
                         if (pl.anti[a].edge == 0) c.anti_t(anti_off(1), a, sl) = tt;
                 }
                 __syncwarp();
-                setP(1, cp + __popc(kb));
-                if (cp + __popc(kb) >= DESCEND) drain(1);
+                np1 += __popc(kb);
             }
         }
-        if (flush_at_end && k > 1 && P(1) > 0) drain(1);
     }
 
-    __device__ void run_task(const Task& tk) {
-        use_query(tk.query);
-        const int i = tk.level;
-        const int nb = q->plan.lv[i].nb;
+    // Put the donated task in slot h into its level's frame as the only parent; returns the level.
+    __device__ int take_task(unsigned long long h) {
+        const Task* t = tasks + h;
+        const uint32_t ql = __ldcg((const uint32_t*)t);     // query, level
+        use_query((int)(ql & 0xFFFFu));
+        const int i = (int)(ql >> 16);
+        const int nb = Hot::nb(hot(i));
         Frame f = frame(i);
         if (lane == 0) {
-            f.tprev(0) = tk.tprev;
-            set_tend(f, 0, tk.tprev, tk.tend);
-            f.beg(0) = tk.beg;
-            f.len(0) = tk.len;
-            f.root(0) = tk.root;
-            for (int s = 0; s < nb; ++s) f.node(s, 0) = tk.node[s];
+            const int64_t tprev = __ldcg(&t->tprev);
+            f.tprev(0) = tprev;
+            set_tend(f, 0, tprev, __ldcg(&t->tend));
+            f.beg(0) = __ldcg(&t->beg);
+            f.len(0) = __ldcg(&t->len);
+            f.root(0) = __ldcg(&t->root);
         }
+        if (lane < nb) f.node(lane, 0) = __ldcg(&t->node[lane]);
         __syncwarp();
-        setP(i, 1);
-        drain(i);
+        return i;
     }
 
     // Global chunk c -> query index (chunks of query j are contiguous).
@@ -786,7 +920,8 @@ struct Search {
         return lo;
     }
 
-    __device__ bool try_pop(Task& out) {
+    // Pop a published task; returns its slot, or NO_CHUNK when none is ready.
+    __device__ unsigned long long try_pop() {
         int got = 0;
         unsigned long long h = 0;
         if (lane == 0) {
@@ -802,17 +937,14 @@ struct Search {
                     __nanosleep(64);
                 }
                 if (st == 1) got = 1;
+                else atomicAdd(&ctrl->done_tasks, 1ULL);   // a void slot holds nothing to run
             }
         }
         got = __shfl_sync(FULL, got, 0);
-        if (!got) return false;
+        if (!got) return NO_CHUNK;
         h = __shfl_sync(FULL, h, 0);
         __threadfence();
-        const uint32_t* src = (const uint32_t*)(tasks + h);
-        uint32_t w = lane < 16 ? __ldcg(src + lane) : 0u;
-        uint32_t* dst = (uint32_t*)&out;
-        for (int j = 0; j < 16; ++j) dst[j] = __shfl_sync(FULL, w, j);
-        return true;
+        return h;
     }
 
     __device__ bool queue_empty() const {
@@ -821,71 +953,139 @@ struct Search {
         return h >= min(r, (unsigned long long)task_cap);
     }
 
-    __device__ void run(int nq, uint64_t total_chunks) {
-        if (MODE == MODE_COUNT && lane == 0) atomicAdd(&ctrl->busy, 1);
-        // phase 1: root chunks
-        while (true) {
-            unsigned long long c = 0;
-            if (lane == 0) c = atomicAdd(&ctrl->next_chunk, 1ULL);
-            c = __shfl_sync(FULL, c, 0);
-            if (c >= total_chunks) break;
-            int j = query_of_chunk(c, nq);
-            if (j != qi) {
-                // frames of the previous query must be empty before switching
-                if (MODE == MODE_COUNT && qi >= 0 && k > 1 && P(1) > 0) drain(1);
-                use_query(j);
-            }
-            uint64_t lc = c - q->chunk_base;
-            const uint64_t cr = (uint64_t)q->plan.tune.chunk_roots;
-            if (MODE == MODE_FILL) {
-                // claim index lc -> the lc-th listed chunk (one holding a match whose
-                // rows start below the cap); past the list's end the rest of this
-                // query is skipped
-                if (lc >= q->chunk_off[q->n_chunks + 1]) {
-                    unsigned long long nxt = (j + 1 < nq) ? qs[j + 1].chunk_base : total_chunks;
-                    if (lane == 0) atomicMax(&ctrl->next_chunk, nxt);
-                    continue;
-                }
-                lc = ((const uint32_t*)(q->chunk_off + q->n_chunks + 2))[lc];
-                out_base = q->chunk_off[lc];
-                out_local = 0;
-            }
-            const uint64_t r0 = q->root_begin + lc * cr;
-            const uint64_t r1 = min(q->root_end, r0 + cr);
-            roots(r0, r1, MODE == MODE_FILL);
-        }
-        if (MODE == MODE_COUNT && qi >= 0 && k > 1 && P(1) > 0) drain(1);
-        // phase 2 (count): help with donated subtrees until no warp holds work
-        if (MODE == MODE_COUNT) {
-            Task tk;
+    // Nothing is left to run and nothing can be donated any more: every chunk's
+    // subtree and every reserved task slot is done.  A donor reserves its slots before it
+    // reports its own chunk or task done, so done_tasks catching up with q_reserve
+    // after that is final.
+    __device__ bool all_done(uint64_t total_chunks) const {
+        if (*(volatile unsigned long long*)&ctrl->done_chunks < total_chunks) return false;
+        const unsigned long long d = *(volatile unsigned long long*)&ctrl->done_tasks;
+        __threadfence();
+        const unsigned long long r = *(volatile unsigned long long*)&ctrl->q_reserve;
+        return d >= min(r, (unsigned long long)task_cap);
+    }
+
+    // Wait for a task (true) or the end of the launch (false).  One warp per block
+    // polls the control block at a time and the block's other idle warps watch
+    // shared memory: thousands of warps polling one line delayed every claim and
+    // donation that goes through it.
+    __device__ bool wait_for_work(uint64_t total_chunks, int* poller, int* finished) {
+        int leave = 0;
+        if (lane == 0) {
+            atomicAdd(&ctrl->idle, 1);
+            const uint64_t t0 = now_ns();
+            unsigned ns = 128;
+            bool polling = false;
             while (true) {
-                if (try_pop(tk)) { run_task(tk); continue; }
-                int leave = 0;
-                if (lane == 0) {
-                    atomicSub(&ctrl->busy, 1);
-                    atomicAdd(&ctrl->idle, 1);
-                    uint64_t t0 = now_ns();
-                    unsigned ns = 256;
-                    while (true) {
-                        if (!queue_empty()) { atomicAdd(&ctrl->busy, 1); break; }
-                        int b = *(volatile int*)&ctrl->busy;
-                        if (b == 0) {
-                            // no warp holds work: leave unless a donation landed meanwhile
-                            __threadfence();
-                            if (queue_empty()) { leave = 1; break; }
+                if (*(volatile int*)finished) { leave = 1; break; }
+                if (!polling) polling = atomicCAS(poller, 0, 1) == 0;
+                if (polling) {
+                    if (!queue_empty()) break;
+                    if (all_done(total_chunks)) { *(volatile int*)finished = 1; leave = 1; break; }
+                }
+                if (now_ns() - t0 > WAIT_NS) { leave = 1; break; }
+                __nanosleep(ns);
+                if (ns < 2048) ns <<= 1;
+            }
+            if (polling) atomicExch(poller, 0);
+            if (!leave) atomicSub(&ctrl->idle, 1);
+        }
+        return __shfl_sync(FULL, leave, 0) == 0;
+    }
+
+    // Find the next frame to drain, in order: roots collected in frame 1 (root
+    // chunks are claimed and scanned until it is full enough or must be emptied), then
+    // donated tasks, until the launch has no work left.  One loop with one drain,
+    // so the search's code exists once per kernel.
+    __device__ void run(int nq, uint64_t total_chunks, int* poller, int* finished) {
+        uint32_t rb = 0, re = 0;                  // roots left of the current chunk
+        unsigned long long held = NO_CHUNK;       // claimed chunk of the next query, waiting for frame 1 to empty
+        bool scanning = true, ending = false;
+        while (true) {
+            int base = 1;
+            uint32_t np = 0;
+            bool is_task = false;
+            if (scanning) {
+                while (np1 < DESCEND) {
+                    if (nbuf >= 32u) { root_batch(); continue; }
+                    if (rb < re) {
+                        scan_roots(rb, re);
+                        rb = (rb & ~1u) + 64u;
+                        continue;
+                    }
+                    // the chunk is scanned; what it left in the root buffer and frame 1
+                    // stays for the next one, except where that belongs to another
+                    // query or (enumeration) writes from another offset
+                    if (MODE == MODE_FILL || held != NO_CHUNK || ending) {
+                        if (nbuf > 0u) { root_batch(); continue; }
+                        if (np1 > 0u) break;
+                        if (ending) { scanning = false; break; }
+                    }
+                    unsigned long long c = held;
+                    held = NO_CHUNK;
+                    if (c == NO_CHUNK) {
+                        if (lane == 0) c = atomicAdd(&ctrl->next_chunk, 1ULL);
+                        c = __shfl_sync(FULL, c, 0);
+                        if (c >= total_chunks) { ending = true; continue; }
+                        ++claimed;
+                    }
+                    const int j = query_of_chunk(c, nq);
+                    if (j != qi) {
+                        // nothing of the previous query may be left when switching
+                        if (np1 + nbuf > 0u) { held = c; continue; }
+                        use_query(j);
+                    }
+                    uint64_t lc = c - q->chunk_base;
+                    const uint64_t cr = (uint64_t)q->plan.tune.chunk_roots;
+                    if (MODE == MODE_FILL) {
+                        // claim index lc -> the lc-th listed chunk (one holding a match whose
+                        // rows start below the cap); past the list's end the rest of this
+                        // query is skipped
+                        if (lc >= q->chunk_off[q->n_chunks + 1]) {
+                            unsigned long long nxt = (j + 1 < nq) ? qs[j + 1].chunk_base : total_chunks;
+                            if (lane == 0) atomicMax(&ctrl->next_chunk, nxt);
                             continue;
                         }
-                        if (now_ns() - t0 > WAIT_NS) { leave = 1; break; }
-                        __nanosleep(ns);     // back off: waiting warps poll one shared line
-                        if (ns < 8192) ns <<= 1;
+                        lc = ((const uint32_t*)(q->chunk_off + q->n_chunks + 2))[lc];
+                        out_base = q->chunk_off[lc];
+                        out_local = 0;
                     }
-                    atomicSub(&ctrl->idle, 1);
+                    rb = (uint32_t)(q->root_begin + lc * cr);
+                    re = (uint32_t)min(q->root_end, (uint64_t)rb + cr);
                 }
-                leave = __shfl_sync(FULL, leave, 0);
-                if (leave) break;
+                np = np1;
+                np1 = 0;
+                if (np == 0) continue;
+            } else {
+                if (MODE == MODE_FILL) break;
+                report_chunks();
+                const unsigned long long slot = try_pop();
+                if (slot != NO_CHUNK) {
+                    base = take_task(slot);
+                    np = 1;
+                    is_task = true;
+                } else {
+                    // a launch of one query that never donates has nothing to wait for
+                    if (nq == 1 && qs[0].plan.tune.split_depth <= 0) break;
+                    if (!wait_for_work(total_chunks, poller, finished)) break;
+                    continue;
+                }
+            }
+            drain(base, np);
+            if (MODE == MODE_COUNT && is_task) {
+                __threadfence();      // donations made by this task are reserved before it counts as done
+                if (lane == 0) atomicAdd(&ctrl->done_tasks, 1ULL);
             }
         }
         flush();
+    }
+
+    // Count this warp's chunks as done, once their subtrees (and the slots they donated) are.
+    __device__ void report_chunks() {
+        if (!claimed) return;
+        __threadfence();
+        if (lane == 0) atomicAdd(&ctrl->done_chunks, (unsigned long long)claimed);
+        claimed = 0;
     }
 };
 
@@ -893,10 +1093,14 @@ template <int MODE, bool STATS, int FEAT>
 __global__ void __maxnreg__(56) search_kernel(const __grid_constant__ GraphView g,
                                                      const QueryDev* __restrict__ qs, int nq, int warp_smem,
                                                      Ctrl* ctrl, Task* tasks, uint8_t* ready, uint64_t task_cap) {
-    extern __shared__ __align__(16) char smem[];
+    __shared__ int poller, finished;
+    if (MODE == MODE_COUNT) {
+        if (threadIdx.x == 0) poller = finished = 0;
+        __syncthreads();
+    }
     const int warp = threadIdx.x >> 5;
-    Search<MODE, STATS, FEAT> s(g, qs, ctrl, tasks, ready, task_cap, smem + (size_t)warp * warp_smem);
-    s.run(nq, ctrl->total_chunks);
+    Search<MODE, STATS, FEAT> s(g, qs, ctrl, tasks, ready, task_cap, (uint32_t)(warp * warp_smem));
+    s.run(nq, ctrl->total_chunks, &poller, &finished);
 }
 
 }  // namespace
@@ -958,13 +1162,16 @@ const void* kernel_of(Mode mode, bool stats, unsigned feat) {
     return kernel_for<MODE_COUNT>(feat);
 }
 
+// dynamic shared memory a block may use beside the kernel's few static bytes
+constexpr int MAX_DYN_SMEM = 232448 - 64;
+
 // Resident blocks per SM for one launch shape, computed once per shape.
 int blocks_per_sm(const tm_graph* g, const void* fn, int kid, int threads, int smem) {
     uint64_t key = ((uint64_t)g->device << 56) | ((uint64_t)kid << 48) | ((uint64_t)threads << 32) | (uint64_t)smem;
     std::lock_guard<std::mutex> lk(g_cfg_mu);
     auto it = g_blocks_per_sm.find(key);
     if (it != g_blocks_per_sm.end()) return it->second;
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
     int blocks = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fn, threads, smem);
     cudaGetLastError();
@@ -974,11 +1181,31 @@ int blocks_per_sm(const tm_graph* g, const void* fn, int kid, int threads, int s
 }
 }  // namespace
 
+// Blocks of a launch: the resident grid, less when the root chunks are too few
+// to give each of its warps one (at least a block per SM stays to take donated
+// subtrees).  Idle warps are not free: claiming, waiting and leaving go
+// through a few shared lines.
+int launch_blocks(const tm_graph* g, const LaunchCfg& c, uint64_t total_chunks) {
+    const uint64_t need = (total_chunks + (uint64_t)c.warps_per_block - 1) / (uint64_t)c.warps_per_block;
+    return (int)std::min<uint64_t>((uint64_t)c.grid, std::max<uint64_t>(need, (uint64_t)g->num_sms));
+}
+
+// Roots a warp claims at a time, of `roots` in the launch.  Too few of them to
+// give each warp of a full grid (about 32 per SM) two chunks: smaller ones, down
+// to 8 roots.  There the longest chain of one warp's chunks is the launch's time,
+// not the number of claims.  Sizes set by the caller or picked by the tuner are kept.
+int effective_chunk(const tm_graph* g, const Plan& p, uint64_t roots) {
+    int cr = p.tune.chunk_roots;
+    if (p.auto_chunk)
+        while (cr > 8 && roots < 64ull * (uint64_t)g->num_sms * (uint64_t)cr) cr >>= 1;
+    return cr;
+}
+
 LaunchCfg search_launch_cfg(const tm_graph* g, Mode mode, int max_warp_smem, int warps_per_block) {
     LaunchCfg c;
     c.warps_per_block = std::max(1, std::min(16, warps_per_block));
-    // keep the block's frames within the 227 KB of shared memory a block may use
-    while (c.warps_per_block > 1 && max_warp_smem * c.warps_per_block > 232448) c.warps_per_block--;
+    // keep the block's frames within the shared memory a block may use
+    while (c.warps_per_block > 1 && max_warp_smem * c.warps_per_block > MAX_DYN_SMEM) c.warps_per_block--;
     c.smem_bytes = max_warp_smem * c.warps_per_block;
     int kid = mode == MODE_FILL ? 8 : 0;
     c.grid = blocks_per_sm(g, kernel_of(mode, false, 0u), kid, c.warps_per_block * 32, c.smem_bytes) * g->num_sms;
@@ -989,7 +1216,7 @@ tm_status launch_search(const tm_graph* g, Mode mode, const QueryDev* qdev_dev, 
                         int warps_per_block, unsigned feat, const Scratch* s, cudaStream_t st, int grid_override,
                         bool stats) {
     LaunchCfg c = search_launch_cfg(g, mode, max_warp_smem, warps_per_block);
-    int grid = grid_override > 0 ? grid_override : c.grid;
+    const int grid = grid_override > 0 ? std::min(grid_override, c.grid) : c.grid;
     if (mode == MODE_FILL) stats = false;
     const void* fn = kernel_of(mode, stats, feat);
     // the instance's shared-memory limit (set once per launch shape)

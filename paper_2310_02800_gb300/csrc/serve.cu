@@ -103,7 +103,7 @@ namespace {
 
 uint64_t req_bytes(const tm_graph* g, const Plan& p, int enumerate, uint64_t cap) {
     if (!enumerate) return 0;
-    uint64_t nch = ((uint64_t)g->v.m + p.tune.chunk_roots - 1) / (uint64_t)p.tune.chunk_roots;
+    uint64_t nch = n_chunks((uint64_t)g->v.m, effective_chunk(g, p, (uint64_t)g->v.m));
     return cap * (uint64_t)p.k * 4 + chunk_buf_bytes(nch) + scan_temp_bytes(nch + 1);
 }
 
@@ -119,11 +119,12 @@ double estimate(const tm_server* s, const Req* r) {
     return it == s->g->serve_cost_ms.end() ? -1.0 : it->second;
 }
 
-// The persistent grid of one launch: the full resident grid, or the configured share of it.
-int launch_grid(const tm_server* s, const LaunchCfg& c) {
-    const int pct = s->cfg.grid_pct;
-    if (pct <= 0 || pct >= 100) return c.grid;
-    return std::max(s->g->num_sms, c.grid * pct / 100);
+// The persistent grid of one launch over `chunks` root chunks: the resident
+// grid those chunks can use, within the configured share of it.
+int launch_grid(const tm_server* s, const LaunchCfg& c, uint64_t chunks) {
+    const int pct = s->cfg.grid_pct, blocks = launch_blocks(s->g, c, chunks);
+    if (pct <= 0 || pct >= 100) return blocks;
+    return std::min(blocks, std::max(s->g->num_sms, c.grid * pct / 100));
 }
 
 tm_status launch_batch(tm_server* s, Slot& sl) {
@@ -138,7 +139,7 @@ tm_status launch_batch(tm_server* s, Slot& sl) {
     // enumerate buffers (stream-ordered allocations: no device-wide sync)
     for (Req* q : sl.batch) {
         if (!q->enumerate) continue;
-        q->nch = (m + q->plan.tune.chunk_roots - 1) / (uint64_t)q->plan.tune.chunk_roots;
+        q->nch = n_chunks(m, effective_chunk(g, q->plan, m));
         TM_CUDA(dev_malloc_async((void**)&q->match, std::max<uint64_t>(q->cap * q->plan.k * 4, 16), sl.st));
         TM_CUDA(dev_malloc_async((void**)&q->chunk, chunk_buf_bytes(q->nch), sl.st));
         TM_CUDA(dev_malloc_async(&q->scan_tmp, scan_temp_bytes(q->nch + 1), sl.st));
@@ -156,9 +157,10 @@ tm_status launch_batch(tm_server* s, Slot& sl) {
         QueryDev* qd = cs.qdev_stage() + j;
         memset(qd, 0, sizeof(QueryDev));
         qd->plan = q->plan;
+        qd->plan.tune.chunk_roots = effective_chunk(g, q->plan, m);
         qd->root_begin = 0;
         qd->root_end = m;
-        qd->n_chunks = (m + q->plan.tune.chunk_roots - 1) / (uint64_t)q->plan.tune.chunk_roots;
+        qd->n_chunks = n_chunks(m, qd->plan.tune.chunk_roots);
         qd->chunk_base = base;
         base += qd->n_chunks;
         qd->total = cs.counters + j;
@@ -173,7 +175,7 @@ tm_status launch_batch(tm_server* s, Slot& sl) {
     TM_CUDA(cudaMemsetAsync(cs.counters, 0, (size_t)nq * 8, sl.st));
     TM_CUDA(cudaMemsetAsync(cs.ready, 0, cs.task_cap, sl.st));
     LaunchCfg lc = search_launch_cfg(g, MODE_COUNT, warp_smem, warps);
-    r = launch_search(g, MODE_COUNT, cs.qdev(), nq, warp_smem, warps, feat, &cs, sl.st, launch_grid(s, lc));
+    r = launch_search(g, MODE_COUNT, cs.qdev(), nq, warp_smem, warps, feat, &cs, sl.st, launch_grid(s, lc, base));
     if (r != TM_OK) return r;
     // fill launch over the enumerate requests
     int ne = 0;
@@ -191,6 +193,7 @@ tm_status launch_batch(tm_server* s, Slot& sl) {
         QueryDev* qd = fs.qdev_stage() + ne;
         memset(qd, 0, sizeof(QueryDev));
         qd->plan = q->plan;
+        qd->plan.tune.chunk_roots = effective_chunk(g, q->plan, m);
         qd->root_begin = 0;
         qd->root_end = m;
         qd->n_chunks = q->nch;
@@ -207,7 +210,7 @@ tm_status launch_batch(tm_server* s, Slot& sl) {
         fc->total_chunks = fbase;
         TM_CUDA(cudaMemcpyAsync(fs.head, fs.stage, fs.head_bytes(ne), cudaMemcpyHostToDevice, sl.st));
         LaunchCfg lf = search_launch_cfg(g, MODE_FILL, fsmem, warps);
-        r = launch_search(g, MODE_FILL, fs.qdev(), ne, fsmem, warps, ffeat, &fs, sl.st, launch_grid(s, lf));
+        r = launch_search(g, MODE_FILL, fs.qdev(), ne, fsmem, warps, ffeat, &fs, sl.st, launch_grid(s, lf, fbase));
         if (r != TM_OK) return r;
     }
     TM_CUDA(cudaMemcpyAsync(cs.counters_host, cs.counters, (size_t)nq * 8, cudaMemcpyDeviceToHost, sl.st));

@@ -133,12 +133,31 @@ struct LevelPlan {
     uint8_t n_look;    // later motif edges (after i+1) whose two nodes are first both bound by edge i
     int8_t look_u[TM_MAX_LOOK];  // their endpoint slots: an edge look_u -> look_v must exist in
     int8_t look_v[TM_MAX_LOOK];  // (t_i, t_root + delta], else no match extends this partial match
-    int8_t pad2[4];
+    uint32_t hot;            // the fields every step needs, packed (see Hot)
     int32_t frame_off;       // byte offset of this level's frame in a warp's shared block (count)
     int32_t frame_off_fill;  // same, enumerate-fill layout (frames also carry edge ids)
     int32_t anti_row_off;    // byte offset of the anti-edge time rows within this level's frame
     int32_t anti_row_off_fill;
     int64_t gap;             // t_i - t_{i-1} bound (INT64_MAX = none)
+};
+
+// LevelPlan::hot.  One 4-byte load per level change tells a step what kind of
+// level it is on, which slots it reads and which optional checks apply; the
+// rest of the plan is read only by the checks that need it.
+struct Hot {
+    static constexpr uint32_t ELABEL = 1u << 18, NLABEL = 1u << 19, ANTI = 1u << 20, LOOK = 1u << 21, GAP = 1u << 22;
+    static uint32_t pack(const LevelPlan& lp) {
+        return (uint32_t)lp.kind | (uint32_t)(lp.a & 7) << 2 | (uint32_t)(lp.b & 7) << 5 | (uint32_t)lp.nb << 8 |
+               (uint32_t)(lp.nx_a + 1) << 12 | (uint32_t)(lp.nx_b + 1) << 15 | (lp.elabel >= 0 ? ELABEL : 0u) |
+               (lp.nl0 >= 0 || lp.nl1 >= 0 ? NLABEL : 0u) | (lp.anti_mask ? ANTI : 0u) | (lp.n_look ? LOOK : 0u) |
+               (lp.gap != INT64_MAX ? GAP : 0u);
+    }
+    __host__ __device__ static int kind(uint32_t h) { return (int)(h & 3u); }
+    __host__ __device__ static int a(uint32_t h) { return (int)(h >> 2 & 7u); }
+    __host__ __device__ static int b(uint32_t h) { return (int)(h >> 5 & 7u); }
+    __host__ __device__ static int nb(uint32_t h) { return (int)(h >> 8 & 15u); }
+    __host__ __device__ static int nx_a(uint32_t h) { return (int)(h >> 12 & 7u) - 1; }
+    __host__ __device__ static int nx_b(uint32_t h) { return (int)(h >> 15 & 7u) - 1; }
 };
 
 // One temporal anti-edge (paper Section 2.1, Section 5.4.3), checked at the
@@ -169,7 +188,11 @@ struct Plan {
     uint64_t shape_hash;
     int32_t n_anti;
     uint8_t anti_mask0;            // anti-edges checked when the root binds edge 0
-    uint8_t pad1[3];
+    uint8_t root_need;             // lists a match rooted at an edge must continue in, one bit per SuccKind: bits 0-3
+                                   // within root_span, bits 4-7 (edge 1's own lists) within root_span_next
+    uint8_t auto_chunk;            // 1: tune.chunk_roots is the default and may shrink on small inputs
+    uint8_t pad1;
+    uint32_t root_span, root_span_next;   // delta, and min(delta, gap_0), as largest word gaps
     AntiPlan anti[TM_MAX_ANTI];
     LevelPlan lv[TM_MAX_EDGES];    // lv[i] for i = 1..k-1 (lv[0]: only the look-ahead of the root)
 };
@@ -203,7 +226,9 @@ inline int frame_bytes(int nb, int level, bool with_eids, int n_anti = 0) {
         return FrameLayout<FCAP_FILL>::NODE + 4 * FCAP_FILL * (nb + level) + 8 * FCAP_FILL * n_anti;
     return FrameLayout<FCAP_COUNT>::NODE + 4 * FCAP_COUNT * nb + 8 * FCAP_COUNT * n_anti;
 }
-constexpr int WARP_HDR = 128;      // per-warp header: level cursors
+// A warp's shared block starts with its root buffer: up to 31 roots left over
+// and the 64 of one scan step.
+constexpr int ROOT_BUF_BYTES = 96 * 4;
 
 tm_status build_plan(const tm_graph* g, const tm_motif* m, Plan* out);
 uint64_t plan_shape_hash(const tm_motif* m);
@@ -233,11 +258,13 @@ struct Ctrl {
     unsigned long long pad1[15];
     unsigned long long q_reserve;    // task slots reserved by donors
     unsigned long long q_head;       // next task slot to pop
-    int busy;                        // warps holding work
+    int pad3;
     int idle;                        // warps waiting for tasks
     unsigned int err;                // 0 or TM_E_TIMEOUT
     unsigned int donated;            // tasks donated (diagnostic)
-    unsigned long long pad2[12];
+    unsigned long long done_chunks;  // root chunks whose whole subtree has been searched
+    unsigned long long done_tasks;   // task slots run (or found void)
+    unsigned long long pad2[10];
 };
 static_assert(sizeof(Ctrl) == 384, "control block is three 128-byte lines");
 
@@ -325,10 +352,12 @@ struct LaunchGroup {
     int warp_smem;       // frame bytes per warp (largest of the group)
     int warps;           // warps per block
     unsigned feat;       // union of the group's plan features
+    int grid;            // blocks
 };
-// Groups of nq plans for `mode`; order[i] = index of the query at grouped position i.
-std::vector<LaunchGroup> occupancy_groups(const tm_graph* g, Mode mode, const Plan* const* plans, int nq,
-                                          int* order);
+// Groups of nq plans for `mode`, query j having nch[j] root chunks; order[i] =
+// index of the query at grouped position i.
+std::vector<LaunchGroup> occupancy_groups(const tm_graph* g, Mode mode, const Plan* const* plans,
+                                          const uint64_t* nch, int nq, int* order);
 
 // Launch the persistent search over nq queries (qdev already on the device).
 // Ctrl (incl. total_chunks) and qdev must already be initialised on the stream.
@@ -338,6 +367,9 @@ tm_status launch_search(const tm_graph* g, Mode mode, const QueryDev* qdev_dev, 
                         int max_warp_smem, int warps_per_block, unsigned feat,
                         const Scratch* s, cudaStream_t st, int grid_override = 0, bool stats = false);
 
+int launch_blocks(const tm_graph* g, const LaunchCfg& c, uint64_t total_chunks);
+int effective_chunk(const tm_graph* g, const Plan& p, uint64_t roots);
+uint64_t n_chunks(uint64_t roots, int chunk_roots);
 LaunchCfg search_launch_cfg(const tm_graph* g, Mode mode, int max_warp_smem, int warps_per_block);
 
 // ------------------------------------------------------------- primitives

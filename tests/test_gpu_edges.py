@@ -1,0 +1,86 @@
+"""Sizes at which the search's work splitting can go wrong, against the CPU oracle.
+
+Whole numbers throughout: results are equal or wrong.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def tmg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2310_02800_gb300 as m
+    m.lib()
+    return m
+
+
+def graph(n, m, span, seed, loops=True):
+    rng = np.random.default_rng(seed)
+    src = rng.integers(0, n, m).astype(np.int32)
+    dst = rng.integers(0, n, m).astype(np.int32)
+    if not loops:
+        dst = np.where(dst == src, (dst + 1) % n, dst).astype(np.int32)
+    t = rng.integers(0, span, m).astype(np.int64)
+    el = rng.integers(0, 3, m).astype(np.uint8)
+    nl = rng.integers(0, 2, n).astype(np.uint8)
+    return n, src, dst, t, el, nl
+
+
+MOTIFS = [
+    synth.Motif([(0, 1)], 0), synth.Motif([(0, 1)], 5, elabel=[1]),
+    synth.Motif([(0, 1), (1, 2)], 60), synth.Motif([(0, 1), (2, 3)], 40),
+    synth.Motif([(0, 1), (1, 0), (0, 1)], 200), synth.cycle(3, 300), synth.Motif([(0, 1), (1, 2), (2, 0)], 300, [90, 200]),
+    synth.out_star(3, 90), synth.in_star(3, 90), synth.Motif([(0, 1), (1, 2), (2, 3)], 120, elabel=[2, -1, 0]),
+    synth.Motif([(0, 1), (1, 2), (2, 3), (3, 0)], 400, nlabel=[1, -1, 0, -1]),
+    synth.Motif([(0, 1), (1, 2), (2, 0)], 300, anti=[(1, 0, 0, 100)]),
+]
+
+
+@pytest.mark.parametrize("m", [1, 2, 31, 32, 33, 63, 64, 65, 127, 129, 511, 2047, 5001])
+def test_root_scan_edges(tmg, m):
+    """Graphs around the 64-root scan step and the smallest chunks; root ranges that start and
+    end on odd edges: totals, per-root counts and every row."""
+    n, src, dst, t, el, nl = graph(max(3, min(24, m)), m, max(8, m * 2), seed=m)
+    og = oracle.Graph(n, src, dst, t, el, nl)
+    gg = tmg.Graph.load(n, src, dst, t, el, nl)
+    for mo in MOTIFS:
+        q = gg.compile(mo)
+        want, want_pr = og.count(mo, per_root=True)
+        pr = torch.full((m,), -1, dtype=torch.int64, device="cuda")
+        assert q.count(per_root=pr) == want, mo
+        assert np.array_equal(pr.cpu().numpy(), want_pr.astype(np.int64)), mo
+        for a, b in ((0, m), (1, m), (m // 3, m - m // 5), (m // 2, m // 2), (m - 1, m)):
+            part = torch.full((b - a,), -1, dtype=torch.int64, device="cuda")
+            assert q.count_roots(a, b, per_root=part) == int(want_pr[a:b].sum()), (mo, a, b)
+            assert np.array_equal(part.cpu().numpy(), want_pr[a:b].astype(np.int64)), (mo, a, b)
+        rows = og.enumerate(mo, cap=want + 1)[0]
+        out = torch.full((want + 1, mo.k), -7, dtype=torch.int32, device="cuda")
+        assert q.enumerate(out)[:2] == (want, want), mo
+        assert np.array_equal(out[:want].cpu().numpy(), rows), mo
+
+
+@pytest.mark.parametrize("nq", [1, 7, 64])
+def test_many_queries_on_a_small_graph(tmg, nq):
+    """A batch whose warps switch queries with roots still buffered: totals of every batched form."""
+    n, src, dst, t, el, nl = graph(30, 3001, 6000, seed=nq)
+    og = oracle.Graph(n, src, dst, t, el, nl)
+    gg = tmg.Graph.load(n, src, dst, t, el, nl)
+    mos = [MOTIFS[(5 * j) % len(MOTIFS)] for j in range(nq)]
+    qs = [gg.compile(mo) for mo in mos]
+    want = [og.count(mo, per_root=True)[0] for mo in mos]
+    assert gg.count_batch(qs) == want
+    tot = torch.zeros(nq, dtype=torch.int64, device="cuda")
+    assert gg.count_batch_noalloc(qs, tot).tolist() == want
+    outs = [torch.full((max(1, w), mo.k), -7, dtype=torch.int32, device="cuda") for w, mo in zip(want, mos)]
+    nw, tots, trunc = gg.enumerate_batch(qs, outs)
+    assert tots == want and nw == want and not trunc
+    for mo, w, o in zip(mos, want, outs):
+        assert np.array_equal(o[:w].cpu().numpy(), og.enumerate(mo, cap=w + 1)[0]), mo
