@@ -50,106 +50,125 @@ __global__ void check_kernel(const int32_t* __restrict__ src, const int32_t* __r
     }
 }
 
+template <typename K>
 __global__ void time_keys_kernel(const int64_t* __restrict__ t, int64_t m, unsigned long long tmin,
-                                 uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        keys[i] = (uint64_t)t[i] - tmin;
-        vals[i] = (uint32_t)i;
-    }
-}
-
-__global__ void iota_kernel(uint32_t* __restrict__ v, int64_t m) {
+                                 K* __restrict__ keys) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
-        v[i] = (uint32_t)i;
+        keys[i] = (K)((uint64_t)t[i] - tmin);
 }
 
-__global__ void gather_edges_kernel(const uint32_t* __restrict__ perm, int64_t m, const int32_t* __restrict__ src,
+// Elements a thread of the gather kernels takes at a time: their loads are all
+// issued before the first is used, since each is a sector from anywhere in the column.
+constexpr int GATHER = 4;
+
+// Edge columns in edge-id order.  The sorted keys are the times; without them
+// (keys null) the input is in time order already and perm is null too.
+template <typename K>
+__global__ void gather_edges_kernel(const uint32_t* __restrict__ perm, const K* __restrict__ keys,
+                                    unsigned long long tmin, int64_t m, const int32_t* __restrict__ src,
                                     const int32_t* __restrict__ dst, const int64_t* __restrict__ t,
                                     const uint8_t* __restrict__ el, int32_t* __restrict__ src_o,
                                     int32_t* __restrict__ dst_o, int64_t* __restrict__ t_o, uint8_t* __restrict__ el_o,
                                     int32_t* __restrict__ perm_o) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t i = perm[e];
-        src_o[e] = src[i];
-        dst_o[e] = dst[i];
-        t_o[e] = t[i];
-        if (el) el_o[e] = el[i];
-        perm_o[e] = (int32_t)i;
-    }
-}
-
-// Degree histogram.  Lanes of a warp holding the same node add once for the
-// group: on power-law inputs a hub takes a large share of all endpoints, and
-// one atomic per edge on its counter serialises.  blockDim is a multiple of 32.
-__global__ void degree_kernel(const int32_t* __restrict__ node, int64_t m, unsigned long long* __restrict__ deg) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < m; base += stride) {
-        const int64_t e = base + threadIdx.x;
-        const unsigned act = __ballot_sync(0xffffffffu, e < m);
-        if (e >= m) continue;
-        const int32_t v = node[e];
-        const unsigned grp = __match_any_sync(act, v);
-        if ((int)(threadIdx.x & 31) == __ffs(grp) - 1) atomicAdd(&deg[v], (unsigned long long)__popc(grp));
+    for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e0 < m; e0 += GATHER * stride) {
+        uint32_t i[GATHER];
+        int32_t s[GATHER], d[GATHER];
+        int64_t tt[GATHER];
+#pragma unroll
+        for (int j = 0; j < GATHER; ++j) {
+            const int64_t e = e0 + j * stride;
+            i[j] = e >= m ? 0u : perm ? perm[e] : (uint32_t)e;
+        }
+#pragma unroll
+        for (int j = 0; j < GATHER; ++j) {
+            const int64_t e = e0 + j * stride;
+            s[j] = src[i[j]];
+            d[j] = dst[i[j]];
+            tt[j] = e >= m ? 0 : keys ? (int64_t)((unsigned long long)keys[e] + tmin) : t[e];
+        }
+#pragma unroll
+        for (int j = 0; j < GATHER; ++j) {
+            const int64_t e = e0 + j * stride;
+            if (e >= m) break;
+            src_o[e] = s[j];
+            dst_o[e] = d[j];
+            t_o[e] = tt[j];
+            if (el) el_o[e] = el[i[j]];
+            perm_o[e] = (int32_t)i[j];
+        }
     }
 }
 
-__global__ void node_keys_kernel(const int32_t* __restrict__ node, int64_t m, uint32_t* __restrict__ keys,
-                                 uint32_t* __restrict__ vals) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        keys[e] = (uint32_t)node[e];
-        vals[e] = (uint32_t)e;
+// List offsets from the list's sorted node column: off[v] = first entry of a
+// node >= v.  (A binary search per node, neighbouring threads on neighbouring nodes:
+// a degree histogram by atomics took 190 and 280 us for 10M edges, this 20.)
+__global__ void offsets_kernel(const uint32_t* __restrict__ nodes, int64_t m, int64_t n1, uint32_t* __restrict__ off) {
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n1; v += (int64_t)gridDim.x * blockDim.x) {
+        uint32_t lo = 0, hi = (uint32_t)m;
+        while (lo < hi) {
+            const uint32_t mid = lo + ((hi - lo) >> 1);
+            if ((int64_t)nodes[mid] < v) lo = mid + 1; else hi = mid;
+        }
+        off[v] = lo;
     }
 }
 
-__global__ void offsets_kernel(const unsigned long long* __restrict__ off64, int64_t n1, uint32_t* __restrict__ off) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n1; i += (int64_t)gridDim.x * blockDim.x)
-        off[i] = (uint32_t)off64[i];
-}
-
+// List columns (time, other endpoint, edge id) from the list's edge ids.
 __global__ void list_columns_kernel(const uint32_t* __restrict__ eids, int64_t m, const int64_t* __restrict__ t,
                                     const int32_t* __restrict__ other, int64_t* __restrict__ at,
-                                    int32_t* __restrict__ anbr, int32_t* __restrict__ aeid,
-                                    uint32_t* __restrict__ pos_of_edge) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t e = eids[i];
-        at[i] = t[e];
-        anbr[i] = other[e];
-        aeid[i] = (int32_t)e;
-        pos_of_edge[e] = (uint32_t)i;
+                                    int32_t* __restrict__ anbr, int32_t* __restrict__ aeid) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < m; i0 += GATHER * stride) {
+        uint32_t e[GATHER];
+        int64_t tt[GATHER];
+        int32_t o[GATHER];
+#pragma unroll
+        for (int j = 0; j < GATHER; ++j) e[j] = i0 + j * stride < m ? eids[i0 + j * stride] : 0u;
+#pragma unroll
+        for (int j = 0; j < GATHER; ++j) {
+            tt[j] = t[e[j]];
+            o[j] = other[e[j]];
+        }
+#pragma unroll
+        for (int j = 0; j < GATHER; ++j) {
+            const int64_t i = i0 + j * stride;
+            if (i >= m) break;
+            at[i] = tt[j];
+            anbr[i] = o[j];
+            aeid[i] = (int32_t)e[j];
+        }
     }
 }
 
-// Successor index by list position (see GraphView::pnx): the words of the
-// edge at each list position.
+// Successor index by list position (see GraphView::pnx), the two words that
+// were found in the other direction's order: position i's edge's word.
 __global__ void successor_by_position_kernel(int64_t m, const int32_t* __restrict__ aeid_out,
-                                             const int32_t* __restrict__ aeid_in, const uint2* __restrict__ so_src,
-                                             const uint2* __restrict__ so_dst, const uint2* __restrict__ si_dst,
-                                             const uint2* __restrict__ si_src, uint2* __restrict__ p_out_same,
-                                             uint2* __restrict__ p_out_dst, uint2* __restrict__ p_in_same,
+                                             const int32_t* __restrict__ aeid_in, const uint2* __restrict__ so_dst,
+                                             const uint2* __restrict__ si_src, uint2* __restrict__ p_out_dst,
                                              uint2* __restrict__ p_in_src) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t eo = aeid_out[i], ei = aeid_in[i];
-        p_out_same[i] = so_src[eo];
-        p_out_dst[i] = so_dst[eo];
-        p_in_same[i] = si_dst[ei];
-        p_in_src[i] = si_src[ei];
-    }
-}
-
-__global__ void keys_by_perm_kernel(const int32_t* __restrict__ node, const uint32_t* __restrict__ perm, int64_t m,
-                                    uint32_t* __restrict__ keys) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
-        keys[i] = (uint32_t)node[perm[i]];
-}
-
-__global__ void pair_columns_kernel(const uint32_t* __restrict__ eids, int64_t m, const int64_t* __restrict__ t,
-                                    const int32_t* __restrict__ dst, int32_t* __restrict__ pnbr,
-                                    int64_t* __restrict__ pt, int32_t* __restrict__ peid) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t e = eids[i];
-        pnbr[i] = dst[e];
-        pt[i] = t[e];
-        peid[i] = (int32_t)e;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < m; i0 += GATHER * stride) {
+        int32_t eo[GATHER], ei[GATHER];
+        uint2 wo[GATHER], wi[GATHER];
+#pragma unroll
+        for (int j = 0; j < GATHER; ++j) {
+            const int64_t i = i0 + j * stride;
+            eo[j] = i < m ? aeid_out[i] : 0;
+            ei[j] = i < m ? aeid_in[i] : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < GATHER; ++j) {
+            wo[j] = so_dst[eo[j]];
+            wi[j] = si_src[ei[j]];
+        }
+#pragma unroll
+        for (int j = 0; j < GATHER; ++j) {
+            const int64_t i = i0 + j * stride;
+            if (i >= m) break;
+            p_out_dst[i] = wo[j];
+            p_in_src[i] = wi[j];
+        }
     }
 }
 
@@ -184,31 +203,30 @@ __device__ __forceinline__ uint2 succ_word(const int64_t* __restrict__ t, uint32
     return make_uint2(p, d < SUCC_FAR ? (uint32_t)d : SUCC_FAR);
 }
 
-// Successor index: for every edge e = (u, v, t), the first position after t in
-// each of the four lists that touch it: out(u), in(v) (where e itself sits,
-// so the search starts just past e), out(v) and in(u), with the time gap to
-// that entry.  A search level whose candidate list belongs to an endpoint of
+// Successor index of one direction's lists, in list order.  Entry i of node v's
+// list is edge e at time te: the first later entry of the same list (the search
+// starts just past i) and the first later entry of v's list in the other direction,
+// each with its time gap.  A search level whose candidate list belongs to an endpoint of
 // the previous level's edge reads its window start here instead of
 // binary-searching the list, and skips the window when the gap already
-// exceeds it.
-__global__ void successor_kernel(int64_t m, const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
-                                 const int64_t* __restrict__ t, const uint32_t* __restrict__ off_out,
-                                 const int64_t* __restrict__ at_out, const uint32_t* __restrict__ off_in,
-                                 const int64_t* __restrict__ at_in, const uint32_t* __restrict__ pos_out,
-                                 const uint32_t* __restrict__ pos_in, uint2* __restrict__ so_src,
-                                 uint2* __restrict__ si_dst, uint2* __restrict__ so_dst,
-                                 uint2* __restrict__ si_src) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t u = src[e], v = dst[e];
-        const int64_t te = t[e];
-        uint32_t hi = off_out[u + 1];
-        so_src[e] = succ_word(at_out, first_later_from(at_out, pos_out[e] + 1, hi, te), hi, te);
-        hi = off_in[v + 1];
-        si_dst[e] = succ_word(at_in, first_later_from(at_in, pos_in[e] + 1, hi, te), hi, te);
-        hi = off_out[v + 1];
-        so_dst[e] = succ_word(at_out, first_later(at_out, off_out[v], hi, te), hi, te);
-        hi = off_in[u + 1];
-        si_src[e] = succ_word(at_in, first_later(at_in, off_in[u], hi, te), hi, te);
+// exceeds it.  In list order, neighbouring threads search the same node's lists
+// around the same times, so the searches stay in L1; by edge id every
+// thread of a warp searched another node's list.
+__global__ void successor_kernel(int64_t m, const uint32_t* __restrict__ nodes, const int32_t* __restrict__ eid,
+                                 const uint32_t* __restrict__ off, const int64_t* __restrict__ at,
+                                 const uint32_t* __restrict__ off_x, const int64_t* __restrict__ at_x,
+                                 uint2* __restrict__ same_by_pos, uint2* __restrict__ same_by_edge,
+                                 uint2* __restrict__ cross_by_edge) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t v = nodes[i];
+        const int32_t e = eid[i];
+        const int64_t te = at[i];
+        uint32_t hi = off[v + 1];
+        const uint2 w = succ_word(at, first_later_from(at, (uint32_t)i + 1u, hi, te), hi, te);
+        same_by_pos[i] = w;
+        same_by_edge[e] = w;
+        hi = off_x[v + 1];
+        cross_by_edge[e] = succ_word(at_x, first_later(at_x, off_x[v], hi, te), hi, te);
     }
 }
 
@@ -349,26 +367,17 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
         return TM_E_INVALID;
     }
     // 2. time order
-    uint32_t *perm_a, *perm_b;
-    TRY(tmp.get(&perm_a, m));
-    TRY(tmp.get(&perm_b, m));
-    size_t rtemp_bytes = radix_temp_bytes((uint64_t)m);
+    const uint64_t um = (uint64_t)m;
+    const int grid = grid_for(m, sms), grid4 = grid_for((m + GATHER - 1) / GATHER, sms);
+    uint32_t *ka[2], *kb[2], *va[2], *keys_of[2];
+    for (int j = 0; j < 2; ++j) {
+        TRY(tmp.get(&ka[j], m));
+        TRY(tmp.get(&kb[j], m));
+        TRY(tmp.get(&va[j], m));
+    }
+    size_t rtemp_bytes = radix_temp_bytes(um);
     void* rtemp;
     TRY(tmp.get((char**)&rtemp, rtemp_bytes));
-    if (m > 0 && hc.descents > 0) {
-        uint64_t *ka, *kb;
-        TRY(tmp.get(&ka, m));
-        TRY(tmp.get(&kb, m));
-        time_keys_kernel<<<grid_for(m, sms), 256, 0, st>>>(t, m, hc.tmin, ka, perm_a);
-        note_launches(1);
-        TM_CUDA(cudaGetLastError());
-        TRY(radix_sort_pairs(ka, kb, perm_a, perm_b, (uint64_t)m, bits_for(hc.tmax - hc.tmin), rtemp, rtemp_bytes, st));
-    } else if (m > 0) {
-        iota_kernel<<<grid_for(m, sms), 256, 0, st>>>(perm_a, m);
-        note_launches(1);
-        TM_CUDA(cudaGetLastError());
-    }
-    // 3. edge columns in edge-id order
     int32_t *s_o, *d_o, *p_o;
     int64_t* t_o;
     uint8_t* el_o = nullptr;
@@ -377,25 +386,40 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
     TRY(owned(g, &t_o, m));
     TRY(owned(g, &p_o, m));
     if (el) TRY(owned(g, &el_o, m));
+    // 3. edge columns in edge-id order
     if (m > 0) {
-        gather_edges_kernel<<<grid_for(m, sms), 256, 0, st>>>(perm_a, m, src, dst, t, el, s_o, d_o, t_o, el_o, p_o);
+        const int tbits = bits_for(hc.tmax - hc.tmin);
+        int w = 0;
+        if (hc.descents == 0) {
+            gather_edges_kernel<uint32_t><<<grid4, 256, 0, st>>>(nullptr, nullptr, 0, m, src, dst, t, el, s_o, d_o, t_o,
+                                                                 el_o, p_o);
+        } else if (tbits <= 32) {
+            // a time range below 2^32: 4-byte keys
+            time_keys_kernel<uint32_t><<<grid, 256, 0, st>>>(t, m, hc.tmin, kb[0]);
+            note_launches(1);
+            TM_CUDA(cudaGetLastError());
+            TRY(radix_sort_pairs<uint32_t>(kb[0], nullptr, ka, va, um, tbits, rtemp, rtemp_bytes, st, &w));
+            gather_edges_kernel<uint32_t><<<grid4, 256, 0, st>>>(va[w], ka[w], hc.tmin, m, src, dst, t, el, s_o, d_o, t_o,
+                                                                 el_o, p_o);
+        } else {
+            uint64_t *k0, *k8[2];
+            TRY(tmp.get(&k0, m));
+            TRY(tmp.get(&k8[0], m));
+            TRY(tmp.get(&k8[1], m));
+            time_keys_kernel<uint64_t><<<grid, 256, 0, st>>>(t, m, hc.tmin, k0);
+            note_launches(1);
+            TM_CUDA(cudaGetLastError());
+            TRY(radix_sort_pairs<uint64_t>(k0, nullptr, k8, va, um, tbits, rtemp, rtemp_bytes, st, &w));
+            gather_edges_kernel<uint64_t><<<grid4, 256, 0, st>>>(va[w], k8[w], hc.tmin, m, src, dst, t, el, s_o, d_o, t_o,
+                                                                 el_o, p_o);
+        }
         note_launches(1);
         TM_CUDA(cudaGetLastError());
     }
     v.src = s_o; v.dst = d_o; v.t = t_o; v.elabel = el_o;
     g->perm = p_o;
-    // 4. adjacency lists
-    unsigned long long* deg;
-    TRY(tmp.get(&deg, n + 1));
-    size_t stemp_bytes = scan_temp_bytes((uint64_t)(n + 1));
-    void* stemp;
-    TRY(tmp.get((char**)&stemp, stemp_bytes));
-    uint32_t *nk_a, *nk_b, *pos_edge[2];
-    TRY(tmp.get(&nk_a, m));
-    TRY(tmp.get(&nk_b, m));
-    TRY(tmp.get(&pos_edge[0], m));
-    TRY(tmp.get(&pos_edge[1], m));
-    int nbits = bits_for((unsigned long long)(n > 0 ? n - 1 : 0));
+    // 4. adjacency lists: edge ids sorted by endpoint, stably, are in time order per node
+    const int nbits = bits_for((unsigned long long)(n > 0 ? n - 1 : 0));
     for (int dir = 0; dir < 2; ++dir) {
         const int32_t* key_node = dir == 0 ? s_o : d_o;
         const int32_t* other = dir == 0 ? d_o : s_o;
@@ -406,30 +430,23 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
         TRY(owned(g, &at, m));
         TRY(owned(g, &anbr, m));
         TRY(owned(g, &aeid, m));
-        TM_CUDA(cudaMemsetAsync(deg, 0, (n + 1) * sizeof(unsigned long long), st));
-        if (m > 0) {
-            degree_kernel<<<grid_for(m, sms), 256, 0, st>>>(key_node, m, deg);
-            note_launches(1);
-            TM_CUDA(cudaGetLastError());
-        }
-        TRY(exclusive_scan_u64(deg, deg, (uint64_t)(n + 1), stemp, st));
-        offsets_kernel<<<grid_for(n + 1, sms), 256, 0, st>>>(deg, n + 1, off);
+        uint32_t** nk = dir == 0 ? ka : kb;       // both directions' sorted nodes stay for step 6
+        int w = 0;
+        TRY(radix_sort_pairs<uint32_t>((const uint32_t*)key_node, nullptr, nk, va, um, nbits, rtemp, rtemp_bytes, st, &w));
+        keys_of[dir] = nk[w];
+        offsets_kernel<<<grid_for(n + 1, sms), 256, 0, st>>>(keys_of[dir], m, n + 1, off);
         note_launches(1);
         TM_CUDA(cudaGetLastError());
         if (m > 0) {
-            node_keys_kernel<<<grid_for(m, sms), 256, 0, st>>>(key_node, m, nk_a, perm_a);
-            note_launches(1);
-            TM_CUDA(cudaGetLastError());
-            TRY(radix_sort_pairs32(nk_a, nk_b, perm_a, perm_b, (uint64_t)m, nbits, rtemp, rtemp_bytes, st));
-            list_columns_kernel<<<grid_for(m, sms), 256, 0, st>>>(perm_a, m, t_o, other, at, anbr, aeid,
-                                                                   pos_edge[dir]);
+            list_columns_kernel<<<grid4, 256, 0, st>>>(va[w], m, t_o, other, at, anbr, aeid);
             note_launches(1);
             TM_CUDA(cudaGetLastError());
         }
         v.off[dir] = off; v.at[dir] = at; v.anbr[dir] = anbr; v.aeid[dir] = aeid;
     }
-    // 5. pair-ordered out-lists: stable sorts of the time-ordered edge ids by
-    //    destination, then by source, give (source, destination, time) order
+    // 5. pair-ordered out-lists: the in-lists hold the edges by (destination, time) with
+    //    their sources beside them, so one more stable sort, by source, gives
+    //    (source, destination, time) order
     {
         int32_t *pn, *pe;
         int64_t* ptm;
@@ -437,40 +454,32 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
         TRY(owned(g, &ptm, m));
         TRY(owned(g, &pe, m));
         if (m > 0) {
-            node_keys_kernel<<<grid_for(m, sms), 256, 0, st>>>(d_o, m, nk_a, perm_a);
-            note_launches(1);
-            TM_CUDA(cudaGetLastError());
-            TRY(radix_sort_pairs32(nk_a, nk_b, perm_a, perm_b, (uint64_t)m, nbits, rtemp, rtemp_bytes, st));
-            keys_by_perm_kernel<<<grid_for(m, sms), 256, 0, st>>>(s_o, perm_a, m, nk_a);
-            note_launches(1);
-            TM_CUDA(cudaGetLastError());
-            TRY(radix_sort_pairs32(nk_a, nk_b, perm_a, perm_b, (uint64_t)m, nbits, rtemp, rtemp_bytes, st));
-            pair_columns_kernel<<<grid_for(m, sms), 256, 0, st>>>(perm_a, m, t_o, d_o, pn, ptm, pe);
+            uint32_t* pk[2];                      // the sorted sources are not needed
+            for (int j = 0; j < 2; ++j) TRY(tmp.get(&pk[j], m));
+            int w = 0;
+            TRY(radix_sort_pairs<uint32_t>((const uint32_t*)v.anbr[1], (const uint32_t*)v.aeid[1], pk, va, um, nbits,
+                                           rtemp, rtemp_bytes, st, &w));
+            list_columns_kernel<<<grid4, 256, 0, st>>>(va[w], m, t_o, d_o, ptm, pn, pe);
             note_launches(1);
             TM_CUDA(cudaGetLastError());
         }
         v.pnbr = pn; v.pt = ptm; v.peid = pe;
     }
     // 6. successor index (window starts for lists that touch the previous edge)
-    uint2* nx[4];
+    uint2 *nx[4], *px[4];
     for (int j = 0; j < 4; ++j) TRY(owned(g, &nx[j], m));
+    for (int j = 0; j < 4; ++j) TRY(owned(g, &px[j], m));
     if (m > 0) {
-        successor_kernel<<<grid_for(m, sms), 256, 0, st>>>(m, s_o, d_o, t_o, v.off[0], v.at[0], v.off[1], v.at[1],
-                                                           pos_edge[0], pos_edge[1], nx[NX_OUT_SRC], nx[NX_IN_DST],
-                                                           nx[NX_OUT_DST], nx[NX_IN_SRC]);
-        note_launches(1);
+        successor_kernel<<<grid, 256, 0, st>>>(m, keys_of[0], v.aeid[0], v.off[0], v.at[0], v.off[1], v.at[1], px[0],
+                                               nx[NX_OUT_SRC], nx[NX_IN_SRC]);
+        successor_kernel<<<grid, 256, 0, st>>>(m, keys_of[1], v.aeid[1], v.off[1], v.at[1], v.off[0], v.at[0], px[2],
+                                               nx[NX_IN_DST], nx[NX_OUT_DST]);
+        successor_by_position_kernel<<<grid4, 256, 0, st>>>(m, v.aeid[0], v.aeid[1], nx[NX_OUT_DST], nx[NX_IN_SRC],
+                                                           px[1], px[3]);
+        note_launches(3);
         TM_CUDA(cudaGetLastError());
     }
     for (int j = 0; j < 4; ++j) v.nxt[j] = nx[j];
-    uint2* px[4];
-    for (int j = 0; j < 4; ++j) TRY(owned(g, &px[j], m));
-    if (m > 0) {
-        successor_by_position_kernel<<<grid_for(m, sms), 256, 0, st>>>(
-            m, v.aeid[0], v.aeid[1], nx[NX_OUT_SRC], nx[NX_OUT_DST], nx[NX_IN_DST], nx[NX_IN_SRC], px[0], px[1], px[2],
-            px[3]);
-        note_launches(1);
-        TM_CUDA(cudaGetLastError());
-    }
     for (int j = 0; j < 4; ++j) v.pnx[j] = px[j];
     TM_CUDA(cudaStreamSynchronize(st));
     return TM_OK;

@@ -380,12 +380,13 @@ size_t scan_temp_bytes(uint64_t n);
 tm_status exclusive_scan_u64(const unsigned long long* in, unsigned long long* out, uint64_t n,
                              void* temp, cudaStream_t st);
 
-// Stable LSD radix sort of (key, value) pairs on the low `bits` bits of key.
-// keys/vals are double-buffered: on return *_a holds the result.
-tm_status radix_sort_pairs(uint64_t* keys_a, uint64_t* keys_b, uint32_t* vals_a, uint32_t* vals_b,
-                           uint64_t n, int bits, void* temp, size_t temp_bytes, cudaStream_t st);
-tm_status radix_sort_pairs32(uint32_t* keys_a, uint32_t* keys_b, uint32_t* vals_a, uint32_t* vals_b,
-                             uint64_t n, int bits, void* temp, size_t temp_bytes, cudaStream_t st);
+// Stable LSD radix sort of (key, value) pairs on the low `bits` bits of the key
+// (K: uint32_t or uint64_t).  keys_in / vals_in are read only (vals_in may be null:
+// the values are then 0 .. n-1); keys[] and vals[] are two buffers each, of which
+// number *which holds the result.
+template <typename K>
+tm_status radix_sort_pairs(const K* keys_in, const uint32_t* vals_in, K* const keys[2], uint32_t* const vals[2],
+                           uint64_t n, int bits, void* temp, size_t temp_bytes, cudaStream_t st, int* which);
 size_t radix_temp_bytes(uint64_t n);
 
 }  // namespace tmg
