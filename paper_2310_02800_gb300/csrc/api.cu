@@ -179,12 +179,6 @@ tm_status build_plan(const tm_graph* g, const tm_motif* m, Plan* out) {
         }
         for (int a = 0; a < m->n_anti; ++a)
             if (anti_level[a] == i) lp.anti_mask |= (uint8_t)(1u << a);
-        lp.frame_off = off_c;
-        lp.frame_off_fill = off_f;
-        lp.anti_row_off = frame_bytes(lp.nb, i, false);
-        lp.anti_row_off_fill = frame_bytes(lp.nb, i, true);
-        off_c += frame_bytes(lp.nb, i, false, m->n_anti);
-        off_f += frame_bytes(lp.nb, i, true, m->n_anti);
     }
     for (int a = 0; a < m->n_anti; ++a) {
         p.anti[a].xs = (int8_t)slot[m->anti_src[a]];
@@ -214,6 +208,26 @@ tm_status build_plan(const tm_graph* g, const tm_motif* m, Plan* out) {
         L.n_look++;
     }
     for (int i = 0; i < k; ++i) p.lv[i].hot = Hot::pack(p.lv[i]);
+    for (int i = 1; i < k; ++i) {
+        LevelPlan& lp = p.lv[i];
+        const bool filter = (lp.hot & Hot::FILT) != 0;
+        if (filter) {
+            // a look-ahead pair joins the new node (slot nb) and a bound one
+            lp.fdir = lp.look_u[0] == lp.nb ? 1 : 0;
+            lp.fx = lp.fdir ? lp.look_v[0] : lp.look_u[0];
+            const int px = slot[m->esrc[i - 1]], py = slot[m->edst[i - 1]];
+            lp.fnx = lp.fx == px ? (lp.fdir ? NX_IN_SRC : NX_OUT_SRC)
+                   : lp.fx == py ? (lp.fdir ? NX_IN_DST : NX_OUT_DST) : NX_NONE;
+        }
+        lp.frame_off = off_c;
+        lp.frame_off_fill = off_f;
+        lp.anti_row_off = frame_bytes(lp.nb, i, false);
+        lp.anti_row_off_fill = frame_bytes(lp.nb, i, true);
+        lp.filt_off = frame_bytes(lp.nb, i, false, m->n_anti);
+        lp.filt_off_fill = frame_bytes(lp.nb, i, true, m->n_anti);
+        off_c += frame_bytes(lp.nb, i, false, m->n_anti, filter);
+        off_f += frame_bytes(lp.nb, i, true, m->n_anti, filter);
+    }
     p.warp_smem = (off_c + 15) & ~15;
     p.warp_smem_fill = (off_f + 15) & ~15;
     // lists of the root's two nodes that some later edge is drawn from or closes

@@ -51,6 +51,8 @@
 //    graph edge must join their images later in the root's window; the
 //    pair-ordered out-list answers that with two searches, and partial
 //    matches without one are dropped before their subtrees are searched.
+//    Before those searches, candidates go through a signature of the chord's
+//    list window, one per parent.
 //  * Enumeration is two launches of this kernel: a count launch leaves
 //    per-chunk match counts, a device scan turns them into row offsets,
 //    list_chunks_kernel lists the chunks holding a match below the cap, and a fill
@@ -206,6 +208,7 @@ template <int MODE, bool STATS, int FEAT>
 struct Search {
     static constexpr bool ANTI = (FEAT & FEAT_ANTI) != 0;   // anti-edge checks compiled in
     static constexpr bool LOOK = (FEAT & FEAT_LOOK) != 0;   // look-ahead checks compiled in
+    static constexpr bool FILTER = LOOK && !STATS;          // ... with their candidate filter
     static constexpr int CAP = MODE == MODE_FILL ? FCAP_FILL : FCAP_COUNT;   // parents per frame
     static constexpr uint32_t DESCEND = CAP - 32;   // a child frame this full is drained next
     using Frame = FrameT<CAP>;
@@ -222,7 +225,7 @@ struct Search {
     const QueryDev* q;
     int k;
     // cursors of the suspended levels: lane j holds level j's next candidate and total
-    uint32_t myOff, myT, myNp;
+    uint32_t myOff, myT, myNp, myPend;
     uint32_t np1;             // parents in frame 1 (warp-uniform)
     uint32_t nbuf;            // roots in the root buffer (warp-uniform)
     Acc acc;
@@ -235,7 +238,7 @@ struct Search {
         : g(g_), qs(qs_), ctrl(c), tasks(t), ready(r), task_cap(cap), wbase(wb) {
         lane = threadIdx.x & 31;
         qi = -1; q = nullptr; k = 0;
-        myOff = myT = myNp = 0;
+        myOff = myT = myNp = myPend = 0;
         np1 = nbuf = 0;
         acc.total = 0;
         if (STATS) for (int i = 0; i < W_LEN; ++i) acc.w[i] = 0;
@@ -446,11 +449,13 @@ struct Search {
     // Start frame i, which holds np parents: its window lengths become their
     // exclusive prefix (the flattened position each window starts at; entries past
     // np never start), computed once per frame.  Returns the flattened total.
-    __device__ uint32_t begin_frame(Frame f, uint32_t np) const {
+    __device__ uint32_t begin_frame(Frame f, uint32_t np) const { return begin_row(&f.pre2(0), np); }
+
+    __device__ uint32_t begin_row(uint2* row, uint32_t np) const {
         const uint32_t a = 2u * lane;
         uint32_t tot = 0;
         uint2 l = make_uint2(0u, 0u);
-        if (a < (uint32_t)CAP) l = f.pre2(lane);
+        if (a < (uint32_t)CAP) l = row[lane];
         if (a >= np) l.x = 0u;
         if (a + 1u >= np) l.y = 0u;
         const uint32_t s = l.x + l.y;
@@ -461,7 +466,7 @@ struct Search {
         }
         tot = __shfl_sync(FULL, inc, 31);
         const uint32_t pa = inc - s;
-        if (a < (uint32_t)CAP) f.pre2(lane) = make_uint2(a < np ? pa : NEVER, a + 1u < np ? pa + l.x : NEVER);
+        if (a < (uint32_t)CAP) row[lane] = make_uint2(a < np ? pa : NEVER, a + 1u < np ? pa + l.x : NEVER);
         __syncwarp();
         return tot;
     }
@@ -482,6 +487,143 @@ struct Search {
         if (db - 1u < 31u) mk |= 1u << db;
         starts = __reduce_or_sync(FULL, mk);
         return p0 + __popc(starts & ((2u << lane) - 1u));
+    }
+
+    // ---------------------------------------------------- candidate filter
+    //
+    // A level whose look-ahead joins its new node to a bound node x keeps, per
+    // parent, a 256-bit signature (two bits per entry) of x's list in (tprev, tend]:
+    // a candidate whose two bits are not both set has no such edge.  The filter reads the
+    // neighbour column only; what passes is collected in order and goes through step() 32 at
+    // a time, so the exact check's dependent searches run on full warps.  Without
+    // it every candidate paid those searches (a hub's list: ~20 loads each): the chorded
+    // 4-cycle on 100M hub-skewed edges 222 -> 53 ms.
+
+    __device__ uint32_t filt(Frame f, int i) const {
+        return f.o + (uint32_t)__ldg(MODE == MODE_FILL ? &q->plan.lv[i].filt_off_fill : &q->plan.lv[i].filt_off);
+    }
+    __device__ static uint32_t& filt_u32(uint32_t area, int row, int s) { return ((uint32_t*)(smem + area + row))[s]; }
+    __device__ static uint32_t* filt_sig(uint32_t area, int s) {
+        return (uint32_t*)(smem + area + CandidateFilter::SIG) + CandidateFilter::WORDS * s;
+    }
+    __device__ static uint32_t filt_hash(int32_t x) { return (uint32_t)x * 2654435761u; }   // bits 31-24 and 23-16
+
+    // Window of x's list for the filter of level i, for a partial match as in locate() with a
+    // level-i window of clen candidates; 0 when no candidate can pass.  A long list window saturates
+    // its signature, and one much longer than the candidates' costs more to read than
+    // their searches (about 8 entries a search): those parents pass everything (beg = NEVER).
+    __device__ uint32_t filt_window(int i, Frame pf, int ps, int nb, int32_t n0, int32_t n1, int32_t prev_e, int cdir,
+                                    uint32_t cpos, int64_t tprev, int64_t tend, uint32_t clen, uint32_t& beg) const {
+        const LevelPlan& lp = q->plan.lv[i];
+        const int fx = lp.fx, dir = lp.fdir, nx = lp.fnx;
+        const int32_t x = fx < nb ? pf.node(fx, ps) : (fx == nb ? n0 : n1);
+        const int64_t* ta = g.at[dir];
+        const uint32_t hi = __ldg(g.off[dir] + x + 1);
+        uint32_t b;
+        if (nx >= 0 && cdir >= 0) {
+            const uint2 w = successor(nx, cdir, cpos, prev_e);
+            if (word_shows_empty(w, (uint64_t)(tend - tprev))) return 0u;
+            b = w.x;
+        } else {
+            b = upper_bound_t(ta, __ldg(g.off[dir] + x), hi, tprev);
+            if (b >= hi || __ldg(ta + b) > tend) return 0u;
+        }
+        const uint32_t most = 8u * min(clen, 32u);
+        const uint32_t e = window_end(ta, b, min(hi, b + most + 1u), tend);
+        beg = b;
+        if (e - b <= most) return e - b;
+        beg = NEVER;
+        return 1u;
+    }
+
+    // The signatures of frame f's np parents.
+    __device__ void build_filter(Frame f, int i, uint32_t np) const {
+        const uint32_t area = filt(f, i);
+        for (uint32_t s = lane; s < np; s += 32u) {
+            const uint32_t v = filt_u32(area, CandidateFilter::BEG, s) == NEVER ? FULL : 0u;
+            uint4* sig = (uint4*)filt_sig(area, s);
+            sig[0] = sig[1] = make_uint4(v, v, v, v);
+        }
+        uint2* row = (uint2*)(smem + area + CandidateFilter::LEN);
+        const uint32_t tot = begin_row(row, np);
+        const uint2 pr = 2 * lane < CAP ? row[lane] : make_uint2(NEVER, NEVER);
+        const int32_t* __restrict__ nbr = g.anbr[q->plan.lv[i].fdir];
+        for (uint32_t off = 0; off < tot; off += 32u) {
+            unsigned starts;
+            const int p = lane_parent(pr, off, starts);
+            if (off + lane < tot) {
+                const uint32_t b = filt_u32(area, CandidateFilter::BEG, p);
+                if (b != NEVER) {
+                    const uint32_t h = filt_hash(__ldg(nbr + b + (off + lane - filt_u32(area, CandidateFilter::LEN, p))));
+                    uint32_t* sig = filt_sig(area, p);
+                    atomicOr(sig + (h >> 29), 1u << (h >> 24 & 31u));
+                    atomicOr(sig + (h >> 21 & 7u), 1u << (h >> 16 & 31u));
+                }
+            }
+        }
+        __syncwarp();
+    }
+
+    // Filter candidates [off, off + 64) of frame f's tot; those that pass join the
+    // pend pending ones.  Returns their new number.
+    __device__ uint32_t filter_step(int i, uint32_t h, Frame f, uint32_t off, uint32_t tot, uint32_t pend) const {
+        const uint32_t area = filt(f, i);
+        const int32_t* __restrict__ nbr = g.anbr[Hot::kind(h) == EXT_IN ? 1 : 0];
+        const uint2 pr = 2 * lane < CAP ? f.pre2(lane) : make_uint2(NEVER, NEVER);
+        unsigned starts;
+        uint32_t pos[2];
+        int32_t x[2];
+        int p[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const uint32_t idx = off + 32u * j + lane;
+            p[j] = lane_parent(pr, off + 32u * j, starts);
+            if (idx >= tot) { p[j] = -1; continue; }
+            pos[j] = (f.beg(p[j]) & POSMASK) + (idx - f.pre(p[j]));
+            x[j] = __ldg(nbr + pos[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            bool pass = p[j] >= 0;
+            if (pass) {
+                const uint32_t hx = filt_hash(x[j]);
+                const uint32_t* sig = filt_sig(area, p[j]);
+                pass = (sig[hx >> 29] >> (hx >> 24 & 31u) & sig[hx >> 21 & 7u] >> (hx >> 16 & 31u) & 1u) != 0u;
+            }
+            const unsigned b = __ballot_sync(FULL, pass);
+            if (pass) {
+                const uint32_t at = pend + __popc(b & ((1u << lane) - 1u));
+                filt_u32(area, CandidateFilter::POS, at) = pos[j];
+                ((uint8_t*)(smem + area + CandidateFilter::PAR))[at] = (uint8_t)p[j];
+            }
+            pend += __popc(b);
+        }
+        __syncwarp();
+        return pend;
+    }
+
+    // Take the first 32 of frame f's pend pending candidates: this lane's position, and its
+    // parent or -1.  The rest move up.
+    __device__ int pop_pending(int i, Frame f, uint32_t pend, uint32_t& pos) const {
+        const uint32_t area = filt(f, i);
+        uint8_t* par = (uint8_t*)(smem + area + CandidateFilter::PAR);
+        uint32_t ps[3];
+        int pp[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const uint32_t a = 32u * j + lane;
+            ps[j] = filt_u32(area, CandidateFilter::POS, a);
+            pp[j] = par[a];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 1; j < 3; ++j) {
+            filt_u32(area, CandidateFilter::POS, 32 * (j - 1) + lane) = ps[j];
+            par[32 * (j - 1) + lane] = (uint8_t)pp[j];
+        }
+        __syncwarp();
+        pos = ps[0];
+        return lane < pend ? pp[0] : -1;
     }
 
     // Emit survivors of the last level (or of the root level when k == 1).
@@ -516,16 +658,27 @@ struct Search {
     // One 32-candidate step of frame f at level i < k - 1 (or of the last level,
     // where survivors are emitted): candidates [off, off + 32) of its tot.  h, hc: packed plans of
     // levels i and i + 1; survivors with a window join child frame c after its cp
-    // parents.  Returns the child frame's new size.
+    // parents.  On a filtered level the candidates are the first of its pend
+    // pending ones.  Returns the child frame's new size.
     __device__ uint32_t step(int i, uint32_t h, uint32_t hc, Frame f, Frame c, uint32_t off, uint32_t tot,
-                                          uint32_t cp) {
+                                          uint32_t cp, uint32_t pend) {
         const int nb = Hot::nb(h), kind = Hot::kind(h);
-        const uint2 pr = f.pre2(2 * lane < CAP ? lane : 0);
-        unsigned starts;
-        const uint32_t idx = off + lane;
-        const bool act = idx < tot;
-        const int pl_ = lane_parent(2 * lane < CAP ? pr : make_uint2(NEVER, NEVER), off, starts);
-        const int p = act ? pl_ : 0;
+        uint32_t pos = 0;
+        bool act;
+        int p;
+        if (FILTER && (h & Hot::FILT)) {
+            p = pop_pending(i, f, pend, pos);
+            act = p >= 0;
+            if (!act) p = 0;
+        } else {
+            const uint2 pr = f.pre2(2 * lane < CAP ? lane : 0);
+            unsigned starts;
+            const uint32_t idx = off + lane;
+            act = idx < tot;
+            const int pl_ = lane_parent(2 * lane < CAP ? pr : make_uint2(NEVER, NEVER), off, starts);
+            p = act ? pl_ : 0;
+            if (act) pos = (f.beg(p) & POSMASK) + (idx - f.pre(p));
+        }
         int32_t n0 = -1, n1 = -1, ceid = -1;
         int64_t ct = 0;
         bool ok = act;
@@ -533,11 +686,9 @@ struct Search {
         // the next level's successor lookup loads it only if it needs it
         const bool need_eid = (MODE == MODE_FILL) || (h & Hot::ELABEL);
         int cdir = 2;
-        uint32_t pos = 0;
         uint2 wa = make_uint2(0u, 0u), wb = wa;   // next level's successor words, read with the candidate
         if (act) {
-            uint32_t bw = f.beg(p);
-            pos = (bw & POSMASK) + (idx - f.pre(p));
+            const uint32_t bw = f.beg(p);
             cdir = (bw & PAIRLIST) ? 3 : (kind == FREE ? 2 : ((bw & INLIST) ? 1 : 0));
             if (PREFETCH && !STATS && i < k - 1) next_words(hc, cdir, pos, wa, wb);
             if (bw & PAIRLIST) {
@@ -584,11 +735,13 @@ struct Search {
         }
         // expand survivors into frame i+1
         const int nb_c = Hot::nb(hc);
-        uint32_t cbeg = 0, clen = 0;
+        uint32_t cbeg = 0, clen = 0, fbeg = 0, flen = 1;
         int64_t tend = 0;
         if (ok) {
             tend = tend_of(f, p);
             clen = locate(i + 1, hc, f, p, nb, n0, n1, ceid, cdir, pos, ct, tend, cbeg, wa, wb);
+            if (FILTER && (hc & Hot::FILT) && clen > 0)
+                flen = filt_window(i + 1, f, p, nb, n0, n1, ceid, cdir, pos, ct, tend, clen, fbeg);
         }
         if (STATS) {
             unsigned b = __ballot_sync(FULL, ok);
@@ -599,7 +752,7 @@ struct Search {
                 acc.w[W_ENTRIES + (i + 1)] += l;
             }
         }
-        bool keep = ok && clen > 0;
+        bool keep = ok && clen > 0 && flen > 0;
         unsigned kb = __ballot_sync(FULL, keep);
         if (!kb) return cp;
         if (keep) {
@@ -612,6 +765,10 @@ struct Search {
             c.beg(s) = cbeg;
             c.len(s) = clen;
             c.root(s) = root;
+            if (FILTER && (hc & Hot::FILT)) {
+                filt_u32(filt(c, i + 1), CandidateFilter::BEG, s) = fbeg;
+                filt_u32(filt(c, i + 1), CandidateFilter::LEN, s) = flen;
+            }
             if (MODE == MODE_FILL) {
                 for (int j = 0; j < i; ++j) c.eid(nb_c, j, s) = f.eid(nb, j, p);
                 c.eid(nb_c, i, s) = ceid;
@@ -728,22 +885,30 @@ struct Search {
         int lvl = base;
         uint32_t h = hot(lvl), hc = lvl + 1 < k ? hot(lvl + 1) : 0u;
         Frame f = frame(lvl), c = lvl + 1 < k ? frame(lvl + 1) : f;
-        uint32_t off = 0, tot = begin_frame(f, np), nch = 0;
+        uint32_t off = 0, tot = begin_frame(f, np), nch = 0, pend = 0;
+        if (FILTER && (h & Hot::FILT)) build_filter(f, lvl, np);
         while (true) {
             if (MODE == MODE_COUNT && !STATS && lvl == k - 1 && Hot::kind(h) <= EXT_IN &&
                 !(h & (Hot::ELABEL | Hot::NLABEL | Hot::ANTI))) {
                 count_ext(lvl, h, f, np, tot);
                 off = tot;
             }
-            while (off < tot) {
-                if (MODE == MODE_COUNT) tot = maybe_donate(lvl, f, np, off, tot);
-                nch = step(lvl, h, hc, f, c, off, tot, nch);
-                off += 32;
+            while (off < tot || (FILTER && pend > 0)) {
+                if (MODE == MODE_COUNT && off < tot) tot = maybe_donate(lvl, f, np, off, tot);
+                if (FILTER && (h & Hot::FILT)) {
+                    for (; pend < 32u && off < tot; off += 64u) pend = filter_step(lvl, h, f, off, tot, pend);
+                    if (pend == 0) break;
+                    nch = step(lvl, h, hc, f, c, 0u, 0u, nch, pend);
+                    pend -= min(pend, 32u);
+                } else {
+                    nch = step(lvl, h, hc, f, c, off, tot, nch, 0u);
+                    off += 32;
+                }
                 if (nch >= DESCEND) break;
             }
             if (nch > 0) {
                 // down into the child frame
-                if (lane == lvl) { myOff = off; myT = tot; myNp = np; }
+                if (lane == lvl) { myOff = off; myT = tot; myNp = np; if (FILTER) myPend = pend; }
                 ++lvl;
                 np = nch;
                 nch = 0;
@@ -752,6 +917,10 @@ struct Search {
                 if (lvl + 1 < k) { hc = hot(lvl + 1); c = frame(lvl + 1); }
                 off = 0;
                 tot = begin_frame(f, np);
+                if (FILTER) {
+                    pend = 0;
+                    if (h & Hot::FILT) build_filter(f, lvl, np);
+                }
                 continue;
             }
             if (lvl == base) break;
@@ -764,6 +933,7 @@ struct Search {
             off = __shfl_sync(FULL, myOff, lvl);
             tot = __shfl_sync(FULL, myT, lvl);
             np = __shfl_sync(FULL, myNp, lvl);
+            if (FILTER) pend = __shfl_sync(FULL, myPend, lvl);
         }
     }
 
@@ -851,11 +1021,13 @@ struct Search {
                 emit(ok, r, Frame{wbase}, 0, 0, (int32_t)r);
                 return;
             }
-            uint32_t cbeg = 0, clen = 0;
+            uint32_t cbeg = 0, clen = 0, fbeg = 0, flen = 1;
             int64_t tend = 0;
             if (ok) {
                 tend = sat_add(tt, pl.delta);
                 clen = locate(1, hc, Frame{wbase}, 0, 0, s, d, (int32_t)r, 2, (uint32_t)r, tt, tend, cbeg, wa, wb);
+                if (FILTER && (hc & Hot::FILT) && clen > 0)
+                    flen = filt_window(1, Frame{wbase}, 0, 0, s, d, (int32_t)r, 2, (uint32_t)r, tt, tend, clen, fbeg);
             }
             if (STATS) {
                 unsigned b = __ballot_sync(FULL, ok);
@@ -866,7 +1038,7 @@ struct Search {
                     acc.w[W_ENTRIES + 1] += l;
                 }
             }
-            bool keep = ok && clen > 0;
+            bool keep = ok && clen > 0 && flen > 0;
             unsigned kb = __ballot_sync(FULL, keep);
             if (kb) {
                 Frame c = frame(1);
@@ -879,6 +1051,10 @@ struct Search {
                     c.beg(sl) = cbeg;
                     c.len(sl) = clen;
                     c.root(sl) = (uint32_t)r;
+                    if (FILTER && (hc & Hot::FILT)) {
+                        filt_u32(filt(c, 1), CandidateFilter::BEG, sl) = fbeg;
+                        filt_u32(filt(c, 1), CandidateFilter::LEN, sl) = flen;
+                    }
                     if (MODE == MODE_FILL) c.eid(2, 0, sl) = (int32_t)r;
                     for (int a = 0; ANTI && a < pl.n_anti; ++a)
                         if (pl.anti[a].edge == 0) c.anti_t(anti_off(1), a, sl) = tt;
@@ -906,6 +1082,15 @@ struct Search {
             f.root(0) = __ldcg(&t->root);
         }
         if (lane < nb) f.node(lane, 0) = __ldcg(&t->node[lane]);
+        __syncwarp();
+        if (FILTER && (hot(i) & Hot::FILT) && lane == 0) {
+            // the edge just bound is not in the task: the list is searched for its time
+            const int64_t tprev = f.tprev(0);
+            uint32_t fbeg = NEVER;
+            const uint32_t flen = filt_window(i, f, 0, nb, -1, -1, -1, -1, 0u, tprev, tend_of(f, 0), f.len(0), fbeg);
+            filt_u32(filt(f, i), CandidateFilter::BEG, 0) = flen ? fbeg : NEVER;
+            filt_u32(filt(f, i), CandidateFilter::LEN, 0) = max(flen, 1u);
+        }
         __syncwarp();
         return i;
     }

@@ -133,11 +133,15 @@ struct LevelPlan {
     uint8_t n_look;    // later motif edges (after i+1) whose two nodes are first both bound by edge i
     int8_t look_u[TM_MAX_LOOK];  // their endpoint slots: an edge look_u -> look_v must exist in
     int8_t look_v[TM_MAX_LOOK];  // (t_i, t_root + delta], else no match extends this partial match
+    int8_t fx, fdir;         // candidate filter (Hot::FILT): new nodes must be in bound slot fx's list of direction fdir
+    int8_t fnx;              // SuccKind giving the start of that list's window, after edge i - 1
     uint32_t hot;            // the fields every step needs, packed (see Hot)
     int32_t frame_off;       // byte offset of this level's frame in a warp's shared block (count)
     int32_t frame_off_fill;  // same, enumerate-fill layout (frames also carry edge ids)
     int32_t anti_row_off;    // byte offset of the anti-edge time rows within this level's frame
     int32_t anti_row_off_fill;
+    int32_t filt_off;        // byte offset of the candidate filter within this level's frame
+    int32_t filt_off_fill;
     int64_t gap;             // t_i - t_{i-1} bound (INT64_MAX = none)
 };
 
@@ -146,11 +150,13 @@ struct LevelPlan {
 // rest of the plan is read only by the checks that need it.
 struct Hot {
     static constexpr uint32_t ELABEL = 1u << 18, NLABEL = 1u << 19, ANTI = 1u << 20, LOOK = 1u << 21, GAP = 1u << 22;
+    // the level's look-ahead on its new node is filtered first (see CandidateFilter)
+    static constexpr uint32_t FILT = 1u << 23;
     static uint32_t pack(const LevelPlan& lp) {
         return (uint32_t)lp.kind | (uint32_t)(lp.a & 7) << 2 | (uint32_t)(lp.b & 7) << 5 | (uint32_t)lp.nb << 8 |
                (uint32_t)(lp.nx_a + 1) << 12 | (uint32_t)(lp.nx_b + 1) << 15 | (lp.elabel >= 0 ? ELABEL : 0u) |
                (lp.nl0 >= 0 || lp.nl1 >= 0 ? NLABEL : 0u) | (lp.anti_mask ? ANTI : 0u) | (lp.n_look ? LOOK : 0u) |
-               (lp.gap != INT64_MAX ? GAP : 0u);
+               (lp.gap != INT64_MAX ? GAP : 0u) | (lp.n_look && lp.kind <= EXT_IN ? FILT : 0u);
     }
     __host__ __device__ static int kind(uint32_t h) { return (int)(h & 3u); }
     __host__ __device__ static int a(uint32_t h) { return (int)(h >> 2 & 7u); }
@@ -220,11 +226,25 @@ struct FrameLayout {
     static constexpr int ROOT = LEN + 4 * CAP;
     static constexpr int NODE = ROOT + 4 * CAP;
 };
+// A frame's candidate filter (levels with Hot::FILT, after the anti-edge rows).  The
+// list windows the signatures are built from are needed until the frame is begun, the
+// pending candidates only after, so the two share their bytes.
+struct CandidateFilter {
+    static constexpr int WORDS = 8;                // signature words per parent
+    static constexpr int PEND = 96;                // up to 31 pending candidates and the 64 of a filter step
+    static constexpr int BEG = 0, LEN = 256;       // u32 per parent: window of the list the signature covers
+    static constexpr int POS = 0, PAR = 4 * PEND;  // u32 list position, u8 parent of each pending candidate
+    static constexpr int SIG = 512;                // WORDS words per parent
+    static constexpr int bytes(int cap) { return SIG + 4 * WORDS * cap; }
+};
+static_assert(4 * FCAP_FILL <= 256 && CandidateFilter::PAR + CandidateFilter::PEND <= CandidateFilter::SIG,
+              "candidate filter rows overlap");
+
 // Count frames (no edge ids) or fill frames (edge ids of the bound edges).
-inline int frame_bytes(int nb, int level, bool with_eids, int n_anti = 0) {
-    if (with_eids)
-        return FrameLayout<FCAP_FILL>::NODE + 4 * FCAP_FILL * (nb + level) + 8 * FCAP_FILL * n_anti;
-    return FrameLayout<FCAP_COUNT>::NODE + 4 * FCAP_COUNT * nb + 8 * FCAP_COUNT * n_anti;
+inline int frame_bytes(int nb, int level, bool with_eids, int n_anti = 0, bool filter = false) {
+    const int cap = with_eids ? FCAP_FILL : FCAP_COUNT;
+    return FrameLayout<FCAP_FILL>::NODE / FCAP_FILL * cap + 4 * cap * (nb + (with_eids ? level : 0)) + 8 * cap * n_anti +
+           (filter ? CandidateFilter::bytes(cap) : 0);
 }
 // A warp's shared block starts with its root buffer: up to 31 roots left over
 // and the 64 of one scan step.

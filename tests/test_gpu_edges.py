@@ -84,3 +84,45 @@ def test_many_queries_on_a_small_graph(tmg, nq):
     assert tots == want and nw == want and not trunc
     for mo, w, o in zip(mos, want, outs):
         assert np.array_equal(o[:w].cpu().numpy(), og.enumerate(mo, cap=w + 1)[0]), mo
+
+
+CHORDS = [
+    synth.chorded_four_cycle(1000), synth.chorded_four_cycle(400),
+    synth.Motif([(0, 1), (1, 2), (2, 3), (2, 0)], 1000),               # the new node sends the chord
+    synth.Motif([(0, 1), (2, 1), (2, 3), (0, 2)], 700),                # the new node is found in an in-list
+    synth.Motif([(0, 1), (1, 2), (2, 3), (3, 1), (0, 3)], 900),        # a chord node the previous edge does not touch
+    synth.Motif([(0, 1), (1, 2), (2, 3), (0, 2)], 1000, [500, 1000, 1000], elabel=[-1, 1, -1, -1]),
+    synth.Motif([(0, 1), (1, 2), (2, 3), (2, 0)], 1000, anti=[(1, 0, 0, 30)]),
+]
+
+
+@pytest.mark.parametrize("w", [1, 7, 31, 33, 64, 65, 255, 257, 1500])
+def test_chord_filter_edges(tmg, w):
+    """Chorded motifs where two hubs send w edges each into one window: candidate windows and filtered lists
+    around the step sizes, the longest list that is filtered and windows long enough to be donated."""
+    rng = np.random.default_rng(w)
+    leaves = 4 + w // 8
+    n = leaves + 2
+
+    def leaf(k):
+        return rng.integers(2, n, k)
+
+    src = np.concatenate([np.repeat([0, 1], w), leaf(leaves), leaf(leaves), np.array([0, 1, 0, 1, 0])])
+    dst = np.concatenate([leaf(2 * w), leaf(leaves), rng.integers(0, 2, leaves), np.array([1, 0, 1, 0, 0])])
+    m = len(src)
+    t = rng.integers(0, 1000, m).astype(np.int64)
+    t[-5:] = rng.integers(0, 60, 5)
+    el, nl = rng.integers(0, 3, m).astype(np.uint8), np.zeros(n, np.uint8)
+    src, dst = src.astype(np.int32), dst.astype(np.int32)
+    og = oracle.Graph(n, src, dst, t, el, nl)
+    gg = tmg.Graph.load(n, src, dst, t, el, nl)
+    for mo in CHORDS:
+        q = gg.compile(mo)
+        want, want_pr = og.count(mo, per_root=True)
+        pr = torch.full((m,), -1, dtype=torch.int64, device="cuda")
+        assert q.count(per_root=pr) == want, mo
+        assert np.array_equal(pr.cpu().numpy(), want_pr.astype(np.int64)), mo
+        rows = og.enumerate(mo, cap=min(want, 20_000) + 1)[0][: min(want, 20_000)]
+        out = torch.full((max(1, len(rows)), mo.k), -7, dtype=torch.int32, device="cuda")
+        assert q.enumerate(out)[:2] == (len(rows), want), mo
+        assert np.array_equal(out[: len(rows)].cpu().numpy(), rows), mo
