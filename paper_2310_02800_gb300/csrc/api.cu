@@ -231,17 +231,21 @@ tm_status build_plan(const tm_graph* g, const tm_motif* m, Plan* out) {
     p.warp_smem = (off_c + 15) & ~15;
     p.warp_smem_fill = (off_f + 15) & ~15;
     // lists of the root's two nodes that some later edge is drawn from or closes
-    // into: each needs an entry in (t_root, t_root + delta], else the root has no match
-    auto word_span = [](int64_t d) { return (uint32_t)std::min<int64_t>(d, (int64_t)SUCC_FAR); };
-    p.root_span = word_span(m->delta);
-    p.root_span_next = k > 1 ? word_span(std::min(m->delta, m->gap[0])) : p.root_span;
+    // into: each needs an entry in (t_root, t_root + delta], sooner where the gaps up to that
+    // edge add up to less, else the root has no match
+    uint8_t code[4];
+    memset(code, GAP_CODE_END, sizeof code);
+    int64_t reach = 0;
     for (int j = 1; j < k; ++j) {
-        const int sh = j == 1 ? 4 : 0;
-        if (m->esrc[j] == m->esrc[0]) p.root_need |= (uint8_t)(1u << (NX_OUT_SRC + sh));
-        if (m->esrc[j] == m->edst[0]) p.root_need |= (uint8_t)(1u << (NX_OUT_DST + sh));
-        if (m->edst[j] == m->edst[0]) p.root_need |= (uint8_t)(1u << (NX_IN_DST + sh));
-        if (m->edst[j] == m->esrc[0]) p.root_need |= (uint8_t)(1u << (NX_IN_SRC + sh));
+        reach = m->gap[j - 1] > m->delta - reach ? m->delta : reach + m->gap[j - 1];
+        const uint8_t c = (uint8_t)gap_code((uint32_t)std::min<int64_t>(reach, (int64_t)SUCC_FAR));
+        auto need = [&](int kind) { code[succ_byte(kind)] = std::min(code[succ_byte(kind)], c); };
+        if (m->esrc[j] == m->esrc[0]) need(NX_OUT_SRC);
+        if (m->esrc[j] == m->edst[0]) need(NX_OUT_DST);
+        if (m->edst[j] == m->edst[0]) need(NX_IN_DST);
+        if (m->edst[j] == m->esrc[0]) need(NX_IN_SRC);
     }
+    for (int b = 0; b < 4; ++b) p.root_codes |= (uint32_t)code[b] << (8 * b);
     p.tune.warps_per_block = 4;
     p.tune.chunk_roots = 64;
     p.auto_chunk = 1;

@@ -230,6 +230,17 @@ __global__ void successor_kernel(int64_t m, const uint32_t* __restrict__ nodes, 
     }
 }
 
+// Root filter (see GraphView::rcode) from the four words of each edge.  A streaming pass of its own:
+// storing the two bytes of a direction from successor_kernel, whose edges come in list
+// order, is a partial sector per edge and cost ten times as much (0.5 ms for 10M edges).
+__global__ void root_codes_kernel(int64_t m, const uint2* __restrict__ out_src, const uint2* __restrict__ in_dst,
+                                  const uint2* __restrict__ out_dst, const uint2* __restrict__ in_src,
+                                  uint32_t* __restrict__ rcode) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x)
+        rcode[e] = gap_code(out_src[e].y) << (8 * succ_byte(NX_OUT_SRC)) | gap_code(in_dst[e].y) << (8 * succ_byte(NX_IN_DST)) |
+                   gap_code(out_dst[e].y) << (8 * succ_byte(NX_OUT_DST)) | gap_code(in_src[e].y) << (8 * succ_byte(NX_IN_SRC));
+}
+
 int bits_for(unsigned long long x) {
     int b = 0;
     while (b < 64 && (x >> b) != 0) ++b;
@@ -273,7 +284,7 @@ size_t storage_bytes(int64_t n, int64_t m, bool node_labels, bool edge_labels) {
     if (edge_labels) b += col_bytes(m, 1);
     b += 2 * (col_bytes(n + 1, 4) + col_bytes(m, 8) + col_bytes(m, 4) * 2);  // out / in lists
     b += col_bytes(m, 4) + col_bytes(m, 8) + col_bytes(m, 4);               // pair-ordered list
-    b += 8 * col_bytes(m, sizeof(uint2));                                     // successor words
+    b += 8 * col_bytes(m, sizeof(uint2)) + col_bytes(m, 4);                   // successor words, root filter
     return b;
 }
 
@@ -469,6 +480,8 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
     uint2 *nx[4], *px[4];
     for (int j = 0; j < 4; ++j) TRY(owned(g, &nx[j], m));
     for (int j = 0; j < 4; ++j) TRY(owned(g, &px[j], m));
+    uint32_t* codes;
+    TRY(owned(g, &codes, m));
     if (m > 0) {
         successor_kernel<<<grid, 256, 0, st>>>(m, keys_of[0], v.aeid[0], v.off[0], v.at[0], v.off[1], v.at[1], px[0],
                                                nx[NX_OUT_SRC], nx[NX_IN_SRC]);
@@ -476,11 +489,13 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
                                                nx[NX_IN_DST], nx[NX_OUT_DST]);
         successor_by_position_kernel<<<grid4, 256, 0, st>>>(m, v.aeid[0], v.aeid[1], nx[NX_OUT_DST], nx[NX_IN_SRC],
                                                            px[1], px[3]);
-        note_launches(3);
+        root_codes_kernel<<<grid, 256, 0, st>>>(m, nx[NX_OUT_SRC], nx[NX_IN_DST], nx[NX_OUT_DST], nx[NX_IN_SRC], codes);
+        note_launches(4);
         TM_CUDA(cudaGetLastError());
     }
     for (int j = 0; j < 4; ++j) v.nxt[j] = nx[j];
     for (int j = 0; j < 4; ++j) v.pnx[j] = px[j];
+    v.rcode = codes;
     TM_CUDA(cudaStreamSynchronize(st));
     return TM_OK;
 }

@@ -5,12 +5,15 @@
 // Section 5.1.2 deciding where candidates come from and which mapped nodes a
 // new node must differ from.  The GPU organisation is our own:
 //
-//  * Roots are filtered before anything else of them is read: 64 at a time, two
-//    successor words per lane and list the motif continues in, since most edges
-//    have no later edge in the window at one of their nodes.  The survivors are
-//    buffered and taken 32 at a time, so the searches that start a window
-//    run on full warps.  (10M-edge power-law graph, 1 h windows: the cycles'
-//    roots fall to the tenth whose source is answered within the window.)
+//  * Roots are filtered before anything else of them is read, since most edges
+//    have no later edge in the window at one of their nodes: one byte per list
+//    (its successor gap, rounded down) decides, four lists of a root in one word, four
+//    roots per lane, 128 per step.  The survivors are buffered and taken 32 at a
+//    time, so the searches that start a window run on full warps.  (10M-edge
+//    power-law graph, 1 h windows: the cycles' roots fall to the tenth whose
+//    source is answered within the window.)  With the 8-byte successor words
+//    read instead, 64 roots per step, and every warp claiming for itself: 1/61 of
+//    10M edges 107 -> 83 us a call, labelled 5-path on 20M edges 450 -> 348 us.
 //  * A warp owns a stack of FRAMES, one per motif edge i >= 1.  Frame i holds
 //    up to 48 (count) or 64 (fill) partial matches of i edges ("parents"), each with its candidate
 //    window for edge i: the entries of one time-ordered adjacency list with
@@ -204,6 +207,23 @@ struct Acc {             // per-warp accumulators for the current query
     unsigned long long w[W_LEN];   // stats launches; lane-0 values except W_PROBE (per lane)
 };
 
+// What the warps of a block share.  One global atomic claims chunks for all of them, and one
+// reports what they finished: returning atomics on one address take 1.9 ns each
+// on a GB300 however they are spread, so 5,472 warps claiming, reporting and going
+// idle one by one took 56 us without any search (200k edges, a query without a single window;
+// 10M edges: 103 us); per block they take 31 (58) us.
+struct Block {
+    int lock;                     // guards cn, left, grow, claimed_at, ended
+    int ended;                    // no chunks are left to claim
+    unsigned long long cn;        // claimed chunks nobody took yet: cn .. cn + left
+    uint32_t left, grow;
+    uint32_t claimed_at;          // clock at the last claim
+    int poller, finished;         // see wait_for_work()
+    unsigned unreported;          // finished chunks not added to done_chunks yet
+    int arrived;                  // warps that have left the search, of a launch of one query,
+    unsigned long long total;     // ... and their matches
+};
+
 template <int MODE, bool STATS, int FEAT>
 struct Search {
     static constexpr bool ANTI = (FEAT & FEAT_ANTI) != 0;   // anti-edge checks compiled in
@@ -232,10 +252,12 @@ struct Search {
     // enumerate fill
     unsigned long long out_base, out_local;
     unsigned polls;           // donation checks (warp-uniform)
-    uint32_t claimed;         // root chunks this warp has claimed (warp-uniform)
+    uint32_t claimed;         // root chunks this warp has taken (warp-uniform)
+    Block* blk;
 
-    __device__ Search(const GraphView& g_, const QueryDev* qs_, Ctrl* c, Task* t, uint8_t* r, uint64_t cap, uint32_t wb)
-        : g(g_), qs(qs_), ctrl(c), tasks(t), ready(r), task_cap(cap), wbase(wb) {
+    __device__ Search(const GraphView& g_, const QueryDev* qs_, Ctrl* c, Task* t, uint8_t* r, uint64_t cap, uint32_t wb,
+                      Block* b)
+        : g(g_), qs(qs_), ctrl(c), tasks(t), ready(r), task_cap(cap), wbase(wb), blk(b) {
         lane = threadIdx.x & 31;
         qi = -1; q = nullptr; k = 0;
         myOff = myT = myNp = myPend = 0;
@@ -939,53 +961,53 @@ struct Search {
 
     __device__ uint32_t& root_buf(uint32_t j) const { return ((uint32_t*)(smem + wbase))[j]; }
 
-    // Scan 64 root edges from rb (rounded down to even) up to re: those whose
-    // successor words leave them a chance of a match join the root buffer, in order.  A
+    // Scan 128 root edges from rb (rounded down to a multiple of 4) up to re: those whose
+    // gap codes leave them a chance of a match join the root buffer, in order.  A
     // root dies when a list the motif draws a later edge from -- any of the out- and
-    // in-lists of its two nodes -- has no entry in (t, t + delta].  The words are
-    // read two per lane and nothing else of a dead root is read.
+    // in-lists of its two nodes -- has no entry soon enough; a code says so when it is above
+    // the query's byte for that list (both below 128: the subtraction borrows from no neighbour).
     __device__ void scan_roots(uint32_t rb, uint32_t re) {
-        const uint32_t r = (rb & ~1u) + 2u * lane;
-        bool a = r >= rb && r < re, b = r + 1u < re;
+        const uint32_t base = rb & ~3u, r = base + 4u * lane;
+        // the columns are padded past the last edge: no read is out of range
+        unsigned alive = 0;
         if (STATS) {
-            if (lane == 0) acc.w[W_ROOTS] += min(re, (rb & ~1u) + 64u) - rb;
-        } else if (a || b) {
+            alive = 15u;
+            if (lane == 0) acc.w[W_ROOTS] += min(re, base + 128u) - rb;
+        } else if (r < re) {
             const Plan& pl = q->plan;
+            const uint32_t most = __ldg(&pl.root_codes) | 0x80808080u;
+            const uint4 c = __ldg((const uint4*)(g.rcode + r));
+            alive = ((most - c.x) & 0x80808080u) == 0x80808080u ? 1u : 0u;
+            alive |= ((most - c.y) & 0x80808080u) == 0x80808080u ? 2u : 0u;
+            alive |= ((most - c.z) & 0x80808080u) == 0x80808080u ? 4u : 0u;
+            alive |= ((most - c.w) & 0x80808080u) == 0x80808080u ? 8u : 0u;
             if (pl.elabel0 >= 0) {
-                a = a && g.elabel[r] == (uint8_t)pl.elabel0;
-                b = b && g.elabel[r + 1] == (uint8_t)pl.elabel0;
-            }
-            if (a || b) {
-                const unsigned need = __ldg(&pl.root_need);
-                const uint32_t near = __ldg(&pl.root_span_next), far = __ldg(&pl.root_span);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (!(need & (0x11u << j))) continue;
-                    // the column is padded to an even number of words
-                    const uint4 w = __ldg((const uint4*)(g.nxt[j] + r));
-                    const uint32_t span = need & (0x10u << j) ? near : far;
-                    a = a && w.y <= span;
-                    b = b && w.w <= span;
-                }
+                const uchar4 l = __ldg((const uchar4*)(g.elabel + r));
+                const uint8_t want = (uint8_t)pl.elabel0;
+                alive &= (l.x == want ? 1u : 0u) | (l.y == want ? 2u : 0u) | (l.z == want ? 4u : 0u) | (l.w == want ? 8u : 0u);
             }
         }
-        const unsigned ba = __ballot_sync(FULL, a), bb = __ballot_sync(FULL, b);
-        if (!(ba | bb)) return;
+        if (r < rb) alive &= 15u << (rb - r);             // rb - r < 4: only lane 0's word
+        if (r + 4u > re) alive &= r < re ? 15u >> (r + 4u - re) : 0u;
+        if (!__any_sync(FULL, alive != 0u)) return;
         const unsigned lt = (1u << lane) - 1u;
-        const uint32_t at = nbuf + __popc(ba & lt) + __popc(bb & lt);
-        if (a) root_buf(at) = r;
-        if (b) root_buf(at + (a ? 1u : 0u)) = r + 1u;
-        nbuf += __popc(ba) + __popc(bb);
+        uint32_t at = nbuf;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const unsigned b = __ballot_sync(FULL, alive >> j & 1u);
+            at += __popc(b & lt);
+            nbuf += __popc(b);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (alive >> j & 1u) root_buf(at++) = r + j;
         __syncwarp();
     }
 
-    // Drop the first n of the buffered roots.
+    // Drop the first n of the buffered roots: 32 of them, or all.
     __device__ void pop_roots(uint32_t n) {
         const uint32_t left = nbuf - n;
-        const uint32_t x = lane < left ? root_buf(n + lane) : 0u, y = lane + 32u < left ? root_buf(n + 32u + lane) : 0u;
-        __syncwarp();
-        if (lane < left) root_buf(lane) = x;
-        if (lane + 32u < left) root_buf(lane + 32u) = y;
+        for (uint32_t j = lane; j < left; j += 32u) root_buf(j) = root_buf(32u + j);   // each lane its own slots
         __syncwarp();
         nbuf = left;
     }
@@ -1133,8 +1155,8 @@ struct Search {
     }
 
     __device__ bool queue_empty() const {
-        unsigned long long h = *(volatile unsigned long long*)&ctrl->q_head;
-        unsigned long long r = *(volatile unsigned long long*)&ctrl->q_reserve;
+        unsigned long long r, h;
+        asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(r), "=l"(h) : "l"(&ctrl->q_reserve));
         return h >= min(r, (unsigned long long)task_cap);
     }
 
@@ -1151,41 +1173,92 @@ struct Search {
     }
 
     // Wait for a task (true) or the end of the launch (false).  One warp per block
-    // polls the control block at a time and the block's other idle warps watch
-    // shared memory: thousands of warps polling one line delayed every claim and
-    // donation that goes through it.
-    __device__ bool wait_for_work(uint64_t total_chunks, int* poller, int* finished) {
+    // polls the control block at a time, and stands for the block in the idle count; the
+    // block's other idle warps watch shared memory: thousands of warps polling one line delayed
+    // every claim and donation that goes through it.
+    __device__ bool wait_for_work(uint64_t total_chunks) {
         int leave = 0;
         if (lane == 0) {
-            atomicAdd(&ctrl->idle, 1);
             const uint64_t t0 = now_ns();
-            unsigned ns = 128;
+            // a poll is two loads of a line that every block polls: sooner ones only delay each other
+            unsigned ns = 512;
             bool polling = false;
             while (true) {
-                if (*(volatile int*)finished) { leave = 1; break; }
-                if (!polling) polling = atomicCAS(poller, 0, 1) == 0;
+                if (*(volatile int*)&blk->finished) { leave = 1; break; }
+                if (!polling && atomicCAS(&blk->poller, 0, 1) == 0) {
+                    polling = true;
+                    atomicAdd(&ctrl->idle, 1);
+                }
                 if (polling) {
+                    const unsigned n = atomicExch(&blk->unreported, 0u);
+                    if (n) {
+                        __threadfence();
+                        atomicAdd(&ctrl->done_chunks, (unsigned long long)n);
+                    }
                     if (!queue_empty()) break;
-                    if (all_done(total_chunks)) { *(volatile int*)finished = 1; leave = 1; break; }
+                    if (all_done(total_chunks)) { *(volatile int*)&blk->finished = 1; leave = 1; break; }
                 }
                 if (now_ns() - t0 > WAIT_NS) { leave = 1; break; }
                 __nanosleep(ns);
                 if (ns < 2048) ns <<= 1;
             }
-            if (polling) atomicExch(poller, 0);
-            if (!leave) atomicSub(&ctrl->idle, 1);
+            if (polling) {
+                if (!leave) atomicSub(&ctrl->idle, 1);
+                atomicExch(&blk->poller, 0);
+            }
         }
         return __shfl_sync(FULL, leave, 0) == 0;
+    }
+
+    // Take chunks for this warp from the block's, claiming more for the block when it has none: up to
+    // `n` of them from `c` on; 0 when the launch has none left.
+    __device__ uint32_t take_chunks(uint64_t total_chunks, unsigned long long& c) {
+        uint32_t n = 0;
+        if (lane == 0) {
+            const uint64_t t0 = now_ns();
+            bool mine = true;
+            while (atomicCAS(&blk->lock, 0, 1) != 0) {
+                if (now_ns() - t0 > READY_NS) { atomicMax(&ctrl->err, (unsigned)TM_E_TIMEOUT); mine = false; break; }
+                __nanosleep(32);
+            }
+            if (mine) {
+                __threadfence_block();
+                volatile Block* b = blk;
+                if (b->left == 0u && !b->ended) {
+                    const uint32_t warps = blockDim.x >> 5, now = (uint32_t)clock();
+                    const unsigned long long seen = b->cn;    // where the cursor stood at the last claim
+                    uint32_t grow = MODE == MODE_FILL ? 1u : claim_size(b->grow, now - b->claimed_at, total_chunks - seen, warps);
+                    const unsigned long long at = atomicAdd(&ctrl->next_chunk, (unsigned long long)(grow * warps));
+                    b->grow = grow;
+                    b->claimed_at = now;
+                    if (at >= total_chunks) {
+                        b->ended = 1;
+                    } else {
+                        b->cn = at;
+                        b->left = (uint32_t)min((unsigned long long)(grow * warps), total_chunks - at);
+                    }
+                }
+                n = min(b->left, b->grow);
+                c = b->cn;
+                b->cn = c + n;
+                b->left = b->left - n;
+                __threadfence_block();
+                atomicExch(&blk->lock, 0);
+            }
+        }
+        c = __shfl_sync(FULL, c, 0);
+        return __shfl_sync(FULL, n, 0);
     }
 
     // Find the next frame to drain, in order: roots collected in frame 1 (root
     // chunks are claimed and scanned until it is full enough or must be emptied), then
     // donated tasks, until the launch has no work left.  One loop with one drain,
     // so the search's code exists once per kernel.
-    __device__ void run(int nq, uint64_t total_chunks, int* poller, int* finished) {
-        uint32_t rb = 0, re = 0;                  // roots left of the current chunk
-        unsigned long long held = NO_CHUNK;       // claimed chunk of the next query, waiting for frame 1 to empty
-        bool scanning = true, ending = false;
+    __device__ void run(int nq, uint64_t total_chunks) {
+        uint32_t rb = 0, re = 0;                  // roots left of the current chunks
+        unsigned long long cn = 0;                // chunks taken and not scanned yet: cn .. cn + left
+        uint32_t left = 0;
+        bool scanning = true, switching = false, ending = false, ran_task = false;
         while (true) {
             int base = 1;
             uint32_t np = 0;
@@ -1195,48 +1268,51 @@ struct Search {
                     if (nbuf >= 32u) { root_batch(); continue; }
                     if (rb < re) {
                         scan_roots(rb, re);
-                        rb = (rb & ~1u) + 64u;
+                        rb = (rb & ~3u) + 128u;
                         continue;
                     }
-                    // the chunk is scanned; what it left in the root buffer and frame 1
-                    // stays for the next one, except where that belongs to another
-                    // query or (enumeration) writes from another offset
-                    if (MODE == MODE_FILL || held != NO_CHUNK || ending) {
+                    // the chunks are scanned; what they left in the root buffer and frame 1
+                    // stays for the next ones, except where those belong to another
+                    // query or (enumeration) write from another offset
+                    if (MODE == MODE_FILL || switching || ending) {
                         if (nbuf > 0u) { root_batch(); continue; }
                         if (np1 > 0u) break;
                         if (ending) { scanning = false; break; }
+                        switching = false;
                     }
-                    unsigned long long c = held;
-                    held = NO_CHUNK;
-                    if (c == NO_CHUNK) {
-                        if (lane == 0) c = atomicAdd(&ctrl->next_chunk, 1ULL);
-                        c = __shfl_sync(FULL, c, 0);
-                        if (c >= total_chunks) { ending = true; continue; }
-                        ++claimed;
+                    if (left == 0u) {
+                        left = take_chunks(total_chunks, cn);
+                        if (left == 0u) { ending = true; continue; }
+                        claimed += left;
                     }
-                    const int j = query_of_chunk(c, nq);
-                    if (j != qi) {
+                    if (q == nullptr || cn < q->chunk_base || cn - q->chunk_base >= q->n_chunks) {
                         // nothing of the previous query may be left when switching
-                        if (np1 + nbuf > 0u) { held = c; continue; }
-                        use_query(j);
+                        if (np1 + nbuf > 0u) { switching = true; continue; }
+                        use_query(query_of_chunk(cn, nq));
                     }
-                    uint64_t lc = c - q->chunk_base;
+                    uint64_t lc = cn - q->chunk_base;
                     const uint64_t cr = (uint64_t)q->plan.tune.chunk_roots;
+                    uint32_t n = 1;
                     if (MODE == MODE_FILL) {
                         // claim index lc -> the lc-th listed chunk (one holding a match whose
                         // rows start below the cap); past the list's end the rest of this
                         // query is skipped
                         if (lc >= q->chunk_off[q->n_chunks + 1]) {
-                            unsigned long long nxt = (j + 1 < nq) ? qs[j + 1].chunk_base : total_chunks;
+                            unsigned long long nxt = (qi + 1 < nq) ? qs[qi + 1].chunk_base : total_chunks;
                             if (lane == 0) atomicMax(&ctrl->next_chunk, nxt);
+                            left = 0u;
                             continue;
                         }
                         lc = ((const uint32_t*)(q->chunk_off + q->n_chunks + 2))[lc];
                         out_base = q->chunk_off[lc];
                         out_local = 0;
+                    } else {
+                        n = (uint32_t)min((uint64_t)left, q->n_chunks - lc);
                     }
+                    cn += n;
+                    left -= n;
                     rb = (uint32_t)(q->root_begin + lc * cr);
-                    re = (uint32_t)min(q->root_end, (uint64_t)rb + cr);
+                    re = (uint32_t)min(q->root_end, (uint64_t)rb + n * cr);
                 }
                 np = np1;
                 np1 = 0;
@@ -1244,17 +1320,19 @@ struct Search {
             } else {
                 if (MODE == MODE_FILL) break;
                 report_chunks();
+                // a launch of one query that never donates has nothing to wait for; after a task, more of
+                // them are likely; before the first, the block's poller looks
+                const bool alone = nq == 1 && qs[0].plan.tune.split_depth <= 0;
+                if (!alone && !ran_task && !wait_for_work(total_chunks)) break;
                 const unsigned long long slot = try_pop();
-                if (slot != NO_CHUNK) {
-                    base = take_task(slot);
-                    np = 1;
-                    is_task = true;
-                } else {
-                    // a launch of one query that never donates has nothing to wait for
-                    if (nq == 1 && qs[0].plan.tune.split_depth <= 0) break;
-                    if (!wait_for_work(total_chunks, poller, finished)) break;
+                ran_task = slot != NO_CHUNK;
+                if (!ran_task) {
+                    if (alone) break;
                     continue;
                 }
+                base = take_task(slot);
+                np = 1;
+                is_task = true;
             }
             drain(base, np);
             if (MODE == MODE_COUNT && is_task) {
@@ -1262,30 +1340,59 @@ struct Search {
                 if (lane == 0) atomicAdd(&ctrl->done_tasks, 1ULL);
             }
         }
-        flush();
+        if (STATS || nq != 1) flush(); else leave();
+    }
+
+    // The end of a launch of one query: the block's last warp adds the matches of all of them.
+    __device__ void leave() {
+        for (int d = 16; d > 0; d >>= 1) acc.total += __shfl_down_sync(FULL, acc.total, d);
+        if (lane == 0) {
+            if (acc.total) atomicAdd(&blk->total, acc.total);
+            __threadfence_block();
+            if (atomicAdd(&blk->arrived, 1) == (int)(blockDim.x >> 5) - 1) {
+                __threadfence_block();
+                const unsigned long long all = atomicAdd(&blk->total, 0ULL);
+                if (all) atomicAdd(qs[0].total, all);
+            }
+        }
+    }
+
+    // Chunks per warp of a block's next claim.  Chunks without matches are scanned in less than
+    // a claim takes, so the size doubles (up to 16) when the last claim of `last` was gone within 16k cycles,
+    // about 8 us, and starts over when it was not: roots held by a busy warp wait for it.
+    // With `ahead` chunks unclaimed it is at most a quarter of the warp's share.
+    __device__ static uint32_t claim_size(uint32_t last, uint32_t cycles, unsigned long long ahead, uint32_t warps) {
+        if (cycles > 16384u) return 1u;
+        const uint32_t share = (uint32_t)min(ahead / (4ull * warps * gridDim.x), 16ull);
+        return max(min(2u * last, share), 1u);
     }
 
     // Count this warp's chunks as done, once their subtrees (and the slots they donated) are.
     __device__ void report_chunks() {
         if (!claimed) return;
         __threadfence();
-        if (lane == 0) atomicAdd(&ctrl->done_chunks, (unsigned long long)claimed);
+        if (lane == 0) atomicAdd(&blk->unreported, claimed);
         claimed = 0;
     }
 };
 
+// 64 registers: 32 warps per SM, which the frames' shared memory allows about half of the motifs
+// anyway.  At 56 (36 warps) the candidate loops spilled: 4-path over 15 h windows 21.5 ms
+// against 20.0, 64-query batch 19.2 against 16.7.
 template <int MODE, bool STATS, int FEAT>
-__global__ void __maxnreg__(56) search_kernel(const __grid_constant__ GraphView g,
+__global__ void __maxnreg__(64) search_kernel(const __grid_constant__ GraphView g,
                                                      const QueryDev* __restrict__ qs, int nq, int warp_smem,
                                                      Ctrl* ctrl, Task* tasks, uint8_t* ready, uint64_t task_cap) {
-    __shared__ int poller, finished;
-    if (MODE == MODE_COUNT) {
-        if (threadIdx.x == 0) poller = finished = 0;
-        __syncthreads();
+    __shared__ Block blk;
+    if (threadIdx.x == 0) {
+        blk = Block{};
+        blk.grow = 1;
+        blk.claimed_at = (uint32_t)clock();
     }
+    __syncthreads();
     const int warp = threadIdx.x >> 5;
-    Search<MODE, STATS, FEAT> s(g, qs, ctrl, tasks, ready, task_cap, (uint32_t)(warp * warp_smem));
-    s.run(nq, ctrl->total_chunks, &poller, &finished);
+    Search<MODE, STATS, FEAT> s(g, qs, ctrl, tasks, ready, task_cap, (uint32_t)(warp * warp_smem), &blk);
+    s.run(nq, ctrl->total_chunks);
 }
 
 }  // namespace
@@ -1348,7 +1455,7 @@ const void* kernel_of(Mode mode, bool stats, unsigned feat) {
 }
 
 // dynamic shared memory a block may use beside the kernel's few static bytes
-constexpr int MAX_DYN_SMEM = 232448 - 64;
+constexpr int MAX_DYN_SMEM = 232448 - 128;
 
 // Resident blocks per SM for one launch shape, computed once per shape.
 int blocks_per_sm(const tm_graph* g, const void* fn, int kid, int threads, int smem) {

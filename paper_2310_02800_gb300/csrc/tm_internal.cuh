@@ -68,6 +68,10 @@ struct GraphView {
     // entry -> next later in that out-list, [1] out-list entry -> out(its neighbour),
     // [2] in-list entry -> next later in that in-list, [3] in-list entry -> in(its neighbour)
     const uint2* pnx[4];
+    // root filter, by edge id: the gaps of the edge's four successor words as gap_code()
+    // bytes (byte succ_byte(kind)), rounded down, so that one load tells for four lists
+    // whether they have an entry soon enough
+    const uint32_t* rcode;
     // out-lists again, ordered by (neighbour, time) within each node (offsets off[0]):
     // the edges u -> v form one contiguous, time-ordered range
     const int32_t* pnbr;
@@ -79,6 +83,22 @@ constexpr uint32_t SUCC_END = 0xFFFFFFFFu;   // successor word: no later entry i
 constexpr uint32_t SUCC_FAR = 0xFFFFFFFEu;   // successor word: time gap >= this
 
 enum SuccKind : int8_t { NX_OUT_SRC = 0, NX_IN_DST = 1, NX_OUT_DST = 2, NX_IN_SRC = 3, NX_NONE = -1 };
+
+// A time gap as a 7-bit floating code (5 bits of exponent, 2 of mantissa, rounded down): larger gaps never
+// have smaller codes.  GAP_CODE_END (SUCC_END) is above the code of any gap.
+constexpr uint32_t GAP_CODE_END = 127;
+__host__ __device__ inline uint32_t gap_code(uint32_t gap) {
+    if (gap == SUCC_END) return GAP_CODE_END;
+    if (gap < 4u) return gap;
+#ifdef __CUDA_ARCH__
+    const uint32_t e = 31u - (uint32_t)__clz((int)gap);
+#else
+    const uint32_t e = 31u - (uint32_t)__builtin_clz(gap);
+#endif
+    return (e - 1u) << 2 | (gap >> (e - 2u) & 3u);
+}
+// Byte of rcode that holds a list's code.
+__host__ __device__ constexpr int succ_byte(int kind) { return kind; }
 
 struct TuneKey {
     uint64_t shape;     // motif structure hash
@@ -194,11 +214,10 @@ struct Plan {
     uint64_t shape_hash;
     int32_t n_anti;
     uint8_t anti_mask0;            // anti-edges checked when the root binds edge 0
-    uint8_t root_need;             // lists a match rooted at an edge must continue in, one bit per SuccKind: bits 0-3
-                                   // within root_span, bits 4-7 (edge 1's own lists) within root_span_next
     uint8_t auto_chunk;            // 1: tune.chunk_roots is the default and may shrink on small inputs
-    uint8_t pad1;
-    uint32_t root_span, root_span_next;   // delta, and min(delta, gap_0), as largest word gaps
+    uint16_t pad1;
+    uint32_t root_codes;           // lists a match rooted at an edge must continue in: the largest gap allowed, as
+                                   // bytes laid out like GraphView::rcode (GAP_CODE_END: the list is not needed)
     AntiPlan anti[TM_MAX_ANTI];
     LevelPlan lv[TM_MAX_EDGES];    // lv[i] for i = 1..k-1 (lv[0]: only the look-ahead of the root)
 };
@@ -247,8 +266,8 @@ inline int frame_bytes(int nb, int level, bool with_eids, int n_anti = 0, bool f
            (filter ? CandidateFilter::bytes(cap) : 0);
 }
 // A warp's shared block starts with its root buffer: up to 31 roots left over
-// and the 64 of one scan step.
-constexpr int ROOT_BUF_BYTES = 96 * 4;
+// and the 128 of one scan step.
+constexpr int ROOT_BUF_BYTES = 160 * 4;
 
 tm_status build_plan(const tm_graph* g, const tm_motif* m, Plan* out);
 uint64_t plan_shape_hash(const tm_motif* m);
@@ -277,9 +296,9 @@ struct Ctrl {
     unsigned long long next_chunk;   // root-chunk cursor (own line)
     unsigned long long pad1[15];
     unsigned long long q_reserve;    // task slots reserved by donors
-    unsigned long long q_head;       // next task slot to pop
+    unsigned long long q_head;       // next task slot to pop (read together with q_reserve)
     int pad3;
-    int idle;                        // warps waiting for tasks
+    int idle;                        // blocks with a warp waiting for tasks
     unsigned int err;                // 0 or TM_E_TIMEOUT
     unsigned int donated;            // tasks donated (diagnostic)
     unsigned long long done_chunks;  // root chunks whose whole subtree has been searched
