@@ -208,6 +208,11 @@ tm_status build_plan(const tm_graph* g, const tm_motif* m, Plan* out) {
         L.n_look++;
     }
     for (int i = 0; i < k; ++i) p.lv[i].hot = Hot::pack(p.lv[i]);
+    if (k >= 3) {
+        LevelPlan &l = p.lv[k - 2], &z = p.lv[k - 1];
+        const uint32_t plain = Hot::ELABEL | Hot::NLABEL | Hot::ANTI | Hot::LOOK | Hot::GAP;
+        if (l.kind == z.kind && l.kind <= EXT_IN && l.a == z.a && !((l.hot | z.hot) & plain)) l.hot |= Hot::PAIRS;
+    }
     for (int i = 1; i < k; ++i) {
         LevelPlan& lp = p.lv[i];
         const bool filter = (lp.hot & Hot::FILT) != 0;
@@ -426,7 +431,8 @@ static tm_status run_count(tm_graph* g, tm_query* q, uint64_t rb, uint64_t re, c
     if (per_root && re > rb) TM_CUDA(cudaMemsetAsync(per_root, 0, (re - rb) * 8, st));
     if (chunk_counts) TM_CUDA(cudaMemsetAsync(s.chunk_cnt, 0, (nch + 2) * 8, st));   // counts + list length
     if (q->profile) TM_CUDA(cudaEventRecord(q->ev[0], st));
-    const LaunchCfg lc = search_launch_cfg(g, MODE_COUNT, q->plan.warp_smem, q->plan.tune.warps_per_block);
+    const LaunchCfg lc = search_launch_cfg(g, MODE_COUNT, q->plan.warp_smem, q->plan.tune.warps_per_block,
+                                           plan_features(q->plan), work);
     r = launch_search(g, MODE_COUNT, s.qdev(), 1, q->plan.warp_smem, q->plan.tune.warps_per_block,
                       plan_features(q->plan), &s, st, launch_blocks(g, lc, nch), work);
     if (r != TM_OK) return r;
@@ -605,7 +611,8 @@ extern "C" tm_status tm_enumerate(tm_graph* g, tm_query* q, void* stream, int32_
         qd->total = sc.counters + 1;
         TM_CUDA(cudaMemcpyAsync(sc.head, sc.stage, sc.head_bytes(1), cudaMemcpyHostToDevice, st));
         if (q->profile) TM_CUDA(cudaEventRecord(q->ev[2], st));
-        const LaunchCfg lc = search_launch_cfg(g, MODE_FILL, q->plan.warp_smem_fill, q->plan.tune.warps_per_block);
+        const LaunchCfg lc = search_launch_cfg(g, MODE_FILL, q->plan.warp_smem_fill, q->plan.tune.warps_per_block,
+                                               plan_features(q->plan));
         s = launch_search(g, MODE_FILL, sc.qdev(), 1, q->plan.warp_smem_fill, q->plan.tune.warps_per_block,
                          plan_features(q->plan), &sc, st, launch_blocks(g, lc, nch));
         if (s != TM_OK) return s;
@@ -624,12 +631,14 @@ namespace tmg {
 std::vector<LaunchGroup> occupancy_groups(const tm_graph* g, Mode mode, const Plan* const* plans,
                                           const uint64_t* nch, int nq, int* order) {
     std::vector<int> grid(nq), wpb(nq);
+    std::vector<unsigned> kind(nq);            // queries that count pairs have a kernel instance of their own
     for (int j = 0; j < nq; ++j) {
         const Plan& p = *plans[j];
         LaunchCfg c = search_launch_cfg(g, mode, mode == MODE_FILL ? p.warp_smem_fill : p.warp_smem,
-                                        p.tune.warps_per_block);
+                                        p.tune.warps_per_block, plan_features(p));
         grid[j] = c.grid;
         wpb[j] = c.warps_per_block;
+        kind[j] = mode == MODE_COUNT ? plan_features(p) & FEAT_PAIRS : 0u;
         order[j] = j;
     }
     // highest occupancy first; within a group the likely most expensive queries
@@ -639,6 +648,7 @@ std::vector<LaunchGroup> occupancy_groups(const tm_graph* g, Mode mode, const Pl
     std::stable_sort(order, order + nq, [&](int a, int b) {
         if (grid[a] != grid[b]) return grid[a] > grid[b];
         if (wpb[a] != wpb[b]) return wpb[a] > wpb[b];
+        if (kind[a] != kind[b]) return kind[a] > kind[b];
         if (plans[a]->k != plans[b]->k) return plans[a]->k > plans[b]->k;
         return plans[a]->delta > plans[b]->delta;
     });
@@ -646,7 +656,8 @@ std::vector<LaunchGroup> occupancy_groups(const tm_graph* g, Mode mode, const Pl
     for (int i = 0; i < nq; ++i) {
         const int j = order[i];
         const Plan& p = *plans[j];
-        if (out.empty() || grid[order[out.back().first]] != grid[j] || wpb[order[out.back().first]] != wpb[j])
+        const int lead = out.empty() ? j : order[out.back().first];
+        if (out.empty() || grid[lead] != grid[j] || wpb[lead] != wpb[j] || kind[lead] != kind[j])
             out.push_back(LaunchGroup{i, 0, 16, wpb[j], 0u, 0});
         LaunchGroup& lg = out.back();
         lg.count++;
@@ -656,7 +667,7 @@ std::vector<LaunchGroup> occupancy_groups(const tm_graph* g, Mode mode, const Pl
     for (LaunchGroup& lg : out) {
         uint64_t chunks = 0;
         for (int i = lg.first; i < lg.first + lg.count; ++i) chunks += nch[order[i]];
-        lg.grid = launch_blocks(g, search_launch_cfg(g, mode, lg.warp_smem, lg.warps), chunks);
+        lg.grid = launch_blocks(g, search_launch_cfg(g, mode, lg.warp_smem, lg.warps, lg.feat), chunks);
     }
     return out;
 }

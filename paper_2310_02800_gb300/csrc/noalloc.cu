@@ -139,7 +139,7 @@ extern "C" tm_status tm_count_batch_noalloc(tm_graph* g, tm_query* const* qs, in
     view.ready = base + OFF_READY;
     view.task_cap = NOALLOC_TASKS;
     s = launch_search(g, MODE_COUNT, (const QueryDev*)(base + OFF_QDEV), nq, warp_smem, warps, feat, &view, st,
-                      launch_blocks(g, search_launch_cfg(g, MODE_COUNT, warp_smem, warps), total_chunks));
+                      launch_blocks(g, search_launch_cfg(g, MODE_COUNT, warp_smem, warps, feat), total_chunks));
     if (s != TM_OK) return s;
     Ctrl done;
     TM_CUDA(cudaMemcpyAsync(&done, base + OFF_CTRL, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));

@@ -62,8 +62,10 @@
 //    launch searches only the listed chunks again, each writing its rows in
 //    lexicographic order from its offset.
 //  * The kernel is instantiated per mode (count, enumeration fill), with or
-//    without work counters, and per feature set (anti-edges, look-ahead), so
-//    a plain motif runs code holding neither.
+//    without work counters, and per feature set (anti-edges, look-ahead, last
+//    edges counted as pairs), so a plain motif runs code holding none: registers
+//    and instruction cache are short (the pair code alone, in the plain instance,
+//    made a 4-edge path 22% slower).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -85,6 +87,7 @@ constexpr uint32_t POSMASK = 0x3FFFFFFFu;
 constexpr unsigned long long NO_CHUNK = ~0ull;
 constexpr uint32_t NEVER = 0xFFFFFFFFu;      // prefix entry past a frame's last parent
 constexpr uint32_t SPAN_FAR = 0xFFFFFFFFu;   // frame window end: recompute from the root
+constexpr uint32_t PAIRS_MAX = 256;          // longest window whose last two edges are counted as pairs
 constexpr uint32_t PAIR_MIN_DEG = 1024;     // closing lookups on shorter lists scan the time window
 constexpr uint32_t PAIR_MIN_WINDOW = 768;   // ... and so do windows shorter than this
 constexpr uint64_t WAIT_NS = 20ull * 1000 * 1000 * 1000;      // idle-wait deadline
@@ -229,6 +232,7 @@ struct Search {
     static constexpr bool ANTI = (FEAT & FEAT_ANTI) != 0;   // anti-edge checks compiled in
     static constexpr bool LOOK = (FEAT & FEAT_LOOK) != 0;   // look-ahead checks compiled in
     static constexpr bool FILTER = LOOK && !STATS;          // ... with their candidate filter
+    static constexpr bool PAIRS = MODE == MODE_COUNT && (FEAT & FEAT_PAIRS) != 0;   // last two edges as pairs
     static constexpr int CAP = MODE == MODE_FILL ? FCAP_FILL : FCAP_COUNT;   // parents per frame
     static constexpr uint32_t DESCEND = CAP - 32;   // a child frame this full is drained next
     using Frame = FrameT<CAP>;
@@ -472,6 +476,15 @@ struct Search {
     // exclusive prefix (the flattened position each window starts at; entries past
     // np never start), computed once per frame.  Returns the flattened total.
     __device__ uint32_t begin_frame(Frame f, uint32_t np) const { return begin_row(&f.pre2(0), np); }
+
+    __device__ static bool pair_level(uint32_t h) { return PAIRS && (h & Hot::PAIRS); }
+
+    // Whether a frame, not begun yet, has only windows that count_pairs() takes.
+    __device__ bool short_windows(Frame f, uint32_t np) const {
+        bool longer = lane < np && f.len(lane) > PAIRS_MAX;
+        if (lane + 32u < np) longer = longer || f.len(lane + 32) > PAIRS_MAX;
+        return !__any_sync(FULL, longer);
+    }
 
     __device__ uint32_t begin_row(uint2* row, uint32_t np) const {
         const uint32_t a = 2u * lane;
@@ -858,6 +871,105 @@ struct Search {
         return mid;
     }
 
+    // Of the lanes in v, those after this lane in its window whose entry is later than t and another
+    // neighbour than x.  starts: bit j = a window starts at lane j > 0; the lanes are in list order.
+    __device__ unsigned later_others(unsigned v, unsigned starts, int64_t t, int32_t x) const {
+        const unsigned above = ~((2u << lane) - 1u), next = starts & above;
+        unsigned m = v & above & (next ? (next & (0u - next)) - 1u : FULL);
+        const int64_t t1 = __shfl_down_sync(FULL, t, 1);
+        if (__any_sync(FULL, (m >> lane & 2u) != 0u && t1 == t)) m &= ~__match_any_sync(FULL, (long long)t);
+        return m & ~__match_any_sync(FULL, x);
+    }
+
+    // Level k - 2 of a count-mode search whose last two edges extend by new nodes from one list (out-stars and
+    // the like): the last edge's window is what follows the candidate in its own window, so the
+    // pairs are counted with ballots, without a frame entry, a window search and another pass
+    // per candidate.  A step takes whole windows, as many as fit 32 lanes; a longer window is taken
+    // in tiles of 32, each against itself and those after it.  Frames with a window above
+    // PAIRS_MAX go the general way, whose subtrees can be donated: tiles cost its square.
+    // 8 queries on 200k edges 361 -> 246 us, four queries' counts and rows on 10M edges 2.32 -> 1.87 ms.
+    __device__ void count_pairs(uint32_t h, Frame f, uint32_t tot) {
+        const int nb = Hot::nb(h), dir = Hot::kind(h) == EXT_IN ? 1 : 0;
+        const int32_t* __restrict__ nbr = g.anbr[dir];
+        const int64_t* __restrict__ ta = g.at[dir];
+        const uint2 pr = 2 * lane < CAP ? f.pre2(lane) : make_uint2(NEVER, NEVER);
+        const bool attrib = q->per_root || q->chunk_cnt;
+        // an entry of parent p's window: false when its neighbour is bound already
+        auto entry = [&](bool act, int p, uint32_t pos, int32_t& x, int64_t& t) -> bool {
+            x = -1;
+            t = 0;
+            if (!act) return false;
+            x = __ldg(nbr + pos);
+            t = __ldg(ta + pos);
+            bool ok = true;
+            for (int j = 0; j < nb; ++j) ok &= f.node(j, p) != x;
+            return ok;
+        };
+        unsigned long long sum = 0;
+        uint32_t off = 0;
+        while (off < tot) {
+            unsigned starts;
+            int p = lane_parent(pr, off, starts);
+            uint32_t n = min(tot - off, 32u);      // entries of whole windows in this step
+            if (off + 32u < tot && !__any_sync(FULL, pr.x == off + 32u || pr.y == off + 32u)) n = starts ? 31u - __clz(starts) : 0u;
+            int32_t x;
+            int64_t t;
+            if (n > 0u) {
+                if (lane >= n) p = 0;
+                const bool ok = entry(lane < n, p, (f.beg(p) & POSMASK) + (off + lane - f.pre(p)), x, t);
+                uint32_t c = __popc(later_others(__ballot_sync(FULL, ok), starts, t, x));
+                if (!ok) c = 0;
+                sum += c;
+                if (attrib) attribute_lanes(f.root(p), c);
+                off += n;
+                continue;
+            }
+            // one window, from off to end
+            p = __shfl_sync(FULL, p, 0);
+            const uint32_t end = p + 1 < CAP ? min(f.pre(p + 1), tot) : tot, b = f.beg(p) & POSMASK, len = end - off;
+            for (uint32_t a = 0; a < len; a += 32u) {
+                const bool ok = entry(a + lane < len, p, b + a + lane, x, t);
+                uint32_t c = __popc(later_others(__ballot_sync(FULL, ok), 0u, t, x));
+                for (uint32_t o = a + 32u; o < len; o += 32u) {
+                    int32_t xo;
+                    int64_t to;
+                    unsigned v = __ballot_sync(FULL, entry(o + lane < len, p, b + o + lane, xo, to));
+                    const int64_t t_last = __shfl_sync(FULL, t, 31);
+                    const bool tie = __shfl_sync(FULL, to, 0) == t_last;
+                    for (int j = 0; j < 32; ++j) {
+                        unsigned same = __shfl_sync(FULL, xo, j) == x ? 1u : 0u;
+                        if (tie) same |= __shfl_sync(FULL, to, j) == t ? 1u : 0u;
+                        v &= ~(same << j);
+                    }
+                    c += __popc(v);
+                }
+                if (!ok) c = 0;
+                sum += c;
+                if (attrib) attribute_lanes(f.root(p), c);
+            }
+            off = end;
+        }
+        acc.total += sum;
+    }
+
+    // Add each lane's c matches of its root, lanes in root order (per-root or per-chunk counts asked for).
+    __device__ void attribute_lanes(uint32_t root, uint32_t c) const {
+        if (!q->per_root) {
+            // one chunk for all of them, mostly
+            const uint32_t cr = (uint32_t)q->plan.tune.chunk_roots, ch = (root - (uint32_t)q->root_begin) / cr;
+            const unsigned with = __ballot_sync(FULL, c > 0u);
+            if (!with) return;
+            const int l = __ffs(with) - 1;
+            const uint32_t first = __shfl_sync(FULL, ch, l);
+            if (!__any_sync(FULL, c > 0u && ch != first)) {
+                const unsigned all = __reduce_add_sync(FULL, c);
+                if (lane == l) atomicAdd(q->chunk_cnt + ch, (unsigned long long)all);
+                return;
+            }
+        }
+        if (c) attribute(root, c);
+    }
+
     // The last level of a count-mode search whose last edge extends by one new
     // node without labels or anti-edges: a candidate survives when its neighbour is none of the
     // bound nodes, so only the neighbour column is read and lanes count on their own.
@@ -903,10 +1015,12 @@ struct Search {
     }
 
     // Drain frame `base`, holding np parents (and everything below it), to completion.
-    __device__ void drain(int base, uint32_t np) {
+    // whole: the windows end where the search's do (a donated task's is a part of one).
+    __device__ void drain(int base, uint32_t np, bool whole) {
         int lvl = base;
         uint32_t h = hot(lvl), hc = lvl + 1 < k ? hot(lvl + 1) : 0u;
         Frame f = frame(lvl), c = lvl + 1 < k ? frame(lvl + 1) : f;
+        bool pairs = pair_level(h) && whole && short_windows(f, np);
         uint32_t off = 0, tot = begin_frame(f, np), nch = 0, pend = 0;
         if (FILTER && (h & Hot::FILT)) build_filter(f, lvl, np);
         while (true) {
@@ -914,6 +1028,10 @@ struct Search {
                 !(h & (Hot::ELABEL | Hot::NLABEL | Hot::ANTI))) {
                 count_ext(lvl, h, f, np, tot);
                 off = tot;
+            } else if (pairs) {
+                count_pairs(h, f, tot);
+                off = tot;
+                pairs = false;
             }
             while (off < tot || (FILTER && pend > 0)) {
                 if (MODE == MODE_COUNT && off < tot) tot = maybe_donate(lvl, f, np, off, tot);
@@ -938,6 +1056,7 @@ struct Search {
                 f = c;
                 if (lvl + 1 < k) { hc = hot(lvl + 1); c = frame(lvl + 1); }
                 off = 0;
+                pairs = pair_level(h) && short_windows(f, np);
                 tot = begin_frame(f, np);
                 if (FILTER) {
                     pend = 0;
@@ -1334,7 +1453,7 @@ struct Search {
                 np = 1;
                 is_task = true;
             }
-            drain(base, np);
+            drain(base, np, !is_task);
             if (MODE == MODE_COUNT && is_task) {
                 __threadfence();      // donations made by this task are reserved before it counts as done
                 if (lane == 0) atomicAdd(&ctrl->done_tasks, 1ULL);
@@ -1376,11 +1495,19 @@ struct Search {
     }
 };
 
-// 64 registers: 32 warps per SM, which the frames' shared memory allows about half of the motifs
-// anyway.  At 56 (36 warps) the candidate loops spilled: 4-path over 15 h windows 21.5 ms
-// against 20.0, 64-query batch 19.2 against 16.7.
+// Registers per thread of an instance.  Plain motifs of up to 4 edges: 64, which is 32 warps per SM (at 56 the
+// candidate loops spilled: 4-path over 15 h windows 21.5 ms, at 64 20.0, at 72 21.3, at
+// 80 22.1).  Where shared memory allows WIDE_WARPS warps or fewer (5 edges: 28) the registers of the others are
+// there to take, and without spills at 80 fewer warps are faster: labelled 5-path on 20M edges
+// 344 us at 64, 313 at 72, 265 at 80.  Pairs (8 queries on 200k edges 278, 259, 247 us),
+// anti-edges (109, 106, 104) and look-ahead (chorded 4-cycle on 100M edges 52, 49, 48 ms) likewise.
+// Fills have the widest frames and 64 did best (four queries' counts and rows 1.85 ms, at 72 1.92).
+constexpr int search_regs(int mode, bool stats, int feat) { return stats || mode == MODE_FILL || feat == 0 ? 64 : 80; }
+constexpr unsigned FEAT_WIDE = 8u;     // a plain count with 80 registers
+constexpr int WIDE_WARPS = 28;
+
 template <int MODE, bool STATS, int FEAT>
-__global__ void __maxnreg__(64) search_kernel(const __grid_constant__ GraphView g,
+__global__ void __maxnreg__(search_regs(MODE, STATS, FEAT)) search_kernel(const __grid_constant__ GraphView g,
                                                      const QueryDev* __restrict__ qs, int nq, int warp_smem,
                                                      Ctrl* ctrl, Task* tasks, uint8_t* ready, uint64_t task_cap) {
     __shared__ Block blk;
@@ -1441,6 +1568,9 @@ std::unordered_map<uint64_t, int> g_blocks_per_sm;   // (device, kernel, warps, 
 // runs the instance holding only the code its plan needs.
 template <int MODE>
 const void* kernel_for(unsigned feat) {
+    // pairs are only faster, not needed: beside a query with checks they are searched like any level
+    if (MODE == MODE_COUNT && (feat & 7u) == FEAT_PAIRS) return (const void*)search_kernel<MODE_COUNT, false, FEAT_PAIRS>;
+    if (MODE == MODE_COUNT && feat == FEAT_WIDE) return (const void*)search_kernel<MODE_COUNT, false, FEAT_WIDE>;
     switch (feat & 3u) {
         case 0: return (const void*)search_kernel<MODE, false, 0>;
         case 1: return (const void*)search_kernel<MODE, false, 1>;
@@ -1493,34 +1623,38 @@ int effective_chunk(const tm_graph* g, const Plan& p, uint64_t roots) {
     return cr;
 }
 
-LaunchCfg search_launch_cfg(const tm_graph* g, Mode mode, int max_warp_smem, int warps_per_block) {
+LaunchCfg search_launch_cfg(const tm_graph* g, Mode mode, int max_warp_smem, int warps_per_block, unsigned feat,
+                            bool stats) {
     LaunchCfg c;
     c.warps_per_block = std::max(1, std::min(16, warps_per_block));
     // keep the block's frames within the shared memory a block may use
     while (c.warps_per_block > 1 && max_warp_smem * c.warps_per_block > MAX_DYN_SMEM) c.warps_per_block--;
     c.smem_bytes = max_warp_smem * c.warps_per_block;
-    int kid = mode == MODE_FILL ? 8 : 0;
-    c.grid = blocks_per_sm(g, kernel_of(mode, false, 0u), kid, c.warps_per_block * 32, c.smem_bytes) * g->num_sms;
+    feat &= 7u;
+    // 228 KB per SM, of which a block takes 1 KB beside its own
+    if (feat == 0 && mode == MODE_COUNT && !stats &&
+        228 * 1024 / (c.smem_bytes + (int)sizeof(Block) + 1024) * c.warps_per_block <= WIDE_WARPS)
+        feat = FEAT_WIDE;
+    c.fn = kernel_of(mode, stats, feat);
+    c.grid = blocks_per_sm(g, c.fn, (mode == MODE_FILL ? 32 : 0) + (stats ? 16 : 0) + (int)feat, c.warps_per_block * 32,
+                           c.smem_bytes) * g->num_sms;
     return c;
 }
 
 tm_status launch_search(const tm_graph* g, Mode mode, const QueryDev* qdev_dev, int nq, int max_warp_smem,
                         int warps_per_block, unsigned feat, const Scratch* s, cudaStream_t st, int grid_override,
                         bool stats) {
-    LaunchCfg c = search_launch_cfg(g, mode, max_warp_smem, warps_per_block);
-    const int grid = grid_override > 0 ? std::min(grid_override, c.grid) : c.grid;
     if (mode == MODE_FILL) stats = false;
-    const void* fn = kernel_of(mode, stats, feat);
-    // the instance's shared-memory limit (set once per launch shape)
-    blocks_per_sm(g, fn, (mode == MODE_FILL ? 8 : 0) + (stats ? 4 : 0) + (int)(feat & 3u), c.warps_per_block * 32,
-                  c.smem_bytes);
+    // sets the instance's shared-memory limit too (once per launch shape)
+    LaunchCfg c = search_launch_cfg(g, mode, max_warp_smem, warps_per_block, feat, stats);
+    const int grid = grid_override > 0 ? std::min(grid_override, c.grid) : c.grid;
     GraphView v = g->v;
     Ctrl* ctrl = s->ctrl();
     Task* tasks = s->tasks;
     uint8_t* ready = s->ready;
     uint64_t cap = s->task_cap;
     void* args[] = {&v, (void*)&qdev_dev, &nq, &max_warp_smem, &ctrl, &tasks, &ready, &cap};
-    TM_CUDA(cudaLaunchKernel(fn, dim3(grid), dim3(c.warps_per_block * 32), args, (size_t)c.smem_bytes, st));
+    TM_CUDA(cudaLaunchKernel(c.fn, dim3(grid), dim3(c.warps_per_block * 32), args, (size_t)c.smem_bytes, st));
     note_launches(1);
     return TM_OK;
 }

@@ -174,7 +174,7 @@ tm_status launch_batch(tm_server* s, Slot& sl) {
     TM_CUDA(cudaMemcpyAsync(cs.head, cs.stage, cs.head_bytes(nq), cudaMemcpyHostToDevice, sl.st));
     TM_CUDA(cudaMemsetAsync(cs.counters, 0, (size_t)nq * 8, sl.st));
     TM_CUDA(cudaMemsetAsync(cs.ready, 0, cs.task_cap, sl.st));
-    LaunchCfg lc = search_launch_cfg(g, MODE_COUNT, warp_smem, warps);
+    LaunchCfg lc = search_launch_cfg(g, MODE_COUNT, warp_smem, warps, feat);
     r = launch_search(g, MODE_COUNT, cs.qdev(), nq, warp_smem, warps, feat, &cs, sl.st, launch_grid(s, lc, base));
     if (r != TM_OK) return r;
     // fill launch over the enumerate requests
@@ -209,7 +209,7 @@ tm_status launch_batch(tm_server* s, Slot& sl) {
     if (ne > 0) {
         fc->total_chunks = fbase;
         TM_CUDA(cudaMemcpyAsync(fs.head, fs.stage, fs.head_bytes(ne), cudaMemcpyHostToDevice, sl.st));
-        LaunchCfg lf = search_launch_cfg(g, MODE_FILL, fsmem, warps);
+        LaunchCfg lf = search_launch_cfg(g, MODE_FILL, fsmem, warps, ffeat);
         r = launch_search(g, MODE_FILL, fs.qdev(), ne, fsmem, warps, ffeat, &fs, sl.st, launch_grid(s, lf, fbase));
         if (r != TM_OK) return r;
     }
@@ -465,7 +465,8 @@ extern "C" tm_status tm_serve_submit(tm_server* s, tm_query* q, int enumerate, u
     r->need = req_bytes(s->g, r->plan, r->enumerate, r->cap);
     r->key = cost_key(r->plan, r->enumerate);
     TM_ENTER(s->g->device);   // the launch shape may query the device's occupancy once
-    const LaunchCfg lc = search_launch_cfg(s->g, MODE_COUNT, r->plan.warp_smem, r->plan.tune.warps_per_block);
+    const LaunchCfg lc = search_launch_cfg(s->g, MODE_COUNT, r->plan.warp_smem, r->plan.tune.warps_per_block,
+                                           plan_features(r->plan));
     r->occ = lc.grid * 32 + lc.warps_per_block;
     if (r->need > s->cfg.mem_budget_bytes) {
         set_error("request needs more device memory than the serving budget");

@@ -172,6 +172,9 @@ struct Hot {
     static constexpr uint32_t ELABEL = 1u << 18, NLABEL = 1u << 19, ANTI = 1u << 20, LOOK = 1u << 21, GAP = 1u << 22;
     // the level's look-ahead on its new node is filtered first (see CandidateFilter)
     static constexpr uint32_t FILT = 1u << 23;
+    // level k - 2, when the last two edges extend by new nodes from one list, without labels,
+    // gaps, anti-edges or look-ahead: their pairs are counted from the window itself
+    static constexpr uint32_t PAIRS = 1u << 24;
     static uint32_t pack(const LevelPlan& lp) {
         return (uint32_t)lp.kind | (uint32_t)(lp.a & 7) << 2 | (uint32_t)(lp.b & 7) << 5 | (uint32_t)lp.nb << 8 |
                (uint32_t)(lp.nx_a + 1) << 12 | (uint32_t)(lp.nx_b + 1) << 15 | (lp.elabel >= 0 ? ELABEL : 0u) |
@@ -222,12 +225,12 @@ struct Plan {
     LevelPlan lv[TM_MAX_EDGES];    // lv[i] for i = 1..k-1 (lv[0]: only the look-ahead of the root)
 };
 
-// Code a plan needs beyond plain search: anti-edge checks, look-ahead checks.
-constexpr unsigned FEAT_ANTI = 1u, FEAT_LOOK = 2u;
+// Code a plan needs beyond plain search: anti-edge checks, look-ahead checks; or can use: pairs.
+constexpr unsigned FEAT_ANTI = 1u, FEAT_LOOK = 2u, FEAT_PAIRS = 4u;
 inline unsigned plan_features(const Plan& p) {
     unsigned f = p.n_anti > 0 ? FEAT_ANTI : 0u;
     for (int i = 0; i < TM_MAX_EDGES; ++i)
-        if (p.lv[i].n_look) f |= FEAT_LOOK;
+        f |= (p.lv[i].n_look ? FEAT_LOOK : 0u) | (p.lv[i].hot & Hot::PAIRS ? FEAT_PAIRS : 0u);
     return f;
 }
 
@@ -377,6 +380,7 @@ void scratch_free(Scratch* s);
 enum Mode { MODE_COUNT = 0, MODE_FILL = 1 };
 
 struct LaunchCfg {
+    const void* fn;      // kernel instance
     int warps_per_block;
     int grid;
     int smem_bytes;      // per block
@@ -409,7 +413,8 @@ tm_status launch_search(const tm_graph* g, Mode mode, const QueryDev* qdev_dev, 
 int launch_blocks(const tm_graph* g, const LaunchCfg& c, uint64_t total_chunks);
 int effective_chunk(const tm_graph* g, const Plan& p, uint64_t roots);
 uint64_t n_chunks(uint64_t roots, int chunk_roots);
-LaunchCfg search_launch_cfg(const tm_graph* g, Mode mode, int max_warp_smem, int warps_per_block);
+LaunchCfg search_launch_cfg(const tm_graph* g, Mode mode, int max_warp_smem, int warps_per_block, unsigned feat,
+                            bool stats = false);
 
 // ------------------------------------------------------------- primitives
 

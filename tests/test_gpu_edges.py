@@ -126,3 +126,42 @@ def test_chord_filter_edges(tmg, w):
         out = torch.full((max(1, len(rows)), mo.k), -7, dtype=torch.int32, device="cuda")
         assert q.enumerate(out)[:2] == (len(rows), want), mo
         assert np.array_equal(out[: len(rows)].cpu().numpy(), rows), mo
+
+
+FANS = [
+    synth.out_star(3, 1000), synth.in_star(3, 1000), synth.out_star(3, 300), synth.Motif([(0, 1), (1, 2), (1, 3)], 1000),
+    synth.Motif([(0, 1), (2, 0), (3, 0)], 900), synth.Motif([(0, 1), (0, 2), (0, 3)], 1000, [1000, 50]),
+    synth.Motif([(0, 1), (0, 2), (0, 3)], 1000, [50, 1000]), synth.Motif([(0, 1), (0, 2), (0, 3)], 1000, elabel=[-1, -1, 1]),
+    synth.out_star(4, 1000),
+]
+
+
+@pytest.mark.parametrize("w", [2, 31, 32, 33, 63, 64, 65, 96, 255, 256, 257, 300])
+def test_fan_window_edges(tmg, w):
+    """Motifs whose last two edges leave (enter) one node, counted as pairs within a window of w entries: around
+    the 32-lane steps and tiles and the longest window taken, with equal times and repeated neighbours, next to
+    many one- and two-entry windows."""
+    rng = np.random.default_rng(100 + w)
+    n = 40 + w
+    hub = np.zeros(w + 1, np.int64)
+    leaf = rng.integers(1, 10 + w // 4, w + 1)
+    few = rng.integers(1, n, 3 * n)
+    src = np.concatenate([hub, leaf, few, rng.integers(0, n, 3 * n)]).astype(np.int32)
+    dst = np.concatenate([leaf, hub, rng.integers(0, n, 3 * n), few]).astype(np.int32)
+    m = len(src)
+    t = np.concatenate([rng.integers(0, max(3, 2 * w // 3), 2 * (w + 1)), rng.integers(0, 20_000, m - 2 * (w + 1))]).astype(np.int64)
+    t[: 2 * (w + 1)] *= 900 // max(3, 2 * w // 3)
+    el, nl = rng.integers(0, 3, m).astype(np.uint8), np.zeros(n, np.uint8)
+    og = oracle.Graph(n, src, dst, t, el, nl)
+    gg = tmg.Graph.load(n, src, dst, t, el, nl)
+    for mo in FANS[: 9 if w <= 65 else 8]:
+        q = gg.compile(mo)
+        want, want_pr = og.count(mo, per_root=True)
+        pr = torch.full((m,), -1, dtype=torch.int64, device="cuda")
+        assert q.count(per_root=pr) == want, mo
+        assert np.array_equal(pr.cpu().numpy(), want_pr.astype(np.int64)), mo
+        assert q.count() == want, mo
+        rows = og.enumerate(mo, cap=5_000)[0]
+        out = torch.full((5_000, mo.k), -7, dtype=torch.int32, device="cuda")
+        assert q.enumerate(out)[:2] == (len(rows), want), mo
+        assert np.array_equal(out[: len(rows)].cpu().numpy(), rows), mo
