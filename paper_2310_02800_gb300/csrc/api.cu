@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <atomic>
 #include <chrono>
+#include <cstddef>
 #include <cstring>
 #include <map>
 #include <memory>
@@ -394,59 +395,113 @@ void query_plan(tm_query* q, Plan* out) {
     *out = q->plan;
 }
 
-// Stage and run one single-query count (optionally with per-root, per-chunk
-// or work outputs).  Leaves results in scratch counters; does not sync.
+// A single query's launches.  Its Scratch::counters hold the control blocks of its count and its fill
+// launch, then the total and the work counters, so that one copy reads all of them back; its
+// Scratch::head holds the two launch records after the (unused) control block.
+constexpr uint64_t CTRL_WORDS = sizeof(Ctrl) / 8, SINGLE_WORK = 2 * CTRL_WORDS + 1,
+                   SINGLE_WORDS = SINGLE_WORK + sizeof(tm_work) / 8 + 1;
+
+struct SingleInit {
+    QueryDev q[2];                       // count, fill
+    unsigned long long* counters;
+    QueryDev* qdev;
+    uint64_t total_chunks, reserved;     // reserved: task slots taken before the launch (fault injection)
+    unsigned long long* zero[3];         // also cleared: task flags, chunk counts, per-root counts
+    uint64_t zero_words[3];
+};
+
+// Everything a single query's launches start from, in one launch: a staged copy and three or four
+// memsets before a kernel of 20 us were 15 us of a small call.
+__global__ void single_init_kernel(const __grid_constant__ SingleInit in) {
+    const uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
+    if (blockIdx.x == 0) {
+        for (uint64_t i = threadIdx.x; i < SINGLE_WORDS; i += blockDim.x)
+            in.counters[i] = i == offsetof(Ctrl, total_chunks) / 8 || i == CTRL_WORDS + offsetof(Ctrl, total_chunks) / 8 ? in.total_chunks
+                             : i == offsetof(Ctrl, q_reserve) / 8 ? in.reserved : 0;
+        for (uint32_t i = threadIdx.x; i < 2 * sizeof(QueryDev) / 4; i += blockDim.x)
+            ((uint32_t*)in.qdev)[i] = ((const uint32_t*)in.q)[i];
+    }
+#pragma unroll
+    for (int z = 0; z < 3; ++z)
+        for (uint64_t i = i0; i < in.zero_words[z]; i += stride) in.zero[z][i] = 0;
+}
+
+// The scratch one of a single query's launches sees.
+static Scratch single_view(const Scratch& s, int which) {
+    Scratch v;
+    v.head = (char*)(s.counters + which * CTRL_WORDS);
+    v.tasks = s.tasks;
+    v.ready = s.ready;
+    v.task_cap = s.task_cap;
+    return v;
+}
+
+// Run one single-query count (optionally with per-root, per-chunk or work outputs);
+// rows and cap: also what the fill launch of an enumeration starts from.  Leaves results in
+// scratch counters; does not sync.
 static tm_status run_count(tm_graph* g, tm_query* q, uint64_t rb, uint64_t re, cudaStream_t st,
-                           unsigned long long* per_root, bool chunk_counts, bool work) {
+                           unsigned long long* per_root, bool chunk_counts, bool work, int32_t* rows = nullptr,
+                           uint64_t cap = 0) {
     Scratch& s = q->scratch;
     const int cr = effective_chunk(g, q->plan, re - rb);
     uint64_t nch = n_chunks(re - rb, cr);
-    tm_status r = scratch_reserve(&s, g->device, 1, 1 + (2 + 2 * TM_MAX_EDGES + 1), chunk_counts ? nch : 0,
-                                  DEFAULT_TASK_CAP);
+    tm_status r = scratch_reserve(&s, g->device, 2, SINGLE_WORDS, chunk_counts ? nch : 0, DEFAULT_TASK_CAP);
     if (r != TM_OK) return r;
-    Ctrl* c = s.ctrl_stage();
-    memset(c, 0, sizeof(Ctrl));
-    c->total_chunks = nch;
+    SingleInit in;
+    memset(&in, 0, sizeof in);
+    in.counters = s.counters;
+    in.qdev = s.qdev();
+    in.total_chunks = nch;
     if (q->inject == 1) {
         // one reserved task slot that no warp will ever publish: a warp that
         // pops it waits out its bounded wait and reports TM_E_TIMEOUT
-        c->q_reserve = 1;
+        in.reserved = 1;
         q->inject = 0;
     }
-    QueryDev* qd = s.qdev_stage();
-    memset(qd, 0, sizeof(QueryDev));
+    QueryDev* qd = in.q;
     qd->plan = q->plan;
     qd->plan.tune.chunk_roots = cr;
     qd->root_begin = rb;
     qd->root_end = re;
     qd->n_chunks = nch;
     qd->chunk_base = 0;
-    qd->total = s.counters;
+    qd->total = s.counters + 2 * CTRL_WORDS;
+    in.q[1] = in.q[0];
     qd->per_root = per_root;
     qd->chunk_cnt = chunk_counts ? s.chunk_cnt : nullptr;
-    qd->work = work ? s.counters + 1 : nullptr;
-    TM_CUDA(cudaMemcpyAsync(s.head, s.stage, s.head_bytes(1), cudaMemcpyHostToDevice, st));
-    TM_CUDA(cudaMemsetAsync(s.counters, 0, s.counters_len * 8, st));
-    TM_CUDA(cudaMemsetAsync(s.ready, 0, s.task_cap, st));
-    if (per_root && re > rb) TM_CUDA(cudaMemsetAsync(per_root, 0, (re - rb) * 8, st));
-    if (chunk_counts) TM_CUDA(cudaMemsetAsync(s.chunk_cnt, 0, (nch + 2) * 8, st));   // counts + list length
+    qd->work = work ? s.counters + SINGLE_WORK : nullptr;
+    in.q[1].total = s.counters + SINGLE_WORDS - 1;
+    in.q[1].chunk_off = s.chunk_cnt;
+    in.q[1].match_out = rows;
+    in.q[1].cap = cap;
+    in.zero[0] = (unsigned long long*)s.ready;
+    in.zero_words[0] = s.task_cap / 8;
+    in.zero[1] = s.chunk_cnt;
+    in.zero_words[1] = chunk_counts ? nch + 2 : 0;       // counts + list length
+    in.zero[2] = per_root;
+    in.zero_words[2] = per_root ? re - rb : 0;
+    const uint64_t most = std::max(std::max(in.zero_words[0], in.zero_words[1]), in.zero_words[2]);
+    single_init_kernel<<<(unsigned)std::min<uint64_t>((most + 1023) / 1024, (uint64_t)g->num_sms * 8), 256, 0, st>>>(in);
+    note_launches(1);
+    TM_CUDA(cudaGetLastError());
     if (q->profile) TM_CUDA(cudaEventRecord(q->ev[0], st));
     const LaunchCfg lc = search_launch_cfg(g, MODE_COUNT, q->plan.warp_smem, q->plan.tune.warps_per_block,
                                            plan_features(q->plan), work);
+    const Scratch v = single_view(s, 0);
     r = launch_search(g, MODE_COUNT, s.qdev(), 1, q->plan.warp_smem, q->plan.tune.warps_per_block,
-                      plan_features(q->plan), &s, st, launch_blocks(g, lc, nch), work);
+                      plan_features(q->plan), &v, st, launch_blocks(g, lc, nch), work);
     if (r != TM_OK) return r;
     if (q->profile) TM_CUDA(cudaEventRecord(q->ev[1], st));
     q->fill_timed = false;
     return TM_OK;
 }
 
-static tm_status read_back(Scratch& s, cudaStream_t st, uint64_t n_counters) {
-    TM_CUDA(cudaMemcpyAsync(s.counters_host, s.counters, n_counters * 8, cudaMemcpyDeviceToHost, st));
-    TM_CUDA(cudaMemcpyAsync(s.stage, s.head, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
+static tm_status read_back(Scratch& s, cudaStream_t st) {
+    TM_CUDA(cudaMemcpyAsync(s.counters_host, s.counters, SINGLE_WORDS * 8, cudaMemcpyDeviceToHost, st));
     TM_CUDA(cudaStreamSynchronize(st));
-    note_search_stats(*s.ctrl_stage());
-    if (s.ctrl_stage()->err) {
+    const Ctrl *c = (const Ctrl*)s.counters_host, *f = (const Ctrl*)(s.counters_host + CTRL_WORDS);
+    note_search_stats(*c);
+    if (c->err || f->err) {
         set_error("a bounded device wait timed out");
         return TM_E_TIMEOUT;
     }
@@ -539,9 +594,9 @@ extern "C" tm_status tm_count_roots(tm_graph* g, tm_query* q, int64_t rb, int64_
     }
     tm_status s = run_count(g, q, (uint64_t)rb, (uint64_t)re, st, (unsigned long long*)per_root_dev, false, false);
     if (s != TM_OK) return s;
-    s = read_back(q->scratch, st, 1);
+    s = read_back(q->scratch, st);
     if (s != TM_OK) return s;
-    *total = q->scratch.counters_host[0];
+    *total = q->scratch.counters_host[2 * CTRL_WORDS];
     return TM_OK;
 }
 
@@ -559,9 +614,9 @@ extern "C" tm_status tm_query_work(tm_graph* g, tm_query* q, void* stream, tm_wo
     if (g->v.m == 0) return TM_OK;
     tm_status s = run_count(g, q, 0, (uint64_t)g->v.m, st, nullptr, false, true);
     if (s != TM_OK) return s;
-    s = read_back(q->scratch, st, 1 + sizeof(tm_work) / 8);
+    s = read_back(q->scratch, st);
     if (s != TM_OK) return s;
-    memcpy(out, q->scratch.counters_host + 1, sizeof(tm_work));
+    memcpy(out, q->scratch.counters_host + SINGLE_WORK, sizeof(tm_work));
     return TM_OK;
 }
 
@@ -581,44 +636,30 @@ extern "C" tm_status tm_enumerate(tm_graph* g, tm_query* q, void* stream, int32_
         return TM_OK;
     }
     // pass 1: per-chunk match counts
-    tm_status s = run_count(g, q, 0, m, st, nullptr, true, false);
+    tm_status s = run_count(g, q, 0, m, st, nullptr, true, false, match_dev, cap);
     if (s != TM_OK) return s;
     Scratch& sc = q->scratch;
     const uint64_t nch = n_chunks(m, effective_chunk(g, q->plan, m));
     // pass 2: chunk offsets, and the chunks the fill pass must search
-    s = exclusive_scan_u64(sc.chunk_cnt, sc.chunk_cnt, nch + 1, sc.scan_tmp, st);
+    s = chunk_offsets(sc.chunk_cnt, nch, cap, sc.scan_tmp, g->num_sms, st);
     if (s != TM_OK) return s;
     if (cap > 0) {
-        s = list_chunks(sc.chunk_cnt, nch, cap, g->num_sms, st);
-        if (s != TM_OK) return s;
-    }
-    s = read_back(sc, st, 1);
-    if (s != TM_OK) return s;
-    const uint64_t tot = sc.counters_host[0];
-    const uint64_t nw = std::min(tot, cap);
-    if (nw > 0) {
-        // pass 3: fill rows in lexicographic order from each chunk's offset
-        Ctrl* c = sc.ctrl_stage();
-        memset(c, 0, sizeof(Ctrl));
-        c->total_chunks = nch;
-        QueryDev* qd = sc.qdev_stage();
-        qd->per_root = nullptr;
-        qd->chunk_cnt = nullptr;
-        qd->chunk_off = sc.chunk_cnt;
-        qd->match_out = match_dev;
-        qd->cap = cap;
-        qd->work = nullptr;
-        qd->total = sc.counters + 1;
-        TM_CUDA(cudaMemcpyAsync(sc.head, sc.stage, sc.head_bytes(1), cudaMemcpyHostToDevice, st));
+        // pass 3: fill rows in lexicographic order from each chunk's offset (nothing to do
+        // when no chunk is listed: cheaper than reading the total first)
         if (q->profile) TM_CUDA(cudaEventRecord(q->ev[2], st));
         const LaunchCfg lc = search_launch_cfg(g, MODE_FILL, q->plan.warp_smem_fill, q->plan.tune.warps_per_block,
                                                plan_features(q->plan));
-        s = launch_search(g, MODE_FILL, sc.qdev(), 1, q->plan.warp_smem_fill, q->plan.tune.warps_per_block,
-                         plan_features(q->plan), &sc, st, launch_blocks(g, lc, nch));
+        const Scratch v = single_view(sc, 1);
+        s = launch_search(g, MODE_FILL, sc.qdev() + 1, 1, q->plan.warp_smem_fill, q->plan.tune.warps_per_block,
+                         plan_features(q->plan), &v, st, launch_blocks(g, lc, nch));
         if (s != TM_OK) return s;
-        if (q->profile) { TM_CUDA(cudaEventRecord(q->ev[3], st)); q->fill_timed = true; }
-        TM_CUDA(cudaStreamSynchronize(st));
+        if (q->profile) TM_CUDA(cudaEventRecord(q->ev[3], st));
     }
+    s = read_back(sc, st);
+    if (s != TM_OK) return s;
+    const uint64_t tot = sc.counters_host[2 * CTRL_WORDS];
+    const uint64_t nw = std::min(tot, cap);
+    q->fill_timed = q->profile && nw > 0;
     *total = tot;
     *n_written = nw;
     return tot > cap ? TM_E_TRUNCATED : TM_OK;
@@ -929,13 +970,8 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
     if (kernel_ms) TM_CUDA(cudaEventRecord(bc->ev[1], st));
     // pass 2: chunk offsets, and the chunks the fill pass must search
     for (int j = 0; j < nq; ++j) {
-        s = exclusive_scan_u64(qs[j]->scratch.chunk_cnt, qs[j]->scratch.chunk_cnt, nch[j] + 1,
-                               qs[j]->scratch.scan_tmp, st);
+        s = chunk_offsets(qs[j]->scratch.chunk_cnt, nch[j], caps[j], qs[j]->scratch.scan_tmp, g->num_sms, st);
         if (s != TM_OK) return s;
-        if (caps[j] > 0) {
-            s = list_chunks(qs[j]->scratch.chunk_cnt, nch[j], caps[j], g->num_sms, st);
-            if (s != TM_OK) return s;
-        }
     }
     // pass 3: rows of the queries with room for some, written from each chunk's
     // offset on the device (chunks past the cap or without matches are skipped)

@@ -1548,10 +1548,78 @@ __global__ void list_chunks_kernel(unsigned long long* buf, uint64_t nch, uint64
     }
 }
 
+// Scan and list of a small chunk buffer in one block: a launch each for the scan's two levels and the
+// list took 15 us between the passes of a 100 us call.
+constexpr int SMALL_THREADS = 1024, SMALL_ITEMS = 4;
+constexpr uint64_t SMALL_CHUNKS = 16384;      // four rounds of the block; longer buffers scan faster on many
+
+__global__ void __launch_bounds__(SMALL_THREADS) small_offsets_kernel(unsigned long long* buf, uint32_t nch, uint64_t cap) {
+    __shared__ unsigned long long wsum[SMALL_THREADS / 32];
+    __shared__ uint32_t wkeep[SMALL_THREADS / 32];
+    uint32_t* list = (uint32_t*)(buf + nch + 2);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long carry = 0;
+    uint32_t listed = 0;
+    for (uint32_t base = 0; base <= nch; base += SMALL_THREADS * SMALL_ITEMS) {
+        const uint32_t c0 = base + threadIdx.x * SMALL_ITEMS;
+        unsigned long long v[SMALL_ITEMS], sum = 0;
+#pragma unroll
+        for (int j = 0; j < SMALL_ITEMS; ++j) {
+            v[j] = c0 + j < nch ? buf[c0 + j] : 0;        // entry nch, past the counts, becomes the total
+            sum += v[j];
+        }
+        unsigned long long inc = sum;
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned long long u = __shfl_up_sync(FULL, inc, d);
+            if (lane >= d) inc += u;
+        }
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        unsigned long long at = carry + inc - sum;
+        for (int w = 0; w < SMALL_THREADS / 32; ++w) {
+            if (w < warp) at += wsum[w];
+            carry += wsum[w];
+        }
+        uint32_t keep = 0;
+#pragma unroll
+        for (int j = 0; j < SMALL_ITEMS; ++j) {
+            if (c0 + j <= nch) buf[c0 + j] = at;
+            if (v[j] > 0 && at < cap) keep |= 1u << j;
+            at += v[j];
+        }
+        uint32_t kin = __popc(keep);
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t u = __shfl_up_sync(FULL, kin, d);
+            if (lane >= d) kin += u;
+        }
+        if (lane == 31) wkeep[warp] = kin;
+        __syncthreads();
+        uint32_t to = listed + kin - __popc(keep);
+        for (int w = 0; w < SMALL_THREADS / 32; ++w) {
+            if (w < warp) to += wkeep[w];
+            listed += wkeep[w];
+        }
+#pragma unroll
+        for (int j = 0; j < SMALL_ITEMS; ++j)
+            if (keep >> j & 1u) list[to++] = c0 + j;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) buf[nch + 1] = listed;
+}
+
 }  // namespace
 
-tm_status list_chunks(unsigned long long* chunk_buf, uint64_t nch, uint64_t cap, int num_sms, cudaStream_t st) {
+tm_status chunk_offsets(unsigned long long* chunk_buf, uint64_t nch, uint64_t cap, void* scan_tmp, int num_sms,
+                        cudaStream_t st) {
     if (nch == 0) return TM_OK;
+    if (nch <= SMALL_CHUNKS) {
+        small_offsets_kernel<<<1, SMALL_THREADS, 0, st>>>(chunk_buf, (uint32_t)nch, cap);
+        note_launches(1);
+        TM_CUDA(cudaGetLastError());
+        return TM_OK;
+    }
+    tm_status s = exclusive_scan_u64(chunk_buf, chunk_buf, nch + 1, scan_tmp, st);
+    if (s != TM_OK || cap == 0) return s;
     const uint64_t blocks = std::min<uint64_t>((nch + 255) / 256, (uint64_t)num_sms * 8);
     list_chunks_kernel<<<(unsigned)blocks, 256, 0, st>>>(chunk_buf, nch, cap);
     note_launches(1);

@@ -165,3 +165,21 @@ def test_fan_window_edges(tmg, w):
         out = torch.full((5_000, mo.k), -7, dtype=torch.int32, device="cuda")
         assert q.enumerate(out)[:2] == (len(rows), want), mo
         assert np.array_equal(out[: len(rows)].cpu().numpy(), rows), mo
+
+
+@pytest.mark.parametrize("chunks", [1, 4095, 4096, 4097, 16384, 16385])
+def test_row_offsets_edges(tmg, chunks):
+    """Enumerations whose chunk counts end around a round of the one-block offset scan and around its
+    largest buffer: every row, and buffers that hold none, one, half and all but one of them."""
+    m = 8 * chunks
+    n, src, dst, t, el, nl = graph(max(4, min(50, m)), m, 4 * m, seed=chunks)
+    og = oracle.Graph(n, src, dst, t, el, nl)
+    gg = tmg.Graph.load(n, src, dst, t, el, nl)
+    for mo in (synth.Motif([(0, 1), (1, 0)], 400), synth.out_star(2, 60)):
+        q = gg.compile(mo)
+        rows = og.enumerate(mo)[0]
+        for cap in sorted({0, 1, len(rows) // 2, max(0, len(rows) - 1), len(rows) + 1}):
+            out = torch.full((cap, mo.k), -7, dtype=torch.int32, device="cuda")
+            w = min(cap, len(rows))
+            assert q.enumerate(out) == (w, len(rows), len(rows) > cap), (mo, cap)
+            assert np.array_equal(out[:w].cpu().numpy(), rows[:w]) and (out[w:] == -7).all(), (mo, cap)
