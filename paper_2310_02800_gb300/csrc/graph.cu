@@ -20,17 +20,16 @@ namespace {
 
 struct Check {
     unsigned long long tmin, tmax;
-    unsigned long long bad;       // count of out-of-range ids / negative times
+    unsigned long long bad;       // count of negative times
     unsigned long long descents;  // count of t[i] > t[i+1]
+    unsigned long long bad_nodes; // not 0: some id is out of range
 };
 
-__global__ void check_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
-                             const int64_t* __restrict__ t, int64_t m, int64_t n, Check* out) {
+__global__ void check_times_kernel(const int64_t* __restrict__ t, int64_t m, Check* out) {
     unsigned long long tmin = ~0ULL, tmax = 0, bad = 0, desc = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t s = src[i], d = dst[i];
-        int64_t ti = t[i];
-        if (s < 0 || s >= n || d < 0 || d >= n || ti < 0) bad++;
+        const int64_t ti = t[i];
+        if (ti < 0) bad++;
         unsigned long long u = (unsigned long long)(ti < 0 ? 0 : ti);
         tmin = min(tmin, u);
         tmax = max(tmax, u);
@@ -50,6 +49,16 @@ __global__ void check_kernel(const int32_t* __restrict__ src, const int32_t* __r
     }
 }
 
+__global__ void check_nodes_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t m, int64_t n,
+                                   Check* out) {
+    bool bad = false;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t s = src[i], d = dst[i];
+        bad = bad || s < 0 || s >= n || d < 0 || d >= n;
+    }
+    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicAdd(&out->bad_nodes, 1ULL);
+}
+
 template <typename K>
 __global__ void time_keys_kernel(const int64_t* __restrict__ t, int64_t m, unsigned long long tmin,
                                  K* __restrict__ keys) {
@@ -61,7 +70,14 @@ __global__ void time_keys_kernel(const int64_t* __restrict__ t, int64_t m, unsig
 // issued before the first is used, since each is a sector from anywhere in the column.
 constexpr int GATHER = 4;
 
-// Edge columns in edge-id order.  The sorted keys are the times; without them
+// An edge as one 16-byte record, for the gathers into list order: one sector per entry, where
+// the time and the endpoint columns are two.
+struct __align__(16) EdgeRec {
+    int64_t t;
+    int32_t src, dst;
+};
+
+// Edge columns in edge-id order, and the same as records.  The sorted keys are the times; without them
 // (keys null) the input is in time order already and perm is null too.
 template <typename K>
 __global__ void gather_edges_kernel(const uint32_t* __restrict__ perm, const K* __restrict__ keys,
@@ -69,7 +85,7 @@ __global__ void gather_edges_kernel(const uint32_t* __restrict__ perm, const K* 
                                     const int32_t* __restrict__ dst, const int64_t* __restrict__ t,
                                     const uint8_t* __restrict__ el, int32_t* __restrict__ src_o,
                                     int32_t* __restrict__ dst_o, int64_t* __restrict__ t_o, uint8_t* __restrict__ el_o,
-                                    int32_t* __restrict__ perm_o) {
+                                    int32_t* __restrict__ perm_o, EdgeRec* __restrict__ rec_o) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e0 < m; e0 += GATHER * stride) {
         uint32_t i[GATHER];
@@ -95,6 +111,7 @@ __global__ void gather_edges_kernel(const uint32_t* __restrict__ perm, const K* 
             dst_o[e] = d[j];
             t_o[e] = tt[j];
             if (el) el_o[e] = el[i[j]];
+            rec_o[e] = EdgeRec{tt[j], s[j], d[j]};
             perm_o[e] = (int32_t)i[j];
         }
     }
@@ -114,28 +131,25 @@ __global__ void offsets_kernel(const uint32_t* __restrict__ nodes, int64_t m, in
     }
 }
 
-// List columns (time, other endpoint, edge id) from the list's edge ids.
-__global__ void list_columns_kernel(const uint32_t* __restrict__ eids, int64_t m, const int64_t* __restrict__ t,
-                                    const int32_t* __restrict__ other, int64_t* __restrict__ at,
-                                    int32_t* __restrict__ anbr, int32_t* __restrict__ aeid) {
+// List columns (time, other endpoint, edge id) from the list's edge ids.  Bound by its
+// random sectors: 10M edges took 180 us from the time and endpoint columns, 158 from records.
+template <bool IN>
+__global__ void list_columns_kernel(const uint32_t* __restrict__ eids, int64_t m, const EdgeRec* __restrict__ rec,
+                                    int64_t* __restrict__ at, int32_t* __restrict__ anbr, int32_t* __restrict__ aeid) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < m; i0 += GATHER * stride) {
         uint32_t e[GATHER];
-        int64_t tt[GATHER];
-        int32_t o[GATHER];
+        int4 r[GATHER];
 #pragma unroll
         for (int j = 0; j < GATHER; ++j) e[j] = i0 + j * stride < m ? eids[i0 + j * stride] : 0u;
 #pragma unroll
-        for (int j = 0; j < GATHER; ++j) {
-            tt[j] = t[e[j]];
-            o[j] = other[e[j]];
-        }
+        for (int j = 0; j < GATHER; ++j) r[j] = __ldg((const int4*)(rec + e[j]));
 #pragma unroll
         for (int j = 0; j < GATHER; ++j) {
             const int64_t i = i0 + j * stride;
             if (i >= m) break;
-            at[i] = tt[j];
-            anbr[i] = o[j];
+            at[i] = (int64_t)((uint64_t)(uint32_t)r[j].x | (uint64_t)(uint32_t)r[j].y << 32);
+            anbr[i] = IN ? r[j].z : r[j].w;
             aeid[i] = (int32_t)e[j];
         }
     }
@@ -159,8 +173,8 @@ __global__ void successor_by_position_kernel(int64_t m, const int32_t* __restric
         }
 #pragma unroll
         for (int j = 0; j < GATHER; ++j) {
-            wo[j] = so_dst[eo[j]];
-            wi[j] = si_src[ei[j]];
+            wo[j] = so_dst[2u * (uint32_t)eo[j]];
+            wi[j] = si_src[2u * (uint32_t)ei[j]];
         }
 #pragma unroll
         for (int j = 0; j < GATHER; ++j) {
@@ -206,7 +220,9 @@ __device__ __forceinline__ uint2 succ_word(const int64_t* __restrict__ t, uint32
 // Successor index of one direction's lists, in list order.  Entry i of node v's
 // list is edge e at time te: the first later entry of the same list (the search
 // starts just past i) and the first later entry of v's list in the other direction,
-// each with its time gap.  A search level whose candidate list belongs to an endpoint of
+// each with its time gap.  Both go to the edge in one 16-byte store: 10M edges took 690 us per
+// direction when they were two stores to anywhere, 349 as one (reading them back in list order
+// takes 352 us instead of 238, from columns twice as wide).  A search level whose candidate list belongs to an endpoint of
 // the previous level's edge reads its window start here instead of
 // binary-searching the list, and skips the window when the gap already
 // exceeds it.  In list order, neighbouring threads search the same node's lists
@@ -215,8 +231,7 @@ __device__ __forceinline__ uint2 succ_word(const int64_t* __restrict__ t, uint32
 __global__ void successor_kernel(int64_t m, const uint32_t* __restrict__ nodes, const int32_t* __restrict__ eid,
                                  const uint32_t* __restrict__ off, const int64_t* __restrict__ at,
                                  const uint32_t* __restrict__ off_x, const int64_t* __restrict__ at_x,
-                                 uint2* __restrict__ same_by_pos, uint2* __restrict__ same_by_edge,
-                                 uint2* __restrict__ cross_by_edge) {
+                                 uint2* __restrict__ same_by_pos, uint4* __restrict__ by_edge) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t v = nodes[i];
         const int32_t e = eid[i];
@@ -224,21 +239,22 @@ __global__ void successor_kernel(int64_t m, const uint32_t* __restrict__ nodes, 
         uint32_t hi = off[v + 1];
         const uint2 w = succ_word(at, first_later_from(at, (uint32_t)i + 1u, hi, te), hi, te);
         same_by_pos[i] = w;
-        same_by_edge[e] = w;
         hi = off_x[v + 1];
-        cross_by_edge[e] = succ_word(at_x, first_later(at_x, off_x[v], hi, te), hi, te);
+        const uint2 x = succ_word(at_x, first_later(at_x, off_x[v], hi, te), hi, te);
+        by_edge[e] = make_uint4(w.x, w.y, x.x, x.y);
     }
 }
 
 // Root filter (see GraphView::rcode) from the four words of each edge.  A streaming pass of its own:
 // storing the two bytes of a direction from successor_kernel, whose edges come in list
 // order, is a partial sector per edge and cost ten times as much (0.5 ms for 10M edges).
-__global__ void root_codes_kernel(int64_t m, const uint2* __restrict__ out_src, const uint2* __restrict__ in_dst,
-                                  const uint2* __restrict__ out_dst, const uint2* __restrict__ in_src,
+__global__ void root_codes_kernel(int64_t m, const uint4* __restrict__ by_out, const uint4* __restrict__ by_in,
                                   uint32_t* __restrict__ rcode) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x)
-        rcode[e] = gap_code(out_src[e].y) << (8 * succ_byte(NX_OUT_SRC)) | gap_code(in_dst[e].y) << (8 * succ_byte(NX_IN_DST)) |
-                   gap_code(out_dst[e].y) << (8 * succ_byte(NX_OUT_DST)) | gap_code(in_src[e].y) << (8 * succ_byte(NX_IN_SRC));
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
+        const uint4 o = by_out[e], i = by_in[e];
+        rcode[e] = gap_code(o.y) << (8 * succ_byte(NX_OUT_SRC)) | gap_code(o.w) << (8 * succ_byte(NX_IN_SRC)) |
+                   gap_code(i.y) << (8 * succ_byte(NX_IN_DST)) | gap_code(i.w) << (8 * succ_byte(NX_OUT_DST));
+    }
 }
 
 int bits_for(unsigned long long x) {
@@ -268,6 +284,37 @@ struct Pool {  // temporary device allocations, stream-ordered, freed at scope e
     }
 };
 
+// Host edge lists of at least this many edges copy their endpoints on a stream of their own, beside
+// the time sort; below, the stream and its events cost what the overlap gives.
+constexpr int64_t OVERLAP_MIN = 1 << 19;
+
+// That stream: after what st held when it was opened; st goes on after it once joined.  It is
+// drained before the buffers it writes (declared earlier) are freed.
+struct Side {
+    cudaStream_t st, cs = nullptr;
+    cudaEvent_t ev = nullptr;
+    explicit Side(cudaStream_t s) : st(s) {}
+    tm_status open() {
+        TM_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+        TM_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        TM_CUDA(cudaEventRecord(ev, st));
+        TM_CUDA(cudaStreamWaitEvent(cs, ev, 0));
+        return TM_OK;
+    }
+    tm_status join() {
+        TM_CUDA(cudaEventRecord(ev, cs));
+        TM_CUDA(cudaStreamWaitEvent(st, ev, 0));
+        return TM_OK;
+    }
+    ~Side() {
+        if (cs) {
+            cudaStreamSynchronize(cs);
+            cudaStreamDestroy(cs);
+        }
+        if (ev) cudaEventDestroy(ev);
+    }
+};
+
 // Graph storage is one allocation (one cudaMalloc at load, one cudaFree at
 // free, instead of one per column: ~2 ms less per load/free cycle of a
 // 10M-edge graph), carved into 256-byte aligned columns.
@@ -284,7 +331,8 @@ size_t storage_bytes(int64_t n, int64_t m, bool node_labels, bool edge_labels) {
     if (edge_labels) b += col_bytes(m, 1);
     b += 2 * (col_bytes(n + 1, 4) + col_bytes(m, 8) + col_bytes(m, 4) * 2);  // out / in lists
     b += col_bytes(m, 4) + col_bytes(m, 8) + col_bytes(m, 4);               // pair-ordered list
-    b += 8 * col_bytes(m, sizeof(uint2)) + col_bytes(m, 4);                   // successor words, root filter
+    b += 2 * col_bytes(m, sizeof(uint4)) + 4 * col_bytes(m, sizeof(uint2));   // successor words
+    b += col_bytes(m, 4);                                                     // root filter
     return b;
 }
 
@@ -333,22 +381,21 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
     const int32_t *src = e->src, *dst = e->dst;
     const int64_t* t = e->t;
     const uint8_t* el = e->elabel;
-    if (!e->on_device && m > 0) {
-        int32_t *s2, *d2;
+    const bool host = !e->on_device && m > 0;
+    // host endpoints and labels are copied and checked beside the time sort
+    Side side(st);
+    const bool overlap = host && m >= OVERLAP_MIN;
+    cudaStream_t cs = st;
+    int32_t *s2 = nullptr, *d2 = nullptr;
+    uint8_t* el2 = nullptr;
+    if (host) {
         int64_t* t2;
         TRY(tmp.get(&s2, m));
         TRY(tmp.get(&d2, m));
         TRY(tmp.get(&t2, m));
-        TM_CUDA(cudaMemcpyAsync(s2, src, m * 4, cudaMemcpyHostToDevice, st));
-        TM_CUDA(cudaMemcpyAsync(d2, dst, m * 4, cudaMemcpyHostToDevice, st));
+        if (el) TRY(tmp.get(&el2, m));
         TM_CUDA(cudaMemcpyAsync(t2, t, m * 8, cudaMemcpyHostToDevice, st));
-        src = s2; dst = d2; t = t2;
-        if (el) {
-            uint8_t* e2;
-            TRY(tmp.get(&e2, m));
-            TM_CUDA(cudaMemcpyAsync(e2, el, m, cudaMemcpyHostToDevice, st));
-            el = e2;
-        }
+        t = t2;
     }
     GraphView& v = g->v;
     v.n = n; v.m = m;
@@ -363,24 +410,47 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
     // 1. validate
     Check* chk;
     TRY(tmp.get(&chk, 1));
-    Check init{~0ULL, 0ULL, 0ULL, 0ULL};
+    Check init{~0ULL, 0ULL, 0ULL, 0ULL, 0ULL}, hc;
     TM_CUDA(cudaMemcpyAsync(chk, &init, sizeof(Check), cudaMemcpyHostToDevice, st));
+    if (overlap) {
+        TRY(side.open());              // ordered after the allocations and the cleared counters
+        cs = side.cs;
+    }
     if (m > 0) {
-        check_kernel<<<grid_for(m, sms), 256, 0, st>>>(src, dst, t, m, n, chk);
+        check_times_kernel<<<grid_for(m, sms), 256, 0, st>>>(t, m, chk);
         note_launches(1);
         TM_CUDA(cudaGetLastError());
     }
-    Check hc;
-    TM_CUDA(cudaMemcpyAsync(&hc, chk, sizeof(Check), cudaMemcpyDeviceToHost, st));
-    TM_CUDA(cudaStreamSynchronize(st));
-    if (hc.bad) {
-        set_error("edge endpoint out of [0, n_nodes) or negative timestamp");
-        return TM_E_INVALID;
-    }
+    // the endpoints, on cs: copied where they come from the host, then checked
+    auto endpoints = [&]() -> tm_status {
+        if (host) {
+            TM_CUDA(cudaMemcpyAsync(s2, src, m * 4, cudaMemcpyHostToDevice, cs));
+            TM_CUDA(cudaMemcpyAsync(d2, dst, m * 4, cudaMemcpyHostToDevice, cs));
+            if (el) TM_CUDA(cudaMemcpyAsync(el2, el, m, cudaMemcpyHostToDevice, cs));
+            src = s2; dst = d2; el = el2;
+        }
+        if (m > 0) {
+            check_nodes_kernel<<<grid_for(m, sms), 256, 0, cs>>>(src, dst, m, n, chk);
+            note_launches(1);
+            TM_CUDA(cudaGetLastError());
+        }
+        return TM_OK;
+    };
+    auto read_check = [&](cudaStream_t on) -> tm_status {
+        TM_CUDA(cudaMemcpyAsync(&hc, chk, sizeof(Check), cudaMemcpyDeviceToHost, on));
+        TM_CUDA(cudaStreamSynchronize(on));
+        if (hc.bad || hc.bad_nodes) {
+            set_error("edge endpoint out of [0, n_nodes) or negative timestamp");
+            return TM_E_INVALID;
+        }
+        return TM_OK;
+    };
+    if (!overlap) TRY(endpoints());
+    TRY(read_check(st));
     // 2. time order
     const uint64_t um = (uint64_t)m;
     const int grid = grid_for(m, sms), grid4 = grid_for((m + GATHER - 1) / GATHER, sms);
-    uint32_t *ka[2], *kb[2], *va[2], *keys_of[2];
+    uint32_t *ka[2], *kb[2], *va[2], *keys_of[2], *spare[2];
     for (int j = 0; j < 2; ++j) {
         TRY(tmp.get(&ka[j], m));
         TRY(tmp.get(&kb[j], m));
@@ -397,23 +467,21 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
     TRY(owned(g, &t_o, m));
     TRY(owned(g, &p_o, m));
     if (el) TRY(owned(g, &el_o, m));
-    // 3. edge columns in edge-id order
+    EdgeRec* rec;
+    TRY(tmp.get(&rec, m));
     if (m > 0) {
         const int tbits = bits_for(hc.tmax - hc.tmin);
+        const bool sorted = hc.descents == 0, narrow = tbits <= 32;
         int w = 0;
-        if (hc.descents == 0) {
-            gather_edges_kernel<uint32_t><<<grid4, 256, 0, st>>>(nullptr, nullptr, 0, m, src, dst, t, el, s_o, d_o, t_o,
-                                                                 el_o, p_o);
-        } else if (tbits <= 32) {
+        uint64_t* k8[2] = {nullptr, nullptr};
+        if (!sorted && narrow) {
             // a time range below 2^32: 4-byte keys
             time_keys_kernel<uint32_t><<<grid, 256, 0, st>>>(t, m, hc.tmin, kb[0]);
             note_launches(1);
             TM_CUDA(cudaGetLastError());
             TRY(radix_sort_pairs<uint32_t>(kb[0], nullptr, ka, va, um, tbits, rtemp, rtemp_bytes, st, &w));
-            gather_edges_kernel<uint32_t><<<grid4, 256, 0, st>>>(va[w], ka[w], hc.tmin, m, src, dst, t, el, s_o, d_o, t_o,
-                                                                 el_o, p_o);
-        } else {
-            uint64_t *k0, *k8[2];
+        } else if (!sorted) {
+            uint64_t* k0;
             TRY(tmp.get(&k0, m));
             TRY(tmp.get(&k8[0], m));
             TRY(tmp.get(&k8[1], m));
@@ -421,9 +489,22 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
             note_launches(1);
             TM_CUDA(cudaGetLastError());
             TRY(radix_sort_pairs<uint64_t>(k0, nullptr, k8, va, um, tbits, rtemp, rtemp_bytes, st, &w));
-            gather_edges_kernel<uint64_t><<<grid4, 256, 0, st>>>(va[w], k8[w], hc.tmin, m, src, dst, t, el, s_o, d_o, t_o,
-                                                                 el_o, p_o);
         }
+        if (overlap) {
+            TRY(endpoints());
+            TRY(read_check(cs));
+            TRY(side.join());
+        }
+        // 3. edge columns in edge-id order
+        if (sorted)
+            gather_edges_kernel<uint32_t><<<grid4, 256, 0, st>>>(nullptr, nullptr, 0, m, src, dst, t, el, s_o, d_o, t_o,
+                                                                 el_o, p_o, rec);
+        else if (narrow)
+            gather_edges_kernel<uint32_t><<<grid4, 256, 0, st>>>(va[w], ka[w], hc.tmin, m, src, dst, t, el, s_o, d_o, t_o,
+                                                                 el_o, p_o, rec);
+        else
+            gather_edges_kernel<uint64_t><<<grid4, 256, 0, st>>>(va[w], k8[w], hc.tmin, m, src, dst, t, el, s_o, d_o, t_o,
+                                                                 el_o, p_o, rec);
         note_launches(1);
         TM_CUDA(cudaGetLastError());
     }
@@ -433,7 +514,6 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
     const int nbits = bits_for((unsigned long long)(n > 0 ? n - 1 : 0));
     for (int dir = 0; dir < 2; ++dir) {
         const int32_t* key_node = dir == 0 ? s_o : d_o;
-        const int32_t* other = dir == 0 ? d_o : s_o;
         uint32_t* off;
         int64_t* at;
         int32_t *anbr, *aeid;
@@ -445,11 +525,13 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
         int w = 0;
         TRY(radix_sort_pairs<uint32_t>((const uint32_t*)key_node, nullptr, nk, va, um, nbits, rtemp, rtemp_bytes, st, &w));
         keys_of[dir] = nk[w];
+        spare[dir] = nk[w ^ 1];
         offsets_kernel<<<grid_for(n + 1, sms), 256, 0, st>>>(keys_of[dir], m, n + 1, off);
         note_launches(1);
         TM_CUDA(cudaGetLastError());
         if (m > 0) {
-            list_columns_kernel<<<grid4, 256, 0, st>>>(va[w], m, t_o, other, at, anbr, aeid);
+            if (dir == 0) list_columns_kernel<false><<<grid4, 256, 0, st>>>(va[w], m, rec, at, anbr, aeid);
+            else list_columns_kernel<true><<<grid4, 256, 0, st>>>(va[w], m, rec, at, anbr, aeid);
             note_launches(1);
             TM_CUDA(cudaGetLastError());
         }
@@ -465,35 +547,35 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
         TRY(owned(g, &ptm, m));
         TRY(owned(g, &pe, m));
         if (m > 0) {
-            uint32_t* pk[2];                      // the sorted sources are not needed
-            for (int j = 0; j < 2; ++j) TRY(tmp.get(&pk[j], m));
-            int w = 0;
-            TRY(radix_sort_pairs<uint32_t>((const uint32_t*)v.anbr[1], (const uint32_t*)v.aeid[1], pk, va, um, nbits,
+            int w = 0;                            // the sorted sources are not needed
+            TRY(radix_sort_pairs<uint32_t>((const uint32_t*)v.anbr[1], (const uint32_t*)v.aeid[1], spare, va, um, nbits,
                                            rtemp, rtemp_bytes, st, &w));
-            list_columns_kernel<<<grid4, 256, 0, st>>>(va[w], m, t_o, d_o, ptm, pn, pe);
+            list_columns_kernel<false><<<grid4, 256, 0, st>>>(va[w], m, rec, ptm, pn, pe);
             note_launches(1);
             TM_CUDA(cudaGetLastError());
         }
         v.pnbr = pn; v.pt = ptm; v.peid = pe;
     }
     // 6. successor index (window starts for lists that touch the previous edge)
-    uint2 *nx[4], *px[4];
-    for (int j = 0; j < 4; ++j) TRY(owned(g, &nx[j], m));
+    uint4* by_edge[2];                            // by out-list order, by in-list order
+    uint2* px[4];
+    for (int j = 0; j < 2; ++j) TRY(owned(g, &by_edge[j], m));
     for (int j = 0; j < 4; ++j) TRY(owned(g, &px[j], m));
     uint32_t* codes;
     TRY(owned(g, &codes, m));
+    v.nxt[NX_OUT_SRC] = (const uint2*)by_edge[0];
+    v.nxt[NX_IN_SRC] = (const uint2*)by_edge[0] + 1;
+    v.nxt[NX_IN_DST] = (const uint2*)by_edge[1];
+    v.nxt[NX_OUT_DST] = (const uint2*)by_edge[1] + 1;
     if (m > 0) {
-        successor_kernel<<<grid, 256, 0, st>>>(m, keys_of[0], v.aeid[0], v.off[0], v.at[0], v.off[1], v.at[1], px[0],
-                                               nx[NX_OUT_SRC], nx[NX_IN_SRC]);
-        successor_kernel<<<grid, 256, 0, st>>>(m, keys_of[1], v.aeid[1], v.off[1], v.at[1], v.off[0], v.at[0], px[2],
-                                               nx[NX_IN_DST], nx[NX_OUT_DST]);
-        successor_by_position_kernel<<<grid4, 256, 0, st>>>(m, v.aeid[0], v.aeid[1], nx[NX_OUT_DST], nx[NX_IN_SRC],
+        successor_kernel<<<grid, 256, 0, st>>>(m, keys_of[0], v.aeid[0], v.off[0], v.at[0], v.off[1], v.at[1], px[0], by_edge[0]);
+        successor_kernel<<<grid, 256, 0, st>>>(m, keys_of[1], v.aeid[1], v.off[1], v.at[1], v.off[0], v.at[0], px[2], by_edge[1]);
+        successor_by_position_kernel<<<grid4, 256, 0, st>>>(m, v.aeid[0], v.aeid[1], v.nxt[NX_OUT_DST], v.nxt[NX_IN_SRC],
                                                            px[1], px[3]);
-        root_codes_kernel<<<grid, 256, 0, st>>>(m, nx[NX_OUT_SRC], nx[NX_IN_DST], nx[NX_OUT_DST], nx[NX_IN_SRC], codes);
+        root_codes_kernel<<<grid, 256, 0, st>>>(m, by_edge[0], by_edge[1], codes);
         note_launches(4);
         TM_CUDA(cudaGetLastError());
     }
-    for (int j = 0; j < 4; ++j) v.nxt[j] = nx[j];
     for (int j = 0; j < 4; ++j) v.pnx[j] = px[j];
     v.rcode = codes;
     TM_CUDA(cudaStreamSynchronize(st));

@@ -153,22 +153,23 @@ tm_status exclusive_scan_u64(const unsigned long long* in, unsigned long long* o
 // is how the scatter's writes fall: an element's destination is anywhere, so
 // writing from registers touches a 32-byte sector per element.  The scatter therefore
 // orders its tile in shared memory first and writes each digit's run with
-// consecutive threads: 4,096 elements over 128 digits are runs of 128 bytes.
+// consecutive threads: 8,192 elements over 128 digits are runs of 256 bytes.
 
 namespace {
-constexpr int RS_THREADS = 256;
-constexpr int RS_WARPS = RS_THREADS / 32;
 constexpr int RS_BINS = 256;
-// elements per thread: small inputs take small tiles, so that their few tiles still cover the SMs
-constexpr int RS_BIG = 16, RS_SMALL = 4;
+// threads and elements per thread: small inputs take small tiles, so that their few tiles still cover the SMs
+struct RsBig { static constexpr int THREADS = 512, ITEMS = 16; };
+struct RsSmall { static constexpr int THREADS = 256, ITEMS = 4; };
 constexpr uint64_t RS_SMALL_N = 1u << 20;
-inline int rs_tile(uint64_t n) { return RS_THREADS * (n <= RS_SMALL_N ? RS_SMALL : RS_BIG); }
+inline int rs_tile(uint64_t n) {
+    return n <= RS_SMALL_N ? RsSmall::THREADS * RsSmall::ITEMS : RsBig::THREADS * RsBig::ITEMS;
+}
 
-template <typename K, int ITEMS>
+template <typename K, int RS_THREADS, int ITEMS>
 __global__ void radix_hist_kernel(const K* __restrict__ keys, uint64_t n, int shift, unsigned mask, uint64_t ntiles,
                                   uint32_t* __restrict__ counts) {
     __shared__ unsigned int h[RS_BINS];
-    h[threadIdx.x] = 0;
+    if (threadIdx.x < RS_BINS) h[threadIdx.x] = 0;
     __syncthreads();
     const uint64_t base = (uint64_t)blockIdx.x * (RS_THREADS * ITEMS);
     K key[ITEMS];
@@ -189,17 +190,17 @@ __global__ void radix_hist_kernel(const K* __restrict__ keys, uint64_t n, int sh
 // Elements of a tile are ranked in input order: warp w holds the tile's w-th
 // part, item by item; __match_any_sync ranks equal digits within an item, the
 // warp's running digit counts rank the items, and a scan over the warps ranks the warps.
-template <typename K, int ITEMS>
-__global__ void __launch_bounds__(RS_THREADS) radix_scatter_kernel(
+template <typename K, int RS_THREADS, int ITEMS>
+__global__ void __launch_bounds__(RS_THREADS, 1024 / RS_THREADS) radix_scatter_kernel(
     const K* __restrict__ kin, const uint32_t* __restrict__ vin, K* __restrict__ kout, uint32_t* __restrict__ vout,
     uint64_t n, int shift, unsigned mask, uint64_t ntiles, const uint32_t* __restrict__ offsets) {
-    constexpr int TILE = RS_THREADS * ITEMS;
+    constexpr int TILE = RS_THREADS * ITEMS, RS_WARPS = RS_THREADS / 32;
     extern __shared__ __align__(16) unsigned char rs_smem[];
     K* skey = (K*)rs_smem;                                   // the tile in digit order
     uint32_t* sval = (uint32_t*)(rs_smem + sizeof(K) * TILE);
     __shared__ uint32_t wc[RS_WARPS][RS_BINS];               // digit counts per warp, then where each warp's run starts
     __shared__ uint32_t dst[RS_BINS];                        // a digit's output start minus its start in the tile
-    __shared__ uint32_t wsum[RS_WARPS];
+    __shared__ uint32_t wsum[RS_BINS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const uint64_t tile0 = (uint64_t)blockIdx.x * TILE;
@@ -207,13 +208,11 @@ __global__ void __launch_bounds__(RS_THREADS) radix_scatter_kernel(
     const int seg = warp * (32 * ITEMS);
     for (int d = lane; d < RS_BINS; d += 32) wc[warp][d] = 0;
     K key[ITEMS];
-    uint32_t val[ITEMS];
     uint32_t rank[ITEMS];
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
         const int i = seg + j * 32 + lane;
         key[j] = i < left ? kin[tile0 + i] : K(0);
-        val[j] = i >= left ? 0u : vin ? vin[tile0 + i] : (uint32_t)(tile0 + i);
     }
     const uint32_t out0 = threadIdx.x <= mask ? offsets[(uint64_t)threadIdx.x * ntiles + blockIdx.x] : 0u;
     __syncwarp();
@@ -230,36 +229,41 @@ __global__ void __launch_bounds__(RS_THREADS) radix_scatter_kernel(
     }
     __syncthreads();
     {
-        // thread d: digit d's total, its start in the tile, and each warp's start within it
+        // thread d < RS_BINS: digit d's total, its start in the tile, and each warp's start within it
+        const bool digit = threadIdx.x < RS_BINS;
         uint32_t tot = 0;
 #pragma unroll
-        for (int w = 0; w < RS_WARPS; ++w) tot += wc[w][threadIdx.x];
+        for (int w = 0; w < RS_WARPS; ++w) tot += digit ? wc[w][threadIdx.x] : 0u;
         uint32_t inc = tot;
 #pragma unroll
         for (int s = 1; s < 32; s <<= 1) {
             const uint32_t u = __shfl_up_sync(0xffffffffu, inc, s);
             if (lane >= s) inc += u;
         }
-        if (lane == 31) wsum[warp] = inc;
+        if (digit && lane == 31) wsum[warp] = inc;
         __syncthreads();
-        uint32_t at = inc - tot;
-        for (int w = 0; w < warp; ++w) at += wsum[w];
-        dst[threadIdx.x] = out0 - at;
+        if (digit) {
+            uint32_t at = inc - tot;
+            for (int w = 0; w < warp; ++w) at += wsum[w];
+            dst[threadIdx.x] = out0 - at;
 #pragma unroll
-        for (int w = 0; w < RS_WARPS; ++w) {
-            const uint32_t c = wc[w][threadIdx.x];
-            wc[w][threadIdx.x] = at;
-            at += c;
+            for (int w = 0; w < RS_WARPS; ++w) {
+                const uint32_t c = wc[w][threadIdx.x];
+                wc[w][threadIdx.x] = at;
+                at += c;
+            }
         }
     }
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
-        if (seg + j * 32 + lane >= left) continue;
+        const int i = seg + j * 32 + lane;
+        if (i >= left) continue;
         const unsigned d = (unsigned)(key[j] >> shift) & mask;
         const uint32_t p = wc[warp][d] + rank[j];
         skey[p] = key[j];
-        sval[p] = val[j];
+        // read only now: values held through the ranking took the registers of half the warps
+        sval[p] = vin ? vin[tile0 + i] : (uint32_t)(tile0 + i);
     }
     __syncthreads();
 #pragma unroll
@@ -273,20 +277,21 @@ __global__ void __launch_bounds__(RS_THREADS) radix_scatter_kernel(
     }
 }
 
-template <typename K, int ITEMS>
+template <typename K, typename T>
 tm_status radix_pass(const K* ki, const uint32_t* vi, K* ko, uint32_t* vo, uint64_t n, int shift, unsigned mask,
                      uint32_t* counts, void* scan_tmp, cudaStream_t st) {
-    const uint64_t ntiles = ceil_div(n, RS_THREADS * ITEMS);
-    constexpr int bytes = RS_THREADS * ITEMS * (int)(sizeof(K) + 4);
-    if (bytes > 40 * 1024)
-        TM_CUDA(cudaFuncSetAttribute(radix_scatter_kernel<K, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    radix_hist_kernel<K, ITEMS><<<(unsigned)ntiles, RS_THREADS, 0, st>>>(ki, n, shift, mask, ntiles, counts);
+    const uint64_t ntiles = ceil_div(n, T::THREADS * T::ITEMS);
+    constexpr int bytes = T::THREADS * T::ITEMS * (int)(sizeof(K) + 4);
+    if (bytes > 24 * 1024)
+        TM_CUDA(cudaFuncSetAttribute(radix_scatter_kernel<K, T::THREADS, T::ITEMS>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    radix_hist_kernel<K, T::THREADS, T::ITEMS><<<(unsigned)ntiles, T::THREADS, 0, st>>>(ki, n, shift, mask, ntiles, counts);
     note_launches(1);
     TM_CUDA(cudaGetLastError());
     tm_status s = exclusive_scan(counts, counts, ntiles * (mask + 1u), (uint32_t*)scan_tmp, st);
     if (s != TM_OK) return s;
-    radix_scatter_kernel<K, ITEMS><<<(unsigned)ntiles, RS_THREADS, bytes, st>>>(ki, vi, ko, vo, n, shift, mask, ntiles,
-                                                                                counts);
+    radix_scatter_kernel<K, T::THREADS, T::ITEMS><<<(unsigned)ntiles, T::THREADS, bytes, st>>>(ki, vi, ko, vo, n, shift, mask,
+                                                                                             ntiles, counts);
     note_launches(1);
     TM_CUDA(cudaGetLastError());
     return TM_OK;
@@ -314,8 +319,8 @@ tm_status radix_sort_pairs(const K* keys_in, const uint32_t* vals_in, K* const k
         const K* ki = p == 0 ? keys_in : keys[*which];
         const uint32_t* vi = p == 0 ? vals_in : vals[*which];
         const int to = p == 0 ? 0 : *which ^ 1;
-        tm_status s = n <= RS_SMALL_N ? radix_pass<K, RS_SMALL>(ki, vi, keys[to], vals[to], n, p * per, mask, counts, scan_tmp, st)
-                                      : radix_pass<K, RS_BIG>(ki, vi, keys[to], vals[to], n, p * per, mask, counts, scan_tmp, st);
+        tm_status s = n <= RS_SMALL_N ? radix_pass<K, RsSmall>(ki, vi, keys[to], vals[to], n, p * per, mask, counts, scan_tmp, st)
+                                      : radix_pass<K, RsBig>(ki, vi, keys[to], vals[to], n, p * per, mask, counts, scan_tmp, st);
         if (s != TM_OK) return s;
         *which = to;
     }

@@ -362,7 +362,7 @@ struct Search {
         if (cdir == 0 && nx == NX_OUT_DST) return __ldg(g.pnx[1] + cpos);
         if (cdir == 1 && nx == NX_IN_DST) return __ldg(g.pnx[2] + cpos);
         if (cdir == 1 && nx == NX_IN_SRC) return __ldg(g.pnx[3] + cpos);
-        return __ldg(g.nxt[nx] + edge_at(cdir, cpos, prev_e));
+        return __ldg(g.nxt[nx] + 2u * (uint32_t)edge_at(cdir, cpos, prev_e));
     }
     // True when successor() is one load (no edge id needed first).
     __device__ static bool successor_direct(int nx, int cdir) {

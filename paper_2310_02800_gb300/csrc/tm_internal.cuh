@@ -62,7 +62,9 @@ struct GraphView {
     // out(u), in(v), out(v), in(u).  Each word is {x: absolute position in the
     // list columns, y: time of that entry minus t, saturated at SUCC_FAR, or
     // SUCC_END when the list has no later entry}, so one load both starts a
-    // window and, for most windows, proves it empty.
+    // window and, for most windows, proves it empty.  Edge e's word is nxt[kind][2 * e]: the
+    // two words found in out-list order (out(u), in(u)) lie side by side, and so do the two found in
+    // in-list order, since each pair is written at once to an edge from anywhere.
     const uint2* nxt[4];
     // the same, indexed by list position for the common continuations: [0] out-list
     // entry -> next later in that out-list, [1] out-list entry -> out(its neighbour),

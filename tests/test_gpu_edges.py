@@ -183,3 +183,26 @@ def test_row_offsets_edges(tmg, chunks):
             w = min(cap, len(rows))
             assert q.enumerate(out) == (w, len(rows), len(rows) > cap), (mo, cap)
             assert np.array_equal(out[:w].cpu().numpy(), rows[:w]) and (out[w:] == -7).all(), (mo, cap)
+
+
+@pytest.mark.parametrize("m", [8191, 8193, (1 << 19) - 1, 1 << 19, 1 << 20, (1 << 20) + 1, (1 << 20) + 8193])
+@pytest.mark.parametrize("span", [1, 5_000, 1 << 40])
+def test_load_edges(tmg, m, span):
+    """Loads around the sort's tiles, its small inputs' end and the size from which host endpoints are copied beside
+    the sort, with equal, 4-byte and 8-byte times: the same graph from host and device arrays, ids in stable
+    time order, invalid endpoints refused, counts against the oracle."""
+    n, src, dst, t, el, nl = graph(50_000, m, span, seed=m)
+    gg = tmg.Graph.load(n, src, dst, t, el, nl)
+    gd = tmg.Graph.load(n, *(torch.from_numpy(x).cuda() for x in (src, dst, t, el, nl)))
+    want = np.argsort(t, kind="stable")
+    assert np.array_equal(gg.edge_perm(), want) and np.array_equal(gd.edge_perm(), want)
+    og = oracle.Graph(n, src, dst, t, el, nl)
+    for mo in (synth.Motif([(0, 1), (1, 0)], span // 9, elabel=[1, -1]), synth.Motif([(0, 1), (1, 2)], span // 9, nlabel=[0, -1, 1])):
+        want = og.count(mo)
+        assert gg.compile(mo).count() == want and gd.compile(mo).count() == want, mo
+    for bad in (-1, n):
+        for col in (src, dst):
+            keep, col[m - 1] = int(col[m - 1]), bad
+            with pytest.raises(tmg.TMError):
+                tmg.Graph.load(n, src, dst, t, el, nl)
+            col[m - 1] = keep
