@@ -257,6 +257,11 @@ __global__ void root_codes_kernel(int64_t m, const uint4* __restrict__ by_out, c
     }
 }
 
+__global__ void widen_kernel(const int32_t* __restrict__ in, int64_t n, int64_t* __restrict__ out) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) out[i] = in[i];
+}
+constexpr int64_t PERM_PART = 1 << 22;        // 32 MB of device memory
+
 int bits_for(unsigned long long x) {
     int b = 0;
     while (b < 64 && (x >> b) != 0) ++b;
@@ -315,9 +320,7 @@ struct Side {
     }
 };
 
-// Graph storage is one allocation (one cudaMalloc at load, one cudaFree at
-// free, instead of one per column: ~2 ms less per load/free cycle of a
-// 10M-edge graph), carved into 256-byte aligned columns.
+// Graph storage is one allocation, carved into 256-byte aligned columns.
 constexpr size_t COL_ALIGN = 256;
 inline size_t col_bytes(size_t count, size_t elem) {
     return (std::max<size_t>(count * elem, 16) + COL_ALIGN - 1) & ~(COL_ALIGN - 1);
@@ -607,23 +610,13 @@ extern "C" tm_status tm_graph_load(const tm_edges* e, int device, void* stream, 
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) { delete g; return cuda_fail(cudaGetLastError(), "props"); }
     g->num_sms = prop.multiProcessorCount;
-    // keep up to 2 GiB of freed build temporaries in the device's stream-ordered
-    // pool, so loading graphs one after another does not go back to the driver
-    cudaMemPool_t pool;
-    if (cudaDeviceGetDefaultMemPool(&pool, device) == cudaSuccess) {
-        uint64_t keep = 0;
-        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-        if (keep < (2ull << 30)) {
-            keep = 2ull << 30;
-            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-        }
-    }
-    cudaGetLastError();
+    InFlight call(&g->unsettled);
     tm_status s = build(g, e, (cudaStream_t)stream);
     if (s != TM_OK) {
         tm_graph_free(g);
         return s;
     }
+    call.settle();
     *out = g;
     return TM_OK;
 }
@@ -632,7 +625,7 @@ extern "C" tm_status tm_graph_free(tm_graph* g) {
     if (!g) return TM_OK;
     cudaSetDevice(g->device);
     drop_batches(g);
-    for (void* p : g->allocs) cudaFree(p);
+    for (void* p : g->allocs) dev_free(p, g->device, g->unsettled == 0);
     delete g;
     return TM_OK;
 }
@@ -649,8 +642,25 @@ extern "C" tm_status tm_graph_edge_perm(const tm_graph* g, int64_t* out_perm) {
     if (!g || (!out_perm && g->v.m > 0)) { set_error("null argument"); return TM_E_INVALID; }
     if (g->v.m == 0) return TM_OK;
     TM_ENTER(g->device);
-    std::vector<int32_t> tmp((size_t)g->v.m);
-    TM_CUDA(cudaMemcpy(tmp.data(), g->perm, g->v.m * 4, cudaMemcpyDeviceToHost));
-    for (int64_t i = 0; i < g->v.m; ++i) out_perm[i] = tmp[i];
+    // widened on the device and copied straight out, PERM_PART ids at a time
+    const int64_t m = g->v.m, part = std::min(m, PERM_PART);
+    int64_t* wide = nullptr;
+    if (dev_malloc((void**)&wide, part * 8) == cudaSuccess) {
+        cudaError_t e = cudaSuccess;
+        for (int64_t i = 0; i < m && e == cudaSuccess; i += part) {
+            const int64_t n = std::min(part, m - i);
+            widen_kernel<<<grid_for(n, g->num_sms), 256>>>(g->perm + i, n, wide);
+            note_launches(1);
+            e = cudaGetLastError();
+            if (e == cudaSuccess) e = cudaMemcpy(out_perm + i, wide, n * 8, cudaMemcpyDeviceToHost);
+        }
+        dev_free(wide, g->device, e == cudaSuccess);
+        return e == cudaSuccess ? TM_OK : cuda_fail(e, "edge permutation");
+    }
+    // no device memory to spare: through a host copy
+    cudaGetLastError();
+    std::vector<int32_t> tmp((size_t)m);
+    TM_CUDA(cudaMemcpy(tmp.data(), g->perm, m * 4, cudaMemcpyDeviceToHost));
+    for (int64_t i = 0; i < m; ++i) out_perm[i] = tmp[i];
     return TM_OK;
 }

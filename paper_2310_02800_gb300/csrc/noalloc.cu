@@ -104,6 +104,7 @@ extern "C" tm_status tm_count_batch_noalloc(tm_graph* g, tm_query* const* qs, in
         if (!qs[j] || query_graph(qs[j]) != g) { set_error("null or mismatched query in batch"); return TM_E_INVALID; }
     // Every call reuses the array: clear the caller's totals, then rewrite the
     // control block and the launch records and clear the task-ready flags.
+    InFlight call(&g->unsettled);
     TM_CUDA(cudaMemsetAsync(totals_dev, 0, (size_t)nq * sizeof(uint64_t), st));
     if (m == 0) return cudaStreamSynchronize(st) == cudaSuccess ? TM_OK : cuda_fail(cudaGetLastError(), "sync");
     {
@@ -144,6 +145,7 @@ extern "C" tm_status tm_count_batch_noalloc(tm_graph* g, tm_query* const* qs, in
     Ctrl done;
     TM_CUDA(cudaMemcpyAsync(&done, base + OFF_CTRL, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
     TM_CUDA(cudaStreamSynchronize(st));
+    call.settle();
     note_search_stats(done);
     if (done.err) { set_error("a bounded device wait timed out"); return TM_E_TIMEOUT; }
     return TM_OK;

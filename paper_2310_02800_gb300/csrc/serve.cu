@@ -387,8 +387,8 @@ void scheduler(tm_server* s) {
 
 void destroy_slots(tm_server* s) {
     for (Slot& sl : s->slots) {
-        scratch_free(&sl.count_s);
-        scratch_free(&sl.fill_s);
+        scratch_free(&sl.count_s, false);
+        scratch_free(&sl.fill_s, false);
         if (sl.start) cudaEventDestroy(sl.start);
         if (sl.done) cudaEventDestroy(sl.done);
         if (sl.st_hi) cudaStreamDestroy(sl.st_hi);
@@ -445,6 +445,7 @@ extern "C" tm_status tm_serve_start(tm_graph* g, const tm_serve_cfg* cfg, tm_ser
         cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
     }
     cudaGetLastError();
+    g->unsettled.fetch_add(1);     // batches in flight, until tm_serve_stop has waited for them
     s->th = std::thread(scheduler, s);
     *out = s;
     return TM_OK;
@@ -542,10 +543,12 @@ extern "C" tm_status tm_serve_stop(tm_server* s) {
     for (auto& kv : s->reqs)
         if (kv.second->match) cudaFreeAsync(kv.second->match, s->free_st);
     cudaStreamSynchronize(s->free_st);
+    bool settled = true;
     for (Slot& sl : s->slots) {
-        if (sl.st_hi) cudaStreamSynchronize(sl.st_hi);
-        if (sl.st_lo) cudaStreamSynchronize(sl.st_lo);
+        if (sl.st_hi) settled = cudaStreamSynchronize(sl.st_hi) == cudaSuccess && settled;
+        if (sl.st_lo) settled = cudaStreamSynchronize(sl.st_lo) == cudaSuccess && settled;
     }
+    if (settled) s->g->unsettled.fetch_sub(1);
     destroy_slots(s);
     delete s;
     return TM_OK;

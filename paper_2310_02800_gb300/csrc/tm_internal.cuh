@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <mutex>
 #include <string>
 #include <unordered_map>
@@ -23,7 +24,12 @@ tm_status cuda_fail(cudaError_t e, const char* what);
 // Every device and pinned-host allocation of the library goes through these,
 // so that tm_inject_alloc_failure can make one of them fail like an
 // out-of-memory device (cudaErrorMemoryAllocation, nothing allocated).
+// dev_malloc returns memory of the device's stream-ordered pool (which keeps up to POOL_KEEP of what was
+// freed and gives the rest back), ready for any stream; dev_free takes it back.  `settled`: nothing
+// in flight uses it any more, else the free waits for the device as cudaFree does.
+constexpr uint64_t POOL_KEEP = 4ull << 30;
 cudaError_t dev_malloc(void** p, size_t bytes);
+void dev_free(void* p, int device, bool settled);
 cudaError_t dev_malloc_async(void** p, size_t bytes, cudaStream_t st);
 cudaError_t host_alloc_pinned(void** p, size_t bytes);
 
@@ -115,6 +121,7 @@ struct TuneKeyHash {
 
 struct tm_graph {
     int device = 0;
+    std::atomic<int> unsettled{0};   // calls on this graph that are running, or ended without having waited for their work
     tmg::GraphView v{};
     std::vector<void*> allocs;     // device buffers owned by the graph
     char* slab = nullptr;          // the graph's columns, carved from one allocation
@@ -131,6 +138,24 @@ struct tm_graph {
 };
 
 namespace tmg {
+
+// A call that puts work on a stream: until it has waited for that work, what the work
+// uses (the graph's columns, a query's scratch) is not settled.
+class InFlight {
+    std::atomic<int>*a, *b;
+
+public:
+    explicit InFlight(std::atomic<int>* x, std::atomic<int>* y = nullptr) : a(x), b(y) {
+        a->fetch_add(1);
+        if (b) b->fetch_add(1);
+    }
+    // the work has been waited for
+    void settle() {
+        if (a) a->fetch_sub(1);
+        if (b) b->fetch_sub(1);
+        a = b = nullptr;
+    }
+};
 
 // --------------------------------------------------------------- the plan
 
@@ -378,7 +403,7 @@ tm_status chunk_offsets(unsigned long long* chunk_buf, uint64_t nch, uint64_t ca
 
 tm_status scratch_reserve(Scratch* s, int device, int nq, uint64_t counters_len, uint64_t chunks,
                           uint64_t task_cap);
-void scratch_free(Scratch* s);
+void scratch_free(Scratch* s, bool settled);
 
 enum Mode { MODE_COUNT = 0, MODE_FILL = 1 };
 
