@@ -49,12 +49,14 @@ __global__ void check_times_kernel(const int64_t* __restrict__ t, int64_t m, Che
     }
 }
 
+// Also packs the two endpoints of an edge side by side, for the gather into time order.
 __global__ void check_nodes_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t m, int64_t n,
-                                   Check* out) {
+                                   Check* out, int2* __restrict__ ends) {
     bool bad = false;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t s = src[i], d = dst[i];
         bad = bad || s < 0 || s >= n || d < 0 || d >= n;
+        ends[i] = make_int2(s, d);
     }
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicAdd(&out->bad_nodes, 1ULL);
 }
@@ -81,15 +83,15 @@ struct __align__(16) EdgeRec {
 // (keys null) the input is in time order already and perm is null too.
 template <typename K>
 __global__ void gather_edges_kernel(const uint32_t* __restrict__ perm, const K* __restrict__ keys,
-                                    unsigned long long tmin, int64_t m, const int32_t* __restrict__ src,
-                                    const int32_t* __restrict__ dst, const int64_t* __restrict__ t,
+                                    unsigned long long tmin, int64_t m, const int2* __restrict__ ends,
+                                    const int64_t* __restrict__ t,
                                     const uint8_t* __restrict__ el, int32_t* __restrict__ src_o,
                                     int32_t* __restrict__ dst_o, int64_t* __restrict__ t_o, uint8_t* __restrict__ el_o,
                                     int32_t* __restrict__ perm_o, EdgeRec* __restrict__ rec_o) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e0 < m; e0 += GATHER * stride) {
         uint32_t i[GATHER];
-        int32_t s[GATHER], d[GATHER];
+        int2 n[GATHER];
         int64_t tt[GATHER];
 #pragma unroll
         for (int j = 0; j < GATHER; ++j) {
@@ -99,19 +101,18 @@ __global__ void gather_edges_kernel(const uint32_t* __restrict__ perm, const K* 
 #pragma unroll
         for (int j = 0; j < GATHER; ++j) {
             const int64_t e = e0 + j * stride;
-            s[j] = src[i[j]];
-            d[j] = dst[i[j]];
+            n[j] = ends[i[j]];
             tt[j] = e >= m ? 0 : keys ? (int64_t)((unsigned long long)keys[e] + tmin) : t[e];
         }
 #pragma unroll
         for (int j = 0; j < GATHER; ++j) {
             const int64_t e = e0 + j * stride;
             if (e >= m) break;
-            src_o[e] = s[j];
-            dst_o[e] = d[j];
+            src_o[e] = n[j].x;
+            dst_o[e] = n[j].y;
             t_o[e] = tt[j];
             if (el) el_o[e] = el[i[j]];
-            rec_o[e] = EdgeRec{tt[j], s[j], d[j]};
+            rec_o[e] = EdgeRec{tt[j], n[j].x, n[j].y};
             perm_o[e] = (int32_t)i[j];
         }
     }
@@ -390,7 +391,9 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
     const bool overlap = host && m >= OVERLAP_MIN;
     cudaStream_t cs = st;
     int32_t *s2 = nullptr, *d2 = nullptr;
+    int2* ends;
     uint8_t* el2 = nullptr;
+    TRY(tmp.get(&ends, m));
     if (host) {
         int64_t* t2;
         TRY(tmp.get(&s2, m));
@@ -433,7 +436,7 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
             src = s2; dst = d2; el = el2;
         }
         if (m > 0) {
-            check_nodes_kernel<<<grid_for(m, sms), 256, 0, cs>>>(src, dst, m, n, chk);
+            check_nodes_kernel<<<grid_for(m, sms), 256, 0, cs>>>(src, dst, m, n, chk, ends);
             note_launches(1);
             TM_CUDA(cudaGetLastError());
         }
@@ -500,13 +503,13 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
         }
         // 3. edge columns in edge-id order
         if (sorted)
-            gather_edges_kernel<uint32_t><<<grid4, 256, 0, st>>>(nullptr, nullptr, 0, m, src, dst, t, el, s_o, d_o, t_o,
+            gather_edges_kernel<uint32_t><<<grid4, 256, 0, st>>>(nullptr, nullptr, 0, m, ends, t, el, s_o, d_o, t_o,
                                                                  el_o, p_o, rec);
         else if (narrow)
-            gather_edges_kernel<uint32_t><<<grid4, 256, 0, st>>>(va[w], ka[w], hc.tmin, m, src, dst, t, el, s_o, d_o, t_o,
+            gather_edges_kernel<uint32_t><<<grid4, 256, 0, st>>>(va[w], ka[w], hc.tmin, m, ends, t, el, s_o, d_o, t_o,
                                                                  el_o, p_o, rec);
         else
-            gather_edges_kernel<uint64_t><<<grid4, 256, 0, st>>>(va[w], k8[w], hc.tmin, m, src, dst, t, el, s_o, d_o, t_o,
+            gather_edges_kernel<uint64_t><<<grid4, 256, 0, st>>>(va[w], k8[w], hc.tmin, m, ends, t, el, s_o, d_o, t_o,
                                                                  el_o, p_o, rec);
         note_launches(1);
         TM_CUDA(cudaGetLastError());
