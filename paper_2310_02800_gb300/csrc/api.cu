@@ -733,7 +733,7 @@ std::vector<LaunchGroup> occupancy_groups(const tm_graph* g, Mode mode, const Pl
                                         p.tune.warps_per_block, plan_features(p));
         grid[j] = c.grid;
         wpb[j] = c.warps_per_block;
-        kind[j] = mode == MODE_COUNT ? plan_features(p) & FEAT_PAIRS : 0u;
+        kind[j] = plan_features(p) & FEAT_PAIRS;
         order[j] = j;
     }
     // highest occupancy first; within a group the likely most expensive queries

@@ -232,7 +232,7 @@ struct Search {
     static constexpr bool ANTI = (FEAT & FEAT_ANTI) != 0;   // anti-edge checks compiled in
     static constexpr bool LOOK = (FEAT & FEAT_LOOK) != 0;   // look-ahead checks compiled in
     static constexpr bool FILTER = LOOK && !STATS;          // ... with their candidate filter
-    static constexpr bool PAIRS = MODE == MODE_COUNT && (FEAT & FEAT_PAIRS) != 0;   // last two edges as pairs
+    static constexpr bool PAIRS = (FEAT & FEAT_PAIRS) != 0;   // last two edges as pairs
     static constexpr int CAP = MODE == MODE_FILL ? FCAP_FILL : FCAP_COUNT;   // parents per frame
     static constexpr uint32_t DESCEND = CAP - 32;   // a child frame this full is drained next
     using Frame = FrameT<CAP>;
@@ -881,29 +881,101 @@ struct Search {
         return m & ~__match_any_sync(FULL, x);
     }
 
-    // Level k - 2 of a count-mode search whose last two edges extend by new nodes from one list (out-stars and
+    // The j-th set bit of m (j < popc(m)).
+    __device__ static int nth_bit(unsigned m, uint32_t j) {
+        int at = 0;
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) {
+            const uint32_t low = __popc(m & ((1u << s) - 1u));
+            if (j >= low) {
+                j -= low;
+                m >>= s;
+                at += s;
+            }
+        }
+        return at;
+    }
+
+    // Write the rows of the pairs (this lane's entry of parent p and edge e, each entry of m), whose first goes
+    // to row `at`: 32 rows of the warp's at a time, each lane one.  eo: the edge of the entry a bit of m stands for.
+    __device__ void write_pairs(Frame f, int nb, int p, unsigned m, unsigned long long at, int32_t e, int32_t eo) const {
+        uint32_t inc = __popc(m);
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t u = __shfl_up_sync(FULL, inc, d);
+            if (lane >= d) inc += u;
+        }
+        const uint32_t total = __shfl_sync(FULL, inc, 31);
+        for (uint32_t t = 0; t < total; t += 32u) {
+            const uint32_t r = min(t + lane, total - 1u);
+            int o = 0;                              // the lane whose pair row r is: as many have theirs before it
+#pragma unroll
+            for (int s = 16; s > 0; s >>= 1)
+                if (__shfl_sync(FULL, inc, o + s - 1) <= r) o += s;
+            const unsigned mo = __shfl_sync(FULL, m, o);
+            const uint32_t j = r - (__shfl_sync(FULL, inc, o) - __popc(mo));
+            const unsigned long long pos = __shfl_sync(FULL, at, o) + j;
+            const int po = __shfl_sync(FULL, p, o);
+            const int32_t ea = __shfl_sync(FULL, e, o), eb = __shfl_sync(FULL, eo, nth_bit(mo, j));
+            if (t + lane < total && pos < q->cap) {
+                int32_t* row = q->match_out + pos * (unsigned long long)k;
+                for (int i = 0; i < k - 2; ++i) row[i] = f.eid(nb, i, po);
+                row[k - 2] = ea;
+                row[k - 1] = eb;
+            }
+        }
+    }
+
+    // Level k - 2 of a search whose last two edges extend by new nodes from one list (out-stars and
     // the like): the last edge's window is what follows the candidate in its own window, so the
-    // pairs are counted with ballots, without a frame entry, a window search and another pass
+    // pairs are counted (enumeration: written) with ballots, without a frame entry, a window search and another pass
     // per candidate.  A step takes whole windows, as many as fit 32 lanes; a longer window is taken
     // in tiles of 32, each against itself and those after it.  Frames with a window above
     // PAIRS_MAX go the general way, whose subtrees can be donated: tiles cost its square.
-    // 8 queries on 200k edges 361 -> 246 us, four queries' counts and rows on 10M edges 2.32 -> 1.87 ms.
-    __device__ void count_pairs(uint32_t h, Frame f, uint32_t tot) {
+    // 8 queries on 200k edges 361 -> 246 us, four queries' counts and rows on 10M edges 2.32 -> 1.87 ms
+    // with the count's pairs, 1.73 ms with the rows' too (out-star fill 726 -> 538 us).
+    __device__ void pairs_of(uint32_t h, Frame f, uint32_t tot) {
         const int nb = Hot::nb(h), dir = Hot::kind(h) == EXT_IN ? 1 : 0;
         const int32_t* __restrict__ nbr = g.anbr[dir];
         const int64_t* __restrict__ ta = g.at[dir];
         const uint2 pr = 2 * lane < CAP ? f.pre2(lane) : make_uint2(NEVER, NEVER);
-        const bool attrib = q->per_root || q->chunk_cnt;
+        const bool attrib = MODE == MODE_COUNT && (q->per_root || q->chunk_cnt);
         // an entry of parent p's window: false when its neighbour is bound already
-        auto entry = [&](bool act, int p, uint32_t pos, int32_t& x, int64_t& t) -> bool {
+        auto entry = [&](bool act, int p, uint32_t pos, int32_t& x, int64_t& t, int32_t& e) -> bool {
             x = -1;
             t = 0;
+            e = 0;
             if (!act) return false;
             x = __ldg(nbr + pos);
             t = __ldg(ta + pos);
+            if (MODE == MODE_FILL) e = __ldg(g.aeid[dir] + pos);
             bool ok = true;
             for (int j = 0; j < nb; ++j) ok &= f.node(j, p) != x;
             return ok;
+        };
+        // a tile's entries [o, o + 32) of a window at b that come after this lane's (t, x) in an earlier tile
+        auto after = [&](int p, uint32_t b, uint32_t o, uint32_t len, int64_t t, int32_t x, int32_t& eo) -> unsigned {
+            int32_t xo;
+            int64_t to;
+            unsigned v = __ballot_sync(FULL, entry(o + lane < len, p, b + o + lane, xo, to, eo));
+            const int64_t t_last = __shfl_sync(FULL, t, 31);
+            const bool tie = __shfl_sync(FULL, to, 0) == t_last;
+            for (int j = 0; j < 32; ++j) {
+                unsigned same = __shfl_sync(FULL, xo, j) == x ? 1u : 0u;
+                if (tie) same |= __shfl_sync(FULL, to, j) == t ? 1u : 0u;
+                v &= ~(same << j);
+            }
+            return v;
+        };
+        // rows of the lanes' c pairs each start here (and the next ones after them)
+        auto place = [&](uint32_t c) -> unsigned long long {
+            uint32_t inc = c;
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t u = __shfl_up_sync(FULL, inc, d);
+                if (lane >= d) inc += u;
+            }
+            const unsigned long long at = out_base + out_local + inc - c;
+            out_local += __shfl_sync(FULL, inc, 31);
+            return at;
         };
         unsigned long long sum = 0;
         uint32_t off = 0;
@@ -912,13 +984,15 @@ struct Search {
             int p = lane_parent(pr, off, starts);
             uint32_t n = min(tot - off, 32u);      // entries of whole windows in this step
             if (off + 32u < tot && !__any_sync(FULL, pr.x == off + 32u || pr.y == off + 32u)) n = starts ? 31u - __clz(starts) : 0u;
-            int32_t x;
+            int32_t x, e;
             int64_t t;
             if (n > 0u) {
                 if (lane >= n) p = 0;
-                const bool ok = entry(lane < n, p, (f.beg(p) & POSMASK) + (off + lane - f.pre(p)), x, t);
-                uint32_t c = __popc(later_others(__ballot_sync(FULL, ok), starts, t, x));
-                if (!ok) c = 0;
+                const bool ok = entry(lane < n, p, (f.beg(p) & POSMASK) + (off + lane - f.pre(p)), x, t, e);
+                unsigned m = later_others(__ballot_sync(FULL, ok), starts, t, x);
+                if (!ok) m = 0;
+                const uint32_t c = __popc(m);
+                if (MODE == MODE_FILL) write_pairs(f, nb, p, m, place(c), e, e);
                 sum += c;
                 if (attrib) attribute_lanes(f.root(p), c);
                 off += n;
@@ -928,28 +1002,29 @@ struct Search {
             p = __shfl_sync(FULL, p, 0);
             const uint32_t end = p + 1 < CAP ? min(f.pre(p + 1), tot) : tot, b = f.beg(p) & POSMASK, len = end - off;
             for (uint32_t a = 0; a < len; a += 32u) {
-                const bool ok = entry(a + lane < len, p, b + a + lane, x, t);
-                uint32_t c = __popc(later_others(__ballot_sync(FULL, ok), 0u, t, x));
-                for (uint32_t o = a + 32u; o < len; o += 32u) {
-                    int32_t xo;
-                    int64_t to;
-                    unsigned v = __ballot_sync(FULL, entry(o + lane < len, p, b + o + lane, xo, to));
-                    const int64_t t_last = __shfl_sync(FULL, t, 31);
-                    const bool tie = __shfl_sync(FULL, to, 0) == t_last;
-                    for (int j = 0; j < 32; ++j) {
-                        unsigned same = __shfl_sync(FULL, xo, j) == x ? 1u : 0u;
-                        if (tie) same |= __shfl_sync(FULL, to, j) == t ? 1u : 0u;
-                        v &= ~(same << j);
+                const bool ok = entry(a + lane < len, p, b + a + lane, x, t, e);
+                int32_t eo;
+                unsigned m = later_others(__ballot_sync(FULL, ok), 0u, t, x);
+                uint32_t c = __popc(m);
+                for (uint32_t o = a + 32u; o < len; o += 32u) c += __popc(after(p, b, o, len, t, x, eo));
+                if (!ok) m = c = 0;
+                if (MODE == MODE_FILL) {
+                    unsigned long long at = place(c);
+                    write_pairs(f, nb, p, m, at, e, e);
+                    at += __popc(m);
+                    for (uint32_t o = a + 32u; o < len; o += 32u) {
+                        unsigned v = after(p, b, o, len, t, x, eo);
+                        if (!ok) v = 0;
+                        write_pairs(f, nb, p, v, at, e, eo);
+                        at += __popc(v);
                     }
-                    c += __popc(v);
                 }
-                if (!ok) c = 0;
                 sum += c;
                 if (attrib) attribute_lanes(f.root(p), c);
             }
             off = end;
         }
-        acc.total += sum;
+        if (MODE == MODE_COUNT) acc.total += sum;
     }
 
     // Add each lane's c matches of its root, lanes in root order (per-root or per-chunk counts asked for).
@@ -1029,7 +1104,7 @@ struct Search {
                 count_ext(lvl, h, f, np, tot);
                 off = tot;
             } else if (pairs) {
-                count_pairs(h, f, tot);
+                pairs_of(h, f, tot);
                 off = tot;
                 pairs = false;
             }
@@ -1501,8 +1576,10 @@ struct Search {
 // there to take, and without spills at 80 fewer warps are faster: labelled 5-path on 20M edges
 // 344 us at 64, 313 at 72, 265 at 80.  Pairs (8 queries on 200k edges 278, 259, 247 us),
 // anti-edges (109, 106, 104) and look-ahead (chorded 4-cycle on 100M edges 52, 49, 48 ms) likewise.
-// Fills have the widest frames and 64 did best (four queries' counts and rows 1.85 ms, at 72 1.92).
-constexpr int search_regs(int mode, bool stats, int feat) { return stats || mode == MODE_FILL || feat == 0 ? 64 : 80; }
+// Plain fills have the widest frames and 64 did best (four queries' counts and rows 1.85 ms, at 72 1.92).
+constexpr int search_regs(int mode, bool stats, int feat) {
+    return stats || feat == 0 || (mode == MODE_FILL && feat != FEAT_PAIRS) ? 64 : 80;
+}
 constexpr unsigned FEAT_WIDE = 8u;     // a plain count with 80 registers
 constexpr int WIDE_WARPS = 28;
 
@@ -1637,7 +1714,7 @@ std::unordered_map<uint64_t, int> g_blocks_per_sm;   // (device, kernel, warps, 
 template <int MODE>
 const void* kernel_for(unsigned feat) {
     // pairs are only faster, not needed: beside a query with checks they are searched like any level
-    if (MODE == MODE_COUNT && (feat & 7u) == FEAT_PAIRS) return (const void*)search_kernel<MODE_COUNT, false, FEAT_PAIRS>;
+    if (feat == FEAT_PAIRS) return (const void*)search_kernel<MODE, false, FEAT_PAIRS>;
     if (MODE == MODE_COUNT && feat == FEAT_WIDE) return (const void*)search_kernel<MODE_COUNT, false, FEAT_WIDE>;
     switch (feat & 3u) {
         case 0: return (const void*)search_kernel<MODE, false, 0>;
