@@ -527,12 +527,13 @@ struct Search {
     // ---------------------------------------------------- candidate filter
     //
     // A level whose look-ahead joins its new node to a bound node x keeps, per
-    // parent, a 256-bit signature (two bits per entry) of x's list in (tprev, tend]:
+    // parent, a 512-bit signature (two bits per entry) of x's list in (tprev, tend]:
     // a candidate whose two bits are not both set has no such edge.  The filter reads the
     // neighbour column only; what passes is collected in order and goes through step() 32 at
     // a time, so the exact check's dependent searches run on full warps.  Without
     // it every candidate paid those searches (a hub's list: ~20 loads each): the chorded
-    // 4-cycle on 100M hub-skewed edges 222 -> 53 ms.
+    // 4-cycle on 100M hub-skewed edges 222 -> 53 ms, with 80 registers 48.  (256 bits and at most 8 list
+    // entries per candidate: 49 ms against 42; 512-entry lists: no more.)
 
     __device__ uint32_t filt(Frame f, int i) const {
         return f.o + (uint32_t)__ldg(MODE == MODE_FILL ? &q->plan.lv[i].filt_off_fill : &q->plan.lv[i].filt_off);
@@ -541,12 +542,12 @@ struct Search {
     __device__ static uint32_t* filt_sig(uint32_t area, int s) {
         return (uint32_t*)(smem + area + CandidateFilter::SIG) + CandidateFilter::WORDS * s;
     }
-    __device__ static uint32_t filt_hash(int32_t x) { return (uint32_t)x * 2654435761u; }   // bits 31-24 and 23-16
+    __device__ static uint32_t filt_hash(int32_t x) { return (uint32_t)x * 2654435761u; }   // bits 31-23 and 22-14
 
     // Window of x's list for the filter of level i, for a partial match as in locate() with a
     // level-i window of clen candidates; 0 when no candidate can pass.  A long list window saturates
     // its signature, and one much longer than the candidates' costs more to read than
-    // their searches (about 8 entries a search): those parents pass everything (beg = NEVER).
+    // their searches (32 entries a search): those parents pass everything (beg = NEVER).
     __device__ uint32_t filt_window(int i, Frame pf, int ps, int nb, int32_t n0, int32_t n1, int32_t prev_e, int cdir,
                                     uint32_t cpos, int64_t tprev, int64_t tend, uint32_t clen, uint32_t& beg) const {
         const LevelPlan& lp = q->plan.lv[i];
@@ -563,7 +564,7 @@ struct Search {
             b = upper_bound_t(ta, __ldg(g.off[dir] + x), hi, tprev);
             if (b >= hi || __ldg(ta + b) > tend) return 0u;
         }
-        const uint32_t most = 8u * min(clen, 32u);
+        const uint32_t most = 32u * min(clen, 8u);
         const uint32_t e = window_end(ta, b, min(hi, b + most + 1u), tend);
         beg = b;
         if (e - b <= most) return e - b;
@@ -577,7 +578,7 @@ struct Search {
         for (uint32_t s = lane; s < np; s += 32u) {
             const uint32_t v = filt_u32(area, CandidateFilter::BEG, s) == NEVER ? FULL : 0u;
             uint4* sig = (uint4*)filt_sig(area, s);
-            sig[0] = sig[1] = make_uint4(v, v, v, v);
+            sig[0] = sig[1] = sig[2] = sig[3] = make_uint4(v, v, v, v);
         }
         uint2* row = (uint2*)(smem + area + CandidateFilter::LEN);
         const uint32_t tot = begin_row(row, np);
@@ -591,8 +592,8 @@ struct Search {
                 if (b != NEVER) {
                     const uint32_t h = filt_hash(__ldg(nbr + b + (off + lane - filt_u32(area, CandidateFilter::LEN, p))));
                     uint32_t* sig = filt_sig(area, p);
-                    atomicOr(sig + (h >> 29), 1u << (h >> 24 & 31u));
-                    atomicOr(sig + (h >> 21 & 7u), 1u << (h >> 16 & 31u));
+                    atomicOr(sig + (h >> 28), 1u << (h >> 23 & 31u));
+                    atomicOr(sig + (h >> 19 & 15u), 1u << (h >> 14 & 31u));
                 }
             }
         }
@@ -623,7 +624,7 @@ struct Search {
             if (pass) {
                 const uint32_t hx = filt_hash(x[j]);
                 const uint32_t* sig = filt_sig(area, p[j]);
-                pass = (sig[hx >> 29] >> (hx >> 24 & 31u) & sig[hx >> 21 & 7u] >> (hx >> 16 & 31u) & 1u) != 0u;
+                pass = (sig[hx >> 28] >> (hx >> 23 & 31u) & sig[hx >> 19 & 15u] >> (hx >> 14 & 31u) & 1u) != 0u;
             }
             const unsigned b = __ballot_sync(FULL, pass);
             if (pass) {

@@ -279,7 +279,7 @@ struct FrameLayout {
 // list windows the signatures are built from are needed until the frame is begun, the
 // pending candidates only after, so the two share their bytes.
 struct CandidateFilter {
-    static constexpr int WORDS = 8;                // signature words per parent
+    static constexpr int WORDS = 16;               // signature words per parent
     static constexpr int PEND = 96;                // up to 31 pending candidates and the 64 of a filter step
     static constexpr int BEG = 0, LEN = 256;       // u32 per parent: window of the list the signature covers
     static constexpr int POS = 0, PAR = 4 * PEND;  // u32 list position, u8 parent of each pending candidate
