@@ -1,13 +1,13 @@
 // Graph ingest (paper Section 4.2 data loader, Section 2.2 layout), on the GPU:
-//   1. validate ids / times and find the time range (one reduction kernel)
+//   1. validate times and find their range, and validate node ids (host lists: the ids are
+//      copied and checked while the times are sorted)
 //   2. stable radix sort by time with the input index as payload -> edge ids
 //      (skipped when the input is already in time order)
-//   3. gather the edge columns into edge-id order
-//   4. per direction: degree histogram + exclusive scan -> list offsets;
-//      stable radix sort of (endpoint, edge id) -> lists in time order;
-//      gather (t, neighbour) columns for the lists.
+//   3. gather the edge columns into edge-id order, and the same as records
+//   4. per direction: stable radix sort of (endpoint, edge id) -> lists in time
+//      order and their offsets; gather (t, neighbour) columns for the lists.
 //   5. out-lists re-ordered by (neighbour, time): closing-edge lookups
-//   6. successor index: per edge, the first later position in its four lists
+//   6. successor index: per edge, the first later position in its four lists; root filter
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -655,6 +655,11 @@ extern "C" tm_status tm_graph_edge_perm(const tm_graph* g, int64_t* out_perm) {
             widen_kernel<<<grid_for(n, g->num_sms), 256>>>(g->perm + i, n, wide);
             note_launches(1);
             e = cudaGetLastError();
+            // pages that the caller never touched are slow to fault in from the device: 5.7M ids into fresh memory
+            // took 11 ms, with a byte of each page written first 1.9
+            volatile char* to = (volatile char*)(out_perm + i);
+            for (int64_t b = 0; b < n * 8; b += 4096) to[b] = 0;
+            to[n * 8 - 1] = 0;
             if (e == cudaSuccess) e = cudaMemcpy(out_perm + i, wide, n * 8, cudaMemcpyDeviceToHost);
         }
         dev_free(wide, g->device, e == cudaSuccess);

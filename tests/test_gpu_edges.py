@@ -206,3 +206,11 @@ def test_load_edges(tmg, m, span):
             with pytest.raises(tmg.TMError):
                 tmg.Graph.load(n, src, dst, t, el, nl)
             col[m - 1] = keep
+
+
+@pytest.mark.parametrize("extra", [-1, 0, 1, 4096])
+def test_edge_permutation_parts(tmg, extra):
+    """The permutation is copied out 2^22 ids at a time: around that many, into memory nobody touched before."""
+    m = (1 << 22) + extra
+    n, src, dst, t, el, nl = graph(1000, m, 1 << 30, seed=m)
+    assert np.array_equal(tmg.Graph.load(n, src, dst, t).edge_perm(), np.argsort(t, kind="stable"))
