@@ -67,8 +67,8 @@
 //    and instruction cache are short (the pair code alone, in the plain instance,
 //    made a 4-edge path 22% slower).  The plain instance was 95 KB of code and warps
 //    waited for instructions a third of the time on 4-cycles: one call site for each large part and
-//    no unrolling of short loops made it 81 KB, the 64-query batch 11.3 -> 9.9 ms and four
-//    queries' counts and rows 1.70 -> 1.52 ms.
+//    no unrolling of short loops made it 81 KB, the 64-query batch 11.3 -> 10.2 ms and four
+//    queries' counts and rows 1.70 -> 1.53 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1610,7 +1610,10 @@ __global__ void __maxnreg__(search_regs(MODE, STATS, FEAT)) search_kernel(const 
     __syncthreads();
     const int warp = threadIdx.x >> 5;
     Search<MODE, STATS, FEAT> s(g, qs, ctrl, tasks, ready, task_cap, (uint32_t)(warp * warp_smem), &blk);
-    s.run(nq, ctrl->total_chunks);
+    uint64_t chunks = ctrl->total_chunks;
+    // a fill of one query ends with its list; of several, each warp finds that out query by query
+    if (MODE == MODE_FILL && nq == 1) chunks = min((unsigned long long)chunks, qs[0].chunk_off[qs[0].n_chunks + 1]);
+    s.run(nq, chunks);
 }
 
 }  // namespace
