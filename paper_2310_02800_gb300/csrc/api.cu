@@ -261,6 +261,7 @@ tm_status build_plan(const tm_graph* g, const tm_motif* m, Plan* out) {
         const uint32_t plain = Hot::ELABEL | Hot::NLABEL | Hot::ANTI | Hot::LOOK | Hot::GAP;
         if (l.kind == z.kind && l.kind <= EXT_IN && l.a == z.a && !((l.hot | z.hot) & plain)) l.hot |= Hot::PAIRS;
     }
+    const int cap = plan_features(p) & FEAT_LOOK ? FCAP_LOOK : FCAP_COUNT;
     for (int i = 1; i < k; ++i) {
         LevelPlan& lp = p.lv[i];
         const bool filter = (lp.hot & Hot::FILT) != 0;
@@ -274,12 +275,12 @@ tm_status build_plan(const tm_graph* g, const tm_motif* m, Plan* out) {
         }
         lp.frame_off = off_c;
         lp.frame_off_fill = off_f;
-        lp.anti_row_off = frame_bytes(lp.nb, i, false);
-        lp.anti_row_off_fill = frame_bytes(lp.nb, i, true);
-        lp.filt_off = frame_bytes(lp.nb, i, false, m->n_anti);
-        lp.filt_off_fill = frame_bytes(lp.nb, i, true, m->n_anti);
-        off_c += frame_bytes(lp.nb, i, false, m->n_anti, filter);
-        off_f += frame_bytes(lp.nb, i, true, m->n_anti, filter);
+        lp.anti_row_off = frame_bytes(lp.nb, i, false, cap);
+        lp.anti_row_off_fill = frame_bytes(lp.nb, i, true, cap);
+        lp.filt_off = frame_bytes(lp.nb, i, false, cap, m->n_anti);
+        lp.filt_off_fill = frame_bytes(lp.nb, i, true, cap, m->n_anti);
+        off_c += frame_bytes(lp.nb, i, false, cap, m->n_anti, filter);
+        off_f += frame_bytes(lp.nb, i, true, cap, m->n_anti, filter);
     }
     p.warp_smem = (off_c + 15) & ~15;
     p.warp_smem_fill = (off_f + 15) & ~15;

@@ -15,7 +15,7 @@
 //    read instead, 64 roots per step, and every warp claiming for itself: 1/61 of
 //    10M edges 107 -> 83 us a call, labelled 5-path on 20M edges 450 -> 348 us.
 //  * A warp owns a stack of FRAMES, one per motif edge i >= 1.  Frame i holds
-//    up to 48 (count) or 64 (fill) partial matches of i edges ("parents"), each with its candidate
+//    up to 48 (count; 40 with look-ahead) or 64 (fill) partial matches of i edges ("parents"), each with its candidate
 //    window for edge i: the entries of one time-ordered adjacency list with
 //    t in (t_prev, min(t_root + delta, t_prev + gap_{i-1})], located by a
 //    binary search for the lower end and a galloping search for the upper end
@@ -241,7 +241,7 @@ struct Search {
     static constexpr bool LOOK = (FEAT & FEAT_LOOK) != 0;   // look-ahead checks compiled in
     static constexpr bool FILTER = LOOK && !STATS;          // ... with their candidate filter
     static constexpr bool PAIRS = (FEAT & FEAT_PAIRS) != 0;   // last two edges as pairs
-    static constexpr int CAP = MODE == MODE_FILL ? FCAP_FILL : FCAP_COUNT;   // parents per frame
+    static constexpr int CAP = MODE == MODE_FILL ? FCAP_FILL : LOOK ? FCAP_LOOK : FCAP_COUNT;   // parents per frame
     static constexpr uint32_t DESCEND = CAP - 32;   // a child frame this full is drained next
     using Frame = FrameT<CAP>;
     const GraphView& g;

@@ -232,6 +232,11 @@ struct AntiPlan {
 // memory footprint leaves more of each SM's unified L1 / shared memory to L1;
 // fill frames carry edge ids and keep 64 (descend at 32).
 constexpr int FCAP_COUNT = 48;
+// Counts with look-ahead: the signatures leave shared memory for 12 warps per SM at 48, for 16 at 40, which
+// is worth more than fuller child frames (chorded 4-cycle on 100M edges 41.5 -> 34.2 ms; plain
+// motifs lose: 4-path over 15 h windows 19.9 -> 21.2 ms).  A launch with look-ahead also runs plans without
+// it, laid out for 48: their frames have room to spare.
+constexpr int FCAP_LOOK = 40;
 constexpr int FCAP_FILL = 64;
 
 struct Plan {
@@ -290,8 +295,8 @@ static_assert(4 * FCAP_FILL <= 256 && CandidateFilter::PAR + CandidateFilter::PE
               "candidate filter rows overlap");
 
 // Count frames (no edge ids) or fill frames (edge ids of the bound edges).
-inline int frame_bytes(int nb, int level, bool with_eids, int n_anti = 0, bool filter = false) {
-    const int cap = with_eids ? FCAP_FILL : FCAP_COUNT;
+inline int frame_bytes(int nb, int level, bool with_eids, int cap_count, int n_anti = 0, bool filter = false) {
+    const int cap = with_eids ? FCAP_FILL : cap_count;
     return FrameLayout<FCAP_FILL>::NODE / FCAP_FILL * cap + 4 * cap * (nb + (with_eids ? level : 0)) + 8 * cap * n_anti +
            (filter ? CandidateFilter::bytes(cap) : 0);
 }
