@@ -85,9 +85,13 @@ cudaError_t dev_malloc(void** p, size_t bytes) {
 
 void dev_free(void* p, int device, bool settled) {
     if (!p) return;
+    if (!settled && cudaDeviceSynchronize() != cudaSuccess) {
+        cudaGetLastError();
+        return;             // better lost than given to another owner under its users
+    }
     cudaStream_t st = nullptr;
     cudaMemPool_t pool = nullptr;
-    if (settled && alloc_stream(device, &st, &pool) == cudaSuccess && cudaFreeAsync(p, st) == cudaSuccess) return;
+    if (alloc_stream(device, &st, &pool) == cudaSuccess && cudaFreeAsync(p, st) == cudaSuccess) return;
     cudaGetLastError();
     cudaFree(p);
 }
@@ -641,7 +645,7 @@ extern "C" tm_status tm_count_roots(tm_graph* g, tm_query* q, int64_t rb, int64_
         *total = 0;
         return TM_OK;
     }
-    InFlight call(&g->unsettled, &q->unsettled);
+    InFlight call(st, &g->unsettled, &q->unsettled);
     tm_status s = run_count(g, q, (uint64_t)rb, (uint64_t)re, st, (unsigned long long*)per_root_dev, false, false);
     if (s != TM_OK) return s;
     s = read_back(q->scratch, st);
@@ -663,7 +667,7 @@ extern "C" tm_status tm_query_work(tm_graph* g, tm_query* q, void* stream, tm_wo
     cudaStream_t st = (cudaStream_t)stream;
     memset(out, 0, sizeof *out);
     if (g->v.m == 0) return TM_OK;
-    InFlight call(&g->unsettled, &q->unsettled);
+    InFlight call(st, &g->unsettled, &q->unsettled);
     tm_status s = run_count(g, q, 0, (uint64_t)g->v.m, st, nullptr, false, true);
     if (s != TM_OK) return s;
     s = read_back(q->scratch, st);
@@ -689,7 +693,7 @@ extern "C" tm_status tm_enumerate(tm_graph* g, tm_query* q, void* stream, int32_
         return TM_OK;
     }
     // pass 1: per-chunk match counts
-    InFlight call(&g->unsettled, &q->unsettled);
+    InFlight call(st, &g->unsettled, &q->unsettled);
     tm_status s = run_count(g, q, 0, m, st, nullptr, true, false, match_dev, cap);
     if (s != TM_OK) return s;
     Scratch& sc = q->scratch;
@@ -797,8 +801,11 @@ struct BatchExec {
                 return false;
         return true;
     }
-    tm_status alloc() {
+    int device = 0;
+    bool settled = false;                      // nothing in flight uses the buffers
+    tm_status alloc(int dev) {
         if (head) return TM_OK;
+        device = dev;
         tm_status s = dev_alloc((void**)&head, head_bytes());
         if (s == TM_OK) s = dev_alloc((void**)&counters, (size_t)nq * 8);
         if (s == TM_OK) s = dev_alloc((void**)&tasks, DEFAULT_TASK_CAP * sizeof(Task));
@@ -809,22 +816,23 @@ struct BatchExec {
             set_error("cudaHostAlloc failed");
             s = TM_E_OOM;
         }
-        if (s != TM_OK) release();
+        if (s != TM_OK) release(true);
         return s;
     }
-    void release() {
+    void release(bool idle) {
+        if (!idle) cudaDeviceSynchronize();    // before the executable and the pinned buffers go, too
         for (auto& e : ev)
             if (e) { cudaEventDestroy(e); e = nullptr; }
         if (exec) cudaGraphExecDestroy(exec);
-        if (head) cudaFree(head);
-        if (counters) cudaFree(counters);
-        if (tasks) cudaFree(tasks);
-        if (ready) cudaFree(ready);
+        dev_free(head, device, idle);
+        dev_free(counters, device, idle);
+        dev_free(tasks, device, idle);
+        dev_free(ready, device, idle);
         if (stage) cudaFreeHost(stage);
         if (counters_host) cudaFreeHost(counters_host);
         exec = nullptr; head = stage = nullptr; counters = counters_host = nullptr; tasks = nullptr; ready = nullptr;
     }
-    ~BatchExec() { release(); }
+    ~BatchExec() { release(settled); }
     Scratch view(size_t gi) const {   // what one group's launch reads: its Ctrl and the task queue
         Scratch v;
         v.head = head + gi * sizeof(Ctrl);
@@ -905,7 +913,7 @@ extern "C" tm_status tm_count_batch(tm_graph* g, tm_query* const* qs, int nq, vo
     std::vector<LaunchGroup> groups = occupancy_groups(g, MODE_COUNT, plans.data(), nch.data(), nq, order.data());
     BatchExec* b = cached_exec(g, nq, groups, MODE_COUNT);
     std::lock_guard<std::mutex> use(b->mu);
-    tm_status s = b->alloc();
+    tm_status s = b->alloc(g->device);
     if (s != TM_OK) return s;
     memset(b->stage, 0, b->ctrl_bytes());
     for (size_t gi = 0; gi < groups.size(); ++gi) {
@@ -929,7 +937,7 @@ extern "C" tm_status tm_count_batch(tm_graph* g, tm_query* const* qs, int nq, vo
         s = capture_batch(g, b);
         if (s != TM_OK) return s;
     }
-    InFlight call(&g->unsettled);
+    InFlight call(st, &g->unsettled);
     TM_CUDA(cudaGraphLaunch(b->exec, st));
     note_launches(1);
     TM_CUDA(cudaStreamSynchronize(st));
@@ -977,10 +985,12 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
     std::vector<const Plan*> plans(nq);
     std::vector<uint64_t> nch(nq);
     std::vector<int> cr(nq);
-    InFlight call(&g->unsettled);
+    // the batch buffers' locks: declared before `call`, so that they are held until it has waited
+    std::unique_lock<std::mutex> lock_c, lock_f;
+    InFlight call(st, &g->unsettled);
     std::vector<InFlight> query_calls;           // each query's scratch holds its chunk counts
     query_calls.reserve(nq);
-    for (int j = 0; j < nq; ++j) query_calls.emplace_back(&qs[j]->unsettled);
+    for (int j = 0; j < nq; ++j) query_calls.emplace_back(st, &qs[j]->unsettled);
     for (int j = 0; j < nq; ++j) {
         apply_cached_tuning(g, qs[j]);
         plans[j] = &qs[j]->plan;
@@ -995,8 +1005,8 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
     std::vector<int> order(nq);
     std::vector<LaunchGroup> cg = occupancy_groups(g, MODE_COUNT, plans.data(), nch.data(), nq, order.data());
     BatchExec* bc = cached_exec(g, nq, cg, MODE_COUNT);
-    std::lock_guard<std::mutex> lock_c(bc->mu);
-    tm_status s = bc->alloc();
+    lock_c = std::unique_lock<std::mutex>(bc->mu);
+    tm_status s = bc->alloc(g->device);
     if (s != TM_OK) return s;
     memset(bc->stage, 0, bc->ctrl_bytes());
     for (size_t gi = 0; gi < cg.size(); ++gi) {
@@ -1040,7 +1050,6 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
     for (int j = 0; j < nq; ++j)
         if (caps[j] > 0) fq.push_back(j);
     BatchExec* bf = nullptr;
-    std::unique_lock<std::mutex> lock_f;
     if (!fq.empty()) {
         const int nf = (int)fq.size();
         std::vector<const Plan*> fplans(nf);
@@ -1050,7 +1059,7 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
         std::vector<LaunchGroup> fg = occupancy_groups(g, MODE_FILL, fplans.data(), fch.data(), nf, forder.data());
         bf = cached_exec(g, nf, fg, MODE_FILL);
         lock_f = std::unique_lock<std::mutex>(bf->mu);
-        s = bf->alloc();
+        s = bf->alloc(g->device);
         if (s != TM_OK) return s;
         memset(bf->stage, 0, bf->ctrl_bytes());
         for (size_t gi = 0; gi < fg.size(); ++gi) {
@@ -1120,7 +1129,10 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
 // Release batch executables of a graph (called from tm_graph_free).
 void tmg::drop_batches(const tm_graph* g) {
     std::lock_guard<std::mutex> lk(g_batch_mu);
-    g_batches.erase(g);
+    auto it = g_batches.find(g);
+    if (it == g_batches.end()) return;
+    for (auto& b : it->second) b->settled = g->unsettled == 0;
+    g_batches.erase(it);
 }
 
 // ------------------------------------------------------------- autotune
@@ -1131,6 +1143,7 @@ extern "C" tm_status tm_autotune(tm_graph* g, tm_query* q, void* stream, tm_tuni
     cudaStream_t st = (cudaStream_t)stream;
     const uint64_t m = (uint64_t)g->v.m;
     tm_tuning best = q->plan.tune;
+    InFlight call(st, &g->unsettled, &q->unsettled);
     if (m > 0) {
         cudaEvent_t e0, e1;
         TM_CUDA(cudaEventCreate(&e0));

@@ -613,9 +613,10 @@ extern "C" tm_status tm_graph_load(const tm_edges* e, int device, void* stream, 
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) { delete g; return cuda_fail(cudaGetLastError(), "props"); }
     g->num_sms = prop.multiProcessorCount;
-    InFlight call(&g->unsettled);
+    InFlight call((cudaStream_t)stream, &g->unsettled);
     tm_status s = build(g, e, (cudaStream_t)stream);
     if (s != TM_OK) {
+        call.wait();
         tm_graph_free(g);
         return s;
     }

@@ -104,7 +104,7 @@ extern "C" tm_status tm_count_batch_noalloc(tm_graph* g, tm_query* const* qs, in
         if (!qs[j] || query_graph(qs[j]) != g) { set_error("null or mismatched query in batch"); return TM_E_INVALID; }
     // Every call reuses the array: clear the caller's totals, then rewrite the
     // control block and the launch records and clear the task-ready flags.
-    InFlight call(&g->unsettled);
+    InFlight call(st, &g->unsettled);
     TM_CUDA(cudaMemsetAsync(totals_dev, 0, (size_t)nq * sizeof(uint64_t), st));
     if (m == 0) return cudaStreamSynchronize(st) == cudaSuccess ? TM_OK : cuda_fail(cudaGetLastError(), "sync");
     {

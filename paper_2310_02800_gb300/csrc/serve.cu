@@ -367,6 +367,8 @@ void scheduler(tm_server* s) {
             free_slot->busy = true;
             lk.unlock();
             tm_status r = launch_batch(s, *free_slot);
+            // the slot's next batch may run on its other stream, over the same buffers
+            if (r != TM_OK) cudaStreamSynchronize(free_slot->st);
             lk.lock();
             if (r != TM_OK) {
                 finish_batch(s, *free_slot, r);

@@ -26,7 +26,8 @@ tm_status cuda_fail(cudaError_t e, const char* what);
 // out-of-memory device (cudaErrorMemoryAllocation, nothing allocated).
 // dev_malloc returns memory of the device's stream-ordered pool (which keeps up to POOL_KEEP of what was
 // freed and gives the rest back), ready for any stream; dev_free takes it back.  `settled`: nothing
-// in flight uses it any more, else the free waits for the device as cudaFree does.
+// in flight uses it any more, else the free waits for the device first: cudaFree does not wait for the
+// users of pool memory.
 constexpr uint64_t POOL_KEEP = 4ull << 30;
 cudaError_t dev_malloc(void** p, size_t bytes);
 void dev_free(void* p, int device, bool settled);
@@ -140,19 +141,31 @@ struct tm_graph {
 namespace tmg {
 
 // A call that puts work on a stream: until it has waited for that work, what the work
-// uses (the graph's columns, a query's scratch) is not settled.
+// uses (the graph's columns, a query's scratch) is not settled.  A call that ends early, on
+// an error, waits too: its caller may free, or use on another stream, whatever the work still reads.
 class InFlight {
+    cudaStream_t st;
     std::atomic<int>*a, *b;
 
 public:
-    explicit InFlight(std::atomic<int>* x, std::atomic<int>* y = nullptr) : a(x), b(y) {
+    InFlight(cudaStream_t s, std::atomic<int>* x, std::atomic<int>* y = nullptr) : st(s), a(x), b(y) {
         a->fetch_add(1);
         if (b) b->fetch_add(1);
     }
+    InFlight(InFlight&& o) noexcept : st(o.st), a(o.a), b(o.b) { o.a = o.b = nullptr; }
+    InFlight(const InFlight&) = delete;
+    ~InFlight() { wait(); }
     // the work has been waited for
     void settle() {
         if (a) a->fetch_sub(1);
         if (b) b->fetch_sub(1);
+        a = b = nullptr;
+    }
+    // Wait for it here.  What could not be waited for stays unsettled.
+    void wait() {
+        if (!a) return;
+        if (cudaStreamSynchronize(st) == cudaSuccess) settle();
+        else cudaGetLastError();
         a = b = nullptr;
     }
 };
