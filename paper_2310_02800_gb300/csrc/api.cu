@@ -260,6 +260,9 @@ tm_status build_plan(const tm_graph* g, const tm_motif* m, Plan* out) {
         L.n_look++;
     }
     for (int i = 0; i < k; ++i) p.lv[i].hot = Hot::pack(p.lv[i]);
+    bool free_level = false;
+    for (int i = 1; i < k; ++i) free_level |= p.lv[i].kind == FREE;
+    p.long_frames = g && long_frames(free_level ? (uint64_t)g->v.m : (uint64_t)g->longest_list);
     if (k >= 3) {
         LevelPlan &l = p.lv[k - 2], &z = p.lv[k - 1];
         const uint32_t plain = Hot::ELABEL | Hot::NLABEL | Hot::ANTI | Hot::LOOK | Hot::GAP;
@@ -731,14 +734,14 @@ namespace tmg {
 std::vector<LaunchGroup> occupancy_groups(const tm_graph* g, Mode mode, const Plan* const* plans,
                                           const uint64_t* nch, int nq, int* order) {
     std::vector<int> grid(nq), wpb(nq);
-    std::vector<unsigned> kind(nq);            // queries that count pairs have a kernel instance of their own
+    std::vector<unsigned> kind(nq);            // queries that count pairs have kernel instances of their own, and so have long frames
     for (int j = 0; j < nq; ++j) {
         const Plan& p = *plans[j];
         LaunchCfg c = search_launch_cfg(g, mode, mode == MODE_FILL ? p.warp_smem_fill : p.warp_smem,
                                         p.tune.warps_per_block, plan_features(p));
         grid[j] = c.grid;
         wpb[j] = c.warps_per_block;
-        kind[j] = plan_features(p) & FEAT_PAIRS;
+        kind[j] = plan_features(p) & (FEAT_PAIRS | FEAT_LONG);
         order[j] = j;
     }
     // highest occupancy first; within a group the likely most expensive queries

@@ -132,6 +132,15 @@ __global__ void offsets_kernel(const uint32_t* __restrict__ nodes, int64_t m, in
     }
 }
 
+__global__ void longest_list_kernel(const uint32_t* __restrict__ off0, const uint32_t* __restrict__ off1, int64_t n,
+                                    uint32_t* __restrict__ longest) {
+    uint32_t most = 0;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+        most = max(most, max(off0[v + 1] - off0[v], off1[v + 1] - off1[v]));
+    most = __reduce_max_sync(0xffffffffu, most);
+    if ((threadIdx.x & 31) == 0) atomicMax(longest, most);
+}
+
 // List columns (time, other endpoint, edge id) from the list's edge ids.  Bound by its
 // random sectors: 10M edges took 180 us from the time and endpoint columns, 158 from records.
 template <bool IN>
@@ -542,6 +551,16 @@ tm_status build(tm_graph* g, const tm_edges* e, cudaStream_t st) {
             TM_CUDA(cudaGetLastError());
         }
         v.off[dir] = off; v.at[dir] = at; v.anbr[dir] = anbr; v.aeid[dir] = aeid;
+    }
+    g->longest_list = (uint32_t)m;
+    if (long_frames(um)) {
+        uint32_t* longest;
+        TRY(tmp.get(&longest, 1));
+        TM_CUDA(cudaMemsetAsync(longest, 0, sizeof *longest, st));
+        longest_list_kernel<<<grid_for(n, sms), 256, 0, st>>>(v.off[0], v.off[1], n, longest);
+        note_launches(1);
+        TM_CUDA(cudaGetLastError());
+        TM_CUDA(cudaMemcpyAsync(&g->longest_list, longest, sizeof *longest, cudaMemcpyDeviceToHost, st));
     }
     // 5. pair-ordered out-lists: the in-lists hold the edges by (destination, time) with
     //    their sources beside them, so one more stable sort, by source, gives

@@ -63,7 +63,7 @@
 //    lexicographic order from its offset.
 //  * The kernel is instantiated per mode (count, enumeration fill), with or
 //    without work counters, and per feature set (anti-edges, look-ahead, last
-//    edges counted as pairs), so a plain motif runs code holding none: registers
+//    edges counted as pairs, frames that may begin in parts), so a plain motif runs code holding none: registers
 //    and instruction cache are short (the pair code alone, in the plain instance,
 //    made a 4-edge path 22% slower).  The plain instance was 95 KB of code and warps
 //    waited for instructions a third of the time on 4-cycles: one call site for each large part and
@@ -90,6 +90,14 @@ constexpr uint32_t POSMASK = 0x3FFFFFFFu;
 constexpr unsigned long long NO_CHUNK = ~0ull;
 constexpr uint32_t NEVER = 0xFFFFFFFFu;      // prefix entry past a frame's last parent
 constexpr uint32_t SPAN_FAR = 0xFFFFFFFFu;   // frame window end: recompute from the root
+// Candidates a frame is searched through at a time: positions in its flattened order, a step's overshoot
+// included, stay below LATER.  One window always fits (n_edges < 2^30 - 1).
+constexpr uint32_t LATER = 0x80000000u;      // prefix entry: a window not begun yet, the other bits its length
+#ifndef TMG_FRAME_MAX        // (the tests build one with small parts, for graphs of fewer edges than that)
+#define TMG_FRAME_MAX (LATER - 256u)
+#endif
+constexpr uint32_t FRAME_MAX = TMG_FRAME_MAX;
+constexpr uint32_t MORE = 0x100u;            // in a frame's number of parents: it has windows not begun yet
 constexpr uint32_t PAIRS_MAX = 256;          // longest window whose last two edges are counted as pairs
 constexpr uint32_t PAIR_MIN_DEG = 1024;     // closing lookups on shorter lists scan the time window
 constexpr uint32_t PAIR_MIN_WINDOW = 768;   // ... and so do windows shorter than this
@@ -241,6 +249,7 @@ struct Search {
     static constexpr bool LOOK = (FEAT & FEAT_LOOK) != 0;   // look-ahead checks compiled in
     static constexpr bool FILTER = LOOK && !STATS;          // ... with their candidate filter
     static constexpr bool PAIRS = (FEAT & FEAT_PAIRS) != 0;   // last two edges as pairs
+    static constexpr bool LONG = (FEAT & FEAT_LONG) != 0;     // frames may begin in parts
     static constexpr int CAP = MODE == MODE_FILL ? FCAP_FILL : LOOK ? FCAP_LOOK : FCAP_COUNT;   // parents per frame
     static constexpr uint32_t DESCEND = CAP - 32;   // a child frame this full is drained next
     using Frame = FrameT<CAP>;
@@ -485,8 +494,54 @@ struct Search {
 
     // Start frame i, which holds np parents: its window lengths become their
     // exclusive prefix (the flattened position each window starts at; entries past
-    // np never start), computed once per frame.  Returns the flattened total.
-    __device__ uint32_t begin_frame(Frame f, uint32_t np) const { return begin_row(&f.pre2(0), np); }
+    // np never start), computed once per frame.  Returns the flattened total.  Windows of a frame may add
+    // up to more than 32 bits hold (a few dozen roots of a long delta, each followed by a FREE
+    // edge, on 100M edges): a frame with one that long begins its first parents only (LONG instances).
+    __device__ uint32_t begin_frame(Frame f, uint32_t& np) const {
+        if (LONG) {
+            bool lng = lane < np && f.len(lane) > FRAME_MAX / CAP;
+            if (lane + 32u < np) lng = lng || f.len(lane + 32) > FRAME_MAX / CAP;
+            if (__any_sync(FULL, lng)) return begin_part(f, np);
+        }
+        return begin_row(&f.pre2(0), np);
+    }
+
+    // Start as many of frame f's np windows as FRAME_MAX holds, at least one with entries; np becomes the number
+    // of parents up to there, with MORE if others are left.  Those keep their lengths, marked LATER, which no
+    // flattened position reaches.
+    __device__ uint32_t begin_part(Frame f, uint32_t& np) const {
+        const uint32_t a = 2u * lane;
+        uint2 l = make_uint2(0u, 0u);
+        if (a < (uint32_t)CAP) l = f.pre2(lane);
+        if (a >= np) l.x = 0u;
+        if (a + 1u >= np) l.y = 0u;
+        uint32_t inc = min(l.x + l.y, FRAME_MAX + 1u);      // sums saturate there
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t u = __shfl_up_sync(FULL, inc, d);
+            if (lane >= d) inc = min(inc + u, FRAME_MAX + 1u);
+        }
+        uint32_t at = __shfl_up_sync(FULL, inc, 1);
+        if (lane == 0) at = 0u;
+        const uint32_t mid = min(at + l.x, FRAME_MAX + 1u);
+        const bool fx = a < np && mid <= FRAME_MAX, fy = a + 1u < np && inc <= FRAME_MAX;
+        const uint32_t taken = __popc(__ballot_sync(FULL, fx)) + __popc(__ballot_sync(FULL, fy));
+        const uint32_t tot = __reduce_max_sync(FULL, fy ? inc : fx ? mid : 0u);
+        if (a < (uint32_t)CAP)
+            f.pre2(lane) = make_uint2(fx ? at : a < np ? l.x | LATER : NEVER, fy ? mid : a + 1u < np ? l.y | LATER : NEVER);
+        __syncwarp();
+        if (taken < np) np = taken | MORE;
+        return tot;
+    }
+
+    // Start the windows that begin_part() left: the parents before them stay, with empty windows.
+    __device__ uint32_t begin_rest(Frame f, uint32_t& np) const {
+        uint2 v = make_uint2(NEVER, NEVER);
+        if (2 * lane < CAP) v = f.pre2(lane);
+        np = __popc(__ballot_sync(FULL, v.x != NEVER)) + __popc(__ballot_sync(FULL, v.y != NEVER));
+        if (2 * lane < CAP) f.pre2(lane) = make_uint2(v.x & LATER ? v.x & ~LATER : 0u, v.y & LATER ? v.y & ~LATER : 0u);
+        __syncwarp();
+        return begin_part(f, np);
+    }
 
     __device__ static bool pair_level(uint32_t h) { return PAIRS && (h & Hot::PAIRS); }
 
@@ -517,8 +572,8 @@ struct Search {
         return tot;
     }
 
-    // Parent whose window holds flattened position x (warp-uniform); every
-    // window of a begun frame is non-empty, so it is the last one starting at or before x.
+    // Parent whose window holds flattened position x (warp-uniform); empty windows of a
+    // begun frame come before all others, so it is the last one starting at or before x.
     __device__ static int parent_of(uint2 pr, uint32_t x) {
         return __popc(__ballot_sync(FULL, pr.x <= x)) + __popc(__ballot_sync(FULL, pr.y <= x)) - 1;
     }
@@ -794,7 +849,7 @@ struct Search {
         }
         if (STATS) {
             unsigned b = __ballot_sync(FULL, ok);
-            uint32_t l = ok ? clen : 0u;
+            unsigned long long l = ok ? clen : 0u;
             for (int d = 16; d > 0; d >>= 1) l += __shfl_down_sync(FULL, l, d);
             if (lane == 0) {
                 acc.w[W_NODES + (i + 1)] += __popc(b);
@@ -849,7 +904,7 @@ struct Search {
         if (mid >= tot || mid <= off) return tot;
         // parent containing mid
         const int p0 = parent_of(2 * lane < CAP ? f.pre2(lane) : make_uint2(NEVER, NEVER), mid);
-        const int ntask = (int)np - p0;
+        const int ntask = (int)(LONG ? np & (MORE - 1u) : np) - p0;
         // a task is one parent's window range: donate only when the tasks carry
         // split_min candidates each on average, else the queue traffic costs
         // more than the work it moves
@@ -866,7 +921,7 @@ struct Search {
         const int nb = q->plan.lv[i].nb;
         for (int j = lane; j < ntask; j += 32) {
             int p = p0 + j;
-            const uint32_t pre = f.pre(p), end = p + 1 < (int)np ? f.pre(p + 1) : tot;
+            const uint32_t pre = f.pre(p), end = p + 1 < p0 + ntask ? f.pre(p + 1) : tot;
             const uint32_t skip = (p == p0) ? (mid - pre) : 0u;
             Task* t = tasks + base + j;
             t->query = (int16_t)qi;
@@ -882,7 +937,7 @@ struct Search {
         for (int j = lane; j < ntask; j += 32) *(volatile uint8_t*)&ready[base + j] = 1;
         __syncwarp();
         if (lane == 0) atomicAdd(&ctrl->donated, (unsigned)ntask);
-        np = (uint32_t)p0 + 1u;
+        np = (LONG ? np & MORE : 0u) | ((uint32_t)p0 + 1u);
         return mid;
     }
 
@@ -1113,8 +1168,9 @@ struct Search {
         uint32_t h = hot(lvl), hc = lvl + 1 < k ? hot(lvl + 1) : 0u;
         Frame f = frame(lvl), c = lvl + 1 < k ? frame(lvl + 1) : f;
         bool pairs = pair_level(h) && whole && short_windows(f, np);
+        const uint32_t all = np;
         uint32_t off = 0, tot = begin_frame(f, np), nch = 0, pend = 0;
-        if (FILTER && (h & Hot::FILT)) build_filter(f, lvl, np);
+        if (FILTER && (h & Hot::FILT)) build_filter(f, lvl, all);
         while (true) {
             if (MODE == MODE_COUNT && !STATS && lvl == k - 1 && Hot::kind(h) <= EXT_IN &&
                 !(h & (Hot::ELABEL | Hot::NLABEL | Hot::ANTI))) {
@@ -1149,11 +1205,17 @@ struct Search {
                 if (lvl + 1 < k) { hc = hot(lvl + 1); c = frame(lvl + 1); }
                 off = 0;
                 pairs = pair_level(h) && short_windows(f, np);
+                const uint32_t all = np;
                 tot = begin_frame(f, np);
                 if (FILTER) {
                     pend = 0;
-                    if (h & Hot::FILT) build_filter(f, lvl, np);
+                    if (h & Hot::FILT) build_filter(f, lvl, all);
                 }
+                continue;
+            }
+            if (LONG && (np & MORE)) {
+                off = 0;
+                tot = begin_rest(f, np);
                 continue;
             }
             if (lvl == base) break;
@@ -1264,7 +1326,7 @@ struct Search {
             }
             if (STATS) {
                 unsigned b = __ballot_sync(FULL, ok);
-                uint32_t l = ok ? clen : 0u;
+                unsigned long long l = ok ? clen : 0u;
                 for (int dd = 16; dd > 0; dd >>= 1) l += __shfl_down_sync(FULL, l, dd);
                 if (lane == 0) {
                     acc.w[W_NODES + 1] += __popc(b);
@@ -1595,6 +1657,7 @@ struct Search {
 // anti-edges (109, 106, 104) and look-ahead (chorded 4-cycle on 100M edges 52, 49, 48 ms) likewise.
 // Plain fills have the widest frames and 64 did best (four queries' counts and rows 1.85 ms, at 72 1.92).
 constexpr int search_regs(int mode, bool stats, int feat) {
+    feat &= ~(int)FEAT_LONG;
     return stats || feat == 0 || (mode == MODE_FILL && feat != FEAT_PAIRS) ? 64 : 80;
 }
 constexpr unsigned FEAT_WIDE = 8u;     // a plain count with 80 registers
@@ -1724,15 +1787,25 @@ tm_status chunk_offsets(unsigned long long* chunk_buf, uint64_t nch, uint64_t ca
     return TM_OK;
 }
 
+bool long_frames(uint64_t longest_window) { return longest_window > FRAME_MAX / FCAP_FILL; }
+
 namespace {
 std::mutex g_cfg_mu;
 std::unordered_map<uint64_t, int> g_blocks_per_sm;   // (device, kernel, warps, smem) -> resident blocks per SM
 
-// Kernel instances: count and fill for each feature set (anti-edge checks,
-// look-ahead checks), and count with work counters (all features).  A query
+// Kernel instances: count and fill for each feature set (anti-edge checks, look-ahead
+// checks, long frames), and count with work counters (all features).  A query
 // runs the instance holding only the code its plan needs.
 template <int MODE>
 const void* kernel_for(unsigned feat) {
+    if (feat & FEAT_LONG) {
+        switch (feat & 3u) {
+            case 0: return (const void*)search_kernel<MODE, false, FEAT_LONG>;
+            case 1: return (const void*)search_kernel<MODE, false, FEAT_LONG | 1>;
+            case 2: return (const void*)search_kernel<MODE, false, FEAT_LONG | 2>;
+            default: return (const void*)search_kernel<MODE, false, FEAT_LONG | 3>;
+        }
+    }
     // pairs are only faster, not needed: beside a query with checks they are searched like any level
     if (feat == FEAT_PAIRS) return (const void*)search_kernel<MODE, false, FEAT_PAIRS>;
     if (MODE == MODE_COUNT && feat == FEAT_WIDE) return (const void*)search_kernel<MODE_COUNT, false, FEAT_WIDE>;
@@ -1745,7 +1818,7 @@ const void* kernel_for(unsigned feat) {
 }
 const void* kernel_of(Mode mode, bool stats, unsigned feat) {
     if (mode == MODE_FILL) return kernel_for<MODE_FILL>(feat);
-    if (stats) return (const void*)search_kernel<MODE_COUNT, true, 3>;
+    if (stats) return (const void*)search_kernel<MODE_COUNT, true, FEAT_LONG | 3>;
     return kernel_for<MODE_COUNT>(feat);
 }
 
@@ -1795,7 +1868,7 @@ LaunchCfg search_launch_cfg(const tm_graph* g, Mode mode, int max_warp_smem, int
     // keep the block's frames within the shared memory a block may use
     while (c.warps_per_block > 1 && max_warp_smem * c.warps_per_block > MAX_DYN_SMEM) c.warps_per_block--;
     c.smem_bytes = max_warp_smem * c.warps_per_block;
-    feat &= 7u;
+    feat &= 7u | FEAT_LONG;
     // 228 KB per SM, of which a block takes 1 KB beside its own
     if (feat == 0 && mode == MODE_COUNT && !stats &&
         228 * 1024 / (c.smem_bytes + (int)sizeof(Block) + 1024) * c.warps_per_block <= WIDE_WARPS)

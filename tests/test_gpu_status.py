@@ -1,0 +1,38 @@
+"""What a call leaves behind when it does not succeed."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def tmg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2310_02800_gb300 as m
+    m.lib()
+    return m
+
+
+@pytest.mark.parametrize("m", [60_000, 1_300_000])
+def test_timed_out_count_writes_no_rows(tmg, m):
+    """An enumeration whose count pass runs out of a bounded wait (one-block and long offset scans): the status, the
+    row buffer as it was, and an exact next call."""
+    g = synth.powerlaw_graph(m // 15, m, 313, span=9.46 * m / 8)
+    gg = tmg.Graph.from_synth(g)
+    mo = synth.cycle(3, 3600)
+    q = gg.compile(mo)
+    cap = 4096
+    out = torch.full((cap, 3), -9, dtype=torch.int32, device="cuda")
+    q.inject_fault(1)
+    with pytest.raises(tmg.TMError) as e:
+        q.enumerate(out)
+    assert e.value.status == tmg.E_TIMEOUT
+    assert bool((out == -9).all())
+    rows, total = oracle.Graph.from_synth(g).enumerate(mo, cap=cap)
+    assert q.enumerate(out) == (cap, total, True) and total > cap
+    assert np.array_equal(out.cpu().numpy(), rows)
