@@ -186,6 +186,7 @@ tm_status tm_count_roots(tm_graph* g, tm_query* q, int64_t root_begin, int64_t r
  * Rows are the lexicographically smallest min(cap, total) matches, in
  * lexicographic order of (e_0, ..., e_{k-1}).  *total is always exact.
  * Returns TM_E_TRUNCATED (non-fatal) when total > cap, with *n_written = cap.
+ * A count pass that ends in TM_E_TIMEOUT writes no row.
  * Synchronises the stream. */
 tm_status tm_enumerate(tm_graph* g, tm_query* q, void* stream, int32_t* match_dev, uint64_t cap,
                        uint64_t* n_written, uint64_t* total);

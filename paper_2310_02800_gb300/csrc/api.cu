@@ -702,7 +702,7 @@ extern "C" tm_status tm_enumerate(tm_graph* g, tm_query* q, void* stream, int32_
     Scratch& sc = q->scratch;
     const uint64_t nch = n_chunks(m, effective_chunk(g, q->plan, m));
     // pass 2: chunk offsets, and the chunks the fill pass must search
-    s = chunk_offsets(sc.chunk_cnt, nch, cap, sc.scan_tmp, g->num_sms, st);
+    s = chunk_offsets(sc.chunk_cnt, nch, cap, single_view(sc, 0).ctrl(), sc.scan_tmp, g->num_sms, st);
     if (s != TM_OK) return s;
     if (cap > 0) {
         // pass 3: fill rows in lexicographic order from each chunk's offset (nothing to do
@@ -1043,9 +1043,13 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
     }
     if (kernel_ms) TM_CUDA(cudaEventRecord(bc->ev[1], st));
     // pass 2: chunk offsets, and the chunks the fill pass must search
-    for (int j = 0; j < nq; ++j) {
-        s = chunk_offsets(qs[j]->scratch.chunk_cnt, nch[j], caps[j], qs[j]->scratch.scan_tmp, g->num_sms, st);
-        if (s != TM_OK) return s;
+    for (size_t gi = 0; gi < cg.size(); ++gi) {
+        const Scratch v = bc->view(gi);
+        for (int i = cg[gi].first; i < cg[gi].first + cg[gi].count; ++i) {
+            const int j = order[i];
+            s = chunk_offsets(qs[j]->scratch.chunk_cnt, nch[j], caps[j], v.ctrl(), qs[j]->scratch.scan_tmp, g->num_sms, st);
+            if (s != TM_OK) return s;
+        }
     }
     // pass 3: rows of the queries with room for some, written from each chunk's
     // offset on the device (chunks past the cap or without matches are skipped)

@@ -1689,8 +1689,10 @@ namespace {
 // The chunks of an enumeration that hold a match and whose rows start below
 // the cap, from the scanned row offsets: their ids are appended (in no
 // particular order) after the offsets and the list length (zeroed by the
-// caller), for the fill pass to claim.
-__global__ void list_chunks_kernel(unsigned long long* buf, uint64_t nch, uint64_t cap) {
+// caller), for the fill pass to claim.  A count that gave up (counted->err) has no rows to fill: nothing
+// is listed, and the fill ends at once.
+__global__ void list_chunks_kernel(unsigned long long* buf, uint64_t nch, uint64_t cap, const Ctrl* __restrict__ counted) {
+    if (counted->err) return;
     const unsigned long long* off = buf;
     unsigned long long* n_list = buf + nch + 1;
     uint32_t* list = (uint32_t*)(buf + nch + 2);
@@ -1713,7 +1715,8 @@ __global__ void list_chunks_kernel(unsigned long long* buf, uint64_t nch, uint64
 constexpr int SMALL_THREADS = 1024, SMALL_ITEMS = 4;
 constexpr uint64_t SMALL_CHUNKS = 16384;      // four rounds of the block; longer buffers scan faster on many
 
-__global__ void __launch_bounds__(SMALL_THREADS) small_offsets_kernel(unsigned long long* buf, uint32_t nch, uint64_t cap) {
+__global__ void __launch_bounds__(SMALL_THREADS) small_offsets_kernel(unsigned long long* buf, uint32_t nch, uint64_t cap,
+                                                                      const Ctrl* __restrict__ counted) {
     __shared__ unsigned long long wsum[SMALL_THREADS / 32];
     __shared__ uint32_t wkeep[SMALL_THREADS / 32];
     uint32_t* list = (uint32_t*)(buf + nch + 2);
@@ -1764,16 +1767,16 @@ __global__ void __launch_bounds__(SMALL_THREADS) small_offsets_kernel(unsigned l
             if (keep >> j & 1u) list[to++] = c0 + j;
         __syncthreads();
     }
-    if (threadIdx.x == 0) buf[nch + 1] = listed;
+    if (threadIdx.x == 0) buf[nch + 1] = counted->err ? 0u : listed;
 }
 
 }  // namespace
 
-tm_status chunk_offsets(unsigned long long* chunk_buf, uint64_t nch, uint64_t cap, void* scan_tmp, int num_sms,
-                        cudaStream_t st) {
+tm_status chunk_offsets(unsigned long long* chunk_buf, uint64_t nch, uint64_t cap, const Ctrl* counted, void* scan_tmp,
+                        int num_sms, cudaStream_t st) {
     if (nch == 0) return TM_OK;
     if (nch <= SMALL_CHUNKS) {
-        small_offsets_kernel<<<1, SMALL_THREADS, 0, st>>>(chunk_buf, (uint32_t)nch, cap);
+        small_offsets_kernel<<<1, SMALL_THREADS, 0, st>>>(chunk_buf, (uint32_t)nch, cap, counted);
         note_launches(1);
         TM_CUDA(cudaGetLastError());
         return TM_OK;
@@ -1781,7 +1784,7 @@ tm_status chunk_offsets(unsigned long long* chunk_buf, uint64_t nch, uint64_t ca
     tm_status s = exclusive_scan_u64(chunk_buf, chunk_buf, nch + 1, scan_tmp, st);
     if (s != TM_OK || cap == 0) return s;
     const uint64_t blocks = std::min<uint64_t>((nch + 255) / 256, (uint64_t)num_sms * 8);
-    list_chunks_kernel<<<(unsigned)blocks, 256, 0, st>>>(chunk_buf, nch, cap);
+    list_chunks_kernel<<<(unsigned)blocks, 256, 0, st>>>(chunk_buf, nch, cap, counted);
     note_launches(1);
     TM_CUDA(cudaGetLastError());
     return TM_OK;

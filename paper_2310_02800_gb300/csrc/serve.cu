@@ -186,7 +186,7 @@ tm_status launch_batch(tm_server* s, Slot& sl) {
     int fsmem = 16;
     for (Req* q : sl.batch) {
         if (!q->enumerate) continue;
-        r = chunk_offsets(q->chunk, q->nch, q->cap, q->scan_tmp, g->num_sms, sl.st);
+        r = chunk_offsets(q->chunk, q->nch, q->cap, cs.ctrl(), q->scan_tmp, g->num_sms, sl.st);
         if (r != TM_OK) return r;
         QueryDev* qd = fs.qdev_stage() + ne;
         memset(qd, 0, sizeof(QueryDev));

@@ -419,9 +419,10 @@ void query_plan(tm_query* q, Plan* out);
 const tm_graph* query_graph(const tm_query* q);
 const tm_motif* query_motif(const tm_query* q);
 
-// Turn a chunk buffer's counts into row offsets and, where cap > 0, list the chunks the fill pass must search.
-tm_status chunk_offsets(unsigned long long* chunk_buf, uint64_t nch, uint64_t cap, void* scan_tmp, int num_sms,
-                        cudaStream_t st);
+// Turn a chunk buffer's counts into row offsets and, where cap > 0, list the chunks the fill pass must search:
+// none when the count launch, whose control block is `counted`, gave up.
+tm_status chunk_offsets(unsigned long long* chunk_buf, uint64_t nch, uint64_t cap, const Ctrl* counted, void* scan_tmp,
+                        int num_sms, cudaStream_t st);
 
 tm_status scratch_reserve(Scratch* s, int device, int nq, uint64_t counters_len, uint64_t chunks,
                           uint64_t task_cap);
