@@ -101,7 +101,10 @@ constexpr uint32_t MORE = 0x100u;            // in a frame's number of parents: 
 constexpr uint32_t PAIRS_MAX = 256;          // longest window whose last two edges are counted as pairs
 constexpr uint32_t PAIR_MIN_DEG = 1024;     // closing lookups on shorter lists scan the time window
 constexpr uint32_t PAIR_MIN_WINDOW = 768;   // ... and so do windows shorter than this
-constexpr uint64_t WAIT_NS = 20ull * 1000 * 1000 * 1000;      // idle-wait deadline
+#ifndef TMG_WAIT_NS          // (a shorter one in a test's build)
+#define TMG_WAIT_NS (20ull * 1000 * 1000 * 1000)
+#endif
+constexpr uint64_t WAIT_NS = TMG_WAIT_NS;                     // idle-wait deadline
 constexpr uint64_t READY_NS = 2ull * 1000 * 1000 * 1000;      // publish-wait deadline
 
 __device__ __forceinline__ int64_t sat_add(int64_t a, int64_t b) {
@@ -1476,7 +1479,8 @@ struct Search {
                 if (ns < 2048) ns <<= 1;
             }
             if (polling) {
-                if (!leave) atomicSub(&ctrl->idle, 1);
+                // also when the block gives up waiting: donors would go on handing out work nobody waits for
+                atomicSub(&ctrl->idle, 1);
                 atomicExch(&blk->poller, 0);
             }
         }
