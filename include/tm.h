@@ -142,7 +142,9 @@ typedef struct tm_server tm_server;
  * `stream`; returns after the build has finished.  *out is library-owned. */
 tm_status tm_graph_load(const tm_edges* edges, int device, void* stream, tm_graph** out);
 
-/* Release a graph and its device memory.  NULL is accepted. */
+/* Release a graph and its device memory.  NULL is accepted.  The library allocates from a memory
+ * pool of its own on each device, which keeps up to 4 GiB of what was freed (or the largest budget of a
+ * running server) for later calls; memory above that goes back to the driver here. */
 tm_status tm_graph_free(tm_graph* g);
 
 /* Sizes of a loaded graph (any pointer may be NULL). */

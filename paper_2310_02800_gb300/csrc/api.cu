@@ -9,7 +9,9 @@
 #include <cstring>
 #include <map>
 #include <memory>
+#include <set>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "tm_internal.cuh"
@@ -40,47 +42,77 @@ static bool alloc_fault_due() {
     return false;
 }
 
-// The stream a device's allocations are ordered on (only allocations and frees of settled memory run there) and
-// its pool.  A 10M-edge graph's cudaMalloc and cudaFree, and those of its query's scratch, left 0.9 ms
+// A device's memory pool of the library's own (the default pool's settings belong to whoever else uses it) and
+// the stream its allocations are ordered on: only allocations and frees of settled memory run there.  A
+// 10M-edge graph's cudaMalloc and cudaFree, and those of its query's scratch, left 0.9 ms
 // of a 5.2 ms load-count-free cycle uncovered; from the pool they take 30 us.
-static cudaError_t alloc_stream(int device, cudaStream_t* st, cudaMemPool_t* pool) {
-    static std::mutex mu;
-    static std::map<int, std::pair<cudaStream_t, cudaMemPool_t>> per_device;
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = per_device.find(device);
-    if (it == per_device.end()) {
-        std::pair<cudaStream_t, cudaMemPool_t> sp{nullptr, nullptr};
-        cudaError_t e = cudaDeviceGetDefaultMemPool(&sp.second, device);
-        if (e != cudaSuccess) return e;
-        uint64_t keep = 0;
-        cudaMemPoolGetAttribute(sp.second, cudaMemPoolAttrReleaseThreshold, &keep);
-        if (keep < POOL_KEEP) {
-            keep = POOL_KEEP;
-            cudaMemPoolSetAttribute(sp.second, cudaMemPoolAttrReleaseThreshold, &keep);
-        }
-        if ((e = cudaStreamCreateWithFlags(&sp.first, cudaStreamNonBlocking)) != cudaSuccess) return e;
-        it = per_device.emplace(device, sp).first;
+struct DevPool {
+    cudaStream_t st = nullptr;
+    cudaMemPool_t pool = nullptr;
+    std::unordered_map<void*, size_t> sizes;   // dev_malloc's
+    uint64_t live = 0;                         // their sum
+    std::multiset<uint64_t> budgets;           // of the running servers
+    uint64_t limit = 0;                        // the release threshold
+
+    // What the pool may hold before it gives memory back: the threshold counts what is in use too, so
+    // that follows.  Small changes wait: setting it for each buffer and small graph would cost more than they matter
+    // (8 us of a 1.08 ms load of 1M edges).
+    void set_limit() {
+        const uint64_t want = live + std::max(POOL_KEEP, budgets.empty() ? 0 : *budgets.rbegin());
+        if (want < limit + (256ull << 20) && limit < want + (256ull << 20)) return;
+        uint64_t v = want;
+        if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &v) == cudaSuccess) limit = want;
     }
-    *st = it->second.first;
-    *pool = it->second.second;
+};
+static std::mutex g_pool_mu;
+
+// The device's pool, made on first use (the device is current, g_pool_mu held).
+static cudaError_t dev_pool(int device, DevPool** out) {
+    static std::map<int, DevPool> per_device;
+    DevPool& d = per_device[device];
+    if (!d.pool) {
+        cudaMemPoolProps props;
+        memset(&props, 0, sizeof props);
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        cudaError_t e;
+        if (!d.st && (e = cudaStreamCreateWithFlags(&d.st, cudaStreamNonBlocking)) != cudaSuccess) return e;
+        if ((e = cudaMemPoolCreate(&d.pool, &props)) != cudaSuccess) { d.pool = nullptr; return e; }
+        d.set_limit();
+    }
+    *out = &d;
     return cudaSuccess;
+}
+
+static cudaError_t from_pool(const DevPool& d, void** p, size_t bytes, cudaStream_t st) {
+    const cudaError_t e = cudaMallocFromPoolAsync(p, bytes, d.pool, st);
+    if (e == cudaSuccess) return e;
+    // what the pool keeps may be in the way
+    cudaGetLastError();
+    cudaMemPoolTrimTo(d.pool, 0);
+    return cudaMallocFromPoolAsync(p, bytes, d.pool, st);
 }
 
 cudaError_t dev_malloc(void** p, size_t bytes) {
     if (alloc_fault_due()) return cudaErrorMemoryAllocation;
     int device = 0;
-    cudaError_t e = cudaGetDevice(&device);
-    if (e != cudaSuccess) return e;
-    cudaStream_t st = nullptr;
-    cudaMemPool_t pool = nullptr;
-    if ((e = alloc_stream(device, &st, &pool)) != cudaSuccess) return e;
-    if (cudaMallocAsync(p, bytes, st) != cudaSuccess) {
-        // what the pool keeps may be in the way
-        cudaGetLastError();
-        cudaMemPoolTrimTo(pool, 0);
-        if ((e = cudaMallocAsync(p, bytes, st)) != cudaSuccess) return e;
+    DevPool* d = nullptr;
+    cudaStream_t st;
+    {
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        cudaError_t e = cudaGetDevice(&device);
+        if (e == cudaSuccess) e = dev_pool(device, &d);
+        if (e == cudaSuccess) e = from_pool(*d, p, bytes, d->st);
+        if (e != cudaSuccess) return e;
+        d->sizes[*p] = bytes;
+        d->live += bytes;
+        d->set_limit();
+        st = d->st;
     }
-    return cudaStreamSynchronize(st);
+    const cudaError_t e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) dev_free(*p, device, true);
+    return e;
 }
 
 void dev_free(void* p, int device, bool settled) {
@@ -89,16 +121,57 @@ void dev_free(void* p, int device, bool settled) {
         cudaGetLastError();
         return;             // better lost than given to another owner under its users
     }
-    cudaStream_t st = nullptr;
-    cudaMemPool_t pool = nullptr;
-    if (alloc_stream(device, &st, &pool) == cudaSuccess && cudaFreeAsync(p, st) == cudaSuccess) return;
-    cudaGetLastError();
-    cudaFree(p);
+    DevPool* d = nullptr;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (dev_pool(device, &d) != cudaSuccess || cudaFreeAsync(p, d->st) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(p);
+        if (!d) return;
+    }
+    auto it = d->sizes.find(p);
+    if (it == d->sizes.end()) return;
+    d->live -= it->second;
+    d->sizes.erase(it);
+    d->set_limit();
 }
 
 cudaError_t dev_malloc_async(void** p, size_t bytes, cudaStream_t st) {
     if (alloc_fault_due()) return cudaErrorMemoryAllocation;
-    return cudaMallocAsync(p, bytes, st);
+    int device = 0;
+    DevPool* d = nullptr;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    cudaError_t e = cudaGetDevice(&device);
+    if (e == cudaSuccess) e = dev_pool(device, &d);
+    return e == cudaSuccess ? from_pool(*d, p, bytes, st) : e;
+}
+
+void pool_give_back(int device) {
+    DevPool* d = nullptr;
+    cudaStream_t st = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        uint64_t held = 0;
+        if (dev_pool(device, &d) == cudaSuccess && cudaMemPoolGetAttribute(d->pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+            held > d->limit)
+            st = d->st;
+    }
+    // the driver looks at the threshold when something is waited for
+    if (st) cudaStreamSynchronize(st);
+    cudaGetLastError();
+}
+
+void pool_budget(int device, uint64_t bytes, bool running) {
+    {
+        DevPool* d = nullptr;
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        if (dev_pool(device, &d) == cudaSuccess) {
+            if (running) d->budgets.insert(bytes);
+            else if (auto it = d->budgets.find(bytes); it != d->budgets.end()) d->budgets.erase(it);
+            d->set_limit();
+        }
+        cudaGetLastError();
+    }
+    if (!running) pool_give_back(device);
 }
 
 cudaError_t host_alloc_pinned(void** p, size_t bytes) {

@@ -649,6 +649,7 @@ extern "C" tm_status tm_graph_free(tm_graph* g) {
     cudaSetDevice(g->device);
     drop_batches(g);
     for (void* p : g->allocs) dev_free(p, g->device, g->unsettled == 0);
+    pool_give_back(g->device);
     delete g;
     return TM_OK;
 }

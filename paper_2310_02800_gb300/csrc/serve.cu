@@ -439,14 +439,9 @@ extern "C" tm_status tm_serve_start(tm_graph* g, const tm_serve_cfg* cfg, tm_ser
         delete s;
         return TM_E_CUDA;
     }
-    // keep freed match buffers in the device's stream-ordered pool instead of
-    // returning them to the driver at every synchronisation
-    cudaMemPool_t pool;
-    if (cudaDeviceGetDefaultMemPool(&pool, g->device) == cudaSuccess) {
-        uint64_t keep = s->cfg.mem_budget_bytes;
-        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    }
-    cudaGetLastError();
+    // freed match buffers stay in the library's pool instead of going back to the
+    // driver at every synchronisation
+    pool_budget(g->device, s->cfg.mem_budget_bytes, true);
     g->unsettled.fetch_add(1);     // batches in flight, until tm_serve_stop has waited for them
     s->th = std::thread(scheduler, s);
     *out = s;
@@ -552,6 +547,7 @@ extern "C" tm_status tm_serve_stop(tm_server* s) {
     }
     if (settled) s->g->unsettled.fetch_sub(1);
     destroy_slots(s);
+    pool_budget(s->g->device, s->cfg.mem_budget_bytes, false);
     delete s;
     return TM_OK;
 }

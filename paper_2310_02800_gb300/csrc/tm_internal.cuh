@@ -24,14 +24,17 @@ tm_status cuda_fail(cudaError_t e, const char* what);
 // Every device and pinned-host allocation of the library goes through these,
 // so that tm_inject_alloc_failure can make one of them fail like an
 // out-of-memory device (cudaErrorMemoryAllocation, nothing allocated).
-// dev_malloc returns memory of the device's stream-ordered pool (which keeps up to POOL_KEEP of what was
-// freed and gives the rest back), ready for any stream; dev_free takes it back.  `settled`: nothing
-// in flight uses it any more, else the free waits for the device first: cudaFree does not wait for the
-// users of pool memory.
+// dev_malloc returns memory of the library's pool on the current device, ready for any stream; dev_free takes it
+// back.  The pool keeps up to POOL_KEEP (or a running server's budget, if that is more) beyond dev_malloc's
+// memory in use; pool_give_back returns what is above that, which the driver otherwise does at the
+// next synchronisation.  `settled`: nothing in flight uses the memory any more, else the free waits for the
+// device first: cudaFree does not wait for the users of pool memory.
 constexpr uint64_t POOL_KEEP = 4ull << 30;
 cudaError_t dev_malloc(void** p, size_t bytes);
 void dev_free(void* p, int device, bool settled);
 cudaError_t dev_malloc_async(void** p, size_t bytes, cudaStream_t st);
+void pool_give_back(int device);
+void pool_budget(int device, uint64_t bytes, bool running);
 cudaError_t host_alloc_pinned(void** p, size_t bytes);
 
 // Select the device and drop any error another library left on this thread,

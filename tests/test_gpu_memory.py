@@ -85,3 +85,64 @@ def test_load_fails_at_every_allocation(tmg, on_device):
         break
     assert (11 if on_device else 15) <= after < 64        # every buffer of the build was refused once
     assert np.array_equal(gg.edge_perm(), np.argsort(cols[2], kind="stable"))
+
+
+def free_mb():
+    return torch.cuda.mem_get_info()[0] >> 20
+
+
+def load(tmg, m, seed=1):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    ends = [torch.randint(0, 100_000, (m,), device="cuda", generator=gen, dtype=torch.int32) for _ in range(2)]
+    t = torch.randint(0, 1 << 30, (m,), device="cuda", generator=gen)
+    torch.cuda.synchronize()
+    return lambda: tmg.Graph.load(100_000, *ends, t)
+
+
+def test_freed_memory_is_kept_and_given_back(tmg):
+    """What the library's pool keeps after frees: something for the next load, whatever servers ran before and
+    whatever graph is resident, at most 4 GiB, at once and without a synchronisation by the caller; and the
+    device's default pool is left alone."""
+    import ctypes
+    rt = ctypes.CDLL("libcudart.so.13")
+    pool, thr = ctypes.c_void_p(), ctypes.c_uint64(12_345)
+    assert rt.cudaDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
+    assert rt.cudaMemPoolSetAttribute(pool, 4, ctypes.byref(thr)) == 0        # cudaMemPoolAttrReleaseThreshold
+    small, big = load(tmg, 2_000_000), load(tmg, 40_000_000)
+
+    def kept(fn):
+        """MB held after fn() and a synchronisation that fn's graphs held, too."""
+        g = fn()
+        torch.cuda.synchronize()
+        held = free_mb()
+        g.free()
+        torch.cuda.synchronize()
+        return g.device_bytes >> 20, free_mb() - held
+
+    mb, returned = kept(small)
+    assert mb > 200 and returned <= 2
+    g = small()
+    srv = g.serve(mem_budget_bytes=1 << 20)
+    srv.stop()
+    g.free()
+    mb, returned = kept(small)
+    assert returned <= 2, "a server's small budget must not stay behind"
+    g = big()
+    assert g.device_bytes > 5 << 30
+    mb, returned = kept(small)
+    assert returned <= 2, "a large resident graph must not use up what is kept"
+    torch.cuda.synchronize()
+    before = free_mb()
+    need = g.device_bytes >> 20
+    g.free()
+    after = free_mb()
+    assert after - before >= need - 4096 - 320, "memory above the limit goes back when the graph is freed"
+    g = big()
+    srv = g.serve(mem_budget_bytes=12 << 30)
+    srv.stop()
+    g.free()
+    assert free_mb() >= after - 320, "a server's large budget must not stay behind"
+    thr.value = 0
+    assert rt.cudaMemPoolGetAttribute(pool, 4, ctypes.byref(thr)) == 0 and thr.value == 12_345
+    thr.value = 0
+    rt.cudaMemPoolSetAttribute(pool, 4, ctypes.byref(thr))
