@@ -101,7 +101,11 @@ typedef struct {
 /* Execution knobs for one query shape (see tm_autotune).
  *   warps_per_block : 1..16 (reduced automatically when the block's search
  *                     frames would not fit in shared memory)
- *   chunk_roots     : root edges a warp claims at a time (multiple of 32)
+ *   chunk_roots     : root edges per chunk (multiple of 32).  A block claims chunks for its
+ *                     warps, up to 16 for each while they go fast.  By default (and for as long
+ *                     as the value that tm_query_get_tuning returned is set back) inputs too
+ *                     small to give every warp two chunks are cut into smaller ones, down to 8
+ *                     roots; another value set, or picked by tm_autotune, is kept
  *   split_depth     : deepest search level whose remaining candidates may be
  *                     donated to idle warps: level i holds the candidate windows
  *                     of motif edge i (1 = the root edges' windows, up to k-1);

@@ -208,6 +208,18 @@ uint64_t plan_shape_hash(const tm_motif* m) {
     return h;
 }
 
+// Roots per chunk unless set or tuned.  Stars of 5+ edges on a hub grow subtrees of C(window, k-1)
+// matches: smaller root chunks spread the hubs' roots over more warps (the tuner
+// picked 32 for every such shape on the power-law workload)
+static int default_chunk(const tm_motif& m) {
+    bool out_star = true, in_star = true;
+    for (int i = 1; i < m.k; ++i) {
+        out_star &= m.esrc[i] == m.esrc[0];
+        in_star &= m.edst[i] == m.edst[0];
+    }
+    return m.k >= 5 && (out_star || in_star) ? 32 : 64;
+}
+
 // Per-level plan of a motif (paper Section 5.1.2): motif nodes get slots in
 // the order they are first bound; level i reads the candidate list of an
 // already-mapped endpoint (out-list of x_i, in-list of y_i, the shorter of the
@@ -381,17 +393,8 @@ tm_status build_plan(const tm_graph* g, const tm_motif* m, Plan* out) {
     }
     for (int b = 0; b < 4; ++b) p.root_codes |= (uint32_t)code[b] << (8 * b);
     p.tune.warps_per_block = 4;
-    p.tune.chunk_roots = 64;
+    p.tune.chunk_roots = default_chunk(*m);
     p.auto_chunk = 1;
-    // stars of 5+ edges on a hub grow subtrees of C(window, k-1) matches:
-    // smaller root chunks spread the hubs' roots over more warps (the tuner
-    // picked 32 for every such shape on the power-law workload)
-    bool out_star = true, in_star = true;
-    for (int i = 1; i < k; ++i) {
-        out_star &= m->esrc[i] == m->esrc[0];
-        in_star &= m->edst[i] == m->edst[0];
-    }
-    if (k >= 5 && (out_star || in_star)) p.tune.chunk_roots = 32;
     p.tune.split_depth = k >= 3 ? 2 : (k == 2 ? 1 : 0);
     p.tune.split_min = 512;
     if (m->n_anti > 0) p.tune.split_depth = 0;   // donated tasks carry no anti-edge times
@@ -511,8 +514,8 @@ static void apply_cached_tuning(tm_graph* g, tm_query* q) {
     std::lock_guard<std::mutex> lk(g->tune_mu);
     auto it = g->tuned.find(key);
     if (it != g->tuned.end()) {
-        q->plan.tune = it->second;
-        q->plan.auto_chunk = 0;
+        q->plan.tune = it->second.tune;
+        q->plan.auto_chunk = it->second.automatic;
     }
 }
 
@@ -672,8 +675,9 @@ extern "C" tm_status tm_query_set_tuning(tm_query* q, const tm_tuning* t) {
         set_error("tuning out of range");
         return TM_E_INVALID;
     }
+    // the chunk size it has had so far, when that follows the input, goes on doing so
+    q->plan.auto_chunk = q->plan.auto_chunk && t->chunk_roots == q->plan.tune.chunk_roots;
     q->plan.tune = *t;
-    q->plan.auto_chunk = 0;
     if (q->plan.n_anti > 0) q->plan.tune.split_depth = 0;   // donated tasks carry no anti-edge times
     q->explicit_tuning = true;
     return TM_OK;
@@ -1222,15 +1226,15 @@ extern "C" tm_status tm_autotune(tm_graph* g, tm_query* q, void* stream, tm_tuni
     TM_ENTER(g->device);
     cudaStream_t st = (cudaStream_t)stream;
     const uint64_t m = (uint64_t)g->v.m;
-    tm_tuning best = q->plan.tune;
+    Tuned best{q->plan.tune, q->plan.auto_chunk != 0};
     InFlight call(st, &g->unsettled, &q->unsettled);
     if (m > 0) {
         cudaEvent_t e0, e1;
         TM_CUDA(cudaEventCreate(&e0));
         TM_CUDA(cudaEventCreate(&e1));
-        auto time_cfg = [&](const tm_tuning& t, float* ms) -> tm_status {
-            q->plan.tune = t;
-            q->plan.auto_chunk = 0;
+        auto time_cfg = [&](const Tuned& t, float* ms) -> tm_status {
+            q->plan.tune = t.tune;
+            q->plan.auto_chunk = t.automatic;
             float best_ms = 1e30f;
             for (int rep = 0; rep < 3; ++rep) {
                 cudaEventRecord(e0, st);
@@ -1253,13 +1257,20 @@ extern "C" tm_status tm_autotune(tm_graph* g, tm_query* q, void* stream, tm_tuni
         const int chunk_c[] = {32, 64, 256};
         const int min_c[] = {128, 512, 4096};
         for (int knob = 0; knob < 4 && s == TM_OK; ++knob) {
-            std::vector<tm_tuning> cands;
+            std::vector<Tuned> cands;
             for (int i = 0; i < 3; ++i) {
-                tm_tuning t = best;
-                if (knob == 0) t.warps_per_block = warps_c[i];
-                if (knob == 1) t.chunk_roots = chunk_c[i];
-                if (knob == 2) { t.split_depth = i; if (t.split_depth > q->plan.k - 1) continue; }
-                if (knob == 3) t.split_min = min_c[i];
+                Tuned t = best;
+                if (knob == 0) t.tune.warps_per_block = warps_c[i];
+                if (knob == 1) { t.tune.chunk_roots = chunk_c[i]; t.automatic = false; }
+                if (knob == 2) { t.tune.split_depth = i; if (i > q->plan.k - 1) continue; }
+                if (knob == 3) t.tune.split_min = min_c[i];
+                cands.push_back(t);
+            }
+            if (knob == 1 && !best.automatic) {
+                // the default, where an earlier choice has replaced it
+                Tuned t = best;
+                t.tune.chunk_roots = default_chunk(q->motif);
+                t.automatic = true;
                 cands.push_back(t);
             }
             for (auto& t : cands) {
@@ -1273,7 +1284,8 @@ extern "C" tm_status tm_autotune(tm_graph* g, tm_query* q, void* stream, tm_tuni
         cudaEventDestroy(e1);
         TM_CUDA(cudaStreamSynchronize(st));
         if (s != TM_OK) return s;
-        q->plan.tune = best;
+        q->plan.tune = best.tune;
+        q->plan.auto_chunk = best.automatic;
         TuneKey key{q->plan.shape_hash, 0};
         int64_t d = q->plan.delta;
         while (d > 0) { key.dbucket++; d >>= 1; }
@@ -1281,7 +1293,7 @@ extern "C" tm_status tm_autotune(tm_graph* g, tm_query* q, void* stream, tm_tuni
         g->tuned[key] = best;
     }
     q->explicit_tuning = false;
-    if (tuned) *tuned = best;
+    if (tuned) *tuned = best.tune;
     return TM_OK;
 }
 

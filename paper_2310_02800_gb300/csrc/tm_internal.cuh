@@ -117,6 +117,11 @@ struct TuneKey {
     int dbucket;        // floor(log2(delta + 1))
     bool operator==(const TuneKey& o) const { return shape == o.shape && dbucket == o.dbucket; }
 };
+// A tuned setting: `automatic` keeps the chunk size that follows the input (see effective_chunk).
+struct Tuned {
+    tm_tuning tune;
+    bool automatic;
+};
 struct TuneKeyHash {
     size_t operator()(const TuneKey& k) const { return (size_t)(k.shape * 1315423911ULL + (uint64_t)k.dbucket); }
 };
@@ -135,7 +140,7 @@ struct tm_graph {
     uint32_t longest_list = 0;     // of any node, in either direction (an upper bound where long_frames(m) is false)
     int num_sms = 0;
     std::mutex tune_mu;
-    std::unordered_map<tmg::TuneKey, tm_tuning, tmg::TuneKeyHash> tuned;
+    std::unordered_map<tmg::TuneKey, tmg::Tuned, tmg::TuneKeyHash> tuned;
     // serving: device ms one request of a (shape, delta bucket, flavour) takes,
     // learnt from timed launches and shared by every server of this graph
     std::mutex cost_mu;
