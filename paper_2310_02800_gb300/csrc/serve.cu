@@ -54,6 +54,7 @@ struct Req {
     int enumerate = 0;
     uint64_t cap = 0;
     uint64_t need = 0;          // admitted device bytes
+    int chunk_roots = 0;        // roots per chunk
     uint64_t key = 0;           // cost-model key: shape, delta bucket, flavour
     double est_ms = -1.0;       // expected device time when batched (< 0: unknown)
     int occ = 0;                // launch shape (resident grid, warps per block) of the request alone
@@ -101,9 +102,9 @@ namespace tmg {
 
 namespace {
 
-uint64_t req_bytes(const tm_graph* g, const Plan& p, int enumerate, uint64_t cap) {
+uint64_t req_bytes(const tm_graph* g, const Plan& p, int enumerate, uint64_t cap, int chunk_roots) {
     if (!enumerate) return 0;
-    uint64_t nch = n_chunks((uint64_t)g->v.m, effective_chunk(g, p, (uint64_t)g->v.m));
+    uint64_t nch = n_chunks((uint64_t)g->v.m, chunk_roots);
     return cap * (uint64_t)p.k * 4 + chunk_buf_bytes(nch) + scan_temp_bytes(nch + 1);
 }
 
@@ -139,7 +140,7 @@ tm_status launch_batch(tm_server* s, Slot& sl) {
     // enumerate buffers (stream-ordered allocations: no device-wide sync)
     for (Req* q : sl.batch) {
         if (!q->enumerate) continue;
-        q->nch = n_chunks(m, effective_chunk(g, q->plan, m));
+        q->nch = n_chunks(m, q->chunk_roots);
         TM_CUDA(dev_malloc_async((void**)&q->match, std::max<uint64_t>(q->cap * q->plan.k * 4, 16), sl.st));
         TM_CUDA(dev_malloc_async((void**)&q->chunk, chunk_buf_bytes(q->nch), sl.st));
         TM_CUDA(dev_malloc_async(&q->scan_tmp, scan_temp_bytes(q->nch + 1), sl.st));
@@ -157,7 +158,7 @@ tm_status launch_batch(tm_server* s, Slot& sl) {
         QueryDev* qd = cs.qdev_stage() + j;
         memset(qd, 0, sizeof(QueryDev));
         qd->plan = q->plan;
-        qd->plan.tune.chunk_roots = effective_chunk(g, q->plan, m);
+        qd->plan.tune.chunk_roots = q->chunk_roots;
         qd->root_begin = 0;
         qd->root_end = m;
         qd->n_chunks = n_chunks(m, qd->plan.tune.chunk_roots);
@@ -191,7 +192,7 @@ tm_status launch_batch(tm_server* s, Slot& sl) {
         QueryDev* qd = fs.qdev_stage() + ne;
         memset(qd, 0, sizeof(QueryDev));
         qd->plan = q->plan;
-        qd->plan.tune.chunk_roots = effective_chunk(g, q->plan, m);
+        qd->plan.tune.chunk_roots = q->chunk_roots;
         qd->root_begin = 0;
         qd->root_end = m;
         qd->n_chunks = q->nch;
@@ -458,7 +459,14 @@ extern "C" tm_status tm_serve_submit(tm_server* s, tm_query* q, int enumerate, u
     r->q = q;
     r->enumerate = enumerate ? 1 : 0;
     r->cap = enumerate ? cap : 0;
-    r->need = req_bytes(s->g, r->plan, r->enumerate, r->cap);
+    // the smaller chunks of a small graph take up to eight times the chunk memory: where that is more than
+    // the server may use, the request runs with the plan's
+    r->chunk_roots = effective_chunk(s->g, r->plan, (uint64_t)s->g->v.m);
+    r->need = req_bytes(s->g, r->plan, r->enumerate, r->cap, r->chunk_roots);
+    if (r->need > s->cfg.mem_budget_bytes) {
+        r->chunk_roots = r->plan.tune.chunk_roots;
+        r->need = req_bytes(s->g, r->plan, r->enumerate, r->cap, r->chunk_roots);
+    }
     r->key = cost_key(r->plan, r->enumerate);
     TM_ENTER(s->g->device);   // the launch shape may query the device's occupancy once
     const LaunchCfg lc = search_launch_cfg(s->g, MODE_COUNT, r->plan.warp_smem, r->plan.tune.warps_per_block,

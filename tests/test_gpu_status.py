@@ -36,3 +36,29 @@ def test_timed_out_count_writes_no_rows(tmg, m):
     rows, total = oracle.Graph.from_synth(g).enumerate(mo, cap=cap)
     assert q.enumerate(out) == (cap, total, True) and total > cap
     assert np.array_equal(out.cpu().numpy(), rows)
+
+
+def test_smallest_budget_of_a_served_enumeration(tmg):
+    """A budget that holds a request's rows and its chunk counts at 64 roots a chunk admits it, also on a graph small
+    enough for smaller chunks; one byte less does not."""
+    m, cap = 77_000, 1000
+    g = synth.powerlaw_graph(5000, m, 313, span=9e6)
+    gg = tmg.Graph.from_synth(g)
+    mo = synth.cycle(3, 3600)
+    q = gg.compile(mo)
+    rows, total = oracle.Graph.from_synth(g).enumerate(mo, cap=cap)
+    nch = -(-m // 64)
+    need = cap * 3 * 4 + (nch + 2) * 8 + nch * 4 + 256         # rows, counts and list, scan scratch
+    srv = gg.serve(mem_budget_bytes=need - 1)
+    with pytest.raises(tmg.TMError) as e:
+        srv.submit(q, True, cap)
+    assert e.value.status == tmg.E_ADMISSION
+    srv.stop()
+    srv = gg.serve(mem_budget_bytes=need)
+    for _ in range(2):
+        tk = srv.submit(q, True, cap)
+        r = srv.wait(tk, 60_000)
+        assert (r.total, r.n_written) == (total, len(rows))
+        assert np.array_equal(srv.matches(r).cpu().numpy(), rows)
+        srv.release(tk)
+    srv.stop()
