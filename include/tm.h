@@ -275,15 +275,16 @@ tm_status tm_query_work(tm_graph* g, tm_query* q, void* stream, tm_work* out);
  * under a fixed memory cap or an allocator that forbids cudaMalloc after
  * start-up, plug-ins whose host framework owns every allocation).
  * Same result as tm_count_batch: the same persistent multi-query count kernel,
- * but its scratch (control block, launch records, donated-task queue) lives in
+ * but its scratch (control blocks, launch records, donated-task queue) lives in
  * one file-scope __device__ array of TM_NOALLOC_SCRATCH_BYTES bytes that every
  * GPU loading this library holds until the process exits; no cudaMalloc,
  * cudaFree or other allocating call is made.
  *   qs, nq     : compiled queries of graph g, 1 <= nq <= TM_NOALLOC_MAX_QUERIES
  *                (TM_E_INVALID beyond that, with a message naming the limit)
  *   totals_dev : device pointer uint64[nq], caller-owned; receives the counts
- * The task queue has TM_NOALLOC_TASKS slots per call: slots are not reused
- * within a call, so once a call has donated that many subtrees, further
+ * The task queue has TM_NOALLOC_TASKS slots per launch (a call makes one, or two
+ * when it mixes queries with look-ahead with others): slots are not reused
+ * within a launch, so once it has donated that many subtrees, further
  * donations stay with the donating warp (results are unchanged).
  * The launch records are staged in a static host buffer of about 60 KB (not on
  * the caller's stack); the call's own stack use is under 1 KB.

@@ -811,14 +811,16 @@ namespace tmg {
 std::vector<LaunchGroup> occupancy_groups(const tm_graph* g, Mode mode, const Plan* const* plans,
                                           const uint64_t* nch, int nq, int* order) {
     std::vector<int> grid(nq), wpb(nq);
-    std::vector<unsigned> kind(nq);            // queries that count pairs have kernel instances of their own, and so have long frames
+    // queries that count pairs have kernel instances of their own, and so have long frames; with a look-ahead one in their launch others
+    // run at its registers, shared memory and frames (two 4-edge paths over half-day windows 66 ms, 127 with one)
+    std::vector<unsigned> kind(nq);
     for (int j = 0; j < nq; ++j) {
         const Plan& p = *plans[j];
         LaunchCfg c = search_launch_cfg(g, mode, mode == MODE_FILL ? p.warp_smem_fill : p.warp_smem,
                                         p.tune.warps_per_block, plan_features(p));
         grid[j] = c.grid;
         wpb[j] = c.warps_per_block;
-        kind[j] = plan_features(p) & (FEAT_PAIRS | FEAT_LONG);
+        kind[j] = plan_features(p) & (FEAT_PAIRS | FEAT_LONG | FEAT_LOOK);
         order[j] = j;
     }
     // highest occupancy first; within a group the likely most expensive queries

@@ -14,7 +14,7 @@
 // The array is g_noalloc_scratch below: TM_NOALLOC_SCRATCH_BYTES bytes, present
 // on every GPU that loads this library until the process exits.  It holds at
 // most TM_NOALLOC_MAX_QUERIES launch records and TM_NOALLOC_TASKS task slots,
-// which one call uses up as it donates (slots are not reused within a call).
+// which one launch uses up as it donates (slots are not reused within it).
 // The launch records are staged in a file-scope host buffer (not on the
 // caller's stack, which may be small in a plug-in's threads); a mutex guards
 // it while the records are copied out.
@@ -35,22 +35,26 @@ constexpr int NOALLOC_MAX_QUERIES = TM_NOALLOC_MAX_QUERIES;
 constexpr uint64_t NOALLOC_TASKS = TM_NOALLOC_TASKS;
 
 // byte layout of the static array
+constexpr int PARTS = 2;                 // launches of a call, see below
+constexpr size_t CTRL_STRIDE = 512;      // a control block for each
 constexpr size_t OFF_CTRL = 0;
-constexpr size_t OFF_QDEV = 512;
+constexpr size_t OFF_QDEV = PARTS * CTRL_STRIDE;
 constexpr size_t OFF_READY = (OFF_QDEV + NOALLOC_MAX_QUERIES * sizeof(QueryDev) + 255) / 256 * 256;
 constexpr size_t OFF_TASKS = (OFF_READY + NOALLOC_TASKS + 255) / 256 * 256;
 constexpr size_t NOALLOC_END = OFF_TASKS + NOALLOC_TASKS * sizeof(Task);
 static_assert(NOALLOC_END <= TM_NOALLOC_SCRATCH_BYTES, "static scratch layout exceeds its stated size");
-static_assert(sizeof(Ctrl) <= OFF_QDEV, "control block overlaps the launch records");
+static_assert(sizeof(Ctrl) <= CTRL_STRIDE, "control blocks overlap");
 
 // The scratch itself.  In host code this name is only a host-side stand-in
 // for the symbol; its device address comes from cudaGetSymbolAddress below.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[TM_NOALLOC_SCRATCH_BYTES];
 
-// Host staging of the control block and launch records (about 60 KB).
+// Host staging of the control blocks and launch records (about 60 KB).
 struct Stage {
-    Ctrl ctrl;
-    unsigned char pad[OFF_QDEV - sizeof(Ctrl)];
+    struct {
+        Ctrl c;
+        unsigned char pad[CTRL_STRIDE - sizeof(Ctrl)];
+    } ctrl[PARTS];
     QueryDev q[NOALLOC_MAX_QUERIES];
 };
 Stage g_stage;
@@ -97,9 +101,6 @@ extern "C" tm_status tm_count_batch_noalloc(tm_graph* g, tm_query* const* qs, in
     tm_status s = scratch_address(g->device, &base);
     if (s != TM_OK) return s;
     const uint64_t m = (uint64_t)g->v.m;
-    int warp_smem = 16, warps = 1;
-    unsigned feat = 0;
-    uint64_t total_chunks = 0;
     for (int j = 0; j < nq; ++j)
         if (!qs[j] || query_graph(qs[j]) != g) { set_error("null or mismatched query in batch"); return TM_E_INVALID; }
     // Every call reuses the array: clear the caller's totals, then rewrite the
@@ -107,46 +108,73 @@ extern "C" tm_status tm_count_batch_noalloc(tm_graph* g, tm_query* const* qs, in
     InFlight call(st, &g->unsettled);
     TM_CUDA(cudaMemsetAsync(totals_dev, 0, (size_t)nq * sizeof(uint64_t), st));
     if (m == 0) return cudaStreamSynchronize(st) == cudaSuccess ? TM_OK : cuda_fail(cudaGetLastError(), "sync");
+    // Queries with look-ahead or long frames in a launch of their own: their instances run all of a launch at their
+    // registers, shared memory and frames, and without pairs (two 4-edge paths over half-day windows on 10M
+    // edges 66 ms, with a chorded 4-cycle in their launch 127).
+    struct Part {
+        int first, count, warp_smem, warps;
+        unsigned feat;
+        uint64_t chunks;
+    } part[PARTS];
     {
         std::lock_guard<std::mutex> lk(g_stage_mu);
-        memset(&g_stage.ctrl, 0, sizeof(Ctrl));
-        uint64_t chunk_base = 0;
-        for (int j = 0; j < nq; ++j) {
-            QueryDev& qd = g_stage.q[j];
-            memset(&qd, 0, sizeof(QueryDev));
-            query_plan(qs[j], &qd.plan);
-            qd.root_begin = 0;
-            qd.root_end = m;
-            qd.plan.tune.chunk_roots = effective_chunk(g, qd.plan, m * (uint64_t)nq);
-            qd.n_chunks = n_chunks(m, qd.plan.tune.chunk_roots);
-            qd.chunk_base = chunk_base;
-            chunk_base += qd.n_chunks;
-            qd.total = (unsigned long long*)totals_dev + j;
-            warp_smem = std::max(warp_smem, qd.plan.warp_smem);
-            warps = std::max(warps, qd.plan.tune.warps_per_block);
-            feat |= plan_features(qd.plan);
+        memset(g_stage.ctrl, 0, sizeof g_stage.ctrl);
+        int at = 0;
+        for (int p = 0; p < PARTS; ++p) {
+            Part& pt = part[p];
+            pt = Part{at, 0, 16, 1, 0u, 0};
+            for (int j = 0; j < nq && at < nq; ++j) {
+                QueryDev& qd = g_stage.q[at];
+                memset(&qd, 0, sizeof(QueryDev));
+                query_plan(qs[j], &qd.plan);
+                if (launch_part(plan_features(qd.plan)) != p) continue;
+                qd.root_begin = 0;
+                qd.root_end = m;
+                qd.plan.tune.chunk_roots = effective_chunk(g, qd.plan, m * (uint64_t)nq);
+                qd.n_chunks = n_chunks(m, qd.plan.tune.chunk_roots);
+                qd.chunk_base = pt.chunks;
+                pt.chunks += qd.n_chunks;
+                qd.total = (unsigned long long*)totals_dev + j;
+                pt.warp_smem = std::max(pt.warp_smem, qd.plan.warp_smem);
+                pt.warps = std::max(pt.warps, qd.plan.tune.warps_per_block);
+                pt.feat |= plan_features(qd.plan);
+                ++at;
+            }
+            pt.count = at - pt.first;
+            g_stage.ctrl[p].c.total_chunks = pt.chunks;
         }
-        g_stage.ctrl.total_chunks = total_chunks = chunk_base;
         // pageable source: the copy has left this buffer when the call returns
         TM_CUDA(cudaMemcpyAsync(base + OFF_CTRL, &g_stage, OFF_QDEV + (size_t)nq * sizeof(QueryDev),
                                 cudaMemcpyHostToDevice, st));
     }
-    TM_CUDA(cudaMemsetAsync(base + OFF_READY, 0, NOALLOC_TASKS, st));
-    Scratch view;                       // points into the static array; never freed
-    view.device = g->device;
-    view.head = (char*)(base + OFF_CTRL);
-    view.qcap = NOALLOC_MAX_QUERIES;
-    view.tasks = (Task*)(base + OFF_TASKS);
-    view.ready = base + OFF_READY;
-    view.task_cap = NOALLOC_TASKS;
-    s = launch_search(g, MODE_COUNT, (const QueryDev*)(base + OFF_QDEV), nq, warp_smem, warps, feat, &view, st,
-                      launch_blocks(g, search_launch_cfg(g, MODE_COUNT, warp_smem, warps, feat), total_chunks));
-    if (s != TM_OK) return s;
-    Ctrl done;
-    TM_CUDA(cudaMemcpyAsync(&done, base + OFF_CTRL, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
-    TM_CUDA(cudaStreamSynchronize(st));
+    for (int p = 0; p < PARTS; ++p) {
+        const Part& pt = part[p];
+        if (pt.count == 0) continue;
+        TM_CUDA(cudaMemsetAsync(base + OFF_READY, 0, NOALLOC_TASKS, st));
+        Scratch view;                       // points into the static array; never freed
+        view.device = g->device;
+        view.head = (char*)(base + OFF_CTRL + p * CTRL_STRIDE);
+        view.qcap = NOALLOC_MAX_QUERIES;
+        view.tasks = (Task*)(base + OFF_TASKS);
+        view.ready = base + OFF_READY;
+        view.task_cap = NOALLOC_TASKS;
+        s = launch_search(g, MODE_COUNT, (const QueryDev*)(base + OFF_QDEV) + pt.first, pt.count, pt.warp_smem, pt.warps,
+                          pt.feat, &view, st,
+                          launch_blocks(g, search_launch_cfg(g, MODE_COUNT, pt.warp_smem, pt.warps, pt.feat), pt.chunks));
+        if (s != TM_OK) return s;
+    }
+    Ctrl done, sum;
+    memset(&sum, 0, sizeof sum);
+    for (int p = 0; p < PARTS; ++p) {
+        if (part[p].count == 0) continue;
+        TM_CUDA(cudaMemcpyAsync(&done, base + OFF_CTRL + p * CTRL_STRIDE, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
+        TM_CUDA(cudaStreamSynchronize(st));
+        sum.donated += done.donated;
+        sum.q_reserve += done.q_reserve;
+        sum.err |= done.err;
+    }
     call.settle();
-    note_search_stats(done);
-    if (done.err) { set_error("a bounded device wait timed out"); return TM_E_TIMEOUT; }
+    note_search_stats(sum);
+    if (sum.err) { set_error("a bounded device wait timed out"); return TM_E_TIMEOUT; }
     return TM_OK;
 }

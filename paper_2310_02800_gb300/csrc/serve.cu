@@ -72,7 +72,7 @@ struct Slot {
     cudaStream_t st_hi = nullptr, st_lo = nullptr;   // high / low priority
     cudaStream_t st = nullptr;                       // the one the current batch runs on
     cudaEvent_t start = nullptr, done = nullptr;
-    Scratch count_s, fill_s;    // staging + scratch of the two launches
+    Scratch count_s[2], fill_s[2];   // staging + scratch of the launches: one for each launch_part()
     std::vector<Req*> batch;
     bool busy = false;
 };
@@ -128,92 +128,105 @@ int launch_grid(const tm_server* s, const LaunchCfg& c, uint64_t chunks) {
     return std::min(blocks, std::max(s->g->num_sms, c.grid * pct / 100));
 }
 
+// Requests of one launch.
+struct Part {
+    std::vector<Req*> reqs;
+    int warp_smem = 16, warps = 1;
+    unsigned feat = 0;
+    uint64_t chunks = 0;
+};
+
+// Launch `mode` over the requests of pt, totals of request j to counters + j.
+tm_status launch_requests(tm_server* s, Slot& sl, Mode mode, Part& pt, Scratch& sc,
+                      const std::vector<unsigned long long*>& totals) {
+    tm_graph* g = s->g;
+    const uint64_t m = (uint64_t)g->v.m;
+    const int nq = (int)pt.reqs.size();
+    memset(sc.ctrl_stage(), 0, sizeof(Ctrl));
+    for (int j = 0; j < nq; ++j) {
+        const Req* q = pt.reqs[j];
+        QueryDev* qd = sc.qdev_stage() + j;
+        memset(qd, 0, sizeof(QueryDev));
+        qd->plan = q->plan;
+        qd->plan.tune.chunk_roots = q->chunk_roots;
+        qd->root_begin = 0;
+        qd->root_end = m;
+        qd->n_chunks = n_chunks(m, q->chunk_roots);
+        qd->chunk_base = pt.chunks;
+        pt.chunks += qd->n_chunks;
+        qd->total = totals[j];
+        if (mode == MODE_FILL) {
+            qd->chunk_off = q->chunk;
+            qd->match_out = q->match;
+            qd->cap = q->cap;
+        } else {
+            qd->chunk_cnt = q->enumerate ? q->chunk : nullptr;
+        }
+        pt.warp_smem = std::max(pt.warp_smem, mode == MODE_FILL ? q->plan.warp_smem_fill : q->plan.warp_smem);
+        pt.warps = std::max(pt.warps, q->plan.tune.warps_per_block);
+        pt.feat |= plan_features(q->plan);
+    }
+    sc.ctrl_stage()->total_chunks = pt.chunks;
+    TM_CUDA(cudaMemcpyAsync(sc.head, sc.stage, sc.head_bytes(nq), cudaMemcpyHostToDevice, sl.st));
+    if (mode == MODE_COUNT) TM_CUDA(cudaMemsetAsync(sc.ready, 0, sc.task_cap, sl.st));
+    const LaunchCfg lc = search_launch_cfg(g, mode, pt.warp_smem, pt.warps, pt.feat);
+    return launch_search(g, mode, sc.qdev(), nq, pt.warp_smem, pt.warps, pt.feat, &sc, sl.st, launch_grid(s, lc, pt.chunks));
+}
+
 tm_status launch_batch(tm_server* s, Slot& sl) {
     tm_graph* g = s->g;
     const int nq = (int)sl.batch.size();
-    const uint64_t m = (uint64_t)g->v.m;
     TM_CUDA(cudaEventRecord(sl.start, sl.st));
-    tm_status r = scratch_reserve(&sl.count_s, g->device, nq, (uint64_t)nq, 0, 1u << 18);
-    if (r != TM_OK) return r;
-    r = scratch_reserve(&sl.fill_s, g->device, nq, (uint64_t)nq, 0, 0);
-    if (r != TM_OK) return r;
+    // requests with look-ahead or long frames have launches of their own: in one with others these run at their
+    // registers, shared memory and frames, up to twice as long
+    Part count[2], fill[2];
+    std::vector<unsigned long long*> totals[2];
+    for (Req* q : sl.batch) {
+        const int p = launch_part(plan_features(q->plan));
+        count[p].reqs.push_back(q);
+        if (q->enumerate) fill[p].reqs.push_back(q);
+    }
+    for (int p = 0; p < 2; ++p) {
+        // the first scratch's counters hold every request's total
+        if (p == 0 || !count[p].reqs.empty()) {
+            tm_status r = scratch_reserve(&sl.count_s[p], g->device, nq, (uint64_t)nq, 0, count[p].reqs.empty() ? 0 : 1u << 18);
+            if (r == TM_OK) r = scratch_reserve(&sl.fill_s[p], g->device, nq, (uint64_t)nq, 0, 0);
+            if (r != TM_OK) return r;
+        }
+        if (sl.count_s[p].stage) memset(sl.count_s[p].ctrl_stage(), 0, sizeof(Ctrl));
+    }
+    for (int j = 0; j < nq; ++j)
+        totals[launch_part(plan_features(sl.batch[j]->plan))].push_back(sl.count_s[0].counters + j);
     // enumerate buffers (stream-ordered allocations: no device-wide sync)
     for (Req* q : sl.batch) {
         if (!q->enumerate) continue;
-        q->nch = n_chunks(m, q->chunk_roots);
+        q->nch = n_chunks((uint64_t)g->v.m, q->chunk_roots);
         TM_CUDA(dev_malloc_async((void**)&q->match, std::max<uint64_t>(q->cap * q->plan.k * 4, 16), sl.st));
         TM_CUDA(dev_malloc_async((void**)&q->chunk, chunk_buf_bytes(q->nch), sl.st));
         TM_CUDA(dev_malloc_async(&q->scan_tmp, scan_temp_bytes(q->nch + 1), sl.st));
         TM_CUDA(cudaMemsetAsync(q->chunk, 0, (q->nch + 2) * 8, sl.st));   // counts + list length
     }
-    // count launch over every request of the batch
-    Scratch& cs = sl.count_s;
-    Ctrl* c = cs.ctrl_stage();
-    memset(c, 0, sizeof(Ctrl));
-    uint64_t base = 0;
-    int warp_smem = 16, warps = 1;
-    unsigned feat = 0, ffeat = 0;
-    for (int j = 0; j < nq; ++j) {
-        Req* q = sl.batch[j];
-        QueryDev* qd = cs.qdev_stage() + j;
-        memset(qd, 0, sizeof(QueryDev));
-        qd->plan = q->plan;
-        qd->plan.tune.chunk_roots = q->chunk_roots;
-        qd->root_begin = 0;
-        qd->root_end = m;
-        qd->n_chunks = n_chunks(m, qd->plan.tune.chunk_roots);
-        qd->chunk_base = base;
-        base += qd->n_chunks;
-        qd->total = cs.counters + j;
-        qd->chunk_cnt = q->enumerate ? q->chunk : nullptr;
-        warp_smem = std::max(warp_smem, q->plan.warp_smem);
-        warps = std::max(warps, q->plan.tune.warps_per_block);
-        feat |= plan_features(q->plan);
-        if (q->enumerate) ffeat |= plan_features(q->plan);
-    }
-    c->total_chunks = base;
-    TM_CUDA(cudaMemcpyAsync(cs.head, cs.stage, cs.head_bytes(nq), cudaMemcpyHostToDevice, sl.st));
-    TM_CUDA(cudaMemsetAsync(cs.counters, 0, (size_t)nq * 8, sl.st));
-    TM_CUDA(cudaMemsetAsync(cs.ready, 0, cs.task_cap, sl.st));
-    LaunchCfg lc = search_launch_cfg(g, MODE_COUNT, warp_smem, warps, feat);
-    r = launch_search(g, MODE_COUNT, cs.qdev(), nq, warp_smem, warps, feat, &cs, sl.st, launch_grid(s, lc, base));
-    if (r != TM_OK) return r;
-    // fill launch over the enumerate requests
-    int ne = 0;
-    Scratch& fs = sl.fill_s;
-    Ctrl* fc = fs.ctrl_stage();
-    memset(fc, 0, sizeof(Ctrl));
-    uint64_t fbase = 0;
-    int fsmem = 16;
-    for (Req* q : sl.batch) {
-        if (!q->enumerate) continue;
-        r = chunk_offsets(q->chunk, q->nch, q->cap, cs.ctrl(), q->scan_tmp, g->num_sms, sl.st);
-        if (r != TM_OK) return r;
-        QueryDev* qd = fs.qdev_stage() + ne;
-        memset(qd, 0, sizeof(QueryDev));
-        qd->plan = q->plan;
-        qd->plan.tune.chunk_roots = q->chunk_roots;
-        qd->root_begin = 0;
-        qd->root_end = m;
-        qd->n_chunks = q->nch;
-        qd->chunk_base = fbase;
-        fbase += q->nch;
-        qd->total = fs.counters + ne;
-        qd->chunk_off = q->chunk;
-        qd->match_out = q->match;
-        qd->cap = q->cap;
-        fsmem = std::max(fsmem, q->plan.warp_smem_fill);
-        ++ne;
-    }
-    if (ne > 0) {
-        fc->total_chunks = fbase;
-        TM_CUDA(cudaMemcpyAsync(fs.head, fs.stage, fs.head_bytes(ne), cudaMemcpyHostToDevice, sl.st));
-        LaunchCfg lf = search_launch_cfg(g, MODE_FILL, fsmem, warps, ffeat);
-        r = launch_search(g, MODE_FILL, fs.qdev(), ne, fsmem, warps, ffeat, &fs, sl.st, launch_grid(s, lf, fbase));
+    TM_CUDA(cudaMemsetAsync(sl.count_s[0].counters, 0, (size_t)nq * 8, sl.st));
+    for (int p = 0; p < 2; ++p) {
+        if (count[p].reqs.empty()) continue;
+        const tm_status r = launch_requests(s, sl, MODE_COUNT, count[p], sl.count_s[p], totals[p]);
         if (r != TM_OK) return r;
     }
-    TM_CUDA(cudaMemcpyAsync(cs.counters_host, cs.counters, (size_t)nq * 8, cudaMemcpyDeviceToHost, sl.st));
-    TM_CUDA(cudaMemcpyAsync(cs.stage, cs.head, sizeof(Ctrl), cudaMemcpyDeviceToHost, sl.st));
+    for (int p = 0; p < 2; ++p) {
+        if (fill[p].reqs.empty()) continue;
+        std::vector<unsigned long long*> unused;
+        for (Req* q : fill[p].reqs) {
+            const tm_status r = chunk_offsets(q->chunk, q->nch, q->cap, sl.count_s[p].ctrl(), q->scan_tmp, g->num_sms, sl.st);
+            if (r != TM_OK) return r;
+            unused.push_back(sl.fill_s[p].counters + unused.size());
+        }
+        const tm_status r = launch_requests(s, sl, MODE_FILL, fill[p], sl.fill_s[p], unused);
+        if (r != TM_OK) return r;
+    }
+    TM_CUDA(cudaMemcpyAsync(sl.count_s[0].counters_host, sl.count_s[0].counters, (size_t)nq * 8, cudaMemcpyDeviceToHost, sl.st));
+    for (int p = 0; p < 2; ++p)
+        if (!count[p].reqs.empty())
+            TM_CUDA(cudaMemcpyAsync(sl.count_s[p].stage, sl.count_s[p].head, sizeof(Ctrl), cudaMemcpyDeviceToHost, sl.st));
     for (Req* q : sl.batch) {
         if (!q->enumerate) continue;
         TM_CUDA(cudaFreeAsync(q->chunk, sl.st));
@@ -253,7 +266,8 @@ void learn(tm_server* s, Slot& sl) {
 
 void finish_batch(tm_server* s, Slot& sl, tm_status launch_status) {
     // caller holds s->mu
-    bool timeout = launch_status == TM_OK && sl.count_s.ctrl_stage()->err != 0;
+    bool timeout = false;
+    for (const Scratch& c : sl.count_s) timeout = timeout || (launch_status == TM_OK && c.stage && c.ctrl_stage()->err != 0);
     if (launch_status == TM_OK && !timeout) learn(s, sl);
     auto now = clk::now();
     for (size_t j = 0; j < sl.batch.size(); ++j) {
@@ -264,7 +278,7 @@ void finish_batch(tm_server* s, Slot& sl, tm_status launch_status) {
         } else if (timeout) {
             q->status = TM_E_TIMEOUT;
         } else {
-            q->total = sl.count_s.counters_host[j];
+            q->total = sl.count_s[0].counters_host[j];
             q->n_written = q->enumerate ? std::min(q->total, q->cap) : 0;
             q->status = (q->enumerate && q->total > q->cap) ? TM_E_TRUNCATED : TM_OK;
         }
@@ -390,8 +404,10 @@ void scheduler(tm_server* s) {
 
 void destroy_slots(tm_server* s) {
     for (Slot& sl : s->slots) {
-        scratch_free(&sl.count_s, false);
-        scratch_free(&sl.fill_s, false);
+        for (int p = 0; p < 2; ++p) {
+            scratch_free(&sl.count_s[p], false);
+            scratch_free(&sl.fill_s[p], false);
+        }
         if (sl.start) cudaEventDestroy(sl.start);
         if (sl.done) cudaEventDestroy(sl.done);
         if (sl.st_hi) cudaStreamDestroy(sl.st_hi);

@@ -291,6 +291,10 @@ inline unsigned plan_features(const Plan& p) {
     return f;
 }
 
+// Launches that take queries of any kind (served batches, the call without allocation) keep two sorts apart: 1 for
+// queries with look-ahead or long frames, whose instances cost the others more than a launch.
+inline int launch_part(unsigned feat) { return feat & (FEAT_LOOK | FEAT_LONG) ? 1 : 0; }
+
 // Frame field offsets (bytes, relative to frame start), CAP entries each.
 //   tprev i64, tend - tprev u32 (0xFFFFFFFF when it does not fit: t_root + delta is
 //   then rebuilt from the root edge), beg u32 (bits 31/30: list kind), len u32, root u32,

@@ -1,0 +1,89 @@
+"""Queries whose kernel instances cost others more than a launch, in calls that mix them."""
+import statistics
+
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def tmg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2310_02800_gb300 as m
+    m.lib()
+    return m
+
+
+def path(k, delta):
+    return synth.Motif([(i, i + 1) for i in range(k)], delta)
+
+
+def test_look_ahead_beside_long_paths(tmg):
+    """Two 4-edge paths over long windows and a chorded 4-cycle, counted without allocation and as a batch: together
+    they take what they take apart (a fifth allowed; in one launch they took nearly twice that)."""
+    g = synth.powerlaw_graph(100_000, 1_000_000, 77, span=9_460_800.0)
+    gg = tmg.Graph.from_synth(g)
+    paths = [gg.compile(path(4, d)) for d in (54_000, 40_000)]
+    chord = [gg.compile(synth.chorded_four_cycle(600))]
+
+    def noalloc(qs):
+        tot = torch.zeros(len(qs), dtype=torch.int64, device="cuda")
+        return lambda: gg.count_batch_noalloc(qs, tot).tolist()
+
+    def ms(fn, n=9):
+        got = []
+        for _ in range(n):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            fn()
+            b.record()
+            b.synchronize()
+            got.append(a.elapsed_time(b))
+        return statistics.median(got)
+
+    want = [q.count() for q in paths + chord]
+    for call in (noalloc, lambda qs: lambda: gg.count_batch(qs)):
+        assert call(paths + chord)() == want and call(chord + paths)() == want[2:] + want[:2]
+        apart = ms(call(paths)) + ms(call(chord))
+        assert ms(call(paths + chord)) < 1.2 * apart
+
+
+def test_served_batches_of_either_sort_and_both(tmg):
+    """One server whose batches hold queries with look-ahead, without, and both, in arrival order and by cost: totals
+    and rows against the oracle."""
+    g = synth.powerlaw_graph(3000, 40_000, 93, span=9.46 * 40_000)
+    og = oracle.Graph.from_synth(g)
+    gg = tmg.Graph.from_synth(g)
+    d = 10_000
+    M = synth.Motif
+    plain = [synth.cycle(3, d), path(3, d), synth.out_star(3, d // 10), M([(0, 1), (1, 2), (2, 0)], d, anti=[(1, 0, 0, d // 4)])]
+    look = [synth.chorded_four_cycle(d), M([(0, 1), (1, 2), (2, 3), (0, 2)], d), M([(0, 1), (1, 2), (2, 3), (0, 2)], d, anti=[(2, 1, 1, d // 2)])]
+    blocker = gg.compile(path(4, 3 * d))
+    block_total = blocker.count()
+    rows = {}
+    for policy in (1, 0):
+        srv = gg.serve(mem_budget_bytes=1 << 30, streams=1, max_batch=16, policy=policy)
+        for mix in (plain, look, plain + look, look, plain[:1] + look[:1], plain):
+            held = srv.submit(blocker)                     # the rest queue behind it and go as batches
+            reqs = []
+            for j, mo in enumerate(mix + mix):
+                q = gg.compile(mo)
+                key = repr(mo)
+                if key not in rows:
+                    rows[key] = og.enumerate(mo, cap=5_000)
+                reqs.append((q, rows[key], j % 2 == 0, srv.submit(q, j % 2 == 0, 5_000 if j % 2 == 0 else 0)))
+            assert srv.wait(held, 60_000).total == block_total
+            srv.release(held)
+            for q, (want, total), listed, tk in reqs:
+                r = srv.wait(tk, 60_000)
+                assert r.total == total
+                if listed:
+                    assert np.array_equal(srv.matches(r).cpu().numpy(), want)
+                srv.release(tk)
+        srv.stop()
