@@ -154,7 +154,8 @@ tm_status tm_graph_free(tm_graph* g);
 /* Sizes of a loaded graph (any pointer may be NULL). */
 tm_status tm_graph_info(const tm_graph* g, int64_t* n_nodes, int64_t* n_edges, uint64_t* device_bytes);
 
-/* Edge id -> input index.  out_perm: int64[n_edges], host pointer. */
+/* Edge id -> input index.  out_perm: int64[n_edges], host pointer.  Uses 8 bytes of device memory per edge
+ * while it runs; without them it widens the ids on the host. */
 tm_status tm_graph_edge_perm(const tm_graph* g, int64_t* out_perm);
 
 /* Validate a motif against a graph and build its search plan (Section 5.1.2:
@@ -244,7 +245,8 @@ tm_status tm_query_inject_fault(tm_query* q, int kind);
  * GPU fault): the device or pinned-host allocation that this library makes
  * after `after` further successful ones fails as if the device were out of
  * memory, and the call that made it returns TM_E_OOM with its outputs
- * untouched (a served request completes with status TM_E_OOM).  Process-wide;
+ * untouched (a served request completes with status TM_E_OOM, and
+ * tm_graph_edge_perm goes on without the allocation).  Process-wide;
  * one failure per arming; after < 0 disarms.  Every later call is unaffected. */
 tm_status tm_inject_alloc_failure(int64_t after);
 

@@ -9,6 +9,8 @@
 //   5. out-lists re-ordered by (neighbour, time): closing-edge lookups
 //   6. successor index: per edge, the first later position in its four lists; root filter
 #include <cuda_runtime.h>
+#include <sys/mman.h>
+#include <unistd.h>
 
 #include <algorithm>
 
@@ -270,7 +272,20 @@ __global__ void root_codes_kernel(int64_t m, const uint4* __restrict__ by_out, c
 __global__ void widen_kernel(const int32_t* __restrict__ in, int64_t n, int64_t* __restrict__ out) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) out[i] = in[i];
 }
-constexpr int64_t PERM_PART = 1 << 22;        // 32 MB of device memory
+
+// Pages that the caller never touched are slow to fault in from the device (5.7M ids into fresh memory took 11 ms,
+// with each page touched first 1.9): have them present, with their contents as they are.
+void populate(void* p, size_t bytes) {
+    char* const end = (char*)p + bytes;
+    const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+    char* from = (char*)((uintptr_t)p & ~(uintptr_t)(page - 1));
+#ifdef MADV_POPULATE_WRITE
+    if (madvise(from, (size_t)(end - from), MADV_POPULATE_WRITE) == 0) return;
+#endif
+    // (a kernel without it, or memory it does not take) a read-modify-write of a byte of each
+    for (char* b = (char*)p; b < end; b += page) __atomic_fetch_or(b, 0, __ATOMIC_RELAXED);
+    __atomic_fetch_or(end - 1, 0, __ATOMIC_RELAXED);
+}
 
 int bits_for(unsigned long long x) {
     int b = 0;
@@ -666,24 +681,19 @@ extern "C" tm_status tm_graph_edge_perm(const tm_graph* g, int64_t* out_perm) {
     if (!g || (!out_perm && g->v.m > 0)) { set_error("null argument"); return TM_E_INVALID; }
     if (g->v.m == 0) return TM_OK;
     TM_ENTER(g->device);
-    // widened on the device and copied straight out, PERM_PART ids at a time
-    const int64_t m = g->v.m, part = std::min(m, PERM_PART);
+    // widened on the device, all of it before any is copied, and copied straight out
+    const int64_t m = g->v.m;
     int64_t* wide = nullptr;
-    if (dev_malloc((void**)&wide, part * 8) == cudaSuccess) {
-        cudaError_t e = cudaSuccess;
-        for (int64_t i = 0; i < m && e == cudaSuccess; i += part) {
-            const int64_t n = std::min(part, m - i);
-            widen_kernel<<<grid_for(n, g->num_sms), 256>>>(g->perm + i, n, wide);
-            note_launches(1);
-            e = cudaGetLastError();
-            // pages that the caller never touched are slow to fault in from the device: 5.7M ids into fresh memory
-            // took 11 ms, with a byte of each page written first 1.9
-            volatile char* to = (volatile char*)(out_perm + i);
-            for (int64_t b = 0; b < n * 8; b += 4096) to[b] = 0;
-            to[n * 8 - 1] = 0;
-            if (e == cudaSuccess) e = cudaMemcpy(out_perm + i, wide, n * 8, cudaMemcpyDeviceToHost);
+    if (dev_malloc((void**)&wide, (size_t)m * 8) == cudaSuccess) {
+        widen_kernel<<<grid_for(m, g->num_sms), 256>>>(g->perm, m, wide);
+        note_launches(1);
+        cudaError_t e = cudaGetLastError();
+        const bool launched = e == cudaSuccess;
+        if (launched) {
+            populate(out_perm, (size_t)m * 8);
+            e = cudaMemcpy(out_perm, wide, (size_t)m * 8, cudaMemcpyDeviceToHost);
         }
-        dev_free(wide, g->device, e == cudaSuccess);
+        dev_free(wide, g->device, !launched || e == cudaSuccess);
         return e == cudaSuccess ? TM_OK : cuda_fail(e, "edge permutation");
     }
     // no device memory to spare: through a host copy

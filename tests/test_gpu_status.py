@@ -62,3 +62,30 @@ def test_smallest_budget_of_a_served_enumeration(tmg):
         assert np.array_equal(srv.matches(r).cpu().numpy(), rows)
         srv.release(tk)
     srv.stop()
+
+
+def test_failed_edge_permutation_leaves_its_array(tmg):
+    """A permutation asked for while a blocking stream is being captured, which the legacy stream it runs on must not
+    join: the CUDA error's status, the array as it was, and a right next call."""
+    import ctypes
+    rt = ctypes.CDLL("libcudart.so.13")
+    n, m = 1000, 30_000
+    rng = np.random.default_rng(2)
+    t = rng.integers(0, 5000, m).astype(np.int64)
+    gg = tmg.Graph.load(n, rng.integers(0, n, m).astype(np.int32), rng.integers(0, n, m).astype(np.int32), t)
+    gg.edge_perm()
+    torch.cuda.synchronize()
+    st, graph = ctypes.c_void_p(), ctypes.c_void_p()
+    assert rt.cudaStreamCreate(ctypes.byref(st)) == 0
+    assert rt.cudaStreamBeginCapture(st, 2) == 0                   # cudaStreamCaptureModeRelaxed
+    keep = 0x7777_7777_7777_7777
+    out = np.full(m, keep, np.int64)
+    status = tmg.lib().tm_graph_edge_perm(gg._h, out.ctypes.data)
+    rt.cudaStreamEndCapture(st, ctypes.byref(graph))
+    if graph.value:
+        rt.cudaGraphDestroy(graph)
+    rt.cudaStreamDestroy(st)
+    rt.cudaGetLastError()
+    assert status == tmg.E_CUDA
+    assert (out == keep).all()
+    assert np.array_equal(gg.edge_perm(), np.argsort(t, kind="stable"))
