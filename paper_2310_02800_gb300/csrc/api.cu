@@ -68,7 +68,8 @@ static std::mutex g_pool_mu;
 
 // The device's pool, made on first use (the device is current, g_pool_mu held).
 static cudaError_t dev_pool(int device, DevPool** out) {
-    static std::map<int, DevPool> per_device;
+    // never destroyed: graphs and batch buffers that the program left alive are freed after static objects are
+    static std::map<int, DevPool>& per_device = *new std::map<int, DevPool>();
     DevPool& d = per_device[device];
     if (!d.pool) {
         cudaMemPoolProps props;

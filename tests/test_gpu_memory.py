@@ -146,3 +146,27 @@ def test_freed_memory_is_kept_and_given_back(tmg):
     assert rt.cudaMemPoolGetAttribute(pool, 4, ctypes.byref(thr)) == 0 and thr.value == 12_345
     thr.value = 0
     rt.cudaMemPoolSetAttribute(pool, 4, ctypes.byref(thr))
+
+
+def test_process_ends_with_everything_alive(tmp_path):
+    """A program that ends without freeing its graph, queries, batch buffers and server ends in order."""
+    import subprocess
+    import sys
+    code = """
+import torch, synth, paper_2310_02800_gb300 as tmg
+for c in (tmg.Graph, tmg.Query):
+    c.free = lambda self: None
+tmg.Server.stop = lambda self: None
+g = synth.powerlaw_graph(2000, 20_000, 3, span=2e5)
+keep = []
+for _ in range(3):
+    gg = tmg.Graph.from_synth(g)
+    qs = [gg.compile(synth.cycle(k, 3600)) for k in (3, 4)]
+    keep.append((gg, qs, gg.count_batch(qs), [q.count() for q in qs]))
+    assert keep[-1][2] == keep[-1][3]
+print("done", flush=True)
+"""
+    import os
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout == "done\n" and not r.stderr, (r.returncode, r.stdout, r.stderr)
