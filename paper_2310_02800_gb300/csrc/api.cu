@@ -26,9 +26,9 @@ void note_launches(uint64_t n) { g_launches.fetch_add(n, std::memory_order_relax
 
 void set_error(const std::string& msg) { g_last_error = msg; }
 
-void note_search_stats(const Ctrl& c) {
-    g_last_donated = c.donated;
-    g_last_reserved = c.q_reserve;
+void note_search_stats(uint64_t donated, uint64_t reserved) {
+    g_last_donated = donated;
+    g_last_reserved = reserved;
 }
 
 // Allocations left before an injected failure (-1: none armed).
@@ -633,7 +633,7 @@ static tm_status read_back(Scratch& s, cudaStream_t st) {
     TM_CUDA(cudaMemcpyAsync(s.counters_host, s.counters, SINGLE_WORDS * 8, cudaMemcpyDeviceToHost, st));
     TM_CUDA(cudaStreamSynchronize(st));
     const Ctrl *c = (const Ctrl*)s.counters_host, *f = (const Ctrl*)(s.counters_host + CTRL_WORDS);
-    note_search_stats(*c);
+    note_search_stats(c->donated, c->q_reserve);
     if (c->err || f->err) {
         set_error("a bounded device wait timed out");
         return TM_E_TIMEOUT;
@@ -1033,7 +1033,7 @@ extern "C" tm_status tm_count_batch(tm_graph* g, tm_query* const* qs, int nq, vo
         sum.q_reserve += c.q_reserve;
         sum.err |= c.err;
     }
-    note_search_stats(sum);
+    note_search_stats(sum.donated, sum.q_reserve);
     if (sum.err) { set_error("a bounded device wait timed out"); return TM_E_TIMEOUT; }
     for (int j = 0; j < nq; ++j) totals[j] = b->counters_host[j];
     return TM_OK;
@@ -1195,7 +1195,7 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
         sum.err |= c.err;
     }
     for (size_t gi = 0; bf && gi < bf->groups.size(); ++gi) sum.err |= ((const Ctrl*)bf->stage)[gi].err;
-    note_search_stats(sum);
+    note_search_stats(sum.donated, sum.q_reserve);
     if (sum.err) { set_error("a bounded device wait timed out"); return TM_E_TIMEOUT; }
     if (kernel_ms) {
         float a = 0.f, b = 0.f;

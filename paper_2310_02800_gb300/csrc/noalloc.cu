@@ -60,6 +60,15 @@ struct Stage {
 Stage g_stage;
 std::mutex g_stage_mu;
 
+// What a call reads back of each control block.
+struct Outcome {
+    unsigned long long q_reserve, q_head;
+    int pad, idle;
+    unsigned err, donated;
+};
+static_assert(offsetof(Ctrl, err) - offsetof(Ctrl, q_reserve) == offsetof(Outcome, err) &&
+              offsetof(Ctrl, donated) - offsetof(Ctrl, q_reserve) == offsetof(Outcome, donated), "control block layout");
+
 constexpr int MAX_DEVICES = 64;
 std::mutex g_setup_mu;
 unsigned char* g_scratch_dev[MAX_DEVICES] = {nullptr};
@@ -163,18 +172,12 @@ extern "C" tm_status tm_count_batch_noalloc(tm_graph* g, tm_query* const* qs, in
                           launch_blocks(g, search_launch_cfg(g, MODE_COUNT, pt.warp_smem, pt.warps, pt.feat), pt.chunks));
         if (s != TM_OK) return s;
     }
-    Ctrl done, sum;
-    memset(&sum, 0, sizeof sum);
-    for (int p = 0; p < PARTS; ++p) {
-        if (part[p].count == 0) continue;
-        TM_CUDA(cudaMemcpyAsync(&done, base + OFF_CTRL + p * CTRL_STRIDE, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));
-        TM_CUDA(cudaStreamSynchronize(st));
-        sum.donated += done.donated;
-        sum.q_reserve += done.q_reserve;
-        sum.err |= done.err;
-    }
+    Outcome done[PARTS];                // of a launch not made: as staged, nothing
+    TM_CUDA(cudaMemcpy2DAsync(done, sizeof(Outcome), base + OFF_CTRL + offsetof(Ctrl, q_reserve), CTRL_STRIDE, sizeof(Outcome), PARTS,
+                              cudaMemcpyDeviceToHost, st));
+    TM_CUDA(cudaStreamSynchronize(st));
     call.settle();
-    note_search_stats(sum);
-    if (sum.err) { set_error("a bounded device wait timed out"); return TM_E_TIMEOUT; }
+    note_search_stats((uint64_t)done[0].donated + done[1].donated, done[0].q_reserve + done[1].q_reserve);
+    if (done[0].err || done[1].err) { set_error("a bounded device wait timed out"); return TM_E_TIMEOUT; }
     return TM_OK;
 }

@@ -422,7 +422,7 @@ void drop_batches(const tm_graph* g);
 
 // Record the donation counters of a finished count-mode launch for
 // tm_last_search_stats (per calling thread).
-void note_search_stats(const Ctrl& c);
+void note_search_stats(uint64_t donated, uint64_t reserved);
 
 // The query's plan with the graph's cached tuning for its shape applied.
 void query_plan(tm_query* q, Plan* out);

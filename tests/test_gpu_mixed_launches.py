@@ -87,3 +87,27 @@ def test_served_batches_of_either_sort_and_both(tmg):
                     assert np.array_equal(srv.matches(r).cpu().numpy(), want)
                 srv.release(tk)
         srv.stop()
+
+
+def test_queries_of_every_kind_without_allocation(tmg):
+    """40 queries of every kind, in several orders and subsets: the call without allocation returns the batch's totals
+    and the single calls', each in its place."""
+    g = synth.powerlaw_graph(6_000, 60_000, 5, span=9.46 * 60_000, n_labels=4)
+    g.nlabel = synth.node_labels(g.n_nodes, 2, 7)
+    gg = tmg.Graph.from_synth(g)
+    M, d = synth.Motif, 3_600
+    mos = [M([(0, 1)], 0), path(2, d), M([(0, 1), (2, 3)], 36), synth.cycle(5, d), M([(0, 1), (1, 2), (2, 0)], d, [d // 4, d // 4]),
+           M([(i % 2, 1 - i % 2) for i in range(8)], d), synth.in_star(3, d // 10), synth.out_star(4, d // 4), path(6, d // 2), path(7, d // 3),
+           M([(0, 1), (1, 2), (2, 0)], d, anti=[(1, 0, 0, d // 4)]), M([(0, 1), (1, 2), (2, 3)], d, anti=[(0, 2, 1, d // 4), (1, 0, 0, d)]),
+           synth.chorded_four_cycle(d), M([(0, 1), (1, 2), (2, 3), (0, 2)], d), M([(0, 1), (1, 2), (2, 3), (0, 2)], d, anti=[(2, 1, 1, d // 2)]),
+           M([(0, 1), (0, 2), (3, 1), (3, 2)], d), M([(0, 1), (1, 2), (1, 3), (1, 4)], d // 4),
+           M([(0, 1), (1, 2), (2, 3), (3, 4)], d, elabel=[1, -1, 2, -1])]
+    rng = np.random.default_rng(4)
+    qs = [gg.compile(mos[j]) for j in rng.integers(0, len(mos), 40)]
+    qs[7].set_tuning(2, 64, 1, 512)
+    qs[21].set_tuning(8, 32, 2, 512)
+    want = [q.count() for q in qs]
+    for pick in (range(40), range(39, -1, -1), [0], [12], range(5, 9), range(0, 40, 3)):
+        sub = [qs[j] for j in pick]
+        tot = torch.full((len(sub),), -1, dtype=torch.int64, device="cuda")
+        assert gg.count_batch_noalloc(sub, tot).tolist() == gg.count_batch(sub) == [want[j] for j in pick]
