@@ -155,7 +155,7 @@ tm_status tm_graph_free(tm_graph* g);
 tm_status tm_graph_info(const tm_graph* g, int64_t* n_nodes, int64_t* n_edges, uint64_t* device_bytes);
 
 /* Edge id -> input index.  out_perm: int64[n_edges], host pointer.  Uses 8 bytes of device memory per edge
- * while it runs; without them it widens the ids on the host. */
+ * while it runs; without them, and for few edges, it widens the ids on the host. */
 tm_status tm_graph_edge_perm(const tm_graph* g, int64_t* out_perm);
 
 /* Validate a motif against a graph and build its search plan (Section 5.1.2:

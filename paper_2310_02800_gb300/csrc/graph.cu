@@ -273,6 +273,10 @@ __global__ void widen_kernel(const int32_t* __restrict__ in, int64_t n, int64_t*
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) out[i] = in[i];
 }
 
+// Permutations of this many ids are widened on the host: 5,000 take 13 us there and 19 by the device's allocation,
+// launch and free, 32,000 19 and 20, 64,000 37 and 21.
+constexpr int64_t PERM_HOST = 1 << 15;
+
 // Pages that the caller never touched are slow to fault in from the device (5.7M ids into fresh memory took 11 ms,
 // with each page touched first 1.9): have them present, with their contents as they are.
 void populate(void* p, size_t bytes) {
@@ -681,10 +685,11 @@ extern "C" tm_status tm_graph_edge_perm(const tm_graph* g, int64_t* out_perm) {
     if (!g || (!out_perm && g->v.m > 0)) { set_error("null argument"); return TM_E_INVALID; }
     if (g->v.m == 0) return TM_OK;
     TM_ENTER(g->device);
-    // widened on the device, all of it before any is copied, and copied straight out
+    // widened on the device, all of it before any is copied, and copied straight out; up to PERM_HOST ids
+    // through the host copy below
     const int64_t m = g->v.m;
     int64_t* wide = nullptr;
-    if (dev_malloc((void**)&wide, (size_t)m * 8) == cudaSuccess) {
+    if (m > PERM_HOST && dev_malloc((void**)&wide, (size_t)m * 8) == cudaSuccess) {
         widen_kernel<<<grid_for(m, g->num_sms), 256>>>(g->perm, m, wide);
         note_launches(1);
         cudaError_t e = cudaGetLastError();
@@ -696,7 +701,7 @@ extern "C" tm_status tm_graph_edge_perm(const tm_graph* g, int64_t* out_perm) {
         dev_free(wide, g->device, !launched || e == cudaSuccess);
         return e == cudaSuccess ? TM_OK : cuda_fail(e, "edge permutation");
     }
-    // no device memory to spare: through a host copy
+    // few ids, or no device memory to spare
     cudaGetLastError();
     std::vector<int32_t> tmp((size_t)m);
     TM_CUDA(cudaMemcpy(tmp.data(), g->perm, m * 4, cudaMemcpyDeviceToHost));

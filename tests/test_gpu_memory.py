@@ -170,3 +170,17 @@ print("done", flush=True)
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and r.stdout == "done\n" and not r.stderr, (r.returncode, r.stdout, r.stderr)
+
+
+@pytest.mark.parametrize("m", [1, 5_000, 32_767, 32_768, 32_769, 60_000])
+def test_permutation_of_few_edges(tmg, m):
+    """Around the size from which ids are widened on the device: the permutation, and one that finds no device memory."""
+    rng = np.random.default_rng(m)
+    t = rng.integers(0, 1 + m // 3, m).astype(np.int64)
+    gg = tmg.Graph.load(100, rng.integers(0, 100, m).astype(np.int32), rng.integers(0, 100, m).astype(np.int32), t)
+    want = np.argsort(t, kind="stable")
+    assert np.array_equal(gg.edge_perm(), want)
+    tmg.inject_alloc_failure(0)
+    assert np.array_equal(gg.edge_perm(), want)
+    tmg.inject_alloc_failure(-1)
+    assert np.array_equal(gg.edge_perm(), want)
