@@ -12,7 +12,9 @@
  * Conventions for every call:
  *   - Every call returns tm_status; no C++ exception crosses this boundary.
  *   - On an error status, outputs are left untouched, except TM_E_TRUNCATED
- *     (non-fatal, see tm_enumerate).
+ *     (non-fatal, see tm_enumerate).  Device buffers that kernels count into
+ *     (per_root_dev, totals_dev) may have been cleared or partly counted by
+ *     then when the status is TM_E_TIMEOUT or TM_E_CUDA.
  *   - "device pointer" means memory of the graph's CUDA device (cudaMalloc,
  *     a torch CUDA tensor's data_ptr, ...); "host pointer" means pageable or
  *     pinned host memory.  Caller-owned buffers stay caller-owned.

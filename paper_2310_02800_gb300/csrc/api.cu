@@ -746,8 +746,10 @@ extern "C" tm_status tm_query_work(tm_graph* g, tm_query* q, void* stream, tm_wo
     TM_ENTER(g->device);
     apply_cached_tuning(g, q);
     cudaStream_t st = (cudaStream_t)stream;
-    memset(out, 0, sizeof *out);
-    if (g->v.m == 0) return TM_OK;
+    if (g->v.m == 0) {
+        memset(out, 0, sizeof *out);
+        return TM_OK;
+    }
     InFlight call(st, &g->unsettled, &q->unsettled);
     tm_status s = run_count(g, q, 0, (uint64_t)g->v.m, st, nullptr, false, true);
     if (s != TM_OK) return s;
@@ -1060,8 +1062,8 @@ extern "C" tm_status tm_enumerate_batch(tm_graph* g, tm_query* const* qs, int nq
     TM_ENTER(g->device);
     cudaStream_t st = (cudaStream_t)stream;
     const uint64_t m = (uint64_t)g->v.m;
-    if (kernel_ms) kernel_ms[0] = kernel_ms[1] = 0.0;
     if (m == 0) {
+        if (kernel_ms) kernel_ms[0] = kernel_ms[1] = 0.0;
         for (int j = 0; j < nq; ++j) totals[j] = n_written[j] = 0;
         return TM_OK;
     }

@@ -89,3 +89,29 @@ def test_failed_edge_permutation_leaves_its_array(tmg):
     assert status == tmg.E_CUDA
     assert (out == keep).all()
     assert np.array_equal(gg.edge_perm(), np.argsort(t, kind="stable"))
+
+
+def test_failed_calls_leave_host_outputs(tmg):
+    """Work counters after a timed-out wait, and the kernel times of a batch that runs out of memory."""
+    import ctypes
+    g = synth.powerlaw_graph(2_000, 30_000, 5, span=3e5)
+    gg = tmg.Graph.from_synth(g)
+    q = gg.compile(synth.cycle(3, 3600))
+    w = tmg._Work()
+    ctypes.memset(ctypes.byref(w), 0x55, ctypes.sizeof(w))
+    q.inject_fault(1)
+    assert tmg.lib().tm_query_work(gg._h, q._h, None, ctypes.byref(w)) == tmg.E_TIMEOUT
+    assert bytes(w) == b"\x55" * ctypes.sizeof(w)
+    assert q.work()["matches"] == q.count()
+    ms = (ctypes.c_double * 2)(7.0, 7.0)
+    q2 = gg.compile(synth.cycle(4, 3600))
+    hs, caps = (ctypes.c_void_p * 2)(q._h.value, q2._h.value), (ctypes.c_uint64 * 2)(0, 0)
+    nw, tot = (ctypes.c_uint64 * 2)(9, 9), (ctypes.c_uint64 * 2)(9, 9)
+    bufs = (ctypes.c_void_p * 2)()
+    args = (gg._h, hs, 2, None, bufs, caps, nw, tot, ms)
+    tmg.inject_alloc_failure(0)
+    assert tmg.lib().tm_enumerate_batch(*args) == tmg.E_OOM
+    tmg.inject_alloc_failure(-1)
+    assert list(ms) == [7.0, 7.0] and list(nw) == [9, 9] and list(tot) == [9, 9]
+    assert tmg.lib().tm_enumerate_batch(*args) == tmg.E_TRUNCATED
+    assert list(tot) == [q.count(), q2.count()] and list(nw) == [0, 0] and 0 < ms[0] < 1e3 and ms[1] == 0
