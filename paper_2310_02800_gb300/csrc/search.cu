@@ -1653,9 +1653,9 @@ struct Search {
     }
 };
 
-// Registers per thread of an instance.  Plain motifs of up to 4 edges: 64, which is 32 warps per SM (at 56 the
-// candidate loops spilled: 4-path over 15 h windows 21.5 ms, at 64 20.0, at 72 21.3, at
-// 80 22.1).  Where shared memory allows WIDE_WARPS warps or fewer (5 edges: 28) the registers of the others are
+// Registers per thread of an instance.  Plain motifs of up to 4 edges: 64, which is 32 warps per SM (4-path over
+// 15 h windows 21.5 ms at 56, 20.0 at 64, 21.3 at 72, 22.1 at 80; at 64 the count still stores 106
+// and loads 60 bytes of spills, fills with look-ahead 112 and 106).  Where shared memory allows WIDE_WARPS warps or fewer (5 edges: 28) the registers of the others are
 // there to take, and without spills at 80 fewer warps are faster: labelled 5-path on 20M edges
 // 344 us at 64, 313 at 72, 265 at 80.  Pairs (8 queries on 200k edges 278, 259, 247 us),
 // anti-edges (109, 106, 104) and look-ahead (chorded 4-cycle on 100M edges 52, 49, 48 ms) likewise.
